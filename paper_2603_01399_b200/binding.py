@@ -118,7 +118,15 @@ def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else t.data_ptr()
 
 
+# The handle of the current stream of the current device.  torch.cuda.current_stream() builds a Stream object for it
+# (3.2 us a call on the measured host); the two calls below read the two numbers (0.3 us).
+_current_device = torch._C._cuda_getDevice if hasattr(torch._C, "_cuda_getDevice") else None
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream() -> int:
+    if _raw_stream is not None and _current_device is not None and torch.cuda.is_initialized():
+        return _raw_stream(_current_device())
     return torch.cuda.current_stream().cuda_stream
 
 
