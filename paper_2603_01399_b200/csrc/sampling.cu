@@ -40,14 +40,15 @@ SegPlan seg_plan(int V) {
 }
 
 // A row starts anywhere (V may be odd), so segments are cut on 16-byte boundaries: `lead` values (0..3) of the first
-// segment lie before the row.  Thread t holds positions 16 t .. 16 t + 15 of the segment.
+// segment lie before the row.
 __device__ __forceinline__ int row_lead(const float* row) { return (int)((reinterpret_cast<uintptr_t>(row) & 15u) >> 2); }
 
-template <typename F>
+// 16 values as four 128-bit loads `stride` positions apart
+template <int stride, typename F>
 __device__ __forceinline__ void load16(const float* row, int first, int V, float fill, F&& put) {
 #pragma unroll
   for (int j = 0; j < kPerThread / 4; ++j) {
-    const int v = first + 4 * j;
+    const int v = first + stride * j;
     if (v >= 0 && v + 4 <= V) {
       const float4 x = __ldg(reinterpret_cast<const float4*>(row + v));
       put(4 * j, x.x); put(4 * j + 1, x.y); put(4 * j + 2, x.z); put(4 * j + 3, x.w);
@@ -58,27 +59,21 @@ __device__ __forceinline__ void load16(const float* row, int first, int V, float
   }
 }
 
-__device__ __forceinline__ float block_max(float v, float* sh) {
+__device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  __syncthreads();
-  float r = sh[0];
-#pragma unroll
-  for (int i = 1; i < kSegThreads / 32; ++i) r = fmaxf(r, sh[i]);
-  __syncthreads();
-  return r;
+  return v;
 }
-__device__ __forceinline__ float block_sum(float v, float* sh) {
+__device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  __syncthreads();
-  float r = 0.f;
-#pragma unroll
-  for (int i = 0; i < kSegThreads / 32; ++i) r += sh[i];   // warps in order
-  __syncthreads();
-  return r;
+  return v;
+}
+// (maximum, sum of exponentials against it) of two parts put together
+__device__ __forceinline__ float2 join(float2 x, float2 y, float inv_t) {
+  const float m = fmaxf(x.x, y.x);
+  if (!(m > -INFINITY)) return make_float2(m, 0.f);
+  return make_float2(m, x.y * expf((x.x - m) * inv_t) + y.y * expf((y.x - m) * inv_t));
 }
 
 // part[(b * T_max + i) * nseg + s] = (maximum, sum of exp((x - maximum) / temperature)) of a segment; also clears the
@@ -86,30 +81,35 @@ __device__ __forceinline__ float block_sum(float v, float* sh) {
 __global__ void __launch_bounds__(kSegThreads)
 softmax_segment_kernel(const float* __restrict__ logits, const int32_t* __restrict__ block_len, int T_max, int V, int nseg,
                        int chunks, float inv_t, float2* __restrict__ part, unsigned* __restrict__ arrivals) {
-  __shared__ float sh[kSegThreads / 32];
+  __shared__ float2 sh[kSegThreads / 32];
   const int s = blockIdx.x, i = blockIdx.y, b = blockIdx.z;
   if (s == 0 && i == 0 && threadIdx.x == 0) arrivals[b] = 0;
   if (i >= block_len[b]) return;
   const float* row = logits + ((size_t)b * T_max + i) * V;
-  float m = -INFINITY, sum = 0.f;
+  float2 acc = make_float2(-INFINITY, 0.f);   // of this warp: one block-wide meeting per segment, not one per reduction
   for (int c = 0; c < chunks; ++c) {
-    const int first = (s * chunks + c) * kChunk + threadIdx.x * kPerThread - row_lead(row);
     float x[kPerThread];
-    load16(row, first, V, -INFINITY, [&](int j, float v) { x[j] = v; });
-    float cm = x[0];
+    load16<kChunk / 4>(row, (s * chunks + c) * kChunk + threadIdx.x * 4 - row_lead(row), V, -INFINITY, [&](int j, float v) { x[j] = v; });
+    float m = x[0];
 #pragma unroll
-    for (int j = 1; j < kPerThread; ++j) cm = fmaxf(cm, x[j]);
-    cm = fmaxf(block_max(cm, sh), m);
-    if (cm > -INFINITY) {
-      float cs = 0.f;
+    for (int j = 1; j < kPerThread; ++j) m = fmaxf(m, x[j]);
+    m = warp_max(m);
+    float sum = 0.f;
+    if (m > -INFINITY) {
 #pragma unroll
-      for (int j = 0; j < kPerThread; ++j) cs += expf((x[j] - cm) * inv_t);
-      cs = block_sum(cs, sh);
-      sum = c == 0 ? cs : sum * expf((m - cm) * inv_t) + cs;
-      m = cm;
+      for (int j = 0; j < kPerThread; ++j) sum += expf((x[j] - m) * inv_t);
     }
+    const float2 part_c = make_float2(m, warp_sum(sum));
+    acc = c == 0 ? part_c : join(acc, part_c, inv_t);
   }
-  if (threadIdx.x == 0) part[((size_t)b * T_max + i) * nseg + s] = make_float2(m, sum);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    acc = sh[0];
+#pragma unroll
+    for (int w = 1; w < kSegThreads / 32; ++w) acc = join(acc, sh[w], inv_t);   // warps in order
+    part[((size_t)b * T_max + i) * nseg + s] = acc;
+  }
 }
 
 struct DrawArgs {
@@ -138,9 +138,9 @@ struct Draw {   // what to draw from: a row, its softmax statistics, and what is
 // The weights of this thread's 16 positions of a chunk of the row.
 __device__ __forceinline__ void draw_weights(const Draw& d, int chunk, int V, float inv_t, int& first, float (&w)[kPerThread]) {
   first = chunk * kChunk + threadIdx.x * kPerThread - row_lead(d.row);
-  load16(d.row, first, V, -INFINITY, [&](int j, float v) { w[j] = expf((v - d.max) * inv_t) * d.inv_sum; });
+  load16<4>(d.row, first, V, -INFINITY, [&](int j, float v) { w[j] = expf((v - d.max) * inv_t) * d.inv_sum; });
   if (d.qrow != nullptr)
-    load16(d.qrow, first, V, 0.f, [&](int j, float v) { w[j] = fmaxf(0.f, w[j] - v); });   // Eq. 3
+    load16<4>(d.qrow, first, V, 0.f, [&](int j, float v) { w[j] = fmaxf(0.f, w[j] - v); });   // Eq. 3
 #pragma unroll
   for (int j = 0; j < kPerThread; ++j)
     if (first + j == d.tok) w[j] = 0.f;                                                   // point-mass drafter
@@ -148,46 +148,63 @@ __device__ __forceinline__ void draw_weights(const Draw& d, int chunk, int V, fl
 
 __global__ void __launch_bounds__(kSegThreads) draw_segment_kernel(DrawArgs a) {
   __shared__ float sh[kSegThreads / 32];
-  __shared__ float4 s_row[QUASAR_MAX_BLOCK];      // per block row: max, sum, p of the next block token, q of it
+  __shared__ float2 s_row[QUASAR_MAX_BLOCK];      // per block row: maximum and sum
+  __shared__ float s_logit[QUASAR_MAX_BLOCK], s_q[QUASAR_MAX_BLOCK], s_r[QUASAR_MAX_BLOCK];   // of the next block token
   __shared__ int s_n, s_rejected, s_last, s_pick, s_seg;
-  __shared__ float s_total, s_begin;
+  __shared__ float s_target, s_begin;
   const int s = blockIdx.x, b = blockIdx.y;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int T = min(a.block_len[b], a.T_max);
+  const float r_sample = a.r_sample[b];
 
-  // ---- row statistics: a warp per row, lanes over the segments ----
-  for (int i = warp; i < T; i += kSegThreads / 32) {
-    const float2* p = a.part + ((size_t)b * a.T_max + i) * a.nseg;
-    float m = -INFINITY;
-    for (int k = lane; k < a.nseg; k += 32) m = fmaxf(m, p[k].x);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    float sum = 0.f;
-    for (int k = lane; k < a.nseg; k += 32) sum += p[k].y * expf((p[k].x - m) * a.inv_t);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (lane == 0) {
-      float p_tok = 0.f, q_tok = 1.f;
-      if (i + 1 < T) {
-        const int tok = a.tokens[b * a.T_max + i + 1];
-        const size_t at = ((size_t)b * a.T_max + i) * a.V + tok;
-        if (tok >= 0 && tok < a.V) {
-          p_tok = expf((a.logits[at] - m) * a.inv_t) / sum;
-          if (a.q_probs != nullptr) q_tok = a.q_probs[at];
-        } else {
-          q_tok = 0.f;   // a token outside the vocabulary can only be rejected
-        }
+  // ---- row statistics: half a warp per row, its lanes over the segments; the last T threads fetch what the walk
+  //      compares them with ----
+  const int t_row = kSegThreads - 1 - (int)threadIdx.x;
+  if (t_row < T) {
+    float x = 0.f, q = 1.f, r = 0.f;
+    if (t_row + 1 < T) {
+      const int tok = a.tokens[b * a.T_max + t_row + 1];
+      const size_t at = ((size_t)b * a.T_max + t_row) * a.V + tok;
+      r = a.r_accept[b * a.T_max + t_row];
+      if (tok >= 0 && tok < a.V) {
+        x = a.logits[at];
+        if (a.q_probs != nullptr) q = a.q_probs[at];
+      } else {
+        q = 0.f;   // a token outside the vocabulary can only be rejected
       }
-      s_row[i] = make_float4(m, sum, p_tok, q_tok);
     }
+    s_logit[t_row] = x;
+    s_q[t_row] = q;
+    s_r[t_row] = r;
+  }
+  for (int i = threadIdx.x >> 4; i < (T + 1) / 2 * 2; i += kSegThreads / 16) {   // (both halves of a warp take every turn)
+    const float2* p = a.part + ((size_t)b * a.T_max + i) * a.nseg;
+    float2 v[kMaxSegments / 16];
+#pragma unroll
+    for (int k = 0; k < kMaxSegments / 16; ++k) {
+      const int at = (threadIdx.x & 15) + 16 * k;
+      v[k] = (i < T && at < a.nseg) ? p[at] : make_float2(-INFINITY, 0.f);
+    }
+    float m = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < kMaxSegments / 16; ++k) m = fmaxf(m, v[k].x);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    float sum = 0.f;
+#pragma unroll
+    for (int k = 0; k < kMaxSegments / 16; ++k)
+      if (v[k].y > 0.f) sum += v[k].y * expf((v[k].x - m) * a.inv_t);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (i < T && (threadIdx.x & 15) == 0) s_row[i] = make_float2(m, sum);
   }
   __syncthreads();
   if (threadIdx.x == 0) {   // Eq. 2 along the chain
     int n = 0, rejected = 0;
     for (int i = 0; i + 1 < T; ++i) {
-      const float p_tok = s_row[i].z, q_tok = s_row[i].w;
+      const float p_tok = expf((s_logit[i] - s_row[i].x) * a.inv_t) / s_row[i].y, q_tok = s_q[i];
       const float ratio = q_tok > 0.f ? fminf(1.f, p_tok / q_tok) : 0.f;
-      if (!(q_tok > 0.f) || !(a.r_accept[b * a.T_max + i] < ratio)) { rejected = 1; break; }
+      if (!(q_tok > 0.f) || !(s_r[i] < ratio)) { rejected = 1; break; }
       ++n;
     }
     s_n = n;
@@ -213,7 +230,12 @@ __global__ void __launch_bounds__(kSegThreads) draw_segment_kernel(DrawArgs a) {
     float local = 0.f;
 #pragma unroll
     for (int j = 0; j < kPerThread; ++j) local += w[j];
-    seg += block_sum(local, sh);
+    local = warp_sum(local);
+    if (lane == 0) sh[warp] = local;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kSegThreads / 32; ++k) seg += sh[k];   // warps in order
+    if (c + 1 < a.chunks) __syncthreads();
   }
   if (threadIdx.x == 0) {
     __stcg(a.seg_sum + (size_t)b * a.nseg + s, seg);
@@ -229,68 +251,57 @@ __global__ void __launch_bounds__(kSegThreads) draw_segment_kernel(DrawArgs a) {
   for (int attempt = 0; attempt < 2; ++attempt) {
     if (warp == 0) {
       // the segments' intervals [begin, end) tile [0, total): 32 at a time, an end is the next one's begin
-      float carry = 0.f;
-      for (int k0 = 0; k0 < a.nseg; k0 += 32) {
-        float v = 0.f;
-        if (k0 + lane < a.nseg) {
+      float own[kMaxSegments / 32], incl[kMaxSegments / 32];
+#pragma unroll
+      for (int k = 0; k < kMaxSegments / 32; ++k) {
+        const int at = lane + 32 * k;
+        own[k] = 0.f;
+        if (at < a.nseg) {
           if (attempt == 0) {
-            v = __ldcg(a.seg_sum + (size_t)b * a.nseg + k0 + lane);
+            own[k] = __ldcg(a.seg_sum + (size_t)b * a.nseg + at);
           } else {   // p itself: its segment sums are known from the statistics
-            const float2 p = a.part[((size_t)b * a.T_max + i) * a.nseg + k0 + lane];
-            v = p.y * expf((p.x - d.max) * a.inv_t) * d.inv_sum;
+            const float2 p = a.part[((size_t)b * a.T_max + i) * a.nseg + at];
+            own[k] = p.y > 0.f ? p.y * expf((p.x - d.max) * a.inv_t) * d.inv_sum : 0.f;
           }
         }
+        incl[k] = own[k];
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-          const float up = __shfl_up_sync(0xffffffffu, v, o);
-          if (lane >= o) v += up;
+          const float up = __shfl_up_sync(0xffffffffu, incl[k], o);
+          if (lane >= o) incl[k] += up;
         }
-        carry += __shfl_sync(0xffffffffu, v, 31);
       }
-      const float total = carry;
-      const float target = a.r_sample[b] * total;
-      int found = -1, last = -1;
-      float begin_found = 0.f;
-      carry = 0.f;
-      for (int k0 = 0; k0 < a.nseg && found < 0; k0 += 32) {
-        float v = 0.f;
-        if (k0 + lane < a.nseg) {
-          if (attempt == 0) {
-            v = __ldcg(a.seg_sum + (size_t)b * a.nseg + k0 + lane);
-          } else {
-            const float2 p = a.part[((size_t)b * a.T_max + i) * a.nseg + k0 + lane];
-            v = p.y * expf((p.x - d.max) * a.inv_t) * d.inv_sum;
-          }
-        }
-        const float own = v;
+      float total = 0.f;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const float up = __shfl_up_sync(0xffffffffu, v, o);
-          if (lane >= o) v += up;
-        }
-        float excl = __shfl_up_sync(0xffffffffu, v, 1);
+      for (int k = 0; k < kMaxSegments / 32; ++k) total += __shfl_sync(0xffffffffu, incl[k], 31);
+      const float target = r_sample * total;
+      int found = -1, last = -1;
+      float begin_found = 0.f, carry = 0.f;
+#pragma unroll
+      for (int k = 0; k < kMaxSegments / 32; ++k) {
+        float excl = __shfl_up_sync(0xffffffffu, incl[k], 1);
         if (lane == 0) excl = 0.f;
-        const unsigned hit = __ballot_sync(0xffffffffu, own > 0.f && carry + excl <= target && target < carry + v);
-        const unsigned pos = __ballot_sync(0xffffffffu, own > 0.f);
-        if (pos) last = k0 + 31 - __clz(pos);
-        if (hit) {
+        const unsigned hit = __ballot_sync(0xffffffffu, own[k] > 0.f && carry + excl <= target && target < carry + incl[k]);
+        const unsigned pos = __ballot_sync(0xffffffffu, own[k] > 0.f);
+        if (pos) last = 32 * k + 31 - __clz(pos);
+        if (hit && found < 0) {
           const int l = __ffs(hit) - 1;
-          found = k0 + l;
+          found = 32 * k + l;
           begin_found = __shfl_sync(0xffffffffu, carry + excl, l);
         }
-        carry += __shfl_sync(0xffffffffu, v, 31);
+        carry += __shfl_sync(0xffffffffu, incl[k], 31);
       }
       if (lane == 0) {
-        s_total = total;
-        s_seg = found >= 0 ? found : last;
+        s_seg = total > 0.f ? (found >= 0 ? found : last) : -1;
         // r_sample * total rounded up to the total: no interval holds it, the last positive token is taken
-        s_begin = found >= 0 ? begin_found : -INFINITY;
+        s_begin = found >= 0 ? begin_found : 0.f;
+        s_target = found >= 0 ? target : INFINITY;
       }
     }
     __syncthreads();
-    if (s_total > 0.f && s_seg >= 0) {
-      const float target = s_begin > -INFINITY ? a.r_sample[b] * s_total : INFINITY;
-      float base = s_begin > -INFINITY ? s_begin : 0.f;
+    if (s_seg >= 0) {
+      const float target = s_target;
+      float base = s_begin;
       int last_pos = -1;
       for (int c = 0; c < a.chunks; ++c) {
         draw_weights(d, s_seg * a.chunks + c, a.V, a.inv_t, first, w);
