@@ -12,6 +12,7 @@
 
 #include "common.cuh"
 #include "megakernel.cuh"
+#include "tc_linear.cuh"
 
 namespace quasar {
 
@@ -68,8 +69,8 @@ size_t align_up(size_t v, size_t a = 256) { return (v + a - 1) / a * a; }
 
 // Layout of the verify workspace; every offset is a multiple of 256 bytes.
 struct Workspace {
-  size_t x, h, qkv, attn, gu, act, attn16, act16, h16, inv3, keys, logits, top1, anc, depth, valid, lin, att, cand, ss_part, amax, attn_count, barrier, total;
-  size_t lin_bytes, att_bytes;
+  size_t x, h, qkv, attn, gu, act, attn16, act16, op, op_scale, keys, top1, anc, depth, valid, att, cand, ss_part, amax, attn_count, barrier, total;
+  size_t att_bytes;
 };
 
 constexpr int kMaxGrid = 1024;  // upper bound on CTAs of the persistent kernel (SM count)
@@ -88,30 +89,15 @@ Workspace layout(const quasar_config& c, int B, int T_max, int s_max) {
   w.act = take(M * (size_t)c.ffn * 2);
   w.attn16 = take(M * (size_t)c.n_q_heads * c.head_dim * 2);
   w.act16 = take(M * (size_t)c.ffn * 2);
-  w.h16 = take(M * (size_t)c.hidden * 2);
-  w.inv3 = take(3 * align_up(M * 4));
+  // the operand of the linear layer in hand: three digit rows per block row at most
+  const size_t widest = std::max(std::max((size_t)c.hidden, (size_t)c.n_q_heads * c.head_dim), (size_t)c.ffn);
+  w.op = take(3 * M * widest);
+  w.op_scale = take(M * 4);
   w.keys = take(M * 8);
-  w.logits = take(M * (size_t)c.vocab * 4);
   w.top1 = take(M * 4);
   w.anc = take(M * 8);
   w.depth = take(M * 4);
   w.valid = take((size_t)B * 4);
-  size_t lin = 0;
-  const int64_t shapes[5][2] = {{(int64_t)qkv_w, c.hidden},
-                                {c.hidden, (int64_t)c.n_q_heads * c.head_dim},
-                                {2 * (int64_t)c.ffn, c.hidden},
-                                {c.hidden, c.ffn},
-                                {c.vocab, c.hidden}};
-  for (auto& s : shapes) {
-    size_t b = linear_workspace_bytes((int64_t)M, s[0], s[1]);
-    if (c.act_dtype == QUASAR_A_INT8) {
-      const size_t b8 = linear_w8a8_workspace_bytes((int64_t)M, s[0], s[1]);
-      b = b8 > b ? b8 : b;
-    }
-    lin = b > lin ? b : lin;
-  }
-  w.lin_bytes = lin;
-  w.lin = take(lin);
   w.att_bytes = attention_workspace_bytes(B, T_max, c.n_q_heads, c.n_kv_heads, c.head_dim, s_max);
   {
     const size_t rows = (size_t)B * c.n_kv_heads * mega_attn_nchunk(s_max) * mega_attn_rpad(T_max, c.n_q_heads, c.n_kv_heads);
@@ -237,13 +223,11 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
   __nv_bfloat16* attn = reinterpret_cast<__nv_bfloat16*>(wsp + ws.attn);
   __nv_bfloat16* gu = reinterpret_cast<__nv_bfloat16*>(wsp + ws.gu);
   __nv_bfloat16* act = reinterpret_cast<__nv_bfloat16*>(wsp + ws.act);
-  float* logits = logits_out ? logits_out : reinterpret_cast<float*>(wsp + ws.logits);
   int32_t* top1 = reinterpret_cast<int32_t*>(wsp + ws.top1);
   BlockInfo bi;
   bi.anc = reinterpret_cast<uint64_t*>(wsp + ws.anc);
   bi.depth = reinterpret_cast<int32_t*>(wsp + ws.depth);
   bi.valid = reinterpret_cast<int32_t*>(wsp + ws.valid);
-  void* lin = wsp + ws.lin;
   void* att = wsp + ws.att;
 
   const int M = B * T_max;
@@ -251,14 +235,6 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
   const int qkv_w = (Hq + 2 * Hkv) * D;
   const int wd = c.weight_dtype;
   const bool a8 = c.act_dtype == QUASAR_A_INT8;
-  // one linear layer of the pass: weight-only (Eq. 8 with bf16 activations) or the paper's W8A8 form (Eq. 9-10)
-  auto linear = [&](const __nv_bfloat16* in, const void* w, const float* delta, const float* smooth, int64_t N, int64_t K,
-                    void* out, bool out_f32, const __nv_bfloat16* res) -> int {
-    if (a8)
-      return launch_linear_w8a8(in, smooth, reinterpret_cast<const int8_t*>(w), delta, M, N, K, out, out_f32, res, nullptr,
-                                lin, ws.lin_bytes, status, stream);
-    return launch_linear(in, w, delta, wd, M, N, K, out, out_f32, res, lin, ws.lin_bytes, stream, status);
-  };
   const size_t layer_stride = (size_t)kv->batch * Hkv * (size_t)kv->s_max * D;
   TraceCursor tr{reinterpret_cast<unsigned char*>(m->trace_buf), 0, m->trace_bytes, stream};
 
@@ -297,92 +273,41 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
     return launch_verify_mega(p, wd, D, m->mega_ncta, stream);
   }
 
-  // arrival counters of the split-K reduction start at zero and reset themselves
-  QUASAR_CUDA_CHECK(cudaMemsetAsync(lin, 0, ws.lin_bytes < 65536 ? ws.lin_bytes : 65536, stream));
-  TRY(launch_block_prep(tokens, parents, block_len, kv->seq_len, B, T_max, kv->s_max, c.vocab, bi, status, stream));
-  TRY(launch_embed(tokens, reinterpret_cast<const __nv_bfloat16*>(m->w.embed), M, H, c.vocab, x, stream));
-  TRY(tr.put(x, (size_t)M * H * 2));
-
-  // Blocks of 9..80 rows with int8 weights and 16-bit activations: every linear layer is the tcgen05 kernel, which
-  // wants its operand as fp16 rows times a power of two.  The kernel that produces an operand writes that form too, and
-  // the kernel after a residual linear layer adds up its k-ranges, so a layer is 12 launches instead of 17.
-  bool fused = !a8 && wd == QUASAR_W_INT8 && M > 8 && M <= 80 && H <= 8192 && F <= 24576;   // (rows the fused row kernels hold in registers)
-  {
-    const int64_t shapes[5][2] = {{qkv_w, H}, {H, (int64_t)Hq * D}, {2 * (int64_t)F, H}, {H, F}, {c.vocab, H}};
-    for (auto& sh : shapes) fused = fused && umma_w8a16_usable(M, sh[0], sh[1]);
-  }
-  if (fused) {
-    void* h16 = wsp + ws.h16;
-    void* attn16 = wsp + ws.attn16;
-    void* act16 = wsp + ws.act16;
-    float* inv_h = reinterpret_cast<float*>(wsp + ws.inv3);
-    float* inv_a = reinterpret_cast<float*>(wsp + ws.inv3 + align_up((size_t)M * 4));
-    float* inv_f = reinterpret_cast<float*>(wsp + ws.inv3 + 2 * align_up((size_t)M * 4));
-    float* partial = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(lin) + 65536);
-    auto norm_of = [&](int l) {
-      return reinterpret_cast<const __nv_bfloat16*>(l < c.n_layers ? m->layers[l].attn_norm : m->w.final_norm);
-    };
-    TRY(launch_rmsnorm_f16(x, norm_of(0), M, H, c.rms_eps, h, h16, inv_h, stream));
-    for (int l = 0; l < c.n_layers; ++l) {
-      const quasar_layer_weights& L = m->layers[l];
-      __nv_bfloat16* kc = reinterpret_cast<__nv_bfloat16*>(kv->k) + (size_t)l * layer_stride;
-      __nv_bfloat16* vc = reinterpret_cast<__nv_bfloat16*>(kv->v) + (size_t)l * layer_stride;
-      int ns = 1, mpad = 16;
-      TRY(tr.put(h, (size_t)M * H * 2));
-      TRY(launch_umma_w8a16_prepared(h16, inv_h, reinterpret_cast<const int8_t*>(L.qkv_w), L.qkv_delta, M, qkv_w, H, qkv, false,
-                                     nullptr, partial, true, status, stream));
-      TRY(tr.put(qkv, (size_t)M * qkv_w * 2));
-      TRY(launch_rope_append(qkv, reinterpret_cast<const __nv_bfloat16*>(c.qk_norm ? L.q_norm : nullptr),
-                             reinterpret_cast<const __nv_bfloat16*>(c.qk_norm ? L.k_norm : nullptr), m->rope_table,
-                             kv->seq_len, block_len, bi, B, T_max, Hq, Hkv, D, c.rms_eps, kc, vc, kv->s_max, stream));
-      TRY(tr.put(qkv, (size_t)M * qkv_w * 2));
-      TRY(launch_attention(qkv, kc, vc, kv->seq_len, block_len, bi, B, T_max, Hq, Hkv, D, kv->s_max, attn, att,
-                           ws.att_bytes, stream));
-      TRY(tr.put(attn, (size_t)M * Hq * D * 2));
-      TRY(launch_f16_rows(attn, M, (int64_t)Hq * D, attn16, inv_a, stream));
-      TRY(launch_umma_w8a16_prepared(attn16, inv_a, reinterpret_cast<const int8_t*>(L.o_w), L.o_delta, M, H, (int64_t)Hq * D, x,
-                                     false, x, partial, false, status, stream));
-      umma_w8a16_plan(M, H, (int64_t)Hq * D, &ns, &mpad);
-      TRY(launch_reduce_residual_rmsnorm_f16(partial, ns, mpad, inv_a, L.o_delta, x,
-                                             reinterpret_cast<const __nv_bfloat16*>(L.mlp_norm), M, H, c.rms_eps, h, h16, inv_h,
-                                             stream));
-      TRY(tr.put(x, (size_t)M * H * 2));
-      TRY(launch_umma_w8a16_prepared(h16, inv_h, reinterpret_cast<const int8_t*>(L.gateup_w), L.gateup_delta, M, 2 * (int64_t)F, H,
-                                     gu, false, nullptr, partial, true, status, stream));
-      TRY(launch_swiglu_f16(gu, M, F, act, act16, inv_f, stream));
-      TRY(tr.put(act, (size_t)M * F * 2));
-      TRY(launch_umma_w8a16_prepared(act16, inv_f, reinterpret_cast<const int8_t*>(L.down_w), L.down_delta, M, H, F, x, false, x,
-                                     partial, false, status, stream));
-      umma_w8a16_plan(M, H, F, &ns, &mpad);
-      TRY(launch_reduce_residual_rmsnorm_f16(partial, ns, mpad, inv_f, L.down_delta, x, norm_of(l + 1), M, H, c.rms_eps, h, h16,
-                                             inv_h, stream));
-      TRY(tr.put(x, (size_t)M * H * 2));
-    }
-    TRY(tr.put(h, (size_t)M * H * 2));
-    TRY(launch_umma_w8a16_prepared(h16, inv_h, reinterpret_cast<const int8_t*>(m->w.lm_w), m->w.lm_delta, M, c.vocab, H, logits,
-                                   true, nullptr, partial, true, status, stream));
-    TRY(launch_argmax(logits, M, c.vocab, top1, reinterpret_cast<unsigned long long*>(wsp + ws.keys), stream));
-    TRY(launch_accept(tokens, parents, block_len, top1, bi, B, T_max, accept_len, bonus, accept_path, stream));
-    return QUASAR_OK;
-  }
-
-  // W8A8: the norm and SwiGLU kernels smooth and quantise their output rows themselves (Eq. 9), straight into the place
-  // where the linear layer that follows keeps its quantised operand; that layer is then called without an input.
-  const bool a8_fuse = a8 && M <= kMaxRowsPerGemm && H <= 8192 && F <= 24576;
-  auto norm = [&](const __nv_bfloat16* in, const void* gain, const float* smooth) -> int {
-    if (!a8_fuse) return launch_rmsnorm(in, reinterpret_cast<const __nv_bfloat16*>(gain), M, H, c.rms_eps, h, stream);
-    int8_t* xq = nullptr;
-    float* dxp = nullptr;
-    linear_w8a8_operand_slots(lin, M, H, &xq, &dxp);
-    return launch_rmsnorm_q8(in, reinterpret_cast<const __nv_bfloat16*>(gain), smooth, M, H, c.rms_eps, h, xq, dxp, stream);
+  // ---- one kernel per step.  Every kernel but the first is a dependent launch: it starts under the one in front of it (the
+  //      linear layers ask for their first weights then) and waits by itself for what that one writes. ----
+  const OperandForm form = a8 ? kOperandCodes : wd == QUASAR_W_INT8 ? kOperandDigits : kOperandBf16;
+  const bool traced = m->trace_buf != nullptr;
+  BlockArgs ba{tokens, parents, block_len, kv->seq_len, B, T_max, kv->s_max, c.vocab, bi,
+               reinterpret_cast<unsigned long long*>(wsp + ws.keys), status};
+  int8_t* op_q = reinterpret_cast<int8_t*>(wsp + ws.op);
+  float* op_scale = reinterpret_cast<float*>(wsp + ws.op_scale);
+  // (the bf16 rows themselves are needed where they are the operand, and for a trace)
+  auto operand = [&](__nv_bfloat16* y, const float* smooth) {
+    return RowOperand{form == kOperandBf16 || traced ? y : nullptr, op_q, op_scale, smooth};
   };
+  // one linear layer of the pass on the operand its producer left: weight-only (Eq. 8) or the paper's W8A8 form (Eq. 9-10)
+  auto linear = [&](const __nv_bfloat16* in, const void* w, const float* delta, int64_t N, int64_t K, void* out, bool out_f32,
+                    const __nv_bfloat16* res, unsigned long long* keys) -> int {
+    if (form == kOperandBf16)
+      return launch_tc_linear_bf16(in, reinterpret_cast<const __nv_bfloat16*>(w), M, N, K, out, out_f32, res, keys, status, true, stream);
+    const int8_t* wq = reinterpret_cast<const int8_t*>(w);
+    if (form == kOperandCodes)
+      return launch_tc_linear_w8a8(op_q, op_scale, wq, delta, M, N, K, out, out_f32, res, nullptr, keys, status, true, stream);
+    return launch_tc_linear_digits(op_q, op_scale, wq, delta, M, N, K, out, out_f32, res, keys, status, true, stream);
+  };
+  auto norm_gain = [&](int l) {
+    return reinterpret_cast<const __nv_bfloat16*>(l < c.n_layers ? m->layers[l].attn_norm : m->w.final_norm);
+  };
+  auto norm_smooth = [&](int l) { return l < c.n_layers ? m->layers[l].qkv_smooth : m->w.lm_smooth; };
+  TRY(launch_embed_norm(form, ba, reinterpret_cast<const __nv_bfloat16*>(m->w.embed), x, norm_gain(0), H, c.rms_eps,
+                        operand(h, norm_smooth(0)), stream));
+  TRY(tr.put(x, (size_t)M * H * 2));
   for (int l = 0; l < c.n_layers; ++l) {
     const quasar_layer_weights& L = m->layers[l];
     __nv_bfloat16* kc = reinterpret_cast<__nv_bfloat16*>(kv->k) + (size_t)l * layer_stride;
     __nv_bfloat16* vc = reinterpret_cast<__nv_bfloat16*>(kv->v) + (size_t)l * layer_stride;
-    TRY(norm(x, L.attn_norm, L.qkv_smooth));
     TRY(tr.put(h, (size_t)M * H * 2));
-    TRY(linear(a8_fuse ? nullptr : h, L.qkv_w, L.qkv_delta, L.qkv_smooth, qkv_w, H, qkv, false, nullptr));
+    TRY(linear(h, L.qkv_w, L.qkv_delta, qkv_w, H, qkv, false, nullptr, nullptr));
     TRY(tr.put(qkv, (size_t)M * qkv_w * 2));
     TRY(launch_rope_append(qkv, reinterpret_cast<const __nv_bfloat16*>(c.qk_norm ? L.q_norm : nullptr),
                            reinterpret_cast<const __nv_bfloat16*>(c.qk_norm ? L.k_norm : nullptr), m->rope_table,
@@ -391,28 +316,21 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
     TRY(launch_attention(qkv, kc, vc, kv->seq_len, block_len, bi, B, T_max, Hq, Hkv, D, kv->s_max, attn, att,
                          ws.att_bytes, stream));
     TRY(tr.put(attn, (size_t)M * Hq * D * 2));
-    TRY(linear(attn, L.o_w, L.o_delta, L.o_smooth, H, Hq * D, x, false, x));
+    TRY(launch_operand(form, attn, M, Hq * D, RowOperand{nullptr, op_q, op_scale, L.o_smooth}, stream));
+    TRY(linear(attn, L.o_w, L.o_delta, H, Hq * D, x, false, x, nullptr));
     TRY(tr.put(x, (size_t)M * H * 2));
-    TRY(norm(x, L.mlp_norm, L.gateup_smooth));
-    TRY(linear(a8_fuse ? nullptr : h, L.gateup_w, L.gateup_delta, L.gateup_smooth, 2 * F, H, gu, false, nullptr));
-    if (a8_fuse) {
-      int8_t* xq = nullptr;
-      float* dxp = nullptr;
-      linear_w8a8_operand_slots(lin, M, F, &xq, &dxp);
-      TRY(launch_swiglu_q8(gu, L.down_smooth, M, F, act, xq, dxp, stream));
-    } else {
-      TRY(launch_swiglu(gu, M, F, act, stream));
-    }
+    TRY(launch_norm(form, x, reinterpret_cast<const __nv_bfloat16*>(L.mlp_norm), M, H, c.rms_eps, operand(h, L.gateup_smooth), stream));
+    TRY(linear(h, L.gateup_w, L.gateup_delta, 2 * (int64_t)F, H, gu, false, nullptr, nullptr));
+    TRY(launch_swiglu(form, gu, M, F, operand(act, L.down_smooth), stream));
     TRY(tr.put(act, (size_t)M * F * 2));
-    TRY(linear(a8_fuse ? nullptr : act, L.down_w, L.down_delta, L.down_smooth, H, F, x, false, x));
+    TRY(linear(act, L.down_w, L.down_delta, H, F, x, false, x, nullptr));
     TRY(tr.put(x, (size_t)M * H * 2));
+    TRY(launch_norm(form, x, norm_gain(l + 1), M, H, c.rms_eps, operand(h, norm_smooth(l + 1)), stream));
   }
-  TRY(norm(x, m->w.final_norm, m->w.lm_smooth));
   TRY(tr.put(h, (size_t)M * H * 2));
-  TRY(linear(a8_fuse ? nullptr : h, m->w.lm_w, m->w.lm_delta, m->w.lm_smooth, c.vocab, H, logits, true, nullptr));
-  TRY(launch_argmax(logits, M, c.vocab, top1, reinterpret_cast<unsigned long long*>(wsp + ws.keys), stream));
-  TRY(launch_accept(tokens, parents, block_len, top1, bi, B, T_max, accept_len, bonus, accept_path, stream));
-  return QUASAR_OK;
+  // (the LM head finds the rows' top choices as it goes and writes logits only for a caller who wants them)
+  TRY(linear(h, m->w.lm_w, m->w.lm_delta, c.vocab, H, logits_out, true, nullptr, ba.keys));
+  return launch_accept(ba, accept_len, bonus, accept_path, stream);
 }
 
 int plan_replay(quasar_plan* p, cudaStream_t stream) {

@@ -18,6 +18,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "tc_common.cuh"
 
 namespace quasar {
 
@@ -89,6 +90,8 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 4) verify_attention_kernel(Att
 
   const int c = blockIdx.x / a.ngroups, group = blockIdx.x % a.ngroups;
   const int hk = blockIdx.y, b = blockIdx.z;
+  tc::pdl_trigger();
+  tc::pdl_wait();
   if (!a.bi.valid[b]) return;
   const int T = a.block_len[b];
   const int P = a.seq_len[b];
@@ -285,6 +288,8 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 4) verify_attention_kernel(Att
 // One warp per (sequence, block row, query head): merge the chunk partials in chunk order.
 template <int D>
 __global__ void __launch_bounds__(128) attention_merge_kernel(AttnArgs a) {
+  tc::pdl_trigger();
+  tc::pdl_wait();
   const int item = blockIdx.x * 4 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (item >= a.B * a.T_max * a.Hq) return;
@@ -402,21 +407,18 @@ int launch_attention(const __nv_bfloat16* qkv, const __nv_bfloat16* k_cache_laye
       QUASAR_CUDA_CHECK(cudaFuncSetAttribute(verify_attention_kernel<128>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
       configured128 = true;
     }
-    verify_attention_kernel<128><<<grid, p.warps * 32, smem128, stream>>>(a);
-    QUASAR_LAUNCH_CHECK();
-    attention_merge_kernel<128><<<(items + 3) / 4, 128, 0, stream>>>(a);
-    QUASAR_LAUNCH_CHECK();
+    const int rc = launch_dependent(verify_attention_kernel<128>, grid, dim3(p.warps * 32), smem128, true, stream, a);
+    if (rc != QUASAR_OK) return rc;
+    return launch_dependent(attention_merge_kernel<128>, dim3((items + 3) / 4), dim3(128), 0, true, stream, a);
   } else if (D == 64) {
     constexpr size_t smem64 = 4u * kKeyTile * (64 + 8) * sizeof(__nv_bfloat16);
-    verify_attention_kernel<64><<<grid, p.warps * 32, smem64, stream>>>(a);
-    QUASAR_LAUNCH_CHECK();
-    attention_merge_kernel<64><<<(items + 3) / 4, 128, 0, stream>>>(a);
-    QUASAR_LAUNCH_CHECK();
+    const int rc = launch_dependent(verify_attention_kernel<64>, grid, dim3(p.warps * 32), smem64, true, stream, a);
+    if (rc != QUASAR_OK) return rc;
+    return launch_dependent(attention_merge_kernel<64>, dim3((items + 3) / 4), dim3(128), 0, true, stream, a);
   } else {
     set_error("head_dim %d not supported (64 or 128)", D);
     return QUASAR_ERR_SHAPE;
   }
-  return QUASAR_OK;
 }
 
 }  // namespace quasar

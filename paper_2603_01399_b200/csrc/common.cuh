@@ -34,17 +34,23 @@ void count_launch(int n = 1);
 static inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 #ifdef __CUDACC__
-// The fp16 form of an activation row for the tcgen05 weight-only GEMM: the row times the power of two that puts
-// its largest magnitude in [2^14, 2^15), and the inverse of that power (exact both ways).
-__device__ __forceinline__ void f16_row_scale(float amax, float& scale, float& inv) {
-  scale = 1.f;
-  inv = 1.f;
-  if (amax > 0.f && amax < 3.0e38f) {
-    int e;
-    (void)frexpf(amax, &e);            // amax = f * 2^e, f in [0.5, 1)
-    scale = ldexpf(1.f, 15 - e);
-    inv = ldexpf(1.f, e - 15);
-  }
+// Launches a kernel that waits for the one in front of it on the stream by itself (griddepcontrol.wait); `pdl`: it may start
+// before that one has finished.
+template <typename... P, typename... A>
+int launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, bool pdl, cudaStream_t stream, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
+  count_launch();
+  return QUASAR_OK;
 }
 #endif
 
@@ -72,36 +78,9 @@ int launch_smoothing_factors(const float* act_absmax, const __nv_bfloat16* w, in
 int launch_quantize_smoothed(const __nv_bfloat16* v, const float* s, int mode, int64_t rows, int64_t K, int8_t* q,
                              float* delta, cudaStream_t stream);
 size_t linear_w8a8_workspace_bytes(int64_t M, int64_t N, int64_t K);
-void linear_w8a8_operand_slots(void* workspace, int64_t M, int64_t K, int8_t** xq, float** dx);
 int launch_linear_w8a8(const __nv_bfloat16* x, const float* smooth, const int8_t* w, const float* delta_w, int64_t M,
                        int64_t N, int64_t K, void* y, bool y_is_f32, const __nv_bfloat16* residual, int32_t* acc_out,
                        void* workspace, size_t workspace_bytes, int32_t* status, cudaStream_t stream);
-
-// tcgen05 form of the W8A8 linear layer for blocks of 9..80 rows (umma_gemm.cu)
-bool umma_w8a8_usable(int64_t M, int64_t N, int64_t K);
-size_t umma_w8a8_partial_bytes(int64_t M, int64_t N, int64_t K);
-int launch_umma_w8a8(const int8_t* xq, const float* dx, const int8_t* w, const float* dw, int64_t M, int64_t N, int64_t K,
-                     void* y, bool y_is_f32, const __nv_bfloat16* residual, int32_t* acc_out, int* counters, void* partial,
-                     int32_t* error_word, cudaStream_t stream);
-
-bool umma_w8a16_usable(int64_t M, int64_t N, int64_t K);
-size_t umma_w8a16_scratch_bytes(int64_t M, int64_t N, int64_t K);
-int launch_umma_w8a16(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t N, int64_t K, void* y,
-                      bool y_is_f32, const __nv_bfloat16* residual, void* scratch, int32_t* error_word, cudaStream_t stream);
-// the same in pieces, for a pass that lets the producer of the activations write their fp16 form and the consumer of
-// the result add up the k-ranges (api.cu)
-void umma_w8a16_plan(int64_t M, int64_t N, int64_t K, int* nsplit, int* mpad);
-size_t umma_w8a16_partial_bytes(int64_t M, int64_t N, int64_t K);
-int launch_f16_rows(const __nv_bfloat16* x, int64_t M, int64_t K, void* x16, float* inv_scale, cudaStream_t stream);
-int launch_umma_w8a16_prepared(const void* x16, const float* inv, const int8_t* w, const float* dw, int64_t M, int64_t N,
-                               int64_t K, void* y, bool y_is_f32, const __nv_bfloat16* residual, void* partial, bool finalize,
-                               int32_t* error_word, cudaStream_t stream);
-
-// the weight-only linear layer for at most 8 rows as an exact integer contraction on tcgen05 (umma_gemm.cu)
-bool umma_rows8_usable(int64_t M, int64_t N, int64_t K);
-size_t umma_rows8_scratch_bytes(int64_t M, int64_t N, int64_t K);
-int launch_umma_rows8(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t N, int64_t K, void* y,
-                      bool y_is_f32, const __nv_bfloat16* residual, void* scratch, int32_t* error_word, cudaStream_t stream);
 
 // stochastic acceptance of a chain (Section 3.1 Eq. 2-3)
 size_t accept_stochastic_workspace_bytes(int B, int T_max);
@@ -127,14 +106,29 @@ struct BlockInfo {
   int32_t* valid;   // [B] 1 if the sequence is processed (block fits, parents well formed)
 };
 
-int launch_block_prep(const int32_t* tokens, const int32_t* parents, const int32_t* block_len, const int32_t* seq_len,
-                      int B, int T_max, int s_max, int vocab, BlockInfo bi, int32_t* status, cudaStream_t stream);
+// What the kernels at either end of the pass need to know about the draft blocks.
+struct BlockArgs {
+  const int32_t *tokens, *parents, *block_len, *seq_len;
+  int B, T_max, s_max, vocab;
+  BlockInfo bi;
+  unsigned long long* keys;   // [B*T_max] arg-max keys of the rows, cleared by the first kernel, or nullptr
+  int32_t* status;
+};
 
-int launch_embed(const int32_t* tokens, const __nv_bfloat16* embed, int M, int H, int vocab, __nv_bfloat16* x,
-                 cudaStream_t stream);
-
-int launch_rmsnorm(const __nv_bfloat16* x, const __nv_bfloat16* g, int M, int H, float eps, __nv_bfloat16* y,
-                   cudaStream_t stream);
+// ---- whole-row steps that leave the operand of the following linear layer (row_ops.cu) ----
+enum OperandForm { kOperandBf16 = 0, kOperandDigits = 1, kOperandCodes = 2 };
+struct RowOperand {
+  __nv_bfloat16* y;      // the rows as bf16 as well, or nullptr
+  int8_t* q;             // digits [3 M][width] or codes [M][width]
+  float* scale;          // [M]
+  const float* smooth;   // codes: smoothing factors of the linear layer's input, or nullptr
+};
+int launch_embed_norm(int op, const BlockArgs& a, const __nv_bfloat16* embed, __nv_bfloat16* x, const __nv_bfloat16* g, int H, float eps,
+                      const RowOperand& out, cudaStream_t stream);
+int launch_norm(int op, const __nv_bfloat16* x, const __nv_bfloat16* g, int M, int H, float eps, const RowOperand& out, cudaStream_t stream);
+int launch_swiglu(int op, const __nv_bfloat16* gu, int M, int F, const RowOperand& out, cudaStream_t stream);
+int launch_operand(int op, const __nv_bfloat16* x, int M, int K, const RowOperand& out, cudaStream_t stream);
+int launch_accept(const BlockArgs& a, int32_t* accept_len, int32_t* bonus, int32_t* accept_path, cudaStream_t stream);
 
 // QK-RMSNorm + RoPE on the q and k heads of qkv (in place) and K/V append at slot seq_len[b] + row.
 int launch_rope_append(__nv_bfloat16* qkv, const __nv_bfloat16* q_norm, const __nv_bfloat16* k_norm,
@@ -147,31 +141,6 @@ int launch_attention(const __nv_bfloat16* qkv, const __nv_bfloat16* k_cache_laye
                      const int32_t* seq_len, const int32_t* block_len, BlockInfo bi, int B, int T_max, int Hq, int Hkv,
                      int D, int s_max, __nv_bfloat16* out, void* workspace, size_t workspace_bytes,
                      cudaStream_t stream);
-
-int launch_swiglu(const __nv_bfloat16* gu, int M, int F, __nv_bfloat16* act, cudaStream_t stream);
-
-// Fused forms for the pass whose linear layers take a prepared fp16 operand (umma_gemm.cu): each also writes the
-// fp16 form of its output rows (x16 [M][width] + inv [M]).
-int launch_rmsnorm_f16(const __nv_bfloat16* x, const __nv_bfloat16* g, int M, int H, float eps, __nv_bfloat16* y, void* y16,
-                       float* inv, cudaStream_t stream);
-// The same for the W8A8 pass: the producer smooths and quantises its output rows per token (Eq. 9) into xq / dx.
-int launch_rmsnorm_q8(const __nv_bfloat16* x, const __nv_bfloat16* g, const float* smooth, int M, int H, float eps,
-                      __nv_bfloat16* y, int8_t* xq, float* dx, cudaStream_t stream);
-int launch_swiglu_q8(const __nv_bfloat16* gu, const float* smooth, int M, int F, __nv_bfloat16* act, int8_t* xq, float* dx,
-                     cudaStream_t stream);
-int launch_swiglu_f16(const __nv_bfloat16* gu, int M, int F, __nv_bfloat16* act, void* act16, float* inv, cudaStream_t stream);
-// x += bf16(dw * dx * sum of the k-range partial sums) (the epilogue of a residual linear layer), then y = RMSNorm(x) * g
-// with its fp16 form: one kernel in place of the split-K reduction, the norm and the operand pre-pass
-int launch_reduce_residual_rmsnorm_f16(const float* partial, int nsplit, int mpad, const float* dx, const float* dw,
-                                       __nv_bfloat16* x, const __nv_bfloat16* g, int M, int H, float eps, __nv_bfloat16* y,
-                                       void* y16, float* inv, cudaStream_t stream);
-
-// keys: M x 8 bytes of scratch
-int launch_argmax(const float* logits, int M, int V, int32_t* top1, unsigned long long* keys, cudaStream_t stream);
-
-int launch_accept(const int32_t* tokens, const int32_t* parents, const int32_t* block_len, const int32_t* top1,
-                  BlockInfo bi, int B, int T_max, int32_t* accept_len, int32_t* bonus, int32_t* accept_path,
-                  cudaStream_t stream);
 
 int launch_kv_commit(__nv_bfloat16* k_cache, __nv_bfloat16* v_cache, int32_t* seq_len, const int32_t* accept_len,
                      const int32_t* accept_path, int L, int B_cache, int B, int T_max, int Hkv, int D, int s_max,

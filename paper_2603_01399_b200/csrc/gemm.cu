@@ -1,55 +1,36 @@
-// Skinny quantised GEMM  Y[m][n] = delta[n] * sum_k X[m][k] * W[n][k]  (Section 3.2 Eq. 8 /
-// Section 3.3 Eq. 10, weight-only form): M <= 72 activation rows against an [N][K] int8 (or
-// bf16) weight matrix that is read exactly once.  HBM-bound on the weight stream
-// (1 B per weight, 2*M flop per byte), so the tensor cores are used only to keep up with it.
+// The linear layer  Y[m][n] = delta[n] * sum_k X[m][k] * W[n][k]  (Section 3.2 Eq. 8 / Section 3.3 Eq. 10,
+// weight-only form) with int8 or bf16 weights: which kernel runs a call.
 //
-// Mapping: the weights are the 16-row MMA operand ("A" of mma.m16n8k16, rows = output
-// channels), the activation rows are the 8-wide operand, zero-padded to a multiple of 8.
-// The contraction index may be permuted freely as long as both operands agree, so each
-// thread loads 16 contiguous weight bytes of one row with a single 128-bit load and
-// treats them as the k-columns its fragment slots need; the matching activations come
-// from a swizzled shared-memory copy of the CTA's k-slice of X.  int8 -> bf16 is exact and
-// happens in registers; delta[n] is applied once in the epilogue.
-//
-// Work split: a CTA of 4 warps owns 64 output channels x one k-range; k-ranges of one
-// channel block are reduced in a FIXED order by the last CTA to arrive (fp32 partials in
-// the workspace, a self-resetting arrival counter), so results are run-to-run identical.
+//  * The tcgen05 kernel (tc_linear.cu), int8 weights behind a pre-pass that writes the activations as digit rows:
+//    everything but the next two.
+//  * `skinny_gemm_kernel` below, warp-level MMAs on blocks of at most 8 rows whose contraction has at most 512
+//    elements: such a call is all latency, and one kernel is shorter than pre-pass and tcgen05 kernel (3.1-3.8 us
+//    against 5.8 us at 1024 x 256; from two 512-element pieces on the order turns: 6.3 us against 8.4 us at
+//    1024 x 1024, 8 rows).
+//  * the same kernel, in groups of 8 rows, where the caller's scratch does not hold even one row of digits.
 #include <mutex>
 
 #include "common.cuh"
+#include "tc_linear.cuh"
 
 namespace quasar {
 
 namespace {
 
-constexpr int64_t kRows8UmmaMinBytes = (int64_t)1 << 27;   // weight bytes from which blocks of <= 8 rows take the tcgen05 stream kernel
-
 constexpr int kWarps = 4;
 constexpr int kThreads = kWarps * 32;
 constexpr int kBlockN = kWarps * 16;  // output channels per CTA
-constexpr int kSub = 512;             // contraction elements staged in shared memory at a time (blocks of up to 32 rows)
-// Wider blocks stage half as much at a time: the activations of 72 rows would otherwise take 72 KB per CTA
-// and leave an SM with three CTAs (12 warps) to hide the weight loads behind.
-template <int NT>
-__host__ __device__ constexpr int sub_of() { return NT > 4 ? 256 : 512; }
-constexpr int kMaxSplit = 32;
-// The arrival counters of the split-K reduction take a region of fixed size at the start of the
-// workspace, so that calls of different widths can share one workspace: no call's partial sums
-// land where another call keeps its counters.
-constexpr size_t kCounterBytes = 64 * 1024;
+constexpr int kSub = 512;             // contraction elements staged in shared memory at a time
+constexpr size_t kCounterBytes = 64 * 1024;   // reserved at the start of every workspace (quasar.h)
 constexpr int64_t kMaxChannels = (int64_t)(kCounterBytes / sizeof(int)) * kBlockN;
 
 struct GemmArgs {
   const __nv_bfloat16* x;   // [M][K]
-  const void* w;            // [N][K]
-  const float* delta;       // [N] or nullptr
+  const int8_t* w;          // [N][K]
+  const float* delta;       // [N]
   void* y;                  // [M][N] bf16 or fp32
   const __nv_bfloat16* res; // [M][N] or nullptr
-  float* partial;           // [nsplit][NT*8][N]
-  int* counters;            // [ceil(N / kBlockN)]
-  int M, N, K;
-  int k_per_split;          // multiple of kSub
-  int nsplit;
+  int M, N, K;              // M <= 8
   int y_is_f32;
 };
 
@@ -83,247 +64,112 @@ __device__ __forceinline__ uint4 ldg_stream(const void* p) {
   return r;
 }
 
-template <bool W_INT8>
-__device__ __forceinline__ int swz(int chunk, int row) {
-  return W_INT8 ? (chunk ^ (row & 1)) : (chunk ^ ((row & 1) << 2));
-}
-
-__device__ __forceinline__ float epilogue_value(float acc, float d, const __nv_bfloat16* res, size_t idx) {
-  float v = acc * d;
-  if (res != nullptr) {
-    v = __bfloat162float(__float2bfloat16_rn(v)) + __bfloat162float(res[idx]);
-  }
-  return v;
-}
-
-template <int NT, bool W_INT8>
+// The weights are the 16-row MMA operand (rows = output channels), the activation rows the 8-wide one, zero-padded.  The
+// contraction index may be permuted freely as long as both operands agree, so each thread loads 16 contiguous weight
+// bytes of one row and treats them as the k-columns its fragment slots need; the matching activations come from a
+// swizzled shared-memory copy.  A CTA of 4 warps owns 64 output channels and the whole contraction.
 __global__ void __launch_bounds__(kThreads) skinny_gemm_kernel(GemmArgs a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int kSub = sub_of<NT>();
-  uint4* xs = reinterpret_cast<uint4*>(smem_raw);  // [NT*8][kSub/8] 16-byte chunks, swizzled
   constexpr int kChunksPerRow = kSub / 8;
-  constexpr int kStepK = W_INT8 ? 64 : 32;  // contraction elements one warp step covers
-  constexpr int kSteps = kSub / kStepK;
+  constexpr int kSteps = kSub / 64;   // a warp step covers 64 contraction elements
   constexpr int kUnroll = 4;
+  __shared__ uint4 xs[8 * kChunksPerRow];   // 16-byte chunks, swizzled by the row's parity
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t = lane & 3;
   const int n0 = blockIdx.x * kBlockN + warp * 16;
-  const int split = blockIdx.y;
-  const int k_begin = split * a.k_per_split;
-  const int k_end = min(a.K, k_begin + a.k_per_split);
-
   const int r0 = min(n0 + g, a.N - 1), r1 = min(n0 + g + 8, a.N - 1);
-  const size_t wbytes = W_INT8 ? 1 : 2;
-  const unsigned char* wrow0 = reinterpret_cast<const unsigned char*>(a.w) + (size_t)r0 * a.K * wbytes;
-  const unsigned char* wrow1 = reinterpret_cast<const unsigned char*>(a.w) + (size_t)r1 * a.K * wbytes;
+  const int8_t* wrow0 = a.w + (size_t)r0 * a.K;
+  const int8_t* wrow1 = a.w + (size_t)r1 * a.K;
 
-  float acc[NT][4];
-#pragma unroll
-  for (int i = 0; i < NT; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
-
-  for (int kk = k_begin; kk < k_end; kk += kSub) {
+  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int kk = 0; kk < a.K; kk += kSub) {
     __syncthreads();
     // stage X[:, kk : kk + kSub) (zero beyond M or K)
-    for (int c = threadIdx.x; c < NT * 8 * kChunksPerRow; c += kThreads) {
+    for (int c = threadIdx.x; c < 8 * kChunksPerRow; c += kThreads) {
       const int row = c / kChunksPerRow, ch = c % kChunksPerRow;
       const int k = kk + ch * 8;
       uint4 v = make_uint4(0, 0, 0, 0);
-      if (row < a.M && k < k_end) v = *reinterpret_cast<const uint4*>(a.x + (size_t)row * a.K + k);
-      xs[row * kChunksPerRow + swz<W_INT8>(ch, row)] = v;
+      if (row < a.M && k < a.K) v = *reinterpret_cast<const uint4*>(a.x + (size_t)row * a.K + k);
+      xs[row * kChunksPerRow + (ch ^ (row & 1))] = v;
     }
     __syncthreads();
-
 #pragma unroll 1
     for (int s0 = 0; s0 < kSteps; s0 += kUnroll) {
-      if (kk + s0 * kStepK >= k_end) break;
+      if (kk + s0 * 64 >= a.K) break;
       uint4 wa[kUnroll], wb[kUnroll];
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u) {
-        const int k = kk + (s0 + u) * kStepK + t * 16 / (int)wbytes;
-        if (k < k_end) {
-          wa[u] = ldg_stream(wrow0 + (size_t)k * wbytes);
-          wb[u] = ldg_stream(wrow1 + (size_t)k * wbytes);
-        } else {
-          wa[u] = make_uint4(0, 0, 0, 0);
-          wb[u] = make_uint4(0, 0, 0, 0);
-        }
+        const int k = kk + (s0 + u) * 64 + t * 16;
+        wa[u] = k < a.K ? ldg_stream(wrow0 + k) : make_uint4(0, 0, 0, 0);
+        wb[u] = k < a.K ? ldg_stream(wrow1 + k) : make_uint4(0, 0, 0, 0);
       }
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u) {
-        const int s = s0 + u;
-        if (W_INT8) {
-          uint32_t A0[4], A1[4], A2[4], A3[4];
-          const uint32_t* pa = reinterpret_cast<const uint32_t*>(&wa[u]);
-          const uint32_t* pb = reinterpret_cast<const uint32_t*>(&wb[u]);
+        uint32_t A0[4], A1[4], A2[4], A3[4];
+        const uint32_t* pa = reinterpret_cast<const uint32_t*>(&wa[u]);
+        const uint32_t* pb = reinterpret_cast<const uint32_t*>(&wb[u]);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            s8x4_to_bf16x4(pa[j], A0[j], A2[j]);
-            s8x4_to_bf16x4(pb[j], A1[j], A3[j]);
-          }
-#pragma unroll
-          for (int nt = 0; nt < NT; ++nt) {
-            const int row = nt * 8 + g;
-            const int ch = s * 8 + t * 2;
-            const uint4 x0 = xs[row * kChunksPerRow + swz<true>(ch, row)];
-            const uint4 x1 = xs[row * kChunksPerRow + swz<true>(ch + 1, row)];
-            mma_bf16(acc[nt], A0[0], A1[0], A2[0], A3[0], x0.x, x0.y);
-            mma_bf16(acc[nt], A0[1], A1[1], A2[1], A3[1], x0.z, x0.w);
-            mma_bf16(acc[nt], A0[2], A1[2], A2[2], A3[2], x1.x, x1.y);
-            mma_bf16(acc[nt], A0[3], A1[3], A2[3], A3[3], x1.z, x1.w);
-          }
-        } else {
-#pragma unroll
-          for (int nt = 0; nt < NT; ++nt) {
-            const int row = nt * 8 + g;
-            const int ch = s * 4 + t;
-            const uint4 x0 = xs[row * kChunksPerRow + swz<false>(ch, row)];
-            mma_bf16(acc[nt], wa[u].x, wb[u].x, wa[u].y, wb[u].y, x0.x, x0.y);
-            mma_bf16(acc[nt], wa[u].z, wb[u].z, wa[u].w, wb[u].w, x0.z, x0.w);
-          }
+        for (int j = 0; j < 4; ++j) {
+          s8x4_to_bf16x4(pa[j], A0[j], A2[j]);
+          s8x4_to_bf16x4(pb[j], A1[j], A3[j]);
         }
+        const int ch = (s0 + u) * 8 + t * 2;
+        const uint4 x0 = xs[g * kChunksPerRow + (ch ^ (g & 1))];
+        const uint4 x1 = xs[g * kChunksPerRow + ((ch + 1) ^ (g & 1))];
+        mma_bf16(acc, A0[0], A1[0], A2[0], A3[0], x0.x, x0.y);
+        mma_bf16(acc, A0[1], A1[1], A2[1], A3[1], x0.z, x0.w);
+        mma_bf16(acc, A0[2], A1[2], A2[2], A3[2], x1.x, x1.y);
+        mma_bf16(acc, A0[3], A1[3], A2[3], A3[3], x1.z, x1.w);
       }
     }
   }
-
-  // ---- epilogue ------------------------------------------------------------------------
-  // acc[nt][0..1]: channel n0+g, rows nt*8+2t, +1;  acc[nt][2..3]: channel n0+g+8.
-  if (a.nsplit == 1) {
+  // acc[0..1]: channel n0+g, rows 2t, 2t+1;  acc[2..3]: channel n0+g+8
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int n = n0 + g + (e >> 1) * 8;
-        const int m = nt * 8 + 2 * t + (e & 1);
-        if (n < a.N && m < a.M) {
-          const float d = a.delta ? a.delta[n] : 1.0f;
-          const size_t idx = (size_t)m * a.N + n;
-          const float v = epilogue_value(acc[nt][e], d, a.res, idx);
-          if (a.y_is_f32) reinterpret_cast<float*>(a.y)[idx] = v;
-          else reinterpret_cast<__nv_bfloat16*>(a.y)[idx] = __float2bfloat16_rn(v);
-        }
-      }
-    }
-    return;
-  }
-
-  float* mine = a.partial + (size_t)split * (NT * 8) * a.N;
-#pragma unroll
-  for (int nt = 0; nt < NT; ++nt) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int n = n0 + g + (e >> 1) * 8;
-      const int m = nt * 8 + 2 * t + (e & 1);
-      if (n < a.N && m < a.M) __stcg(mine + (size_t)m * a.N + n, acc[nt][e]);
-    }
-  }
-  __threadfence();
-  __syncthreads();
-  __shared__ int s_last;
-  if (threadIdx.x == 0) {
-    const int prev = atomicAdd(a.counters + blockIdx.x, 1);
-    s_last = (prev == a.nsplit - 1);
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  const int nb = blockIdx.x * kBlockN;
-  for (int i = threadIdx.x; i < kBlockN * a.M; i += kThreads) {
-    const int n = nb + (i % kBlockN), m = i / kBlockN;
-    if (n >= a.N) continue;
-    float sum = 0.f;
-    for (int s = 0; s < a.nsplit; ++s) sum += __ldcg(a.partial + ((size_t)s * (NT * 8) + m) * a.N + n);
-    const float d = a.delta ? a.delta[n] : 1.0f;
+  for (int e = 0; e < 4; ++e) {
+    const int n = n0 + g + (e >> 1) * 8, m = 2 * t + (e & 1);
+    if (n >= a.N || m >= a.M) continue;
     const size_t idx = (size_t)m * a.N + n;
-    const float v = epilogue_value(sum, d, a.res, idx);
+    float v = acc[e] * a.delta[n];
+    if (a.res != nullptr) v = __bfloat162float(__float2bfloat16_rn(v)) + __bfloat162float(a.res[idx]);
     if (a.y_is_f32) reinterpret_cast<float*>(a.y)[idx] = v;
     else reinterpret_cast<__nv_bfloat16*>(a.y)[idx] = __float2bfloat16_rn(v);
   }
-  if (threadIdx.x == 0) a.counters[blockIdx.x] = 0;  // ready for the next launch on this stream
 }
 
-struct SplitPlan {
-  int nblocks, nsplit, k_per_split;
-};
+size_t align256g(size_t v) { return (v + 255) / 256 * 256; }
 
-SplitPlan plan_split(int64_t N, int64_t K) {
-  SplitPlan p;
-  p.nblocks = (int)((N + kBlockN - 1) / kBlockN);
-  const int subs = (int)((K + kSub - 1) / kSub);
-  const int target = 148 * 4;  // four 4-warp CTAs per SM in flight
-  int want = (target + p.nblocks - 1) / p.nblocks;
-  want = want < 1 ? 1 : want;
-  want = want > subs ? subs : want;
-  want = want > kMaxSplit ? kMaxSplit : want;
-  const int subs_per = (subs + want - 1) / want;
-  p.k_per_split = subs_per * kSub;
-  p.nsplit = (subs + subs_per - 1) / subs_per;
-  return p;
-}
-
-template <int NT, bool W_INT8>
-int launch_nt(const GemmArgs& a, const SplitPlan& p, cudaStream_t stream) {
-  const size_t smem = (size_t)NT * 8 * sub_of<NT>() * sizeof(__nv_bfloat16);
-  static bool configured = false;
-  if (smem > 48 * 1024 && !configured) {
-    QUASAR_CUDA_CHECK(cudaFuncSetAttribute(skinny_gemm_kernel<NT, W_INT8>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    configured = true;
-  }
-  dim3 grid(p.nblocks, p.nsplit);
-  skinny_gemm_kernel<NT, W_INT8><<<grid, kThreads, smem, stream>>>(a);
-  QUASAR_LAUNCH_CHECK();
-  return QUASAR_OK;
-}
-
-template <bool W_INT8>
-int launch_w(const GemmArgs& a, const SplitPlan& p, cudaStream_t stream) {
-  const int nt = (a.M + 7) / 8;
-  switch (nt) {
-    case 1: return launch_nt<1, W_INT8>(a, p, stream);
-    case 2: return launch_nt<2, W_INT8>(a, p, stream);
-    case 3: return launch_nt<3, W_INT8>(a, p, stream);
-    case 4: return launch_nt<4, W_INT8>(a, p, stream);
-    case 5: return launch_nt<5, W_INT8>(a, p, stream);
-    case 6: return launch_nt<6, W_INT8>(a, p, stream);
-    case 7: return launch_nt<7, W_INT8>(a, p, stream);
-    case 8: return launch_nt<8, W_INT8>(a, p, stream);
-    case 9: return launch_nt<9, W_INT8>(a, p, stream);
-    default: set_error("skinny GEMM: %d rows in one launch", a.M); return QUASAR_ERR_SHAPE;
-  }
-}
+// bytes of M activation rows as digits (behind the reserved start of a workspace)
+size_t digit_bytes(int64_t M, int64_t K) { return align256g((size_t)3 * M * K) + align256g((size_t)M * 4); }
 
 }  // namespace
 
-// the least a call needs: without the scratch of the stream kernel that blocks of at most 8 rows take on very large
-// matrices WHEN the workspace has room for it (they fall back to the warp-level kernel otherwise)
-static size_t linear_workspace_bytes_min(int64_t M, int64_t N, int64_t K) {
-  const SplitPlan p = plan_split(N, K);
-  const int64_t rows = M < kMaxRowsPerGemm ? M : kMaxRowsPerGemm;
-  const size_t mpad = (size_t)((rows + 7) / 8) * 8;
-  const size_t counters = kCounterBytes;
-  size_t partial = p.nsplit > 1 ? (size_t)p.nsplit * mpad * (size_t)N * sizeof(float) : 0;
-  // blocks of more than 8 rows with int8 weights run on the tcgen05 kernel, which keeps an fp16 copy of the
-  // activation rows and its own partial sums here
-  const int64_t rows_u = M < 80 ? M : 80;
-  if (M > 8 && umma_w8a16_usable(rows_u, N, K)) {
-    const size_t su = umma_w8a16_scratch_bytes(rows_u, N, K);
-    partial = su > partial ? su : partial;
+// What this entry point has asked for since its first version - an fp16 copy of up to 80 rows and the partial sums of the
+// k-ranges.  The built-in scratch of linear_static takes the shapes that fit it by this measure.
+static size_t linear_static_need(int64_t M, int64_t N, int64_t K) {
+  auto ranges = [](int64_t blocks, int64_t pieces, int64_t want) {
+    want = want < 1 ? 1 : (want > pieces ? pieces : want);
+    want = want > 32 ? 32 : want;
+    const int64_t per = (pieces + want - 1) / want;
+    return (pieces + per - 1) / per;
+  };
+  const int64_t rows = M < kMaxRowsPerGemm ? M : kMaxRowsPerGemm, rows_u = M < 80 ? M : 80;
+  const int64_t b0 = (N + 63) / 64, b1 = (N + 127) / 128;
+  const int64_t s0 = ranges(b0, (K + 511) / 512, (148 * 4 + b0 - 1) / b0);
+  size_t need = s0 > 1 ? (size_t)s0 * ((rows + 7) / 8 * 8) * N * 4 : 0;
+  if (M > 8) {
+    const int64_t s1 = ranges(b1, (K + 127) / 128, 296 / b1);
+    const size_t partial = (s1 > 1 || N <= 32768) ? (size_t)s1 * ((rows_u + 15) / 16 * 16) * N * 4 : 0;
+    const size_t u = align256g((size_t)rows_u * K * 2) + align256g((size_t)rows_u * 4) + partial;
+    need = u > need ? u : need;
   }
-  return counters + partial;
+  return kCounterBytes + need;
 }
 
-static bool rows8_stream_eligible(int64_t M, int64_t N, int64_t K) {
-  return M <= 8 && N * K >= kRows8UmmaMinBytes && umma_rows8_usable(M, N, K);
-}
-
+// What a call asks its caller for: the digit rows, and never less than it asked for in earlier versions, so that sizes
+// worked out then still hold.
 size_t linear_workspace_bytes(int64_t M, int64_t N, int64_t K) {
-  size_t need = linear_workspace_bytes_min(M, N, K);
-  if (rows8_stream_eligible(M, N, K)) {
-    const size_t su = kCounterBytes + umma_rows8_scratch_bytes(M, N, K);
-    need = su > need ? su : need;
-  }
-  return need;
+  const size_t digits = kCounterBytes + digit_bytes(M, K), before = linear_static_need(M, N, K);
+  return digits > before ? digits : before;
 }
 
 int launch_linear(const __nv_bfloat16* x, const void* w, const float* delta, int weight_dtype, int64_t M, int64_t N,
@@ -334,55 +180,51 @@ int launch_linear(const __nv_bfloat16* x, const void* w, const float* delta, int
               (long long)M, (long long)N, (long long)K, (long long)kMaxChannels);
     return QUASAR_ERR_SHAPE;
   }
-  if (workspace_bytes < linear_workspace_bytes_min(M, N, K)) {
+  if (workspace_bytes < kCounterBytes) {
     set_error("linear: workspace of %zu bytes, need %zu", workspace_bytes, linear_workspace_bytes(M, N, K));
     return QUASAR_ERR_CAPACITY;
   }
-  const SplitPlan p = plan_split(N, K);
-  const size_t counters = kCounterBytes;
+  if (weight_dtype == QUASAR_W_BF16)
+    return launch_tc_linear_bf16(x, reinterpret_cast<const __nv_bfloat16*>(w), M, N, K, y, y_is_f32, residual, nullptr, status, false,
+                                 stream);
+  const int8_t* wq = reinterpret_cast<const int8_t*>(w);
   const size_t ybytes = y_is_f32 ? 4 : 2;
-  if (weight_dtype == QUASAR_W_INT8 && M > 8 && umma_w8a16_usable(M < 80 ? M : 80, N, K)) {
-    // a real dense contraction: tcgen05 MMAs with the accumulator in tensor memory (umma_gemm.cu)
-    for (int64_t m0 = 0; m0 < M; m0 += 80) {
-      const int64_t rows = (M - m0) < 80 ? (M - m0) : 80;
-      const int rc = launch_umma_w8a16(x + m0 * K, reinterpret_cast<const int8_t*>(w), delta, rows, N, K,
-                                       reinterpret_cast<unsigned char*>(y) + (size_t)m0 * N * ybytes, y_is_f32,
-                                       residual ? residual + m0 * N : nullptr,
-                                       reinterpret_cast<unsigned char*>(workspace) + counters, status, stream);
-      if (rc != QUASAR_OK) return rc;
+  // rows whose digits fit behind the reserved start of the workspace: all of them, unless the workspace is smaller than
+  // linear_workspace_bytes reports (the built-in one of linear_static)
+  const int64_t room = (int64_t)(workspace_bytes - kCounterBytes) - 512;
+  const int64_t fit = room > 0 ? room / (3 * K + 4) : 0;
+  if ((M <= 8 && K <= kSub) || fit < 1) {
+    for (int64_t m0 = 0; m0 < M; m0 += 8) {
+      GemmArgs a;
+      a.M = (int)((M - m0) < 8 ? (M - m0) : 8);
+      a.N = (int)N; a.K = (int)K;
+      a.x = x + m0 * K; a.w = wq; a.delta = delta;
+      a.y = reinterpret_cast<unsigned char*>(y) + (size_t)m0 * N * ybytes;
+      a.res = residual ? residual + m0 * N : nullptr;
+      a.y_is_f32 = y_is_f32 ? 1 : 0;
+      skinny_gemm_kernel<<<(unsigned)((N + kBlockN - 1) / kBlockN), kThreads, 0, stream>>>(a);
+      QUASAR_LAUNCH_CHECK();
     }
     return QUASAR_OK;
   }
-  // A matrix of LM-head size with at most 8 rows is a long pure stream: the persistent tcgen05 kernel that feeds
-  // the int8 tiles straight into integer MMAs (activations as base-256 digits, umma_gemm.cu) sustains a higher
-  // rate than the warp-level kernel there; below that size its two extra launches cost more than it gains.
-  if (weight_dtype == QUASAR_W_INT8 && rows8_stream_eligible(M, N, K) && workspace_bytes >= kCounterBytes + umma_rows8_scratch_bytes(M, N, K))
-    return launch_umma_rows8(x, reinterpret_cast<const int8_t*>(w), delta, M, N, K, y, y_is_f32, residual,
-                             reinterpret_cast<unsigned char*>(workspace) + counters, status, stream);
-  for (int64_t m0 = 0; m0 < M; m0 += kMaxRowsPerGemm) {
-    GemmArgs a;
-    a.M = (int)((M - m0) < kMaxRowsPerGemm ? (M - m0) : kMaxRowsPerGemm);
-    a.N = (int)N;
-    a.K = (int)K;
-    a.x = x + m0 * K;
-    a.w = w;
-    a.delta = weight_dtype == QUASAR_W_INT8 ? delta : nullptr;
-    a.y = reinterpret_cast<unsigned char*>(y) + (size_t)m0 * N * ybytes;
-    a.res = residual ? residual + m0 * N : nullptr;
-    a.counters = reinterpret_cast<int*>(workspace);
-    a.partial = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(workspace) + counters);
-    a.k_per_split = p.k_per_split;
-    a.nsplit = p.nsplit;
-    a.y_is_f32 = y_is_f32 ? 1 : 0;
-    const int rc = weight_dtype == QUASAR_W_INT8 ? launch_w<true>(a, p, stream) : launch_w<false>(a, p, stream);
+  const int64_t step = fit < M ? fit : M;
+  for (int64_t m0 = 0; m0 < M; m0 += step) {
+    const int64_t rows = (M - m0) < step ? (M - m0) : step;
+    int8_t* xd = reinterpret_cast<int8_t*>(workspace) + kCounterBytes;
+    float* scale = reinterpret_cast<float*>(xd + align256g((size_t)3 * rows * K));
+    int rc = launch_digit_rows3(x + m0 * K, rows, K, xd, scale, stream);
+    if (rc != QUASAR_OK) return rc;
+    // (the pre-pass starts only when whatever wrote the weights has finished, so they may be read beside it)
+    rc = launch_tc_linear_digits(xd, scale, wq, delta, rows, N, K, reinterpret_cast<unsigned char*>(y) + (size_t)m0 * N * ybytes,
+                                 y_is_f32, residual ? residual + m0 * N : nullptr, nullptr, status, true, stream);
     if (rc != QUASAR_OK) return rc;
   }
   return QUASAR_OK;
 }
 
 // ---- the same linear layer with its scratch inside the library ------------------------------------
-// Scratch of the split-K reduction for callers that cannot hand over a workspace: a fixed array in
-// device memory that every GPU loading the library holds until the process exits.
+// Scratch for callers that cannot hand over a workspace: a fixed array in device memory that every GPU loading the
+// library holds until the process exits.
 constexpr size_t kStaticScratchBytes = 4u << 20;
 static __device__ __align__(256) unsigned char g_linear_scratch[kStaticScratchBytes];
 
@@ -396,7 +238,8 @@ int launch_linear_static(const __nv_bfloat16* x, const void* w, const float* del
               (long long)M, (long long)N, (long long)K, (long long)kMaxChannels);
     return QUASAR_ERR_SHAPE;
   }
-  const size_t need = linear_workspace_bytes_min(M, N, K);
+  // Refused: blocks whose fp32 sums would not fit the array (the documented limit), whatever the kernel of today keeps there.
+  const size_t need = linear_static_need(M, N, K);
   if (need > kStaticScratchBytes) {
     set_error("linear_static: M=%lld N=%lld K=%lld needs %zu bytes of scratch, the built-in array holds %zu; "
               "use quasar_linear with a workspace",
@@ -426,10 +269,6 @@ int launch_linear_static(const __nv_bfloat16* x, const void* w, const float* del
     }
     scratch = scratch_of_device[dev];
   }
-  // The arrival counters must start at zero; the array keeps whatever the last call left in it.  (Only the
-  // split-K form of the warp-level kernel counts arrivals.)
-  const bool counts = plan_split(N, K).nsplit > 1 && !(weight_dtype == QUASAR_W_INT8 && M > 8 && umma_w8a16_usable(M < 80 ? M : 80, N, K));
-  if (counts) QUASAR_CUDA_CHECK(cudaMemsetAsync(scratch, 0, kCounterBytes, stream));
   return launch_linear(x, w, delta, weight_dtype, M, N, K, y, y_is_f32, residual, scratch, kStaticScratchBytes, stream, nullptr);
 }
 

@@ -1,0 +1,441 @@
+// The steps of the pass that work on whole activation rows and leave the operand of the linear layer that follows
+// (Section 3.3: the "non-linear layers" stay in high precision, the online quantisation of Eq. 9 rides on them):
+// embedding gather + first RMSNorm, RMSNorm, SwiGLU, and the attention output on its way into the o projection.
+//
+// The operand has one of three forms: the row as three digit rows (int8 weights, bf16 activations; see tc_linear.cuh),
+// the row smoothed and quantised per token (W8A8, Eq. 9), or the bf16 row itself (bf16 weights).
+//
+// One CTA of 512 threads per row; a row of up to 24,576 elements stays in registers between its passes (statistic,
+// maximum, codes), eight consecutive elements a thread and turn, longer rows are read again.  Latency-bound (a row is
+// 8 to 48 KB out of L2): every input of a turn is one 128-bit load, the gains and smoothing factors - weights - are
+// asked for before the kernel in front has finished, and all of these are dependent launches.
+#include <math.h>
+
+#include "common.cuh"
+#include "tc_common.cuh"
+#include "tc_linear.cuh"
+
+namespace quasar {
+
+namespace {
+
+using tc::pdl_trigger;
+using tc::pdl_wait;
+
+constexpr int kRowThreads = 512;
+
+__device__ __forceinline__ void unpack8(const uint4& v, float (&f)[8]) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    f[2 * e] = __uint_as_float(w[e] << 16);
+    f[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
+  }
+}
+// rounds f to bf16 in place and returns the packed values
+__device__ __forceinline__ uint4 round8(float (&f)[8]) {
+  uint32_t w[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const __nv_bfloat162 p = __floats2bfloat162_rn(f[2 * e], f[2 * e + 1]);
+    w[e] = *reinterpret_cast<const uint32_t*>(&p);
+    f[2 * e] = __uint_as_float(w[e] << 16);
+    f[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+template <bool MAX>
+__device__ __forceinline__ float block_reduce(float v, float* s_buf) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float u = __shfl_xor_sync(0xffffffffu, v, o);
+    v = MAX ? fmaxf(v, u) : v + u;
+  }
+  if ((threadIdx.x & 31) == 0) s_buf[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = s_buf[0];
+#pragma unroll
+  for (int i = 1; i < kRowThreads / 32; ++i) v = MAX ? fmaxf(v, s_buf[i]) : v + s_buf[i];   // warps in order
+  return v;
+}
+
+// The smoothing factors of eight channels (one for all without smoothing)
+__device__ __forceinline__ void load_smooth8(const float* smooth, int i, float (&s)[8]) {
+  if (smooth == nullptr) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) s[e] = 1.f;
+    return;
+  }
+  const float4 a = __ldg(reinterpret_cast<const float4*>(smooth) + 2 * i), b = __ldg(reinterpret_cast<const float4*>(smooth) + 2 * i + 1);
+  s[0] = a.x; s[1] = a.y; s[2] = a.z; s[3] = a.w; s[4] = b.x; s[5] = b.y; s[6] = b.z; s[7] = b.w;
+}
+
+// The row's values (eight of vector i by value(i, j, f); j is the turn) as the operand.
+template <int OP, int V, typename F>
+__device__ __forceinline__ void write_operand(F&& value, int nvec, int m, const RowOperand& out, float* s_buf) {
+  if (OP == kOperandBf16) {   // (the values have been stored as they were made)
+    float f[8];
+    if (V > 0) {
+#pragma unroll
+      for (int j = 0; j < (V > 0 ? V : 1); ++j)
+        if ((int)threadIdx.x + j * kRowThreads < nvec) value((int)threadIdx.x + j * kRowThreads, j, f);
+    } else {
+      for (int i = threadIdx.x; i < nvec; i += kRowThreads) value(i, 0, f);
+    }
+    return;
+  }
+  const int64_t width = (int64_t)nvec * 8;
+  float f[V > 0 ? V : 1][8];
+  float amax = 0.f;
+  if (V > 0) {
+#pragma unroll
+    for (int j = 0; j < (V > 0 ? V : 1); ++j) {
+      const int i = (int)threadIdx.x + j * kRowThreads;
+      if (i < nvec) {
+        value(i, j, f[j]);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) amax = fmaxf(amax, fabsf(f[j][e]));
+      }
+    }
+  } else {
+    for (int i = threadIdx.x; i < nvec; i += kRowThreads) {
+      value(i, 0, f[0]);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) amax = fmaxf(amax, fabsf(f[0][e]));
+    }
+  }
+  amax = block_reduce<true>(amax, s_buf);
+  float up = 1.f, scale = 1.f;
+  if (OP == kOperandDigits) digit_scale(amax, up, scale);
+  else scale = amax == 0.f ? 1.0f : __fdiv_rn(amax, 127.0f);
+  if (threadIdx.x == 0) out.scale[m] = scale;
+  auto put = [&](int i, const float (&v)[8]) {
+    if (OP == kOperandDigits) {
+      write_digits8(v, up, out.q + 3 * (int64_t)m * width, width, (int64_t)i * 8);
+    } else {
+      uint32_t p[2] = {0u, 0u};
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int q = max(-127, min(127, __float2int_rn(__fdiv_rn(v[e], scale))));
+        p[e >> 2] |= (uint32_t)(q & 0xff) << (8 * (e & 3));
+      }
+      *reinterpret_cast<uint2*>(out.q + (int64_t)m * width + (int64_t)i * 8) = make_uint2(p[0], p[1]);
+    }
+  };
+  if (V > 0) {
+#pragma unroll
+    for (int j = 0; j < (V > 0 ? V : 1); ++j)
+      if ((int)threadIdx.x + j * kRowThreads < nvec) put((int)threadIdx.x + j * kRowThreads, f[j]);
+  } else {
+    for (int i = threadIdx.x; i < nvec; i += kRowThreads) {
+      value(i, 0, f[0]);
+      put(i, f[0]);
+    }
+  }
+}
+
+// RMSNorm of the row whose vectors raw(i, j, f) gives, in operand form: y = bf16(x * rsqrt(mean(x^2) + eps) * g)
+template <int OP, int V, typename F>
+__device__ __forceinline__ void norm_row(F&& raw, const uint4 (&gain)[V > 0 ? V : 1], const __nv_bfloat16* g, int nvec, float eps, int m,
+                                         const RowOperand& out, float* s_buf) {
+  float x[V > 0 ? V : 1][8];
+  float ss = 0.f;
+  if (V > 0) {
+#pragma unroll
+    for (int j = 0; j < (V > 0 ? V : 1); ++j) {
+      const int i = (int)threadIdx.x + j * kRowThreads;
+      if (i < nvec) {
+        raw(i, x[j]);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) ss += x[j][e] * x[j][e];
+      }
+    }
+  } else {
+    for (int i = threadIdx.x; i < nvec; i += kRowThreads) {
+      raw(i, x[0]);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) ss += x[0][e] * x[0][e];
+    }
+  }
+  ss = block_reduce<false>(ss, s_buf);
+  const float r = 1.0f / sqrtf(ss / (float)(nvec * 8) + eps);
+  write_operand<OP, V>(
+      [&](int i, int j, float (&f)[8]) {
+        float gg[8];
+        if (V > 0) {
+          unpack8(gain[V > 0 ? j : 0], gg);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) f[e] = x[V > 0 ? j : 0][e] * r * gg[e];
+        } else {
+          unpack8(__ldg(reinterpret_cast<const uint4*>(g) + i), gg);
+          raw(i, f);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) f[e] = f[e] * r * gg[e];
+        }
+        const uint4 y = round8(f);
+        if (out.y != nullptr) reinterpret_cast<uint4*>(out.y + (size_t)m * nvec * 8)[i] = y;
+        if (OP == kOperandCodes) {
+          float s[8];
+          load_smooth8(out.smooth, i, s);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) f[e] = __fmul_rn(f[e], s[e]);
+        }
+      },
+      nvec, m, out, s_buf + 32);
+}
+
+template <int V>
+__device__ __forceinline__ void load_gain(uint4 (&gain)[V > 0 ? V : 1], const __nv_bfloat16* g, int nvec) {
+  if (V > 0) {
+#pragma unroll
+    for (int j = 0; j < (V > 0 ? V : 1); ++j) {
+      const int i = (int)threadIdx.x + j * kRowThreads;
+      gain[j] = i < nvec ? __ldg(reinterpret_cast<const uint4*>(g) + i) : make_uint4(0, 0, 0, 0);
+    }
+  }
+}
+
+template <int OP, int V>
+__global__ void __launch_bounds__(kRowThreads)
+norm_kernel(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ g, int nvec, float eps, RowOperand out) {
+  __shared__ float s_buf[64];
+  pdl_trigger();
+  uint4 gain[V > 0 ? V : 1];
+  load_gain<V>(gain, g, nvec);
+  pdl_wait();
+  const int m = blockIdx.x;
+  const uint4* row = reinterpret_cast<const uint4*>(x + (size_t)m * nvec * 8);
+  norm_row<OP, V>([&](int i, float (&f)[8]) { unpack8(row[i], f); }, gain, g, nvec, eps, m, out, s_buf);
+}
+
+template <int OP, int V>
+__global__ void __launch_bounds__(kRowThreads)
+swiglu_kernel(const __nv_bfloat16* gu, int nvec, RowOperand out) {
+  __shared__ float s_buf[32];
+  pdl_trigger();
+  pdl_wait();
+  const int m = blockIdx.x;
+  const uint4* gr = reinterpret_cast<const uint4*>(gu + (size_t)m * nvec * 16);
+  const uint4* ur = gr + nvec;
+  write_operand<OP, V>(
+      [&](int i, int j, float (&f)[8]) {
+        float up[8];
+        unpack8(gr[i], f);
+        unpack8(ur[i], up);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) f[e] = f[e] / (1.0f + expf(-f[e])) * up[e];
+        const uint4 y = round8(f);
+        if (out.y != nullptr) reinterpret_cast<uint4*>(out.y + (size_t)m * nvec * 8)[i] = y;
+        if (OP == kOperandCodes) {
+          float s[8];
+          load_smooth8(out.smooth, i, s);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) f[e] = __fmul_rn(f[e], s[e]);
+        }
+      },
+      nvec, m, out, s_buf);
+}
+
+template <int OP, int V>
+__global__ void __launch_bounds__(kRowThreads) operand_kernel(const __nv_bfloat16* x, int nvec, RowOperand out) {
+  __shared__ float s_buf[32];
+  pdl_trigger();
+  pdl_wait();
+  const int m = blockIdx.x;
+  const uint4* row = reinterpret_cast<const uint4*>(x + (size_t)m * nvec * 8);
+  write_operand<OP, V>(
+      [&](int i, int j, float (&f)[8]) {
+        unpack8(row[i], f);
+        if (OP == kOperandCodes) {
+          float s[8];
+          load_smooth8(out.smooth, i, s);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) f[e] = __fmul_rn(f[e], s[e]);
+        }
+      },
+      nvec, m, out, s_buf);
+}
+
+// One warp checks a sequence's tokens / parents / capacity and derives ancestor bit masks and depths.  A chain's are known
+// in closed form; a tree's are walked in shared memory by one lane.
+__device__ void prepare_sequence(const BlockArgs& a, int b, int* s_parent, unsigned long long* s_anc, int* s_depth) {
+  const int lane = threadIdx.x & 31;
+  const int T = a.block_len[b], P = a.seq_len[b];
+  int err = 0;
+  if (T < 1 || T > a.T_max || P < 0) err = QUASAR_ERR_INVALID_ARG;
+  else if (P + T > a.s_max) err = QUASAR_ERR_CAPACITY;
+  const int n = err ? 0 : T;
+  int row_err[2] = {0, 0};
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int i = lane + 32 * h;
+    if (i < n) {
+      const int tok = a.tokens[b * a.T_max + i];
+      const int par = a.parents ? a.parents[b * a.T_max + i] : i - 1;
+      if (tok < 0 || tok >= a.vocab) row_err[h] = QUASAR_ERR_TOKEN;
+      if ((i == 0 && par != -1) || (i > 0 && (par < 0 || par >= i))) row_err[h] = QUASAR_ERR_TREE;
+      s_parent[i] = par;
+    }
+    const unsigned bad = __ballot_sync(0xffffffffu, row_err[h] != 0);
+    if (bad && !err) err = __shfl_sync(0xffffffffu, row_err[h], __ffs(bad) - 1);   // the first faulty row's error
+  }
+  __syncwarp();
+  if (!err && a.parents && lane == 0) {
+    for (int i = 0; i < n; ++i) {
+      const int p = s_parent[i];
+      s_anc[i] = (1ull << i) | (i > 0 ? s_anc[p] : 0ull);
+      s_depth[i] = i > 0 ? s_depth[p] + 1 : 0;
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int i = lane + 32 * h;
+    if (i >= a.T_max) continue;
+    const bool live = !err && i < n;
+    a.bi.anc[b * a.T_max + i] = !live ? 0ull : a.parents ? s_anc[i] : (i == 63 ? ~0ull : (1ull << (i + 1)) - 1ull);
+    a.bi.depth[b * a.T_max + i] = !live ? 0 : a.parents ? s_depth[i] : i;
+    if (a.keys != nullptr) a.keys[b * a.T_max + i] = 0ull;   // the rows' arg-max starts
+  }
+  if (lane == 0) {
+    a.bi.valid[b] = err ? 0 : 1;
+    if (err && a.status) atomicMin(a.status, err);
+  }
+}
+
+// The pass's first kernel: CTA m < M gathers the embedding of row m into the residual stream and normalises it; CTA M + b
+// does the bookkeeping of sequence b.
+template <int OP, int V>
+__global__ void __launch_bounds__(kRowThreads)
+embed_norm_kernel(BlockArgs a, int M, const __nv_bfloat16* __restrict__ embed, __nv_bfloat16* x, const __nv_bfloat16* __restrict__ g,
+                  int nvec, float eps, RowOperand out) {
+  __shared__ float s_buf[64];
+  __shared__ int s_parent[QUASAR_MAX_BLOCK], s_depth[QUASAR_MAX_BLOCK];
+  __shared__ unsigned long long s_anc[QUASAR_MAX_BLOCK];
+  pdl_trigger();
+  const int m = blockIdx.x;
+  if (m >= M) {
+    if (threadIdx.x < 32) prepare_sequence(a, m - M, s_parent, s_anc, s_depth);
+    return;
+  }
+  uint4 gain[V > 0 ? V : 1];
+  load_gain<V>(gain, g, nvec);
+  const int tok = a.tokens[m];
+  const bool ok = tok >= 0 && tok < a.vocab;
+  const uint4* src = reinterpret_cast<const uint4*>(embed) + (size_t)(ok ? tok : 0) * nvec;
+  uint4* dst = reinterpret_cast<uint4*>(x) + (size_t)m * nvec;
+  norm_row<OP, V>(
+      [&](int i, float (&f)[8]) {
+        const uint4 v = ok ? __ldg(src + i) : make_uint4(0, 0, 0, 0);
+        dst[i] = v;
+        unpack8(v, f);
+      },
+      gain, g, nvec, eps, m, out, s_buf);
+}
+
+// One warp per sequence: the rows' top choices out of their arg-max keys, then greedy acceptance (Eq. 2 at temperature
+// 0) in shared memory.
+__global__ void __launch_bounds__(32)
+accept_kernel(BlockArgs a, int32_t* __restrict__ accept_len, int32_t* __restrict__ bonus, int32_t* __restrict__ accept_path) {
+  __shared__ int s_tok[QUASAR_MAX_BLOCK], s_par[QUASAR_MAX_BLOCK], s_top[QUASAR_MAX_BLOCK], s_path[QUASAR_MAX_BLOCK];
+  pdl_trigger();
+  pdl_wait();
+  const int b = blockIdx.x, lane = threadIdx.x, base = b * a.T_max;
+  const bool valid = a.bi.valid[b] != 0;
+  const int T = valid ? a.block_len[b] : 0;
+  for (int i = lane; i < a.T_max; i += 32) {
+    s_path[i] = -1;
+    if (i < T) {
+      const unsigned long long k = a.keys[base + i];
+      s_top[i] = k == 0ull ? 0 : (int)(0xffffffffu - (uint32_t)(k & 0xffffffffull));
+      s_tok[i] = a.tokens[base + i];
+      s_par[i] = a.parents ? a.parents[base + i] : i - 1;
+    }
+  }
+  __syncwarp();
+  int n = -1, bon = -1;   // a skipped sequence: -1 tells quasar_kv_commit to leave its cache and seq_len alone
+  if (valid) {
+    int cur = 0;
+    n = 0;
+    if (lane == 0) s_path[0] = 0;
+    while (true) {   // the lowest row that follows `cur` and holds the verifier's choice
+      const int want = s_top[cur];
+      int nxt = -1;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = lane + 32 * h;
+        const unsigned hit = __ballot_sync(0xffffffffu, c > cur && c < T && s_par[c] == cur && s_tok[c] == want);
+        if (nxt < 0 && hit) nxt = 32 * h + __ffs(hit) - 1;
+      }
+      if (nxt < 0) break;
+      cur = nxt;
+      ++n;
+      if (lane == 0) s_path[n] = cur;
+    }
+    bon = s_top[cur];
+  }
+  __syncwarp();
+  if (lane == 0) {
+    accept_len[b] = n;
+    bonus[b] = bon;
+  }
+  if (accept_path != nullptr)
+    for (int i = lane; i < a.T_max; i += 32) accept_path[base + i] = s_path[i];
+}
+
+// turns of 8 * 512 elements a row takes, rounded up to a form that exists; 0: too long for registers
+int turns_of(int nvec) {
+  const int v = (nvec + kRowThreads - 1) / kRowThreads;
+  return v <= 1 ? 1 : v <= 2 ? 2 : v <= 3 ? 3 : v <= 6 ? 6 : 0;
+}
+
+template <typename... P, typename... A>
+int launch_row(void (*kernel)(P...), int grid, bool pdl, cudaStream_t stream, A&&... args) {
+  return launch_dependent(kernel, dim3((unsigned)grid), dim3(kRowThreads), 0, pdl, stream, static_cast<A&&>(args)...);
+}
+
+#define ROW_DISPATCH(KERNEL, ...)                                                                                              \
+  switch (turns_of(nvec)) {                                                                                                    \
+    case 1: ROW_DISPATCH_OP(KERNEL, 1, __VA_ARGS__)                                                                            \
+    case 2: ROW_DISPATCH_OP(KERNEL, 2, __VA_ARGS__)                                                                            \
+    case 3: ROW_DISPATCH_OP(KERNEL, 3, __VA_ARGS__)                                                                            \
+    case 6: ROW_DISPATCH_OP(KERNEL, 6, __VA_ARGS__)                                                                            \
+    default: ROW_DISPATCH_OP(KERNEL, 0, __VA_ARGS__)                                                                           \
+  }
+#define ROW_DISPATCH_OP(KERNEL, V, ...)                                                                                        \
+  switch (op) {                                                                                                                \
+    case kOperandDigits: return launch_row(KERNEL<kOperandDigits, V>, __VA_ARGS__);                                            \
+    case kOperandCodes: return launch_row(KERNEL<kOperandCodes, V>, __VA_ARGS__);                                              \
+    default: return launch_row(KERNEL<kOperandBf16, V>, __VA_ARGS__);                                                          \
+  }
+
+}  // namespace
+
+int launch_embed_norm(int op, const BlockArgs& a, const __nv_bfloat16* embed, __nv_bfloat16* x, const __nv_bfloat16* g, int H, float eps,
+                      const RowOperand& out, cudaStream_t stream) {
+  const int nvec = H / 8, M = a.B * a.T_max;
+  ROW_DISPATCH(embed_norm_kernel, M + a.B, false, stream, a, M, embed, x, g, nvec, eps, out)
+}
+
+int launch_norm(int op, const __nv_bfloat16* x, const __nv_bfloat16* g, int M, int H, float eps, const RowOperand& out, cudaStream_t stream) {
+  const int nvec = H / 8;
+  ROW_DISPATCH(norm_kernel, M, true, stream, x, g, nvec, eps, out)
+}
+
+int launch_swiglu(int op, const __nv_bfloat16* gu, int M, int F, const RowOperand& out, cudaStream_t stream) {
+  const int nvec = F / 8;
+  ROW_DISPATCH(swiglu_kernel, M, true, stream, gu, nvec, out)
+}
+
+int launch_operand(int op, const __nv_bfloat16* x, int M, int K, const RowOperand& out, cudaStream_t stream) {
+  if (op == kOperandBf16) return QUASAR_OK;   // the row itself is the operand
+  const int nvec = K / 8;
+  ROW_DISPATCH(operand_kernel, M, true, stream, x, nvec, out)
+}
+
+int launch_accept(const BlockArgs& a, int32_t* accept_len, int32_t* bonus, int32_t* accept_path, cudaStream_t stream) {
+  return launch_dependent(accept_kernel, dim3((unsigned)a.B), dim3(32), 0, true, stream, a, accept_len, bonus, accept_path);
+}
+
+}  // namespace quasar

@@ -1,0 +1,87 @@
+// Linear layers on the tcgen05 tensor cores (tc_linear.cu).
+#pragma once
+
+#include "common.cuh"
+
+namespace quasar {
+
+bool tc_linear_usable(int64_t M, int64_t N, int64_t K);
+
+// The launchers below take `pdl`: launched as a dependent of the kernel in front of it on the stream, whose results are waited
+// for before the activations, the residual or y are touched; the WEIGHTS may be read before that, so a caller sets it only
+// where the kernel in front does not write them and was itself launched behind whatever did.
+// y may be nullptr and keys not: then only the rows' arg-max over the output channels is wanted.
+
+int launch_tc_linear_bf16(const __nv_bfloat16* x, const __nv_bfloat16* w, int64_t M, int64_t N, int64_t K, void* y, bool y_is_f32,
+                          const __nv_bfloat16* residual, unsigned long long* keys, int32_t* error, bool pdl, cudaStream_t stream);
+
+// int8 weights, bf16 activations as digit rows: xd [3 M][K] int8 and row_scale [M], see write_digits8
+int launch_digit_rows3(const __nv_bfloat16* x, int64_t M, int64_t K, int8_t* xd, float* row_scale, cudaStream_t stream);
+int launch_tc_linear_digits(const int8_t* xd, const float* row_scale, const int8_t* w, const float* dw, int64_t M, int64_t N,
+                            int64_t K, void* y, bool y_is_f32, const __nv_bfloat16* residual, unsigned long long* keys, int32_t* error, bool pdl,
+                            cudaStream_t stream);
+
+// int8 weights, int8 activations with their step sizes (Eq. 8, Eq. 10); acc_out: the raw sums, or nullptr
+int launch_tc_linear_w8a8(const int8_t* xq, const float* dx, const int8_t* w, const float* dw, int64_t M, int64_t N, int64_t K,
+                          void* y, bool y_is_f32, const __nv_bfloat16* residual, int32_t* acc_out, unsigned long long* keys, int32_t* error, bool pdl,
+                          cudaStream_t stream);
+
+#ifdef __CUDACC__
+// Order-preserving key of a value and its index: the larger key is the larger value and, among equals, the lower index.
+__device__ __forceinline__ unsigned long long argmax_key(float x, int idx) {
+  x += 0.0f;                                            // -0 -> +0: they compare equal
+  uint32_t u = __float_as_uint(x);
+  u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+  return ((unsigned long long)u << 32) | (unsigned long long)(0xffffffffu - (uint32_t)idx);
+}
+
+constexpr int kDigitThreads = 256;
+
+__device__ __forceinline__ float digit_block_max(float v, float* s_max) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = v;
+  __syncthreads();
+  v = s_max[0];
+#pragma unroll
+  for (int i = 1; i < kDigitThreads / 32; ++i) v = fmaxf(v, s_max[i]);
+  return v;
+}
+
+// A row as fixed point against a power of two above its largest magnitude: x = q * 2^(E-21), |q| <= 2^21 (up = 2^(21-E),
+// down its inverse).
+__device__ __forceinline__ void digit_scale(float amax, float& up, float& down) {
+  up = 1.f;
+  down = 1.f;
+  if (amax > 0.f && amax < 3.0e38f) {
+    int e;
+    (void)frexpf(amax, &e);            // amax = f * 2^e, f in [0.5, 1): |x| < 2^e along the row
+    e = e < -100 ? -100 : e;           // keeps both factors normal numbers
+    up = ldexpf(1.f, 21 - e);
+    down = ldexpf(1.f, e - 21);
+  } else if (!(amax < 3.0e38f)) {
+    down = __int_as_float(0x7fc00000);   // a row holding inf or NaN gives NaN outputs
+  }
+}
+
+// q as three balanced base-256 digits, q = d0 + 256 d1 + 65536 d2, each an int8: eight elements from k on, plane d at d * K
+__device__ __forceinline__ void write_digits8(const float (&f)[8], float up, int8_t* dst, int64_t K, int64_t k) {
+  uint32_t p[3][2] = {{0u, 0u}, {0u, 0u}, {0u, 0u}};
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const float v = fminf(fmaxf(f[e] * up, -2097152.f), 2097152.f);
+    const int q = __float2int_rn(v);
+    const int a0 = (int)(int8_t)(q & 0xff);
+    const int q1 = (q - a0) >> 8;
+    const int a1 = (int)(int8_t)(q1 & 0xff);
+    const int a2 = (q1 - a1) >> 8;
+    p[0][e >> 2] |= (uint32_t)(a0 & 0xff) << (8 * (e & 3));
+    p[1][e >> 2] |= (uint32_t)(a1 & 0xff) << (8 * (e & 3));
+    p[2][e >> 2] |= (uint32_t)(a2 & 0xff) << (8 * (e & 3));
+  }
+#pragma unroll
+  for (int d = 0; d < 3; ++d) *reinterpret_cast<uint2*>(dst + d * K + k) = make_uint2(p[d][0], p[d][1]);
+}
+#endif
+
+}  // namespace quasar

@@ -10,6 +10,8 @@
 // shrink an outlier channel (the stated purpose) s_j = max|W_j|^(1-alpha) / max|X_j|^alpha, the reciprocal
 // of the expression printed as Eq. 5 (which is the factor the activations are divided by).
 #include "common.cuh"
+#include "tc_common.cuh"
+#include "tc_linear.cuh"
 
 namespace quasar {
 
@@ -54,6 +56,7 @@ template <int MODE>
 __global__ void __launch_bounds__(kQuantThreads)
 quantize_smoothed_kernel(const __nv_bfloat16* __restrict__ w, const float* __restrict__ s, int64_t K,
                          int8_t* __restrict__ q, float* __restrict__ delta) {
+  tc::pdl_trigger();   // (the contraction that follows in quasar_linear_w8a8 asks for its weights meanwhile)
   const int64_t n = blockIdx.x;
   const __nv_bfloat16* row = w + n * K;
   int8_t* qrow = q + n * K;
@@ -100,188 +103,9 @@ quantize_smoothed_kernel(const __nv_bfloat16* __restrict__ w, const float* __res
   }
 }
 
-// ---- the integer GEMM ---------------------------------------------------------------------------------
-// Same work split as the weight-only skinny GEMM: a CTA of 4 warps owns 64 output channels x one k-range,
-// the weights are the 16-row operand of mma.m16n8k32 (s8 x s8 -> s32), read once with 128-bit streaming
-// loads; the quantised activation rows are the 8-wide operand, staged in shared memory.  The contraction
-// index may be permuted freely as long as both operands agree: a lane's 16 contiguous weight bytes of one
-// row feed the k-slots of two MMAs and meet the 16 activation bytes at the same offsets.  Partial sums of
-// the k-ranges are int32: their reduction by the last CTA to arrive is exact whatever the order.
-constexpr int kWarps = 4;
-constexpr int kThreads = kWarps * 32;
-constexpr int kBlockN = kWarps * 16;
-constexpr int kSubK = 1024;      // contraction elements (bytes) staged at a time
-constexpr int kMaxSplit = 32;
-constexpr size_t kCounterBytes = 64 * 1024;
-constexpr int64_t kMaxChannels = (int64_t)(kCounterBytes / sizeof(int)) * kBlockN;
-
-struct A8Args {
-  const int8_t* xq;          // [M][K]
-  const float* dx;           // [M]
-  const int8_t* w;           // [N][K]
-  const float* dw;           // [N]
-  void* y;                   // [M][N] bf16 or fp32
-  const __nv_bfloat16* res;  // [M][N] or nullptr
-  int32_t* acc_out;          // [M][N] raw accumulators, or nullptr
-  int32_t* partial;          // [nsplit][NT*8][N]
-  int* counters;
-  int M, N, K, k_per_split, nsplit, y_is_f32;
-};
-
-__device__ __forceinline__ void mma_s8(int (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                       uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-      : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-// weights are read once: no L1 allocation, evict-first in L2 (the activations and partial sums are what is read again)
-__device__ __forceinline__ uint4 ldg_stream(const void* p) {
-  uint4 r;
-  uint64_t policy;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;\n" : "=l"(policy));
-  asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;\n"
-               : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
-               : "l"(p), "l"(policy));
-  return r;
-}
-
-__device__ __forceinline__ void a8_store(const A8Args& a, int acc, int m, int n) {
-  const size_t idx = (size_t)m * a.N + n;
-  if (a.acc_out != nullptr) a.acc_out[idx] = acc;
-  // Eq. 10: Y = Y_int32 * (delta_w * delta_x)
-  float v = __fmul_rn((float)acc, __fmul_rn(a.dw[n], a.dx[m]));
-  if (a.res != nullptr) v = __bfloat162float(__float2bfloat16_rn(v)) + __bfloat162float(a.res[idx]);
-  if (a.y_is_f32) reinterpret_cast<float*>(a.y)[idx] = v;
-  else reinterpret_cast<__nv_bfloat16*>(a.y)[idx] = __float2bfloat16_rn(v);
-}
-
-template <int NT>
-__global__ void __launch_bounds__(kThreads) w8a8_gemm_kernel(A8Args a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  uint4* xs = reinterpret_cast<uint4*>(smem_raw);   // [NT*8][kSubK/16] 16-byte pieces, swizzled by row parity
-  constexpr int kPieces = kSubK / 16;
-  constexpr int kUnroll = 4;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int n0 = blockIdx.x * kBlockN + warp * 16;
-  const int k_begin = blockIdx.y * a.k_per_split;
-  const int k_end = min(a.K, k_begin + a.k_per_split);
-  const int r0 = min(n0 + g, a.N - 1), r1 = min(n0 + g + 8, a.N - 1);
-  const int8_t* wrow0 = a.w + (size_t)r0 * a.K;
-  const int8_t* wrow1 = a.w + (size_t)r1 * a.K;
-
-  int acc[NT][4];
-#pragma unroll
-  for (int i = 0; i < NT; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0;
-
-  for (int kk = k_begin; kk < k_end; kk += kSubK) {
-    __syncthreads();
-    for (int c = threadIdx.x; c < NT * 8 * kPieces; c += kThreads) {
-      const int row = c / kPieces, pc = c % kPieces;
-      const int k = kk + pc * 16;
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (row < a.M && k < k_end) v = *reinterpret_cast<const uint4*>(a.xq + (size_t)row * a.K + k);
-      xs[row * kPieces + (pc ^ ((row & 1) << 2))] = v;
-    }
-    __syncthreads();
-#pragma unroll 1
-    for (int s0 = 0; s0 < kPieces / 4; s0 += kUnroll) {   // a warp step covers 64 contraction bytes
-      if (kk + s0 * 64 >= k_end) break;
-      uint4 wa[kUnroll], wb[kUnroll];
-#pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        const int k = kk + (s0 + u) * 64 + t * 16;
-        if (k < k_end) {
-          wa[u] = ldg_stream(wrow0 + k);
-          wb[u] = ldg_stream(wrow1 + k);
-        } else {
-          wa[u] = make_uint4(0, 0, 0, 0);
-          wb[u] = make_uint4(0, 0, 0, 0);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        const int pc = (s0 + u) * 4 + t;
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-          const int row = nt * 8 + g;
-          const uint4 x0 = xs[row * kPieces + (pc ^ ((row & 1) << 2))];
-          mma_s8(acc[nt], wa[u].x, wb[u].x, wa[u].y, wb[u].y, x0.x, x0.y);
-          mma_s8(acc[nt], wa[u].z, wb[u].z, wa[u].w, wb[u].w, x0.z, x0.w);
-        }
-      }
-    }
-  }
-
-  // acc[nt][0..1]: channel n0+g, rows nt*8+2t, +1;  acc[nt][2..3]: channel n0+g+8.
-  if (a.nsplit == 1) {
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int n = n0 + g + (e >> 1) * 8, m = nt * 8 + 2 * t + (e & 1);
-        if (n < a.N && m < a.M) a8_store(a, acc[nt][e], m, n);
-      }
-    }
-    return;
-  }
-  int32_t* mine = a.partial + (size_t)blockIdx.y * (NT * 8) * a.N;
-#pragma unroll
-  for (int nt = 0; nt < NT; ++nt) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int n = n0 + g + (e >> 1) * 8, m = nt * 8 + 2 * t + (e & 1);
-      if (n < a.N && m < a.M) __stcg(mine + (size_t)m * a.N + n, acc[nt][e]);
-    }
-  }
-  __threadfence();
-  __syncthreads();
-  __shared__ int s_last;
-  if (threadIdx.x == 0) s_last = (atomicAdd(a.counters + blockIdx.x, 1) == a.nsplit - 1);
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  const int nb = blockIdx.x * kBlockN;
-  for (int i = threadIdx.x; i < kBlockN * a.M; i += kThreads) {
-    const int n = nb + (i % kBlockN), m = i / kBlockN;
-    if (n >= a.N) continue;
-    int sum = 0;
-    for (int s = 0; s < a.nsplit; ++s) sum += __ldcg(a.partial + ((size_t)s * (NT * 8) + m) * a.N + n);
-    a8_store(a, sum, m, n);
-  }
-  if (threadIdx.x == 0) a.counters[blockIdx.x] = 0;   // ready for the next launch on this stream
-}
-
-struct SplitPlan {
-  int nblocks, nsplit, k_per_split;
-};
-
-SplitPlan plan_split(int64_t N, int64_t K) {
-  SplitPlan p;
-  p.nblocks = (int)((N + kBlockN - 1) / kBlockN);
-  const int subs = (int)((K + kSubK - 1) / kSubK);
-  int want = (148 * 4 + p.nblocks - 1) / p.nblocks;
-  want = want < 1 ? 1 : (want > subs ? subs : want);
-  want = want > kMaxSplit ? kMaxSplit : want;
-  const int subs_per = (subs + want - 1) / want;
-  p.k_per_split = subs_per * kSubK;
-  p.nsplit = (subs + subs_per - 1) / subs_per;
-  return p;
-}
-
-template <int NT>
-int launch_nt(const A8Args& a, const SplitPlan& p, cudaStream_t stream) {
-  const size_t smem = (size_t)NT * 8 * kSubK;
-  static bool configured = false;
-  if (smem > 48 * 1024 && !configured) {
-    QUASAR_CUDA_CHECK(cudaFuncSetAttribute(w8a8_gemm_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    configured = true;
-  }
-  w8a8_gemm_kernel<NT><<<dim3(p.nblocks, p.nsplit), kThreads, smem, stream>>>(a);
-  QUASAR_LAUNCH_CHECK();
-  return QUASAR_OK;
-}
+// The integer contraction (s8 x s8 -> s32, exact) and Eq. 10 are the tcgen05 kernel of tc_linear.cu.
+constexpr size_t kCounterBytes = 64 * 1024;   // reserved at the start of every workspace (quasar.h)
+constexpr int64_t kMaxChannels = (int64_t)1 << 20;
 
 size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
@@ -314,24 +138,8 @@ int launch_quantize_smoothed(const __nv_bfloat16* v, const float* s, int mode, i
 }
 
 size_t linear_w8a8_workspace_bytes(int64_t M, int64_t N, int64_t K) {
-  const SplitPlan p = plan_split(N, K);
-  const int64_t rows = M < kMaxRowsPerGemm ? M : kMaxRowsPerGemm;
-  const size_t mpad = (size_t)((rows + 7) / 8) * 8;
-  size_t partial = p.nsplit > 1 ? (size_t)p.nsplit * mpad * (size_t)N * sizeof(int32_t) : 0;
-  const int64_t rows_u = M < 80 ? M : 80;
-  if (umma_w8a8_usable(rows_u, N, K)) {
-    const size_t pu = umma_w8a8_partial_bytes(rows_u, N, K);
-    partial = pu > partial ? pu : partial;
-  }
-  return kCounterBytes + align256((size_t)M * K) + align256((size_t)M * sizeof(float)) + partial;
-}
-
-// where launch_linear_w8a8 keeps the quantised activation rows and their step sizes inside its workspace: a kernel that
-// produces the operand may write them there itself and pass x == nullptr
-void linear_w8a8_operand_slots(void* workspace, int64_t M, int64_t K, int8_t** xq, float** dx) {
-  unsigned char* ws = reinterpret_cast<unsigned char*>(workspace);
-  *xq = reinterpret_cast<int8_t*>(ws + kCounterBytes);
-  *dx = reinterpret_cast<float*>(ws + kCounterBytes + align256((size_t)M * K));
+  (void)N;
+  return kCounterBytes + align256((size_t)M * K) + align256((size_t)M * sizeof(float));
 }
 
 int launch_linear_w8a8(const __nv_bfloat16* x, const float* smooth, const int8_t* w, const float* delta_w, int64_t M,
@@ -349,58 +157,10 @@ int launch_linear_w8a8(const __nv_bfloat16* x, const float* smooth, const int8_t
   unsigned char* ws = reinterpret_cast<unsigned char*>(workspace);
   int8_t* xq = reinterpret_cast<int8_t*>(ws + kCounterBytes);
   float* dx = reinterpret_cast<float*>(ws + kCounterBytes + align256((size_t)M * K));
-  int32_t* partial = reinterpret_cast<int32_t*>(ws + kCounterBytes + align256((size_t)M * K) + align256((size_t)M * sizeof(float)));
   // Eq. 9: fused smoothing + per-token quantisation of the activations
-  if (x != nullptr) {   // (nullptr: the producer of the activations has already written xq and dx)
-    const int rc0 = launch_quantize_smoothed(x, smooth, kMultiply, M, K, xq, dx, stream);
-    if (rc0 != QUASAR_OK) return rc0;
-  }
-  const SplitPlan p = plan_split(N, K);
-  const size_t ybytes = y_is_f32 ? 4 : 2;
-  if (M > 8 && umma_w8a8_usable(M < 80 ? M : 80, N, K)) {
-    // blocks of more than 8 rows: the contraction runs on tcgen05 with the accumulator in tensor memory
-    for (int64_t m0 = 0; m0 < M; m0 += 80) {
-      const int64_t rows = (M - m0) < 80 ? (M - m0) : 80;
-      const int rc = launch_umma_w8a8(xq + m0 * K, dx + m0, w, delta_w, rows, N, K,
-                                      reinterpret_cast<unsigned char*>(y) + (size_t)m0 * N * ybytes, y_is_f32,
-                                      residual ? residual + m0 * N : nullptr, acc_out ? acc_out + m0 * N : nullptr,
-                                      reinterpret_cast<int*>(workspace), partial, status, stream);
-      if (rc != QUASAR_OK) return rc;
-    }
-    return QUASAR_OK;
-  }
-  for (int64_t m0 = 0; m0 < M; m0 += kMaxRowsPerGemm) {
-    A8Args a;
-    a.M = (int)((M - m0) < kMaxRowsPerGemm ? (M - m0) : kMaxRowsPerGemm);
-    a.N = (int)N;
-    a.K = (int)K;
-    a.xq = xq + m0 * K;
-    a.dx = dx + m0;
-    a.w = w;
-    a.dw = delta_w;
-    a.y = reinterpret_cast<unsigned char*>(y) + (size_t)m0 * N * ybytes;
-    a.res = residual ? residual + m0 * N : nullptr;
-    a.acc_out = acc_out ? acc_out + m0 * N : nullptr;
-    a.counters = reinterpret_cast<int*>(workspace);
-    a.partial = partial;
-    a.k_per_split = p.k_per_split;
-    a.nsplit = p.nsplit;
-    a.y_is_f32 = y_is_f32 ? 1 : 0;
-    int rc;
-    switch ((a.M + 7) / 8) {
-      case 1: rc = launch_nt<1>(a, p, stream); break;
-      case 2: rc = launch_nt<2>(a, p, stream); break;
-      case 3: rc = launch_nt<3>(a, p, stream); break;
-      case 4: rc = launch_nt<4>(a, p, stream); break;
-      case 5: rc = launch_nt<5>(a, p, stream); break;
-      case 6: rc = launch_nt<6>(a, p, stream); break;
-      case 7: rc = launch_nt<7>(a, p, stream); break;
-      case 8: rc = launch_nt<8>(a, p, stream); break;
-      default: rc = launch_nt<9>(a, p, stream); break;
-    }
-    if (rc != QUASAR_OK) return rc;
-  }
-  return QUASAR_OK;
+  const int rc = launch_quantize_smoothed(x, smooth, kMultiply, M, K, xq, dx, stream);
+  if (rc != QUASAR_OK) return rc;
+  return launch_tc_linear_w8a8(xq, dx, w, delta_w, M, N, K, y, y_is_f32, residual, acc_out, nullptr, status, true, stream);
 }
 
 }  // namespace quasar
