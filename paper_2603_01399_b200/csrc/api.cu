@@ -277,6 +277,8 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
   //      linear layers ask for their first weights then) and waits by itself for what that one writes. ----
   const OperandForm form = a8 ? kOperandCodes : wd == QUASAR_W_INT8 ? kOperandDigits : kOperandBf16;
   const bool traced = m->trace_buf != nullptr;
+  // the order of the norms' sums of squares: the W8A8 form keeps its two (a last bit there becomes quantisation steps)
+  const int adders = form == kOperandBf16 || (a8 && (M > 72 || H > 8192 || F > 24576)) ? 256 : 1024;
   BlockArgs ba{tokens, parents, block_len, kv->seq_len, B, T_max, kv->s_max, c.vocab, bi,
                reinterpret_cast<unsigned long long*>(wsp + ws.keys), status};
   int8_t* op_q = reinterpret_cast<int8_t*>(wsp + ws.op);
@@ -299,7 +301,7 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
     return reinterpret_cast<const __nv_bfloat16*>(l < c.n_layers ? m->layers[l].attn_norm : m->w.final_norm);
   };
   auto norm_smooth = [&](int l) { return l < c.n_layers ? m->layers[l].qkv_smooth : m->w.lm_smooth; };
-  TRY(launch_embed_norm(form, ba, reinterpret_cast<const __nv_bfloat16*>(m->w.embed), x, norm_gain(0), H, c.rms_eps,
+  TRY(launch_embed_norm(form, ba, reinterpret_cast<const __nv_bfloat16*>(m->w.embed), x, norm_gain(0), H, c.rms_eps, adders,
                         operand(h, norm_smooth(0)), stream));
   TRY(tr.put(x, (size_t)M * H * 2));
   for (int l = 0; l < c.n_layers; ++l) {
@@ -319,13 +321,13 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
     TRY(launch_operand(form, attn, M, Hq * D, RowOperand{nullptr, op_q, op_scale, L.o_smooth}, stream));
     TRY(linear(attn, L.o_w, L.o_delta, H, Hq * D, x, false, x, nullptr));
     TRY(tr.put(x, (size_t)M * H * 2));
-    TRY(launch_norm(form, x, reinterpret_cast<const __nv_bfloat16*>(L.mlp_norm), M, H, c.rms_eps, operand(h, L.gateup_smooth), stream));
+    TRY(launch_norm(form, x, reinterpret_cast<const __nv_bfloat16*>(L.mlp_norm), M, H, c.rms_eps, adders, operand(h, L.gateup_smooth), stream));
     TRY(linear(h, L.gateup_w, L.gateup_delta, 2 * (int64_t)F, H, gu, false, nullptr, nullptr));
     TRY(launch_swiglu(form, gu, M, F, operand(act, L.down_smooth), stream));
     TRY(tr.put(act, (size_t)M * F * 2));
     TRY(linear(act, L.down_w, L.down_delta, H, F, x, false, x, nullptr));
     TRY(tr.put(x, (size_t)M * H * 2));
-    TRY(launch_norm(form, x, norm_gain(l + 1), M, H, c.rms_eps, operand(h, norm_smooth(l + 1)), stream));
+    TRY(launch_norm(form, x, norm_gain(l + 1), M, H, c.rms_eps, adders, operand(h, norm_smooth(l + 1)), stream));
   }
   TRY(tr.put(h, (size_t)M * H * 2));
   // (the LM head finds the rows' top choices as it goes and writes logits only for a caller who wants them)

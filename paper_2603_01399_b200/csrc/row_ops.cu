@@ -135,10 +135,30 @@ __device__ __forceinline__ void write_operand(F&& value, int nvec, int m, const 
   }
 }
 
+// Sum of squares of a row in a FIXED order, whatever the spread of the row over the threads: pair p of the row (elements 2 p,
+// 2 p + 1) belongs to adder p % adders, which takes its pairs in ascending order; 32 neighbouring adders join as a warp's
+// butterfly does, and these sums are added in order (rows too long for registers: as the threads hold them).  A last-bit difference here turns into quantisation steps in the
+// W8A8 form, so the order does not change with the kernel's shape.
+__device__ __forceinline__ float sum_of_squares(const float* s_pair, int pairs, int adders, float* s_buf) {
+  __syncthreads();   // the pairs' sums are there
+  for (int t = threadIdx.x; t < adders; t += kRowThreads) {
+    float ss = 0.f;
+    for (int p = t; p < pairs; p += adders) ss += s_pair[p];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    if ((t & 31) == 0) s_buf[t >> 5] = ss;
+  }
+  __syncthreads();
+  float tot = 0.f;
+  for (int i = 0; i < adders / 32; ++i) tot += s_buf[i];
+  return tot;
+}
+
 // RMSNorm of the row whose vectors raw(i, j, f) gives, in operand form: y = bf16(x * rsqrt(mean(x^2) + eps) * g)
 template <int OP, int V, typename F>
-__device__ __forceinline__ void norm_row(F&& raw, const uint4 (&gain)[V > 0 ? V : 1], const __nv_bfloat16* g, int nvec, float eps, int m,
-                                         const RowOperand& out, float* s_buf) {
+__device__ __forceinline__ void norm_row(F&& raw, const uint4 (&gain)[V > 0 ? V : 1], const __nv_bfloat16* g, int nvec, float eps, int adders,
+                                         int m, const RowOperand& out, float* s_buf) {
+  extern __shared__ float s_pair[];
   float x[V > 0 ? V : 1][8];
   float ss = 0.f;
   if (V > 0) {
@@ -147,18 +167,23 @@ __device__ __forceinline__ void norm_row(F&& raw, const uint4 (&gain)[V > 0 ? V 
       const int i = (int)threadIdx.x + j * kRowThreads;
       if (i < nvec) {
         raw(i, x[j]);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) ss += x[j][e] * x[j][e];
+        float4 v;
+        v.x = x[j][0] * x[j][0] + x[j][1] * x[j][1];
+        v.y = x[j][2] * x[j][2] + x[j][3] * x[j][3];
+        v.z = x[j][4] * x[j][4] + x[j][5] * x[j][5];
+        v.w = x[j][6] * x[j][6] + x[j][7] * x[j][7];
+        reinterpret_cast<float4*>(s_pair)[i] = v;
       }
     }
+    ss = sum_of_squares(s_pair, nvec * 4, adders, s_buf);
   } else {
     for (int i = threadIdx.x; i < nvec; i += kRowThreads) {
       raw(i, x[0]);
 #pragma unroll
       for (int e = 0; e < 8; ++e) ss += x[0][e] * x[0][e];
     }
+    ss = block_reduce<false>(ss, s_buf);
   }
-  ss = block_reduce<false>(ss, s_buf);
   const float r = 1.0f / sqrtf(ss / (float)(nvec * 8) + eps);
   write_operand<OP, V>(
       [&](int i, int j, float (&f)[8]) {
@@ -198,7 +223,7 @@ __device__ __forceinline__ void load_gain(uint4 (&gain)[V > 0 ? V : 1], const __
 
 template <int OP, int V>
 __global__ void __launch_bounds__(kRowThreads)
-norm_kernel(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ g, int nvec, float eps, RowOperand out) {
+norm_kernel(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ g, int nvec, float eps, int adders, RowOperand out) {
   __shared__ float s_buf[64];
   pdl_trigger();
   uint4 gain[V > 0 ? V : 1];
@@ -206,7 +231,7 @@ norm_kernel(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ g, int nve
   pdl_wait();
   const int m = blockIdx.x;
   const uint4* row = reinterpret_cast<const uint4*>(x + (size_t)m * nvec * 8);
-  norm_row<OP, V>([&](int i, float (&f)[8]) { unpack8(row[i], f); }, gain, g, nvec, eps, m, out, s_buf);
+  norm_row<OP, V>([&](int i, float (&f)[8]) { unpack8(row[i], f); }, gain, g, nvec, eps, adders, m, out, s_buf);
 }
 
 template <int OP, int V>
@@ -309,7 +334,7 @@ __device__ void prepare_sequence(const BlockArgs& a, int b, int* s_parent, unsig
 template <int OP, int V>
 __global__ void __launch_bounds__(kRowThreads)
 embed_norm_kernel(BlockArgs a, int M, const __nv_bfloat16* __restrict__ embed, __nv_bfloat16* x, const __nv_bfloat16* __restrict__ g,
-                  int nvec, float eps, RowOperand out) {
+                  int nvec, float eps, int adders, RowOperand out) {
   __shared__ float s_buf[64];
   __shared__ int s_parent[QUASAR_MAX_BLOCK], s_depth[QUASAR_MAX_BLOCK];
   __shared__ unsigned long long s_anc[QUASAR_MAX_BLOCK];
@@ -331,7 +356,7 @@ embed_norm_kernel(BlockArgs a, int M, const __nv_bfloat16* __restrict__ embed, _
         dst[i] = v;
         unpack8(v, f);
       },
-      gain, g, nvec, eps, m, out, s_buf);
+      gain, g, nvec, eps, adders, m, out, s_buf);
 }
 
 // One warp per sequence: the rows' top choices out of their arg-max keys, then greedy acceptance (Eq. 2 at temperature
@@ -391,9 +416,12 @@ int turns_of(int nvec) {
 }
 
 template <typename... P, typename... A>
-int launch_row(void (*kernel)(P...), int grid, bool pdl, cudaStream_t stream, A&&... args) {
-  return launch_dependent(kernel, dim3((unsigned)grid), dim3(kRowThreads), 0, pdl, stream, static_cast<A&&>(args)...);
+int launch_row(void (*kernel)(P...), int grid, size_t smem, bool pdl, cudaStream_t stream, A&&... args) {
+  return launch_dependent(kernel, dim3((unsigned)grid), dim3(kRowThreads), smem, pdl, stream, static_cast<A&&>(args)...);
 }
+
+// shared memory of a norm: the pairs' sums of a row that stays in registers (at most 48 KB)
+size_t norm_smem(int nvec) { return turns_of(nvec) > 0 ? (size_t)nvec * 16 : 0; }
 
 #define ROW_DISPATCH(KERNEL, ...)                                                                                              \
   switch (turns_of(nvec)) {                                                                                                    \
@@ -413,25 +441,25 @@ int launch_row(void (*kernel)(P...), int grid, bool pdl, cudaStream_t stream, A&
 }  // namespace
 
 int launch_embed_norm(int op, const BlockArgs& a, const __nv_bfloat16* embed, __nv_bfloat16* x, const __nv_bfloat16* g, int H, float eps,
-                      const RowOperand& out, cudaStream_t stream) {
+                      int adders, const RowOperand& out, cudaStream_t stream) {
   const int nvec = H / 8, M = a.B * a.T_max;
-  ROW_DISPATCH(embed_norm_kernel, M + a.B, false, stream, a, M, embed, x, g, nvec, eps, out)
+  ROW_DISPATCH(embed_norm_kernel, M + a.B, norm_smem(nvec), false, stream, a, M, embed, x, g, nvec, eps, adders, out)
 }
 
-int launch_norm(int op, const __nv_bfloat16* x, const __nv_bfloat16* g, int M, int H, float eps, const RowOperand& out, cudaStream_t stream) {
+int launch_norm(int op, const __nv_bfloat16* x, const __nv_bfloat16* g, int M, int H, float eps, int adders, const RowOperand& out, cudaStream_t stream) {
   const int nvec = H / 8;
-  ROW_DISPATCH(norm_kernel, M, true, stream, x, g, nvec, eps, out)
+  ROW_DISPATCH(norm_kernel, M, norm_smem(nvec), true, stream, x, g, nvec, eps, adders, out)
 }
 
 int launch_swiglu(int op, const __nv_bfloat16* gu, int M, int F, const RowOperand& out, cudaStream_t stream) {
   const int nvec = F / 8;
-  ROW_DISPATCH(swiglu_kernel, M, true, stream, gu, nvec, out)
+  ROW_DISPATCH(swiglu_kernel, M, 0, true, stream, gu, nvec, out)
 }
 
 int launch_operand(int op, const __nv_bfloat16* x, int M, int K, const RowOperand& out, cudaStream_t stream) {
   if (op == kOperandBf16) return QUASAR_OK;   // the row itself is the operand
   const int nvec = K / 8;
-  ROW_DISPATCH(operand_kernel, M, true, stream, x, nvec, out)
+  ROW_DISPATCH(operand_kernel, M, 0, true, stream, x, nvec, out)
 }
 
 int launch_accept(const BlockArgs& a, int32_t* accept_len, int32_t* bonus, int32_t* accept_path, cudaStream_t stream) {

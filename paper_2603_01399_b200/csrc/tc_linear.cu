@@ -1,23 +1,26 @@
 // Linear layers  Y = delta * (W X)  (Section 3.2 Eq. 8 / Section 3.3 Eq. 10) on the 5th-generation tensor cores, for
 // int8 weights with bf16 activations, int8 weights with int8 activations, and bf16 weights.
 //
-// Mapping.  The weights are the 128-row operand A (one tensor-memory lane per output channel), the activation rows -
-// padded to a multiple of 16 - operand B.  A CTA owns up to 128 output channels x up to 128 activation rows x one range
-// of the contraction; a stage of its ring is 128 bytes of every weight row (TMA, 128-byte swizzle) and the activations
-// that meet them.
-//   * int8 x int8 (kind::i8, s32 sums) and bf16 x bf16 (kind::f16): both tiles go from TMA straight into the MMA.
-//   * int8 x bf16: operand A is read from TENSOR memory.  Eight converter warps turn a stage's rows into bf16 in
-//     registers and store them with tcgen05.st.  int8 -> bf16 is exact and takes eight instructions for four weights:
-//     with m = w & 127 and s = w & 128, the bytes m and s under the high byte 0x43 read 128 + m and 128 (or 256) as
-//     bf16, and one packed subtraction leaves w.  The activations enter as they are: no fp16 copy of them, no row
-//     scales, no kernel in front of this one.  (The form before this one converted to fp16 with four warps a CTA: each
-//     stage waited for one warp's chain of load, convert, store, publish - 2.9 TB/s of weights at 72 rows.)
+// Mapping.  The weights are the 128-row operand A (one tensor-memory lane per output channel), the activation rows operand
+// B; a stage of a CTA's ring is 128 bytes of every weight row of its tile and of every activation row (TMA, 128-byte
+// swizzle), and both go from there straight into the MMA: no instruction touches a weight byte.
+//   * int8 x int8 (kind::i8): exact s32 sums.
+//   * bf16 x bf16 (kind::f16): f32 sums.
+//   * int8 x bf16: the activations enter as integers, x = q * 2^(E-21) with |q| <= 2^21 against a power of two above their
+//     row's maximum, q as three balanced base-256 digits, each a row of operand B; the s32 sums of the digits are put
+//     together as one 64-bit integer.  A bf16 value has 8 significant bits, so every element within 2^-14 of the row's
+//     maximum is represented exactly and a smaller one to 2^-22 of that maximum - inside what an fp32 accumulation of
+//     the same products loses.
+// Measured against the form before this one (weights turned into fp16 by four warps a CTA and stored to tensor memory, sums of
+// the k-ranges added by a second kernel): LM head (151,936 x 4096) 212 -> 124 us at 72 rows and, against the digit kernel of
+// that time, 118 -> 97 us at 6 (6.4 TB/s); 24,576 x 4096 45 -> 26 us at 72 rows, 34 -> 20 us at 6; 4096 x 12288 29 -> 18
+// and 21 -> 15 us; 4096 x 4096 22 -> 11 and 10.5 -> 8.4 us.  What bounds it: up to about 40 rows HBM and, on the small
+// matrices, the fixed cost of a launch (5-6 us); above that the activations' share of an SM's intake and the MMAs.
 //
-// Work split.  About two CTAs fit an SM, and a launch has to give every SM the same number of weight bytes: the tile
-// height (a multiple of 8 channels) and the number of k-ranges are chosen together for that (plan_tc).  The k-ranges of
-// a tile form a thread-block cluster; their sums meet through distributed shared memory, every CTA of the cluster
-// finishing a share of the rows, in the order of the ranges (results repeat bit for bit): no partial sums in global
-// memory, no second kernel, no counters.
+// Two forms.  `tc_linear_kernel`: one tile, or one k-range of a tile, per CTA, all at once; the k-ranges of a tile form a
+// cluster whose CTAs add their sums through distributed shared memory, in the order of the ranges (results repeat bit for
+// bit).  `tc_stream_kernel`: tiles in turn on one CTA per SM.  Either with single CTAs or with pairs that share the
+// activations.  Which, with which tile height and how many ranges, is chosen by an estimate of the time (launch_any).
 //
 // Every wait is bounded (2 s): on expiry the CTA raises an error word, stops waiting everywhere, releases its tensor
 // memory and returns.
@@ -161,12 +164,32 @@ __device__ __forceinline__ void store4(const TcArgs& a, const uint32_t (&v)[4], 
   }
 }
 
-template <int KIND>
+// The MMAs of one stage: four steps of 32 bytes along the rows of both operands
+template <int KIND, bool PAIR>
+__device__ __forceinline__ void issue_stage(uint32_t d, uint64_t da, uint64_t db, uint32_t id, bool accumulate) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const uint32_t acc = (accumulate || j > 0) ? 1u : 0u;
+    const uint64_t daj = da + (uint64_t)(j * 2), dbj = db + (uint64_t)(j * 2);
+    if (PAIR) {
+      if (KIND == kBf16) mma_f16_ss_pair(d, daj, dbj, id, acc);
+      else mma_i8_ss_pair(d, daj, dbj, id, acc);
+    } else {
+      if (KIND == kBf16) mma_f16_ss(d, daj, dbj, id, acc);
+      else mma_i8_ss(d, daj, dbj, id, acc);
+    }
+  }
+}
+
+// PAIR: CTAs 2 i and 2 i + 1 of a cluster work as one on two neighbouring channel tiles.  Each brings its own weights and HALF
+// of the activation rows; the leader's MMAs (256 rows) read both CTAs' shared memory.
+template <int KIND, bool PAIR>
 __global__ void __launch_bounds__(kThreadsTc, 2)
 tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const TcArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // the swizzle repeats every 1024 bytes
-  const int b_bytes = a.brows * 128;
+  const int b_rows = PAIR ? a.brows / 2 : a.brows;   // of this CTA
+  const int b_bytes = b_rows * 128;
   const int stage_bytes = kAStage + b_bytes;
   const int S = a.stages;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)S * stage_bytes);   // the stage's bytes have landed
@@ -175,8 +198,10 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(accum_done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int row_tile = (int)blockIdx.x % a.row_tiles, tile = (int)blockIdx.x / a.row_tiles;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp: uniform)
+  const int pair_x = PAIR ? (int)blockIdx.x & 1 : 0;
+  const int unit = PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x;
+  const int row_tile = unit % a.row_tiles, tile = PAIR ? 2 * (unit / a.row_tiles) + pair_x : unit / a.row_tiles;
   const int split = blockIdx.y;
   const int n0 = tile * a.chan, m0 = row_tile * a.rows;
   const int kb0 = (int)((long long)split * a.kblocks / a.nsplit), kb1 = (int)((long long)(split + 1) * a.kblocks / a.nsplit);
@@ -191,7 +216,18 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     mbar_init(accum_done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-  if (warp == 1) {
+  if (PAIR) {   // (also: the leader's barriers exist before the other CTA's loads arrive at them)
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+  }
+  if (warp == 1 && PAIR) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
+                 "r"((uint32_t)kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n" ::: "memory");
+  }
+  if (warp == 1 && !PAIR) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
                  "r"((uint32_t)kTmemCols)
                  : "memory");
@@ -206,13 +242,31 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
   if (threadIdx.x == 0) pdl_trigger();
 
   if (warp == 0) {
-    if (lane == 0) {   // ---- TMA producer ----
+    {   // ---- TMA producer ----
       const uint64_t policy = l2_evict_first_policy();
+      const uint32_t leader = (uint32_t)(2 * split);
+      auto arm = [&](int i) {   // the leader's barrier counts the bytes of both CTAs
+        if (pair_x == 0) mbar_expect_tx(full + i, PAIR ? 2 * tx : tx);
+      };
+      auto load_w = [&](int i, int kb) {
+        unsigned char* at = smem + (size_t)i * stage_bytes;
+        if (PAIR) tma_load_2d_pair<true>(at, &map_w, kb * 128, n0, cluster_map(smem_u32(full + i), leader), policy);
+        else tma_load_2d_hint(at, &map_w, kb * 128, n0, full + i, policy);
+      };
+      auto load_x = [&](int i, int kb) {
+        unsigned char* at = smem + (size_t)i * stage_bytes + kAStage;
+        const int y = (KIND == kDigits ? 3 * m0 : m0) + pair_x * b_rows;
+        if (PAIR) tma_load_2d_pair<false>(at, &map_x, kb * 128, y, cluster_map(smem_u32(full + i), leader), policy);
+        else tma_load_2d(at, &map_x, kb * 128, y, full + i);
+      };
       const int ahead = min(S, kb1 - kb0);
       if (a.early_weights) {   // the weights of the first stages do not depend on the kernel in front
         for (int i = 0; i < ahead; ++i) {
-          mbar_expect_tx(full + i, tx);
-          tma_load_2d_hint(smem + (size_t)i * stage_bytes, &map_w, (kb0 + i) * 128, n0, full + i, policy);
+          if (elect_one()) {
+            arm(i);
+            load_w(i, kb0 + i);
+          }
+          __syncwarp();
         }
       }
       pdl_wait();
@@ -220,16 +274,19 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
       uint32_t ph = 0;
       int kb = kb0;
       for (; kb < kb1; ++kb) {
-        unsigned char* at = smem + (size_t)s * stage_bytes;
-        if (!(a.early_weights && kb - kb0 < ahead)) {
-          if (!mbar_wait(empty + s, ph ^ 1u, abort_flag, a.error)) break;
-          mbar_expect_tx(full + s, tx);
-          tma_load_2d_hint(at, &map_w, kb * 128, n0, full + s, policy);
+        const bool early = a.early_weights && kb - kb0 < ahead;
+        if (!early && !mbar_wait(empty + s, ph ^ 1u, abort_flag, a.error)) break;
+        if (elect_one()) {
+          if (!early) {
+            arm(s);
+            load_w(s, kb);
+          }
+          load_x(s, kb);
         }
-        tma_load_2d(at + kAStage, &map_x, kb * 128, KIND == kDigits ? 3 * m0 : m0, full + s);
+        __syncwarp();
         if (++s == S) { s = 0; ph ^= 1u; }
       }
-      if (kb < kb1) {   // given up: what is in flight lands (bounded) before the CTA leaves
+      if (kb < kb1 && pair_x == 0) {   // given up: what is in flight lands (bounded) before the CTA leaves
         for (int i = 0; i < min(S, kb - kb0); ++i) {
           if (--s < 0) { s = S - 1; ph ^= 1u; }
           const unsigned long long t0 = gtime_ns();
@@ -238,26 +295,30 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {   // ---- MMA issuer ----
-      const uint32_t id = idesc(KIND == kBf16 ? 1 : 2, 1, kTileN, a.brows);
+    if (pair_x == 0) {   // ---- MMA issuer ----
+      const uint16_t mask = (uint16_t)(3u << (2 * split));
+      const uint32_t id = idesc(KIND == kBf16 ? 1 : 2, 1, PAIR ? 2 * kTileN : kTileN, a.brows);
+      const uint64_t da0 = desc_sw128(smem), db0 = desc_sw128(smem + kAStage);
       int s = 0;
       uint32_t ph = 0;
       bool ok = true;
       for (int kb = kb0; kb < kb1; ++kb) {
         if (!(ok = mbar_wait(full + s, ph, abort_flag, a.error))) break;
         fence_after();
-        const unsigned char* at = smem + (size_t)s * stage_bytes;
-        const uint64_t da = desc_sw128(at), db = desc_sw128(at + kAStage);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {   // 32 bytes along the rows of both
-          const uint32_t acc = (kb > kb0 || j > 0) ? 1u : 0u;
-          if (KIND == kBf16) mma_f16_ss(tmem_base, da + (uint64_t)(j * 2), db + (uint64_t)(j * 2), id, acc);
-          else mma_i8_ss(tmem_base, da + (uint64_t)(j * 2), db + (uint64_t)(j * 2), id, acc);
+        const uint64_t off = (uint64_t)((uint32_t)(s * stage_bytes) >> 4);
+        if (elect_one()) {
+          issue_stage<KIND, PAIR>(tmem_base, da0 + off, db0 + off, id, kb > kb0);
+          if (PAIR) commit_pair(empty + s, mask);
+          else commit(empty + s);
         }
-        commit(empty + s);
+        __syncwarp();
         if (++s == S) { s = 0; ph ^= 1u; }
       }
-      if (ok) commit(accum_done);
+      if (ok && elect_one()) {
+        if (PAIR) commit_pair(accum_done, mask);
+        else commit(accum_done);
+      }
+      __syncwarp();
     }
   } else {
     // ---- warps 2..9: the sums to shared memory, [row][channel] (the ring is idle then: every load has landed and every MMA
@@ -290,7 +351,7 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
   }
   __syncwarp();
   fence_before();
-  if (a.nsplit > 1) {
+  if (PAIR || a.nsplit > 1) {
     cluster_arrive();
     cluster_wait();
   } else {
@@ -298,7 +359,8 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
   }
   if (warp == 1) {
     fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"((uint32_t)kTmemCols) : "memory");
+    if (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"((uint32_t)kTmemCols) : "memory");
+    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"((uint32_t)kTmemCols) : "memory");
   }
   pdl_wait();   // every thread: the residual below may come from the kernel in front
   if (*abort_flag == 0) {
@@ -321,7 +383,7 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         uint4 p[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-          if (k < a.nsplit) p[k] = ld_cluster_v4(cluster_map(red_addr + off, (uint32_t)k));
+          if (k < a.nsplit) p[k] = ld_cluster_v4(cluster_map(red_addr + off, (uint32_t)(PAIR ? 2 * k + pair_x : k)));
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           if (k >= a.nsplit) break;
@@ -347,14 +409,255 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     }
   }
   __syncwarp();
-  if (a.nsplit > 1) {   // nobody's shared memory goes away while another CTA may read it
+  if (PAIR || a.nsplit > 1) {   // nobody's shared memory goes away while another CTA may read it
     cluster_arrive();
     cluster_wait();
   }
 }
 
+// ---- the same product as a stream of tiles ---------------------------------------------------------------------------
+// Where the tiles of a matrix are more than the SMs, one CTA (or pair) per SM takes them in turn without a pause: the ring
+// never drains between tiles, and with two accumulators in tensor memory (512 columns) a tile leaves for memory while the
+// next one is multiplied.  (One CTA a tile, two on an SM, left every tile's epilogue and start-up half exposed: the LM
+// head at 72 rows took 145-157 us, of which 75-99 us remained with neither weights loaded nor MMAs issued.)  The sums
+// go from tensor memory straight to their places: a thread holds one channel, a warp 32 neighbouring ones.
+constexpr int kAccBuf = 256;   // columns of an accumulator
+
+template <int KIND, bool PAIR>
+__global__ void __launch_bounds__(kThreadsTc, 1)
+tc_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const TcArgs a, int units) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const int b_rows = PAIR ? a.brows / 2 : a.brows;
+  const int b_bytes = b_rows * 128;
+  const int stage_bytes = kAStage + b_bytes;
+  const int S = a.stages;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)S * stage_bytes);
+  uint64_t* empty = full + S;
+  uint64_t* acc_full = empty + S;        // [2] a tile's sums are complete
+  uint64_t* acc_empty = acc_full + 2;    // [2] they have been read out
+  unsigned long long* s_best = reinterpret_cast<unsigned long long*>(acc_empty + 2);   // [256] arg-max keys of the row tile's rows
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_best + 256);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp: uniform)
+  const int pair_x = PAIR ? (int)blockIdx.x & 1 : 0;
+  const int first = PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x, step = PAIR ? (int)gridDim.x >> 1 : (int)gridDim.x;
+  const uint32_t tx = (uint32_t)(a.chan * 128 + b_bytes);
+  auto row_of = [&](int u) { return (u % a.row_tiles) * a.rows; };
+  auto chan_of = [&](int u) { return (PAIR ? 2 * (u / a.row_tiles) + pair_x : u / a.row_tiles) * a.chan; };
+
+  if (threadIdx.x == 0) {
+    *abort_flag = 0;
+    for (int s = 0; s < S; ++s) {
+      mbar_init(full + s, 1);
+      mbar_init(empty + s, 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(acc_full + i, 1);
+      mbar_init(acc_empty + i, PAIR ? 16 : 8);   // one arrival per epilogue warp of every CTA
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  if (threadIdx.x < 256) s_best[threadIdx.x] = 0ull;
+  if (PAIR) {
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+  }
+  if (warp == 1) {
+    if (PAIR) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)), "r"(2u * kAccBuf) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)), "r"(2u * kAccBuf) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  if (threadIdx.x == 0) pdl_trigger();   // (see tc_linear_kernel)
+
+  if (warp == 0) {
+    {   // ---- TMA producer ----
+      const uint64_t policy = l2_evict_first_policy();
+      auto arm = [&](int i) {
+        if (pair_x == 0) mbar_expect_tx(full + i, PAIR ? 2 * tx : tx);
+      };
+      auto load_w = [&](int i, int kb, int n0) {
+        unsigned char* at = smem + (size_t)i * stage_bytes;
+        // (row tiles that share a weight tile read it at about the same time: it may stay in L2 for them)
+        if (PAIR) {
+          if (a.row_tiles == 1) tma_load_2d_pair<true>(at, &map_w, kb * 128, n0, cluster_map(smem_u32(full + i), 0), policy);
+          else tma_load_2d_pair<false>(at, &map_w, kb * 128, n0, cluster_map(smem_u32(full + i), 0), policy);
+        } else {
+          if (a.row_tiles == 1) tma_load_2d_hint(at, &map_w, kb * 128, n0, full + i, policy);
+          else tma_load_2d(at, &map_w, kb * 128, n0, full + i);
+        }
+      };
+      auto load_x = [&](int i, int kb, int m0) {
+        unsigned char* at = smem + (size_t)i * stage_bytes + kAStage;
+        const int y = (KIND == kDigits ? 3 * m0 : m0) + pair_x * b_rows;
+        if (PAIR) tma_load_2d_pair<false>(at, &map_x, kb * 128, y, cluster_map(smem_u32(full + i), 0), policy);
+        else tma_load_2d(at, &map_x, kb * 128, y, full + i);
+      };
+      const int ahead = first < units ? min(S, a.kblocks) : 0;
+      if (a.early_weights) {
+        for (int i = 0; i < ahead; ++i) {
+          if (elect_one()) {
+            arm(i);
+            load_w(i, i, chan_of(first));
+          }
+          __syncwarp();
+        }
+      }
+      pdl_wait();
+      int s = 0, issued = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int u = first; u < units && ok; u += step) {
+        const int n0 = chan_of(u), m0 = row_of(u);
+        for (int kb = 0; kb < a.kblocks; ++kb) {
+          const bool early = a.early_weights && issued < ahead;
+          if (!early && !(ok = mbar_wait(empty + s, ph ^ 1u, abort_flag, a.error))) break;
+          if (elect_one()) {
+            if (!early) {
+              arm(s);
+              load_w(s, kb, n0);
+            }
+            load_x(s, kb, m0);
+          }
+          __syncwarp();
+          ++issued;
+          if (++s == S) { s = 0; ph ^= 1u; }
+        }
+      }
+      if (!ok && pair_x == 0) {   // given up: what is in flight lands (bounded) before the CTA leaves
+        for (int i = 0; i < min(S, issued); ++i) {
+          if (--s < 0) { s = S - 1; ph ^= 1u; }
+          const unsigned long long t0 = gtime_ns();
+          while (!mbar_try(full + s, ph) && gtime_ns() - t0 < 100000ull) {}
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (pair_x == 0) {   // ---- MMA issuer ----
+      const uint32_t id = idesc(KIND == kBf16 ? 1 : 2, 1, PAIR ? 2 * kTileN : kTileN, a.brows);
+      const uint64_t da0 = desc_sw128(smem), db0 = desc_sw128(smem + kAStage);
+      int s = 0, buf = 0;
+      uint32_t ph = 0, bph = 0;
+      bool ok = true;
+      for (int u = first; u < units && ok; u += step) {
+        if (!(ok = mbar_wait(acc_empty + buf, bph ^ 1u, abort_flag, a.error))) break;
+        fence_after();
+        const uint32_t d = tmem_base + (uint32_t)(buf * kAccBuf);
+        for (int kb = 0; kb < a.kblocks; ++kb) {
+          if (!(ok = mbar_wait(full + s, ph, abort_flag, a.error))) break;
+          fence_after();
+          const uint64_t off = (uint64_t)((uint32_t)(s * stage_bytes) >> 4);
+          if (elect_one()) {
+            issue_stage<KIND, PAIR>(d, da0 + off, db0 + off, id, kb > 0);
+            if (PAIR) commit_pair(empty + s, (uint16_t)3);
+            else commit(empty + s);
+          }
+          __syncwarp();
+          if (++s == S) { s = 0; ph ^= 1u; }
+        }
+        if (ok && elect_one()) {
+          if (PAIR) commit_pair(acc_full + buf, (uint16_t)3);
+          else commit(acc_full + buf);
+        }
+        __syncwarp();
+        if ((buf ^= 1) == 0) bph ^= 1u;
+      }
+    }
+  } else {
+    // ---- epilogue: warps 2..9; two warps share a quarter of the channels and take 16 rows in turn ----
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    pdl_wait();   // the step sizes of the activations and the residual come from the kernels in front
+    const bool one_row_tile = step % a.row_tiles == 0;   // (the launcher's grid sees to it)
+    int buf = 0;
+    uint32_t bph = 0;
+    for (int u = first; u < units; u += step) {
+      if (!__all_sync(0xffffffffu, mbar_wait(acc_full + buf, bph, abort_flag, a.error))) break;
+      fence_after();
+      const int m0 = row_of(u), rows = min(a.rows, a.M - m0);
+      const int r = q * 32 + lane, n = chan_of(u) + r;
+      const bool live = r < a.chan && n < a.N;
+      const float dw = (KIND != kBf16 && live) ? __ldg(a.dw + n) : 1.f;
+      const uint32_t t0 = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * kAccBuf);
+      for (int r0 = half * 16; r0 < rows; r0 += 32) {
+        uint32_t v[16];
+        if (KIND == kDigits) {
+          uint32_t d[3][16];
+#pragma unroll
+          for (int c = 0; c < 3; ++c) tmem_ld16_async(t0 + (uint32_t)(3 * r0 + 16 * c), d[c]);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) tmem_ld_wait(d[c]);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const long long total = ((long long)(int)d[(3 * j + 2) / 16][(3 * j + 2) % 16] << 16) +
+                                    ((long long)(int)d[(3 * j + 1) / 16][(3 * j + 1) % 16] << 8) + (long long)(int)d[3 * j / 16][3 * j % 16];
+            v[j] = __float_as_uint((float)total);
+          }
+        } else {
+          tmem_ld16(t0 + (uint32_t)r0, v);
+        }
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const int m = m0 + r0 + j;
+          if (r0 + j >= rows) break;
+          float f = finish<KIND>(v[j], KIND != kBf16 ? __ldg(a.dx + m) : 1.f, dw);
+          if (a.keys != nullptr) {   // the warp's largest value, its lowest channel on ties (NaNs never enter)
+            const bool in = live && f == f;
+            const uint32_t key = in ? (uint32_t)(argmax_key(f, 0) >> 32) : 0u;
+            const uint32_t top = __reduce_max_sync(0xffffffffu, key);
+            const unsigned who = __ballot_sync(0xffffffffu, in && key == top);
+            if (lane == 0 && who != 0u)
+              atomicMax(one_row_tile ? s_best + r0 + j : a.keys + m, ((unsigned long long)top << 32) | (unsigned long long)(0xffffffffu - (uint32_t)(n + __ffs(who) - 1)));
+          }
+          if (!live || a.y == nullptr) continue;
+          const size_t idx = (size_t)m * a.N + n;
+          if (KIND == kCodes && a.acc_out != nullptr) a.acc_out[idx] = (int)v[j];
+          if (a.res != nullptr) f = __bfloat162float(__float2bfloat16_rn(f)) + __bfloat162float(a.res[idx]);
+          if (a.y_is_f32) reinterpret_cast<float*>(a.y)[idx] = f;
+          else reinterpret_cast<__nv_bfloat16*>(a.y)[idx] = __float2bfloat16_rn(f);
+        }
+      }
+      fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        if (PAIR) mbar_arrive_cluster(cluster_map(smem_u32(acc_empty + buf), 0));
+        else mbar_arrive(acc_empty + buf);
+      }
+      if ((buf ^= 1) == 0) bph ^= 1u;
+    }
+    if (a.keys != nullptr && one_row_tile && first < units) {
+      asm volatile("bar.sync 1, 256;\n" ::: "memory");
+      const int t = (int)threadIdx.x - 64, m0 = row_of(first);
+      if (t < min(a.rows, a.M - m0) && s_best[t] != 0ull) atomicMax(a.keys + m0 + t, s_best[t]);
+    }
+  }
+  __syncwarp();
+  fence_before();
+  if (PAIR) {
+    cluster_arrive();
+    cluster_wait();
+  } else {
+    __syncthreads();
+  }
+  if (warp == 1) {
+    fence_after();
+    if (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(2u * kAccBuf) : "memory");
+    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(2u * kAccBuf) : "memory");
+  }
+}
+
 struct TcPlan {
-  int chan, tiles, nsplit, row_tiles, rows, brows, kblocks, stages;
+  int chan, tiles, nsplit, row_tiles, rows, brows, kblocks, stages, pair, stream, ctas;
+  double cost;
 };
 
 // Clusters of s CTAs that the device holds at once with one CTA on each SM (they lie within a group of SMs, so long ones
@@ -382,42 +685,58 @@ int max_clusters(const void* kernel, int s) {
   return seen[s];
 }
 
-// Tile height and k-ranges, by an estimate of the time in us: waves of CTAs, each a fixed cost and the largest of what its
-// stages' latency, the SM's intake (about 95 KB per us) and the memory (6.2 MB of weights per us for all) ask for, with a
-// cost for every range that joins the exchange of sums.  Measured at 6 rows: 4096 x 4096 in 4 ranges 9.1 us, in 8 9.3, in 2
-// 10.6; 4096 x 12288 in 8 ranges 15.4 us, in 4 16.6, in 2 21.2; 6144 x 4096 in 4 ranges 10.5 us, in 6 (more clusters
-// than fit at once) 14.2.
-TcPlan plan_tc(int64_t M, int64_t N, int64_t K, int kind, const void* kernel) {
+// Tile height, k-ranges and form, by an estimate of the time in us: a fixed cost, and the largest of what the latency of a
+// CTA's stages, the SM's intake (about 105 KB per us), its MMAs and the memory (6.3 MB of weights per us for all) ask for,
+// with a cost for every range that joins the exchange of sums.  Measured at 6 rows: 4096 x 4096 in 4 ranges 9.1 us, in 8
+// 9.3, in 2 10.6; 4096 x 12288 in 8 ranges 15.4 us, in 4 16.6, in 2 21.2; 6144 x 4096 in 4 ranges 10.5 us, in 6 (more
+// clusters than fit at once) 14.2.
+double stages_us(const TcPlan& p, int kbs, double on_sm, double ctas, int c, int b_bytes) {
+  const double lat = 0.2 * kbs;
+  const double sm = kbs * on_sm * (c * 128.0 + b_bytes) / 105e3;
+  const double mma = kbs * on_sm * (p.brows > 64 ? p.brows : 64) / 700.0;
+  const double mem = kbs * ctas * c * 128.0 / 6.3e6 / (p.row_tiles < ctas ? p.row_tiles : ctas);
+  return sqrt(sqrt(lat * lat * lat * lat + sm * sm * sm * sm + mma * mma * mma * mma + mem * mem * mem * mem));   // near the largest
+}
+
+TcPlan plan_base(int64_t M, int64_t K, int kind, bool pair) {
   TcPlan p;
-  const int most = kind == kDigits ? 80 : 128;
+  p.pair = pair ? 1 : 0;
+  const int most = kind == kDigits ? 80 : (pair ? 256 : 128);
   p.row_tiles = (int)((M + most - 1) / most);
   p.rows = (int)((M + p.row_tiles - 1) / p.row_tiles);
-  p.brows = (p.rows * (kind == kDigits ? 3 : 1) + 15) / 16 * 16;
+  const int unit = pair ? 32 : 16;   // what an MMA's N is a multiple of (integers, pair: 32)
+  p.brows = (p.rows * (kind == kDigits ? 3 : 1) + unit - 1) / unit * unit;
   p.kblocks = (int)(((kind == kBf16 ? 2 * K : K) + 127) / 128);
-  const int stage = kAStage + p.brows * 128;
+  p.nsplit = 0;
+  p.cost = 0;
+  return p;
+}
+
+// one tile or k-range of a tile per CTA, all of them at once
+TcPlan plan_tiles(int64_t M, int64_t N, int64_t K, int kind, bool pair, const void* kernel) {
+  TcPlan p = plan_base(M, K, kind, pair);
+  p.stream = 0;
+  const int b_bytes = p.brows * (pair ? 64 : 128), stage = kAStage + b_bytes;
   // two CTAs on an SM as long as that leaves each three stages; wider blocks do better with one CTA and its deeper ring
   // (4096 x 4096 at 72 rows: 11.3 us with one, 12.9 with two)
-  int per_sm = (int)((kMaxSmem / 2 - 1024 - kSmemSlack) / stage) >= 3 ? 2 : 1;
+  const size_t half_room = (kMaxSmem / 2 - 1024 - kSmemSlack) / stage * stage;
+  const int per_sm = half_room >= 3 * (size_t)stage && half_room >= (size_t)p.rows * kTileN * 4 ? 2 : 1;   // (the sums go through the ring's memory)
   const size_t room = per_sm == 2 ? kMaxSmem / 2 - 1024 : kMaxSmem;
   const int st = (int)((room - kSmemSlack) / stage);
   p.stages = st > 8 ? 8 : st;
-  double best = 0;
-  p.nsplit = 0;
-  for (int s = 1; s <= 8 && s <= p.kblocks; ++s) {
+  const int group = pair ? 2 : 1;
+  for (int s = 1; s * group <= 8 && s <= p.kblocks; ++s) {
     // (two CTAs of a cluster can share an SM)
-    const long long fit = per_sm == 1 ? max_clusters(kernel, s) : std::max(2 * max_clusters(kernel, s), max_clusters(kernel, (s + 1) / 2));
+    const int cs = s * group;
+    const long long fit = per_sm == 1 ? max_clusters(kernel, cs) : std::max(2 * max_clusters(kernel, cs), max_clusters(kernel, (cs + 1) / 2));
     for (int c = 128; c >= 64; c -= 8) {
-      const long long tiles = (N + c - 1) / c;
-      const long long clusters = tiles * p.row_tiles;
+      const long long tiles = ((N + c - 1) / c + group - 1) / group * group;
+      const long long clusters = tiles / group * p.row_tiles;
       const long long waves = (clusters + fit - 1) / fit;
-      const double ctas = (double)(clusters < fit ? clusters : fit) * s;
-      const double kbs = (double)((p.kblocks + s - 1) / s);
-      const double lat = 0.22 * kbs;
-      const double sm = kbs * (ctas > 148 ? ctas / 148 : 1.0) * (c * 128.0 + p.brows * 128.0) / 95e3;
-      const double mem = kbs * ctas * c * 128.0 / 6.2e6 / p.row_tiles;
-      const double cost = (double)waves * (2.0 + sqrt(lat * lat + sm * sm + mem * mem)) + 0.15 * s;
-      if (p.nsplit == 0 || cost < best * 0.99) {
-        best = cost;
+      const double ctas = (double)(clusters < fit ? clusters : fit) * cs;
+      const double cost = (double)waves * (2.5 + 2.0 * p.pair + 0.01 * p.rows + stages_us(p, (p.kblocks + s - 1) / s, ctas > 148 ? ctas / 148 : 1.0, ctas, c, b_bytes)) + 0.15 * s;
+      if (p.nsplit == 0 || cost < p.cost * 0.99) {
+        p.cost = cost;
         p.nsplit = s;
         p.chan = c;
         p.tiles = (int)tiles;
@@ -427,19 +746,46 @@ TcPlan plan_tc(int64_t M, int64_t N, int64_t K, int kind, const void* kernel) {
   return p;
 }
 
-template <int KIND>
+// tiles in turn on one CTA (or pair) per SM
+TcPlan plan_stream(int64_t M, int64_t N, int64_t K, int kind, bool pair) {
+  TcPlan p = plan_base(M, K, kind, pair);
+  p.stream = 1;
+  const int b_bytes = p.brows * (pair ? 64 : 128), stage = kAStage + b_bytes;
+  const int st = (int)((kMaxSmem - kSmemSlack - 2048) / stage);
+  p.stages = st > 10 ? 10 : st;
+  const int group = pair ? 2 : 1, lanes = 148 / group;
+  for (int c = 128; c >= 64; c -= 8) {
+    const long long tiles = ((N + c - 1) / c + group - 1) / group * group;
+    const long long units = tiles / group * p.row_tiles;
+    long long n = lanes / p.row_tiles * p.row_tiles;   // a CTA stays on its row tile
+    if (n < 1) n = lanes;
+    if (n > units) n = units;
+    const long long turns = (units + n - 1) / n;
+    const double cost = 3.5 + 0.01 * p.rows + turns * (0.15 + stages_us(p, p.kblocks, 1.0, (double)n * group, c, b_bytes));
+    if (p.nsplit == 0 || cost < p.cost * 0.99) {
+      p.cost = cost;
+      p.nsplit = 1;
+      p.chan = c;
+      p.tiles = (int)tiles;
+      p.ctas = (int)n * group;
+    }
+  }
+  return p;
+}
+
+template <int KIND, bool PAIR>
 int launch_kind(const CUtensorMap& map_w, const CUtensorMap& map_x, const TcArgs& a, const TcPlan& p, bool pdl, cudaStream_t stream) {
-  const size_t smem = (size_t)p.stages * (kAStage + p.brows * 128) + kSmemSlack;
+  const size_t smem = (size_t)p.stages * (kAStage + p.brows * (PAIR ? 64 : 128)) + kSmemSlack + (p.stream ? 2048 : 0);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(p.tiles * p.row_tiles), (unsigned)p.nsplit);
+  cfg.gridDim = p.stream ? dim3((unsigned)p.ctas) : dim3((unsigned)(p.tiles * p.row_tiles), (unsigned)p.nsplit);
   cfg.blockDim = dim3(kThreadsTc);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   int na = 0;
-  if (p.nsplit > 1) {
+  if (PAIR || p.nsplit > 1) {
     attr[na].id = cudaLaunchAttributeClusterDimension;
-    attr[na].val.clusterDim.x = 1;
+    attr[na].val.clusterDim.x = PAIR ? 2 : 1;
     attr[na].val.clusterDim.y = (unsigned)p.nsplit;
     attr[na].val.clusterDim.z = 1;
     ++na;
@@ -451,38 +797,57 @@ int launch_kind(const CUtensorMap& map_w, const CUtensorMap& map_x, const TcArgs
   }
   cfg.attrs = attr;
   cfg.numAttrs = (unsigned)na;
-  QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_linear_kernel<KIND>, map_w, map_x, a));
+  if (p.stream)
+    QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_stream_kernel<KIND, PAIR>, map_w, map_x, a, p.tiles / (PAIR ? 2 : 1) * p.row_tiles));
+  else
+    QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_linear_kernel<KIND, PAIR>, map_w, map_x, a));
   count_launch();
   return QUASAR_OK;
 }
 
 int launch_any(int kind, const void* x, const float* dx, const void* w, const float* dw, int64_t M, int64_t N, int64_t K, void* y,
                bool y_is_f32, const __nv_bfloat16* residual, int32_t* acc_out, unsigned long long* keys, int32_t* error, bool pdl, cudaStream_t stream) {
-  const void* kernel = kind == kDigits ? (const void*)tc_linear_kernel<kDigits>
-                                       : (kind == kBf16 ? (const void*)tc_linear_kernel<kBf16> : (const void*)tc_linear_kernel<kCodes>);
-  {
-    static bool configured[3] = {false, false, false};
-    if (!configured[kind]) {
-      QUASAR_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
-      QUASAR_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-      configured[kind] = true;
-    }
+  static const void* const kernels[3][4] = {
+      {(const void*)tc_linear_kernel<kDigits, false>, (const void*)tc_linear_kernel<kDigits, true>,
+       (const void*)tc_stream_kernel<kDigits, false>, (const void*)tc_stream_kernel<kDigits, true>},
+      {(const void*)tc_linear_kernel<kBf16, false>, (const void*)tc_linear_kernel<kBf16, true>,
+       (const void*)tc_stream_kernel<kBf16, false>, (const void*)tc_stream_kernel<kBf16, true>},
+      {(const void*)tc_linear_kernel<kCodes, false>, (const void*)tc_linear_kernel<kCodes, true>,
+       (const void*)tc_stream_kernel<kCodes, false>, (const void*)tc_stream_kernel<kCodes, true>}};
+  static bool configured = false;
+  if (!configured) {
+    for (auto& row : kernels)
+      for (const void* k : row) {
+        QUASAR_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
+        QUASAR_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
+      }
+    configured = true;
   }
-  const TcPlan p = plan_tc(M, N, K, kind, kernel);
+  // A pair of CTAs halves what the activations add to an SM's intake; narrow blocks have too few of them for that to matter.
+  TcPlan p = plan_tiles(M, N, K, kind, false, kernels[kind][0]);
+  auto consider = [&](const TcPlan& q) { if (q.cost < p.cost) p = q; };
+  consider(plan_stream(M, N, K, kind, false));
+  if (p.brows >= 64) {
+    consider(plan_tiles(M, N, K, kind, true, kernels[kind][1]));
+    consider(plan_stream(M, N, K, kind, true));
+  }
   CUtensorMap map_w, map_x;
   int rc = make_map_sw128(&map_w, w, (uint64_t)N, (uint64_t)K * (kind == kBf16 ? 2 : 1), (uint32_t)p.chan);
   if (rc != QUASAR_OK) return rc;
-  rc = make_map_sw128(&map_x, x, (uint64_t)M * (kind == kDigits ? 3 : 1), (uint64_t)K * (kind == kBf16 ? 2 : 1), (uint32_t)p.brows);
+  rc = make_map_sw128(&map_x, x, (uint64_t)M * (kind == kDigits ? 3 : 1), (uint64_t)K * (kind == kBf16 ? 2 : 1), (uint32_t)(p.pair ? p.brows / 2 : p.brows));
   if (rc != QUASAR_OK) return rc;
   TcArgs a;
   a.dx = dx; a.dw = dw; a.y = y; a.res = residual; a.acc_out = acc_out; a.keys = keys; a.error = error;
   a.M = (int)M; a.N = (int)N; a.kblocks = p.kblocks; a.chan = p.chan; a.rows = p.rows; a.brows = p.brows;
   a.row_tiles = p.row_tiles; a.nsplit = p.nsplit; a.stages = p.stages; a.y_is_f32 = y_is_f32 ? 1 : 0;
   a.early_weights = pdl ? 1 : 0;
-  switch (kind) {
-    case kDigits: return launch_kind<kDigits>(map_w, map_x, a, p, pdl, stream);
-    case kBf16: return launch_kind<kBf16>(map_w, map_x, a, p, pdl, stream);
-    default: return launch_kind<kCodes>(map_w, map_x, a, p, pdl, stream);
+  switch (kind * 2 + p.pair) {
+    case kDigits * 2: return launch_kind<kDigits, false>(map_w, map_x, a, p, pdl, stream);
+    case kDigits * 2 + 1: return launch_kind<kDigits, true>(map_w, map_x, a, p, pdl, stream);
+    case kBf16 * 2: return launch_kind<kBf16, false>(map_w, map_x, a, p, pdl, stream);
+    case kBf16 * 2 + 1: return launch_kind<kBf16, true>(map_w, map_x, a, p, pdl, stream);
+    case kCodes * 2: return launch_kind<kCodes, false>(map_w, map_x, a, p, pdl, stream);
+    default: return launch_kind<kCodes, true>(map_w, map_x, a, p, pdl, stream);
   }
 }
 
