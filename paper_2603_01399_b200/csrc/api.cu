@@ -12,6 +12,7 @@
 
 #include "common.cuh"
 #include "megakernel.cuh"
+#include "tc_attention.cuh"
 #include "tc_linear.cuh"
 
 namespace quasar {
@@ -104,6 +105,7 @@ Workspace layout(const quasar_config& c, int B, int T_max, int s_max) {
     const size_t mega = rows * c.head_dim * sizeof(float) + rows * 2 * sizeof(float);
     if (mega > w.att_bytes) w.att_bytes = mega;
   }
+  w.att_bytes = std::max(w.att_bytes, tc_attention_workspace_bytes(B, T_max, c.n_q_heads, c.n_kv_heads, c.head_dim));
   w.att = take(w.att_bytes);
   w.cand = take((size_t)kMaxGrid * 8 * 2 * sizeof(float));
   w.ss_part = take((size_t)kMaxGrid * 8 * sizeof(float));
@@ -297,6 +299,8 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
       return launch_tc_linear_w8a8(op_q, op_scale, wq, delta, M, N, K, out, out_f32, res, nullptr, keys, status, true, stream);
     return launch_tc_linear_digits(op_q, op_scale, wq, delta, M, N, K, out, out_f32, res, keys, status, true, stream);
   };
+  const AttnList list{kv->seq_len, block_len, bi.valid, bi.anc, B, T_max, Hkv, Hq / Hkv, kv->s_max};
+  const AttnParts parts = tc_attention_parts(att, B, T_max, Hq, Hkv, D);
   auto norm_gain = [&](int l) {
     return reinterpret_cast<const __nv_bfloat16*>(l < c.n_layers ? m->layers[l].attn_norm : m->w.final_norm);
   };
@@ -315,10 +319,15 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
                            reinterpret_cast<const __nv_bfloat16*>(c.qk_norm ? L.k_norm : nullptr), m->rope_table,
                            kv->seq_len, block_len, bi, B, T_max, Hq, Hkv, D, c.rms_eps, kc, vc, kv->s_max, stream));
     TRY(tr.put(qkv, (size_t)M * qkv_w * 2));
-    TRY(launch_attention(qkv, kc, vc, kv->seq_len, block_len, bi, B, T_max, Hq, Hkv, D, kv->s_max, attn, att,
-                         ws.att_bytes, stream));
+    if (a8 || Hq * D > 24576) {   // (longer rows do not fit the merge's shared memory)
+      // (the W8A8 form keeps the order of this kernel's sums: a last bit of the attention output becomes quantisation steps)
+      TRY(launch_attention(qkv, kc, vc, kv->seq_len, block_len, bi, B, T_max, Hq, Hkv, D, kv->s_max, attn, att, ws.att_bytes, stream));
+      TRY(launch_operand(form, attn, M, Hq * D, RowOperand{nullptr, op_q, op_scale, L.o_smooth}, stream));
+    } else {
+      TRY(launch_tc_attention(qkv, kc, vc, list, kv->batch, D, parts, status, stream));
+      TRY(launch_attention_merge(form, list, parts, M, D, operand(attn, nullptr), stream));
+    }
     TRY(tr.put(attn, (size_t)M * Hq * D * 2));
-    TRY(launch_operand(form, attn, M, Hq * D, RowOperand{nullptr, op_q, op_scale, L.o_smooth}, stream));
     TRY(linear(attn, L.o_w, L.o_delta, H, Hq * D, x, false, x, nullptr));
     TRY(tr.put(x, (size_t)M * H * 2));
     TRY(launch_norm(form, x, reinterpret_cast<const __nv_bfloat16*>(L.mlp_norm), M, H, c.rms_eps, adders, operand(h, L.gateup_smooth), stream));

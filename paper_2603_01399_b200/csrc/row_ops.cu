@@ -12,6 +12,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "tc_attention.cuh"
 #include "tc_common.cuh"
 #include "tc_linear.cuh"
 
@@ -282,6 +283,112 @@ __global__ void __launch_bounds__(kRowThreads) operand_kernel(const __nv_bfloat1
       nvec, m, out, s_buf);
 }
 
+// Puts the partial results of the tcgen05 attention together (tc_attention.cuh says where they lie): one CTA per block row, a
+// warp per query head in turn.  A head's parts are the two groups of every CTA whose run of the list touched its segment,
+// added in list order; the finished row goes through shared memory into the operand of the o projection.
+template <int OP, int V, int D>
+__global__ void __launch_bounds__(kRowThreads) attention_merge_operand_kernel(AttnList l, AttnParts parts, int nvec, RowOperand out) {
+  __shared__ float s_buf[32];
+  __shared__ long long s_total, s_unit0;
+  __shared__ int s_seg0;
+  extern __shared__ __align__(16) unsigned char s_row[];   // [Hq * D] bf16
+  pdl_trigger();
+  pdl_wait();
+  const int m = blockIdx.x, b = m / l.T_max, i = m % l.T_max;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool live = l.valid[b] != 0 && i < l.block_len[b];
+  constexpr int kPer = D / 32;
+  const int Hq = l.Hkv * l.G;
+  if (live) {
+    if (warp == 0) {   // units and segments of the sequences before this one
+      long long units = 0, before = 0;
+      int segs = 0;
+      for (int x = lane; x < l.B; x += 32) {
+        int t, r;
+        attn_shape(l, x, t, r);
+        units += (long long)t * r * l.Hkv;
+        if (x < b) { before += (long long)t * r * l.Hkv; segs += r * l.Hkv; }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        units += __shfl_xor_sync(0xffffffffu, units, o);
+        before += __shfl_xor_sync(0xffffffffu, before, o);
+        segs += __shfl_xor_sync(0xffffffffu, segs, o);
+      }
+      if (lane == 0) { s_total = units; s_unit0 = before; s_seg0 = segs; }
+    }
+    __syncthreads();
+    int tiles, row_tiles;
+    attn_shape(l, b, tiles, row_tiles);
+    for (int hq = warp; hq < Hq; hq += kRowThreads / 32) {
+      const int r = i * l.G + hq % l.G, s = (hq / l.G) * row_tiles + r / 128, row = r % 128;
+      const long long u0 = s_unit0 + (long long)s * tiles;
+      const int c0 = (int)(((u0 + 1) * kAttnCtas - 1) / s_total), c1 = (int)(((u0 + tiles) * kAttnCtas - 1) / s_total);
+      const int n = 2 * (c1 - c0 + 1);
+      const size_t at0 = ((size_t)(c0 + s_seg0 + s) * 2) * 128 + row;   // part p: 128 entries further
+      float mx = -INFINITY;
+      for (int p = lane; p < n; p += 32) mx = fmaxf(mx, __ldcg(&parts.ml[at0 + (size_t)p * 128].x));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      float acc[kPer], den = 0.f;
+#pragma unroll
+      for (int e = 0; e < kPer; ++e) acc[e] = 0.f;
+      for (int p0 = 0; p0 < n; p0 += 32) {
+        float2 ml = p0 + lane < n ? __ldcg(&parts.ml[at0 + (size_t)(p0 + lane) * 128]) : make_float2(-INFINITY, 0.f);
+        const float w = ml.x == -INFINITY ? 0.f : exp2f(ml.x - mx);
+        float wl = w * ml.y;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) wl += __shfl_xor_sync(0xffffffffu, wl, o);
+        den += wl;
+        for (int q0 = 0; q0 < 32 && p0 + q0 < n; q0 += 4) {   // four parts' loads at a time
+          float v[4][kPer], wq[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            wq[q] = __shfl_sync(0xffffffffu, w, q0 + q);
+            const float* src = parts.o + (at0 + (size_t)(p0 + q0 + q) * 128) * D + lane * kPer;
+            if (wq[q] != 0.f) {   // (a part without a visible key may never have been written)
+              if constexpr (kPer == 4) {
+                const float4 t = __ldcg(reinterpret_cast<const float4*>(src));
+                v[q][0] = t.x; v[q][1] = t.y; v[q][2] = t.z; v[q][3] = t.w;
+              } else {
+                const float2 t = __ldcg(reinterpret_cast<const float2*>(src));
+                v[q][0] = t.x; v[q][1] = t.y;
+              }
+            } else {
+#pragma unroll
+              for (int e = 0; e < kPer; ++e) v[q][e] = 0.f;
+            }
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int e = 0; e < kPer; ++e) acc[e] += wq[q] * v[q][e];
+        }
+      }
+      const float inv = 1.0f / den;
+      uint32_t pk[kPer / 2];
+#pragma unroll
+      for (int e = 0; e < kPer / 2; ++e) {
+        const __nv_bfloat162 t = __floats2bfloat162_rn(acc[2 * e] * inv, acc[2 * e + 1] * inv);
+        pk[e] = *reinterpret_cast<const uint32_t*>(&t);
+      }
+      uint32_t* dst = reinterpret_cast<uint32_t*>(s_row) + hq * (D / 2) + lane * (kPer / 2);
+#pragma unroll
+      for (int e = 0; e < kPer / 2; ++e) dst[e] = pk[e];
+    }
+  } else {
+    for (int v = threadIdx.x; v < nvec; v += kRowThreads) reinterpret_cast<uint4*>(s_row)[v] = make_uint4(0, 0, 0, 0);
+  }
+  __syncthreads();
+  write_operand<OP, V>(
+      [&](int v, int j, float (&f)[8]) {
+        const uint4 y = reinterpret_cast<const uint4*>(s_row)[v];
+        if (out.y != nullptr) reinterpret_cast<uint4*>(out.y + (size_t)m * nvec * 8)[v] = y;
+        unpack8(y, f);
+      },
+      nvec, m, out, s_buf);
+}
+
 // One warp checks a sequence's tokens / parents / capacity and derives ancestor bit masks and depths.  A chain's are known
 // in closed form; a tree's are walked in shared memory by one lane.
 __device__ void prepare_sequence(const BlockArgs& a, int b, int* s_parent, unsigned long long* s_anc, int* s_depth) {
@@ -460,6 +567,23 @@ int launch_operand(int op, const __nv_bfloat16* x, int M, int K, const RowOperan
   if (op == kOperandBf16) return QUASAR_OK;   // the row itself is the operand
   const int nvec = K / 8;
   ROW_DISPATCH(operand_kernel, M, 0, true, stream, x, nvec, out)
+}
+
+int launch_attention_merge(int op, const AttnList& list, const AttnParts& parts, int M, int D, const RowOperand& out, cudaStream_t stream) {
+  const int K = list.Hkv * list.G * D, nvec = K / 8;
+  const size_t smem = (size_t)K * 2;
+  if (smem > 48 * 1024) { set_error("attention merge: rows of %d elements (at most 24576)", K); return QUASAR_ERR_SHAPE; }
+#define MERGE(OP, V, DD) return launch_row(attention_merge_operand_kernel<OP, V, DD>, M, smem, true, stream, list, parts, nvec, out)
+  const bool digits = op == kOperandDigits, wide = turns_of(nvec) > 2;
+  if (D == 128) {
+    if (wide) { if (digits) MERGE(kOperandDigits, 6, 128); MERGE(kOperandBf16, 6, 128); }
+    if (digits) MERGE(kOperandDigits, 2, 128);
+    MERGE(kOperandBf16, 2, 128);
+  }
+  if (wide) { if (digits) MERGE(kOperandDigits, 6, 64); MERGE(kOperandBf16, 6, 64); }
+  if (digits) MERGE(kOperandDigits, 2, 64);
+  MERGE(kOperandBf16, 2, 64);
+#undef MERGE
 }
 
 int launch_accept(const BlockArgs& a, int32_t* accept_len, int32_t* bonus, int32_t* accept_path, cudaStream_t stream) {
