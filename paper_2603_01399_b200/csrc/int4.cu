@@ -5,42 +5,59 @@
 //   Y[m][n] = sum_g delta[n][g] * sum_{k in g} X[m][k] * code[n][k]
 // The weight stream is a quarter of the bf16 one (Section 3.4's M * bytes / BW term).
 //
-// Kernel: a CTA of 4 warps owns 64 output channels x a range of groups.  A lane reads 8 packed bytes (16
-// codes) of one weight row per step; a code becomes a bf16 by placing (code + 8) under the exponent of 128
-// and subtracting 136 (exact), two codes per instruction.  Shifting by 4 bits pairs code i with code i + 4,
-// so the activation rows are staged in shared memory in that order (0,4,1,5,2,6,3,7 within eight) and the
-// MMA's operands line up without further moves.  mma.m16n8k16 bf16 with fp32 accumulation per group, folded
-// into the running sum with the group's step size.  k-ranges are added in a fixed order by a second kernel.
+// Kernel: a CTA of 8 warps owns 128 output channels x a range of groups, a warp 16 channels.  The weights of up to four
+// groups are asked for at once, 16 bytes a row and group and lane, before the activations of the chunk are staged in shared
+// memory; the groups then run without a barrier between them.  A code becomes a bf16 by placing (code + 8) under the
+// exponent of 128 and subtracting 136 (exact), two codes per instruction.  Shifting by 4 bits pairs code i with code
+// i + 4, so the activations are staged in that order (0,4,1,5,2,6,3,7 within eight) and the operands of mma.m16n8k16 line
+// up without further moves; the contraction index may be permuted freely as long as both operands agree.  fp32
+// accumulation per group, folded into the running sum with the group's step size.  The ranges of a channel block form a
+// cluster and add their sums through distributed shared memory in the order of the ranges.
+#include <algorithm>
+
 #include "common.cuh"
+#include "quant.cuh"
+#include "tc_common.cuh"
 
 namespace quasar {
 
 namespace {
 
 constexpr int kGroup = 128;
-constexpr int kW4Threads = 128;
-constexpr int kW4BlockN = 64;
+constexpr int kW4Threads = 256;
+constexpr int kW4BlockN = 128;
+constexpr int kW4Rows = 64;        // activation rows of a launch
+constexpr int kW4Ahead = 4;        // groups whose weights a lane holds at a time
 
+// A thread takes eight consecutive values; the 16 lanes of a group share its maximum.  Four pieces per thread in flight.
+constexpr int kQ4Pieces = 4;
 __global__ void __launch_bounds__(256)
-quantize_int4_kernel(const __nv_bfloat16* __restrict__ w, int64_t K, uint8_t* __restrict__ packed, float* __restrict__ delta) {
-  const int64_t n = blockIdx.x;
-  const int ngroups = (int)(K / kGroup);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int g = warp; g < ngroups; g += 8) {
-    const uint2 raw = __ldg(reinterpret_cast<const uint2*>(w + n * K + (int64_t)g * kGroup) + lane);   // four bf16
-    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&raw);
-    const float2 a = __bfloat1622float2(h[0]), b = __bfloat1622float2(h[1]);
-    float amax = fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(b.x), fabsf(b.y)));
+quantize_int4_kernel(const __nv_bfloat16* __restrict__ w, int64_t nvec, uint32_t* __restrict__ packed, float* __restrict__ delta) {
+  const int64_t base = (int64_t)blockIdx.x * 256 * kQ4Pieces + threadIdx.x;
+  uint4 raw[kQ4Pieces];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-    const float d = amax == 0.f ? 1.0f : __fdiv_rn(amax, 7.0f);
-    const int q0 = max(-7, min(7, __float2int_rn(__fdiv_rn(a.x, d))));
-    const int q1 = max(-7, min(7, __float2int_rn(__fdiv_rn(a.y, d))));
-    const int q2 = max(-7, min(7, __float2int_rn(__fdiv_rn(b.x, d))));
-    const int q3 = max(-7, min(7, __float2int_rn(__fdiv_rn(b.y, d))));
-    const unsigned short out = (unsigned short)((q0 & 0xF) | ((q1 & 0xF) << 4) | ((q2 & 0xF) << 8) | ((q3 & 0xF) << 12));
-    reinterpret_cast<unsigned short*>(packed + n * (K / 2) + (int64_t)g * (kGroup / 2))[lane] = out;
-    if (lane == 0) delta[n * ngroups + g] = d;
+  for (int j = 0; j < kQ4Pieces; ++j) {
+    const int64_t i = base + j * 256;
+    raw[j] = i < nvec ? __ldg(reinterpret_cast<const uint4*>(w) + i) : make_uint4(0, 0, 0, 0);
+  }
+#pragma unroll
+  for (int j = 0; j < kQ4Pieces; ++j) {
+    const int64_t i = base + j * 256;
+    float f[8], c[8];
+    unpack_bf16x8(raw[j], f);
+    AbsMax m;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) m.take(f[e]);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+      m.num = fmaxf(m.num, __shfl_xor_sync(0xffffffffu, m.num, o));
+      m.bits = max(m.bits, __shfl_xor_sync(0xffffffffu, m.bits, o));
+    }
+    const QuantStep st = quant_step(m.num == 0.f ? 1.0f : __fdiv_rn(m.num, 7.0f), m.has_nan());
+    if (i >= nvec) continue;   // (whole groups: nvec is a multiple of 16)
+    quantize8(f, st, 7, c);
+    packed[i] = pack_nibbles8(c);
+    if ((threadIdx.x & 15) == 0) delta[i >> 4] = st.delta;
   }
 }
 
@@ -50,8 +67,7 @@ struct W4Args {
   const float* delta;        // [N][K/128]
   void* y;
   const __nv_bfloat16* res;
-  float* partial;            // [nsplit][NT*8][N]
-  int M, N, K, groups_per_split, nsplit, y_is_f32;
+  int M, N, K, nsplit, chunk, y_is_f32;   // chunk: groups whose activations are staged at a time
 };
 
 __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
@@ -74,117 +90,189 @@ __device__ __forceinline__ void nib8_to_bf16(uint32_t w, uint32_t (&out)[4]) {
   }
 }
 
-__device__ __forceinline__ void w4_store(const W4Args& a, float v, int m, int n) {
-  const size_t idx = (size_t)m * a.N + n;
-  if (a.res != nullptr) v = __bfloat162float(__float2bfloat16_rn(v)) + __bfloat162float(a.res[idx]);
-  if (a.y_is_f32) reinterpret_cast<float*>(a.y)[idx] = v;
-  else reinterpret_cast<__nv_bfloat16*>(a.y)[idx] = __float2bfloat16_rn(v);
+__device__ __forceinline__ uint4 ldg_once(const void* p) {
+  uint4 r;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
+               : "l"(p));
+  return r;
 }
+
+// where piece p (16 bytes: eight elements of the group) of row `row` lies among a row's 16 pieces of a group: lane t reads its
+// pieces 4 t .. 4 t + 3 one after the other, and no two of eight neighbouring lanes meet in a bank
+__device__ __forceinline__ int piece_at(int p, int row) { return (((p & 3) << 2) | (p >> 2)) ^ ((row & 1) << 2); }
 
 template <int NT>
 __global__ void __launch_bounds__(kW4Threads) w4_gemm_kernel(W4Args a) {
-  // one group (128 input channels) of the activation rows at a time: [NT*8][128] bf16, eight-element blocks
-  // permuted to 0,4,1,5,2,6,3,7, 16-byte pieces swizzled by row parity
-  __shared__ __align__(16) uint4 xs[NT * 8 * 16];
+  extern __shared__ __align__(16) unsigned char smem[];
+  uint4* xs = reinterpret_cast<uint4*>(smem);   // [group of the chunk][NT * 8 rows][16 pieces]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int n0 = blockIdx.x * kW4BlockN + warp * 16;
   const int ngroups = a.K / kGroup;
-  const int g_begin = blockIdx.y * a.groups_per_split, g_end = min(ngroups, g_begin + a.groups_per_split);
+  const int g_begin = (int)((int64_t)blockIdx.y * ngroups / a.nsplit), g_end = (int)((int64_t)(blockIdx.y + 1) * ngroups / a.nsplit);
   const int r0 = min(n0 + g, a.N - 1), r1 = min(n0 + g + 8, a.N - 1);
-  const uint8_t* wrow0 = a.w + (size_t)r0 * (a.K / 2);
-  const uint8_t* wrow1 = a.w + (size_t)r1 * (a.K / 2);
+  const uint8_t* wrow0 = a.w + (size_t)r0 * (a.K / 2) + t * 16;
+  const uint8_t* wrow1 = a.w + (size_t)r1 * (a.K / 2) + t * 16;
+  const float* drow0 = a.delta + (size_t)r0 * ngroups;
+  const float* drow1 = a.delta + (size_t)r1 * ngroups;
   float tot[NT][4];
 #pragma unroll
   for (int i = 0; i < NT; ++i) tot[i][0] = tot[i][1] = tot[i][2] = tot[i][3] = 0.f;
 
-  for (int gi = g_begin; gi < g_end; ++gi) {
-    __syncthreads();
-    for (int c = threadIdx.x; c < NT * 8 * 16; c += kW4Threads) {
-      const int row = c >> 4, pc = c & 15;
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (row < a.M) {
-        const uint4 raw = *reinterpret_cast<const uint4*>(a.x + (size_t)row * a.K + (size_t)gi * kGroup + pc * 8);
-        // halves e0..e7 -> e0,e4,e1,e5,e2,e6,e3,e7
-        v.x = __byte_perm(raw.x, raw.z, 0x5410);
-        v.y = __byte_perm(raw.x, raw.z, 0x7632);
-        v.z = __byte_perm(raw.y, raw.w, 0x5410);
-        v.w = __byte_perm(raw.y, raw.w, 0x7632);
+  for (int c0 = g_begin; c0 < g_end; c0 += a.chunk) {
+    const int cn = min(a.chunk, g_end - c0);
+    uint4 wa[kW4Ahead], wb[kW4Ahead];
+    float d0[kW4Ahead], d1[kW4Ahead];
+    auto fetch = [&](int from) {
+#pragma unroll
+      for (int u = 0; u < kW4Ahead; ++u) {
+        if (from + u < cn) {
+          wa[u] = ldg_once(wrow0 + (size_t)(c0 + from + u) * 64);
+          wb[u] = ldg_once(wrow1 + (size_t)(c0 + from + u) * 64);
+          d0[u] = __ldg(drow0 + c0 + from + u);
+          d1[u] = __ldg(drow1 + c0 + from + u);
+        }
       }
-      xs[row * 16 + (pc ^ ((row & 1) << 2))] = v;
+    };
+    fetch(0);
+    if (c0 > g_begin) __syncthreads();   // the chunk before has been read
+    // staged four pieces a thread at a time, all of them in flight at once
+    const int pieces = NT * 8 * 16 * cn;
+    for (int i0 = threadIdx.x; i0 < pieces; i0 += 4 * kW4Threads) {
+      uint4 raw[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int i = i0 + j * kW4Threads;
+        const int row = (i >> 4) % (NT * 8), gi = (i >> 4) / (NT * 8), pc = i & 15;
+        raw[j] = (i < pieces && row < a.M) ? *reinterpret_cast<const uint4*>(a.x + (size_t)row * a.K + (size_t)(c0 + gi) * kGroup + pc * 8)
+                                           : make_uint4(0, 0, 0, 0);
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int i = i0 + j * kW4Threads;
+        if (i >= pieces) break;
+        const int row = (i >> 4) % (NT * 8), gi = (i >> 4) / (NT * 8), pc = i & 15;
+        uint4 v;   // halves e0..e7 -> e0,e4,e1,e5,e2,e6,e3,e7
+        v.x = __byte_perm(raw[j].x, raw[j].z, 0x5410);
+        v.y = __byte_perm(raw[j].x, raw[j].z, 0x7632);
+        v.z = __byte_perm(raw[j].y, raw[j].w, 0x5410);
+        v.w = __byte_perm(raw[j].y, raw[j].w, 0x7632);
+        xs[(gi * NT * 8 + row) * 16 + piece_at(pc, row)] = v;
+      }
     }
     __syncthreads();
-    const float d0 = __ldg(a.delta + (size_t)r0 * ngroups + gi), d1 = __ldg(a.delta + (size_t)r1 * ngroups + gi);
-    float acc[NT][4];
+    for (int from = 0; from < cn; from += kW4Ahead) {
+      if (from > 0) fetch(from);
 #pragma unroll
-    for (int i = 0; i < NT; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
+      for (int u = 0; u < kW4Ahead; ++u) {
+        if (from + u >= cn) break;
+        float acc[NT][4];
 #pragma unroll
-    for (int s = 0; s < 2; ++s) {                       // a step covers 64 input channels: 16 per lane
-      const uint2 wa = __ldg(reinterpret_cast<const uint2*>(wrow0 + (size_t)gi * 64 + s * 32) + t);
-      const uint2 wb = __ldg(reinterpret_cast<const uint2*>(wrow1 + (size_t)gi * 64 + s * 32) + t);
-      uint32_t a_lo[4], a_hi[4], b_lo[4], b_hi[4];
-      nib8_to_bf16(wa.x, a_lo); nib8_to_bf16(wa.y, a_hi);
-      nib8_to_bf16(wb.x, b_lo); nib8_to_bf16(wb.y, b_hi);
+        for (int i = 0; i < NT; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.f;
+        const uint32_t pa[4] = {wa[u].x, wa[u].y, wa[u].z, wa[u].w}, pb[4] = {wb[u].x, wb[u].y, wb[u].z, wb[u].w};
 #pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        const int row = nt * 8 + g;
-        const int pc = s * 8 + t * 2;
-        const uint4 x0 = xs[row * 16 + (pc ^ ((row & 1) << 2))];
-        const uint4 x1 = xs[row * 16 + ((pc + 1) ^ ((row & 1) << 2))];
-        mma_bf16(acc[nt], a_lo[0], b_lo[0], a_lo[1], b_lo[1], x0.x, x0.y);
-        mma_bf16(acc[nt], a_lo[2], b_lo[2], a_lo[3], b_lo[3], x0.z, x0.w);
-        mma_bf16(acc[nt], a_hi[0], b_hi[0], a_hi[1], b_hi[1], x1.x, x1.y);
-        mma_bf16(acc[nt], a_hi[2], b_hi[2], a_hi[3], b_hi[3], x1.z, x1.w);
+        for (int c = 0; c < 4; ++c) {   // eight codes of each row: two MMAs
+          uint32_t A[4], B[4];
+          nib8_to_bf16(pa[c], A);
+          nib8_to_bf16(pb[c], B);
+#pragma unroll
+          for (int nt = 0; nt < NT; ++nt) {
+            const int row = nt * 8 + g;
+            const uint4 x = xs[((from + u) * NT * 8 + row) * 16 + piece_at(t * 4 + c, row)];
+            mma_bf16(acc[nt], A[0], B[0], A[1], B[1], x.x, x.y);
+            mma_bf16(acc[nt], A[2], B[2], A[3], B[3], x.z, x.w);
+          }
+        }
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+          tot[nt][0] = fmaf(acc[nt][0], d0[u], tot[nt][0]);
+          tot[nt][1] = fmaf(acc[nt][1], d0[u], tot[nt][1]);
+          tot[nt][2] = fmaf(acc[nt][2], d1[u], tot[nt][2]);
+          tot[nt][3] = fmaf(acc[nt][3], d1[u], tot[nt][3]);
+        }
       }
-    }
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-      tot[nt][0] = fmaf(acc[nt][0], d0, tot[nt][0]);
-      tot[nt][1] = fmaf(acc[nt][1], d0, tot[nt][1]);
-      tot[nt][2] = fmaf(acc[nt][2], d1, tot[nt][2]);
-      tot[nt][3] = fmaf(acc[nt][3], d1, tot[nt][3]);
     }
   }
+  // the sums to shared memory, [row][channel of the block]; every CTA of the cluster finishes a share of the rows
+  __syncthreads();
+  float* red = reinterpret_cast<float*>(smem);
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt) {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int n = n0 + g + (e >> 1) * 8, m = nt * 8 + 2 * t + (e & 1);
-      if (n >= a.N || m >= a.M) continue;
-      if (a.nsplit == 1) w4_store(a, tot[nt][e], m, n);
-      else __stcg(a.partial + ((size_t)blockIdx.y * (NT * 8) + m) * a.N + n, tot[nt][e]);
-    }
+    for (int e = 0; e < 4; ++e) red[(nt * 8 + 2 * t + (e & 1)) * kW4BlockN + warp * 16 + g + (e >> 1) * 8] = tot[nt][e];
   }
-}
-
-template <int NT>
-__global__ void __launch_bounds__(256) w4_reduce_kernel(W4Args a) {
-  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (i >= (int64_t)a.M * a.N) return;
-  const int m = (int)(i / a.N), n = (int)(i % a.N);
-  float s = 0.f;
-  for (int k = 0; k < a.nsplit; ++k) s += __ldcg(a.partial + ((size_t)k * (NT * 8) + m) * a.N + n);   // fixed order
-  w4_store(a, s, m, n);
-}
-
-int plan_w4_split(int64_t N, int64_t K, int* groups_per_split) {
-  const int nblocks = (int)((N + kW4BlockN - 1) / kW4BlockN);
-  const int ngroups = (int)(K / kGroup);
-  int want = (148 * 4 + nblocks - 1) / nblocks;
-  want = want < 1 ? 1 : (want > ngroups ? ngroups : want);
-  want = want > 32 ? 32 : want;
-  const int per = (ngroups + want - 1) / want;
-  *groups_per_split = per;
-  return (ngroups + per - 1) / per;
-}
-
-template <int NT>
-int launch_w4_nt(const W4Args& a, cudaStream_t stream) {
-  w4_gemm_kernel<NT><<<dim3((a.N + kW4BlockN - 1) / kW4BlockN, a.nsplit), kW4Threads, 0, stream>>>(a);
-  QUASAR_LAUNCH_CHECK();
   if (a.nsplit > 1) {
-    w4_reduce_kernel<NT><<<(unsigned)(((int64_t)a.M * a.N + 255) / 256), 256, 0, stream>>>(a);
-    QUASAR_LAUNCH_CHECK();
+    tc::cluster_arrive();
+    tc::cluster_wait();
+  } else {
+    __syncthreads();
   }
+  const int per = (a.M + a.nsplit - 1) / a.nsplit, m_begin = (int)blockIdx.y * per, m_end = min(a.M, m_begin + per);
+  const uint32_t red_addr = tc::smem_u32(red);
+  for (int i = threadIdx.x; i < (m_end - m_begin) * kW4BlockN; i += kW4Threads) {
+    const int m = m_begin + i / kW4BlockN, c = i % kW4BlockN, n = blockIdx.x * kW4BlockN + c;
+    if (n >= a.N) continue;
+    const uint32_t off = (uint32_t)(m * kW4BlockN + c) * 4;
+    float v;
+    if (a.nsplit == 1) {
+      v = red[m * kW4BlockN + c];
+    } else {
+      float p[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (k < a.nsplit) p[k] = tc::ld_cluster_f32(tc::cluster_map(red_addr + off, (uint32_t)k));
+      v = p[0];
+#pragma unroll
+      for (int k = 1; k < 8; ++k)
+        if (k < a.nsplit) v += p[k];
+    }
+    const size_t idx = (size_t)m * a.N + n;
+    if (a.res != nullptr) v = __bfloat162float(__float2bfloat16_rn(v)) + __bfloat162float(a.res[idx]);
+    if (a.y_is_f32) reinterpret_cast<float*>(a.y)[idx] = v;
+    else reinterpret_cast<__nv_bfloat16*>(a.y)[idx] = __float2bfloat16_rn(v);
+  }
+  if (a.nsplit > 1) {   // nobody's shared memory goes away while another CTA may read it
+    tc::cluster_arrive();
+    tc::cluster_wait();
+  }
+}
+
+template <int NT>
+int launch_w4_nt(W4Args a, cudaStream_t stream) {
+  const int nblocks = (a.N + kW4BlockN - 1) / kW4BlockN, ngroups = a.K / kGroup;
+  // Ranges: two CTAs on an SM (296 at once); a launch takes waves * (groups of a range + what a range costs besides, about
+  // two groups).  No range shorter than three groups.
+  double best = 0;
+  a.nsplit = 0;
+  for (int s = 1; s <= 8 && (s == 1 || ngroups / s >= 3); ++s) {
+    const double cost = (double)(((long long)nblocks * s + 295) / 296) * ((ngroups + s - 1) / s + 2);
+    if (a.nsplit == 0 || cost < best) { best = cost; a.nsplit = s; }
+  }
+  constexpr int kGroupBytes = NT * 8 * 256;
+  const int per = (ngroups + a.nsplit - 1) / a.nsplit;
+  int chunk = (96 * 1024) / kGroupBytes;
+  if (chunk > kW4Ahead) chunk = chunk / kW4Ahead * kW4Ahead;
+  a.chunk = std::min(chunk, per);
+  const size_t smem = std::max((size_t)a.chunk * kGroupBytes, (size_t)NT * 8 * kW4BlockN * 4);
+  static bool configured = false;
+  if (!configured) {
+    QUASAR_CUDA_CHECK(cudaFuncSetAttribute(w4_gemm_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
+    configured = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)nblocks, (unsigned)a.nsplit);
+  cfg.blockDim = dim3(kW4Threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = 1;
+  attr.val.clusterDim.y = (unsigned)a.nsplit;
+  attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = a.nsplit > 1 ? 1 : 0;
+  QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, w4_gemm_kernel<NT>, a));
+  count_launch();
   return QUASAR_OK;
 }
 
@@ -192,16 +280,16 @@ int launch_w4_nt(const W4Args& a, cudaStream_t stream) {
 
 int launch_quantize_int4(const __nv_bfloat16* w, int64_t N, int64_t K, uint8_t* packed, float* delta, cudaStream_t stream) {
   if (N == 0) return QUASAR_OK;
-  quantize_int4_kernel<<<(unsigned)N, 256, 0, stream>>>(w, K, packed, delta);
+  const int64_t nvec = N * (K / 8), per = 256 * kQ4Pieces;
+  if ((nvec + per - 1) / per > 0x7fffffffLL) { set_error("quantize_int4: matrix too large"); return QUASAR_ERR_SHAPE; }
+  quantize_int4_kernel<<<(unsigned)((nvec + per - 1) / per), 256, 0, stream>>>(w, nvec, reinterpret_cast<uint32_t*>(packed), delta);
   QUASAR_LAUNCH_CHECK();
   return QUASAR_OK;
 }
 
 size_t linear_w4_workspace_bytes(int64_t M, int64_t N, int64_t K) {
-  int per = 0;
-  const int nsplit = plan_w4_split(N, K, &per);
-  const size_t mpad = (size_t)(((M < 48 ? M : 48) + 7) / 8) * 8;
-  return nsplit > 1 ? (size_t)nsplit * mpad * (size_t)N * sizeof(float) : 16;
+  (void)M; (void)N; (void)K;
+  return 16;   // (nothing is kept there any more)
 }
 
 int launch_linear_w4(const __nv_bfloat16* x, const uint8_t* w, const float* delta, int64_t M, int64_t N, int64_t K, void* y,
@@ -216,16 +304,16 @@ int launch_linear_w4(const __nv_bfloat16* x, const uint8_t* w, const float* delt
     set_error("linear_w4: workspace of %zu bytes, need %zu", workspace_bytes, linear_w4_workspace_bytes(M, N, K));
     return QUASAR_ERR_CAPACITY;
   }
+  (void)workspace;
   const size_t ybytes = y_is_f32 ? 4 : 2;
-  for (int64_t m0 = 0; m0 < M; m0 += 48) {              // blocks of at most 48 rows per launch
+  const int64_t blocks = (M + kW4Rows - 1) / kW4Rows, rows = (M + blocks - 1) / blocks;
+  for (int64_t m0 = 0; m0 < M; m0 += rows) {
     W4Args a;
-    a.M = (int)((M - m0) < 48 ? (M - m0) : 48);
+    a.M = (int)((M - m0) < rows ? (M - m0) : rows);
     a.N = (int)N; a.K = (int)K;
     a.x = x + m0 * K; a.w = w; a.delta = delta;
     a.y = reinterpret_cast<unsigned char*>(y) + (size_t)m0 * N * ybytes;
     a.res = residual ? residual + m0 * N : nullptr;
-    a.partial = reinterpret_cast<float*>(workspace);
-    a.nsplit = plan_w4_split(N, K, &a.groups_per_split);
     a.y_is_f32 = y_is_f32 ? 1 : 0;
     int rc;
     switch ((a.M + 7) / 8) {
@@ -234,7 +322,9 @@ int launch_linear_w4(const __nv_bfloat16* x, const uint8_t* w, const float* delt
       case 3: rc = launch_w4_nt<3>(a, stream); break;
       case 4: rc = launch_w4_nt<4>(a, stream); break;
       case 5: rc = launch_w4_nt<5>(a, stream); break;
-      default: rc = launch_w4_nt<6>(a, stream); break;
+      case 6: rc = launch_w4_nt<6>(a, stream); break;
+      case 7: rc = launch_w4_nt<7>(a, stream); break;
+      default: rc = launch_w4_nt<8>(a, stream); break;
     }
     if (rc != QUASAR_OK) return rc;
   }

@@ -46,7 +46,7 @@ __device__ __forceinline__ uint4 round8(float (&f)[8]) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-template <bool MAX>
+template <bool MAX, int THREADS = kRowThreads>
 __device__ __forceinline__ float block_reduce(float v, float* s_buf) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -57,7 +57,7 @@ __device__ __forceinline__ float block_reduce(float v, float* s_buf) {
   __syncthreads();
   v = s_buf[0];
 #pragma unroll
-  for (int i = 1; i < kRowThreads / 32; ++i) v = MAX ? fmaxf(v, s_buf[i]) : v + s_buf[i];   // warps in order
+  for (int i = 1; i < THREADS / 32; ++i) v = MAX ? fmaxf(v, s_buf[i]) : v + s_buf[i];   // warps in order
   return v;
 }
 
@@ -73,16 +73,16 @@ __device__ __forceinline__ void load_smooth8(const float* smooth, int i, float (
 }
 
 // The row's values (eight of vector i by value(i, j, f); j is the turn) as the operand.
-template <int OP, int V, typename F>
+template <int OP, int V, int THREADS = kRowThreads, typename F>
 __device__ __forceinline__ void write_operand(F&& value, int nvec, int m, const RowOperand& out, float* s_buf) {
   if (OP == kOperandBf16) {   // (the values have been stored as they were made)
     float f[8];
     if (V > 0) {
 #pragma unroll
       for (int j = 0; j < (V > 0 ? V : 1); ++j)
-        if ((int)threadIdx.x + j * kRowThreads < nvec) value((int)threadIdx.x + j * kRowThreads, j, f);
+        if ((int)threadIdx.x + j * THREADS < nvec) value((int)threadIdx.x + j * THREADS, j, f);
     } else {
-      for (int i = threadIdx.x; i < nvec; i += kRowThreads) value(i, 0, f);
+      for (int i = threadIdx.x; i < nvec; i += THREADS) value(i, 0, f);
     }
     return;
   }
@@ -92,7 +92,7 @@ __device__ __forceinline__ void write_operand(F&& value, int nvec, int m, const 
   if (V > 0) {
 #pragma unroll
     for (int j = 0; j < (V > 0 ? V : 1); ++j) {
-      const int i = (int)threadIdx.x + j * kRowThreads;
+      const int i = (int)threadIdx.x + j * THREADS;
       if (i < nvec) {
         value(i, j, f[j]);
 #pragma unroll
@@ -100,13 +100,13 @@ __device__ __forceinline__ void write_operand(F&& value, int nvec, int m, const 
       }
     }
   } else {
-    for (int i = threadIdx.x; i < nvec; i += kRowThreads) {
+    for (int i = threadIdx.x; i < nvec; i += THREADS) {
       value(i, 0, f[0]);
 #pragma unroll
       for (int e = 0; e < 8; ++e) amax = fmaxf(amax, fabsf(f[0][e]));
     }
   }
-  amax = block_reduce<true>(amax, s_buf);
+  amax = block_reduce<true, THREADS>(amax, s_buf);
   float up = 1.f, scale = 1.f;
   if (OP == kOperandDigits) digit_scale(amax, up, scale);
   else scale = amax == 0.f ? 1.0f : __fdiv_rn(amax, 127.0f);
@@ -127,9 +127,9 @@ __device__ __forceinline__ void write_operand(F&& value, int nvec, int m, const 
   if (V > 0) {
 #pragma unroll
     for (int j = 0; j < (V > 0 ? V : 1); ++j)
-      if ((int)threadIdx.x + j * kRowThreads < nvec) put((int)threadIdx.x + j * kRowThreads, f[j]);
+      if ((int)threadIdx.x + j * THREADS < nvec) put((int)threadIdx.x + j * THREADS, f[j]);
   } else {
-    for (int i = threadIdx.x; i < nvec; i += kRowThreads) {
+    for (int i = threadIdx.x; i < nvec; i += THREADS) {
       value(i, 0, f[0]);
       put(i, f[0]);
     }
@@ -286,9 +286,11 @@ __global__ void __launch_bounds__(kRowThreads) operand_kernel(const __nv_bfloat1
 // Puts the partial results of the tcgen05 attention together (tc_attention.cuh says where they lie): one CTA per block row, a
 // warp per query head in turn.  A head's parts are the two groups of every CTA whose run of the list touched its segment,
 // added in list order; the finished row goes through shared memory into the operand of the o projection.
+constexpr int kMergeThreads = 1024;   // a warp for each of 32 heads
+
 template <int OP, int V, int D>
-__global__ void __launch_bounds__(kRowThreads) attention_merge_operand_kernel(AttnList l, AttnParts parts, int nvec, RowOperand out) {
-  __shared__ float s_buf[32];
+__global__ void __launch_bounds__(kMergeThreads) attention_merge_operand_kernel(AttnList l, AttnParts parts, int nvec, RowOperand out) {
+  __shared__ float s_buf[kMergeThreads / 32];
   __shared__ long long s_total, s_unit0;
   __shared__ int s_seg0;
   extern __shared__ __align__(16) unsigned char s_row[];   // [Hq * D] bf16
@@ -320,7 +322,7 @@ __global__ void __launch_bounds__(kRowThreads) attention_merge_operand_kernel(At
     __syncthreads();
     int tiles, row_tiles;
     attn_shape(l, b, tiles, row_tiles);
-    for (int hq = warp; hq < Hq; hq += kRowThreads / 32) {
+    for (int hq = warp; hq < Hq; hq += kMergeThreads / 32) {
       const int r = i * l.G + hq % l.G, s = (hq / l.G) * row_tiles + r / 128, row = r % 128;
       const long long u0 = s_unit0 + (long long)s * tiles;
       const int c0 = (int)(((u0 + 1) * kAttnCtas - 1) / s_total), c1 = (int)(((u0 + tiles) * kAttnCtas - 1) / s_total);
@@ -340,10 +342,10 @@ __global__ void __launch_bounds__(kRowThreads) attention_merge_operand_kernel(At
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) wl += __shfl_xor_sync(0xffffffffu, wl, o);
         den += wl;
-        for (int q0 = 0; q0 < 32 && p0 + q0 < n; q0 += 4) {   // four parts' loads at a time
-          float v[4][kPer], wq[4];
+        for (int q0 = 0; q0 < 32 && p0 + q0 < n; q0 += 8) {   // eight parts' loads at a time
+          float v[8][kPer], wq[8];
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
+          for (int q = 0; q < 8; ++q) {
             wq[q] = __shfl_sync(0xffffffffu, w, q0 + q);
             const float* src = parts.o + (at0 + (size_t)(p0 + q0 + q) * 128) * D + lane * kPer;
             if (wq[q] != 0.f) {   // (a part without a visible key may never have been written)
@@ -360,7 +362,7 @@ __global__ void __launch_bounds__(kRowThreads) attention_merge_operand_kernel(At
             }
           }
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
+          for (int q = 0; q < 8; ++q)
 #pragma unroll
             for (int e = 0; e < kPer; ++e) acc[e] += wq[q] * v[q][e];
         }
@@ -377,10 +379,10 @@ __global__ void __launch_bounds__(kRowThreads) attention_merge_operand_kernel(At
       for (int e = 0; e < kPer / 2; ++e) dst[e] = pk[e];
     }
   } else {
-    for (int v = threadIdx.x; v < nvec; v += kRowThreads) reinterpret_cast<uint4*>(s_row)[v] = make_uint4(0, 0, 0, 0);
+    for (int v = threadIdx.x; v < nvec; v += kMergeThreads) reinterpret_cast<uint4*>(s_row)[v] = make_uint4(0, 0, 0, 0);
   }
   __syncthreads();
-  write_operand<OP, V>(
+  write_operand<OP, V, kMergeThreads>(
       [&](int v, int j, float (&f)[8]) {
         const uint4 y = reinterpret_cast<const uint4*>(s_row)[v];
         if (out.y != nullptr) reinterpret_cast<uint4*>(out.y + (size_t)m * nvec * 8)[v] = y;
@@ -573,16 +575,18 @@ int launch_attention_merge(int op, const AttnList& list, const AttnParts& parts,
   const int K = list.Hkv * list.G * D, nvec = K / 8;
   const size_t smem = (size_t)K * 2;
   if (smem > 48 * 1024) { set_error("attention merge: rows of %d elements (at most 24576)", K); return QUASAR_ERR_SHAPE; }
-#define MERGE(OP, V, DD) return launch_row(attention_merge_operand_kernel<OP, V, DD>, M, smem, true, stream, list, parts, nvec, out)
-  const bool digits = op == kOperandDigits, wide = turns_of(nvec) > 2;
+#define MERGE(OP, V, DD)                                                                                                    \
+  return launch_dependent(attention_merge_operand_kernel<OP, V, DD>, dim3((unsigned)M), dim3(kMergeThreads), smem, true, stream, \
+                          list, parts, nvec, out)
+  const bool digits = op == kOperandDigits, wide = nvec > kMergeThreads;   // more than a turn of 8 elements a thread
   if (D == 128) {
-    if (wide) { if (digits) MERGE(kOperandDigits, 6, 128); MERGE(kOperandBf16, 6, 128); }
-    if (digits) MERGE(kOperandDigits, 2, 128);
-    MERGE(kOperandBf16, 2, 128);
+    if (wide) { if (digits) MERGE(kOperandDigits, 3, 128); MERGE(kOperandBf16, 3, 128); }
+    if (digits) MERGE(kOperandDigits, 1, 128);
+    MERGE(kOperandBf16, 1, 128);
   }
-  if (wide) { if (digits) MERGE(kOperandDigits, 6, 64); MERGE(kOperandBf16, 6, 64); }
-  if (digits) MERGE(kOperandDigits, 2, 64);
-  MERGE(kOperandBf16, 2, 64);
+  if (wide) { if (digits) MERGE(kOperandDigits, 3, 64); MERGE(kOperandBf16, 3, 64); }
+  if (digits) MERGE(kOperandDigits, 1, 64);
+  MERGE(kOperandBf16, 1, 64);
 #undef MERGE
 }
 

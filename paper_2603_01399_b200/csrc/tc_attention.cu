@@ -61,6 +61,21 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* f) {
   for (int i = 0; i < 32; ++i) f[i] = __uint_as_float(v[i]);
 }
 
+__device__ __forceinline__ float ex2(float x) {   // 2^x; results below the normal range are zero
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// Which of the 32 keys from key0 on a row may see: all before the block (key < P), in the block those of its ancestor mask
+// (which has no bit beyond the block).
+__device__ __forceinline__ uint32_t visible32(unsigned long long anc, int key0, int P) {
+  const int off = key0 - P;
+  if (off <= -32) return 0xffffffffu;
+  if (off < 0) return (uint32_t)(anc << (-off)) | ((1u << (-off)) - 1u);
+  return off < 64 ? (uint32_t)(anc >> off) : 0u;
+}
+
 // V as operand B: N = d (contiguous, 64 elements = 128 bytes per swizzled row), K = keys; groups of 8 keys 1024 bytes apart,
 // the second 64 of d a sub-tile further
 __device__ __forceinline__ uint64_t desc_v(const void* smem_tile) {
@@ -78,15 +93,15 @@ struct Walk {
   AttnCursor cur;
   long long u, end;
   int b, hk, rt, t0, nt, seg;   // the piece: sequence, kv head, row tile, first key tile, key tiles, ordinal of the segment
-  __device__ Walk(const AttnList& l, int cta, int ncta) {
-    const long long total = attn_total(l);
+  const int2* shapes;
+  __device__ Walk(const AttnList& l, const int2* sh, long long total, int cta, int ncta) : shapes(sh) {
     u = (long long)cta * total / ncta;
     end = (long long)(cta + 1) * total / ncta;
-    cur.start(l);
+    cur.start(l, shapes);
   }
   __device__ bool next(const AttnList& l) {
     if (u >= end) return false;
-    cur.seek(l, u);
+    cur.seek(l, shapes, u);
     b = cur.b;
     const long long in = u - cur.unit0;
     const int s = (int)(in / cur.tiles);
@@ -146,8 +161,21 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
   const uint32_t tmem = *tmem_slot;   // columns: S (then P) of group 0, of group 1, O of group 0, of group 1
   if (threadIdx.x == 0) pdl_trigger();
   pdl_wait();
+  // the sequences' shapes, fetched once and side by side (each role walks them on its own)
+  __shared__ int2 s_shape[kShapes];
+  __shared__ long long s_total;
+  for (int b = (int)threadIdx.x; b < min(a.list.B, kShapes); b += kThreadsA) {
+    int t, r;
+    attn_shape(a.list, b, t, r);
+    s_shape[b] = make_int2(t, r);
+  }
+  if (warp == 2) {
+    const long long total = attn_total(a.list);
+    if (lane == 0) s_total = total;
+  }
+  __syncthreads();
 
-  Walk w(a.list, (int)blockIdx.x, (int)gridDim.x);
+  Walk w(a.list, s_shape, s_total, (int)blockIdx.x, (int)gridDim.x);
   if (warp == 0) {
     // ---- TMA producer ----
     const uint64_t policy = l2_evict_first_policy();
@@ -277,12 +305,9 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
           auto load = [&](int c, float (&s)[32]) {
             tmem_ld32(ts + (uint32_t)(c * 32), s);
             if (edge) {
+              const uint32_t see = visible32(anc, k0 + c * 32, P);
 #pragma unroll
-              for (int j = 0; j < 32; ++j) {
-                const int key = k0 + c * 32 + j;
-                const bool in = key < P || (key < Lk && ((anc >> (key - P)) & 1ull) != 0ull);
-                s[j] = in ? s[j] : -INFINITY;
-              }
+              for (int j = 0; j < 32; ++j) s[j] = (see >> j) & 1u ? s[j] : -INFINITY;
             }
           };
           float mx = -INFINITY;
@@ -324,7 +349,7 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             uint32_t p[32];
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
-              const float p0 = exp2f(fmaf(s[2 * j], scale_log2, -m_use)), p1 = exp2f(fmaf(s[2 * j + 1], scale_log2, -m_use));
+              const float p0 = ex2(fmaf(s[2 * j], scale_log2, -m_use)), p1 = ex2(fmaf(s[2 * j + 1], scale_log2, -m_use));
               sum0 += p0;
               sum1 += p1;
               const __nv_bfloat162 h2 = __floats2bfloat162_rn(p0, p1);

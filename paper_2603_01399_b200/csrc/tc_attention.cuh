@@ -7,6 +7,7 @@
 namespace quasar {
 
 constexpr int kAttnCtas = 148;    // one per SM
+constexpr int kShapes = 128;       // sequences whose shapes a CTA keeps in shared memory (more are looked up as they come)
 
 // Segments in order of sequence, kv head, row tile (128 of the G * T query rows of a kv head); a segment's units are its tiles
 // of 128 keys.  CTA c takes the units [c * total / ctas, (c + 1) * total / ctas), and its partial results for segment s
@@ -56,19 +57,22 @@ __device__ __forceinline__ long long attn_total(const AttnList& l) {
 struct AttnCursor {
   int b, seg0, tiles, row_tiles;
   long long unit0;
-  __device__ __forceinline__ void start(const AttnList& l) {
+  __device__ __forceinline__ void shape(const AttnList& l, const int2* known) {   // known: the first kShapes sequences'
+    if (b < kShapes) { tiles = known[b].x; row_tiles = known[b].y; }
+    else attn_shape(l, b, tiles, row_tiles);
+  }
+  __device__ __forceinline__ void start(const AttnList& l, const int2* known) {
     b = 0;
     seg0 = 0;
     unit0 = 0;
-    attn_shape(l, 0, tiles, row_tiles);
+    shape(l, known);
   }
-  __device__ __forceinline__ void advance(const AttnList& l) {
-    unit0 += (long long)tiles * row_tiles * l.Hkv;
-    seg0 += row_tiles * l.Hkv;
-    if (++b < l.B) attn_shape(l, b, tiles, row_tiles);
-  }
-  __device__ __forceinline__ void seek(const AttnList& l, long long u) {   // the sequence that holds unit u
-    while (b < l.B && u >= unit0 + (long long)tiles * row_tiles * l.Hkv) advance(l);
+  __device__ __forceinline__ void seek(const AttnList& l, const int2* known, long long u) {   // the sequence that holds unit u
+    while (b < l.B && u >= unit0 + (long long)tiles * row_tiles * l.Hkv) {
+      unit0 += (long long)tiles * row_tiles * l.Hkv;
+      seg0 += row_tiles * l.Hkv;
+      if (++b < l.B) shape(l, known);
+    }
   }
 };
 #endif

@@ -10,19 +10,49 @@
 // shrink an outlier channel (the stated purpose) s_j = max|W_j|^(1-alpha) / max|X_j|^alpha, the reciprocal
 // of the expression printed as Eq. 5 (which is the factor the activations are divided by).
 #include "common.cuh"
-#include "tc_common.cuh"
 #include "tc_linear.cuh"
 
 namespace quasar {
 
 namespace {
 
-constexpr int kQuantThreads = 256;
-
 // ---- Eq. 5: column maxima of W, then the factors ----------------------------------------------------
+// A thread keeps the maxima of 8 neighbouring columns over a strip of 64 rows (16-byte loads, eight rows in flight);
+// non-negative floats order like their bit patterns.
 __global__ void __launch_bounds__(256) colmax_kernel(const __nv_bfloat16* __restrict__ w, int64_t N, int64_t K,
                                                      unsigned* __restrict__ colmax_bits) {
-  // block: 256 columns x a strip of 64 rows; non-negative floats order like their bit patterns
+  const int64_t nvec = K / 8, v = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (v >= nvec) return;
+  const int64_t n0 = (int64_t)blockIdx.y * 64;
+  const int64_t n1 = n0 + 64 < N ? n0 + 64 : N;
+  const uint4* p = reinterpret_cast<const uint4*>(w) + v;
+  __nv_bfloat162 m[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) m[e] = __floats2bfloat162_rn(0.f, 0.f);
+  auto take = [&](const uint4& r) {   // (NaNs do not enter)
+    const uint32_t x[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) m[e] = __hmax2(m[e], __habs2(*reinterpret_cast<const __nv_bfloat162*>(&x[e])));
+  };
+  int64_t n = n0;
+  for (; n + 8 <= n1; n += 8) {
+    uint4 r[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) r[i] = __ldg(p + (n + i) * nvec);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) take(r[i]);
+  }
+  for (; n < n1; ++n) take(__ldg(p + n * nvec));
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    atomicMax(colmax_bits + v * 8 + 2 * e, __float_as_uint(__low2float(m[e])));
+    atomicMax(colmax_bits + v * 8 + 2 * e + 1, __float_as_uint(__high2float(m[e])));
+  }
+}
+
+// the same for row lengths that are no multiple of 8: a thread per column
+__global__ void __launch_bounds__(256) colmax_any_kernel(const __nv_bfloat16* __restrict__ w, int64_t N, int64_t K,
+                                                         unsigned* __restrict__ colmax_bits) {
   const int64_t k = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (k >= K) return;
   const int64_t n0 = (int64_t)blockIdx.y * 64;
@@ -42,67 +72,6 @@ __global__ void smooth_factor_kernel(const float* __restrict__ act_absmax, const
   s[k] = out;
 }
 
-// ---- Q(v, delta) per row, v = w (kPlain), w / s (kDivide: offline weights) or x * s (kMultiply: activations) ----
-enum SmoothMode { kPlain = 0, kDivide = 1, kMultiply = 2 };
-
-template <int MODE>
-__device__ __forceinline__ float smoothed(float v, float s) {
-  if (MODE == kDivide) return __fdiv_rn(v, s);
-  if (MODE == kMultiply) return __fmul_rn(v, s);
-  return v;
-}
-
-template <int MODE>
-__global__ void __launch_bounds__(kQuantThreads)
-quantize_smoothed_kernel(const __nv_bfloat16* __restrict__ w, const float* __restrict__ s, int64_t K,
-                         int8_t* __restrict__ q, float* __restrict__ delta) {
-  tc::pdl_trigger();   // (the contraction that follows in quasar_linear_w8a8 asks for its weights meanwhile)
-  const int64_t n = blockIdx.x;
-  const __nv_bfloat16* row = w + n * K;
-  int8_t* qrow = q + n * K;
-  const int nvec = (int)(K / 8);
-
-  float amax = 0.f;
-  for (int v = threadIdx.x; v < nvec; v += kQuantThreads) {
-    const uint4 u = __ldg(reinterpret_cast<const uint4*>(row) + v);
-    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
-    float sv[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) sv[i] = MODE == kPlain ? 1.f : __ldg(s + (int64_t)v * 8 + i);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float2 f = __bfloat1622float2(h[i]);
-      amax = fmaxf(amax, fmaxf(fabsf(smoothed<MODE>(f.x, sv[2 * i])), fabsf(smoothed<MODE>(f.y, sv[2 * i + 1]))));
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-  __shared__ float s_max[kQuantThreads / 32];
-  if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = amax;
-  __syncthreads();
-  amax = s_max[0];
-#pragma unroll
-  for (int i = 1; i < kQuantThreads / 32; ++i) amax = fmaxf(amax, s_max[i]);
-
-  const float d = (amax == 0.f) ? 1.0f : __fdiv_rn(amax, 127.0f);
-  if (threadIdx.x == 0) delta[n] = d;
-
-  for (int v = threadIdx.x; v < nvec; v += kQuantThreads) {
-    const uint4 u = __ldg(reinterpret_cast<const uint4*>(row) + v);
-    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
-    uint32_t out[2] = {0u, 0u};
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float2 f = __bfloat1622float2(h[i >> 1]);
-      const float sv = MODE == kPlain ? 1.f : __ldg(s + (int64_t)v * 8 + i);
-      const float val = smoothed<MODE>((i & 1) ? f.y : f.x, sv);
-      const int qi = max(-127, min(127, __float2int_rn(__fdiv_rn(val, d))));
-      out[i >> 2] |= (uint32_t)(qi & 0xff) << (8 * (i & 3));
-    }
-    reinterpret_cast<uint2*>(qrow)[v] = make_uint2(out[0], out[1]);
-  }
-}
-
 // The integer contraction (s8 x s8 -> s32, exact) and Eq. 10 are the tcgen05 kernel of tc_linear.cu.
 constexpr size_t kCounterBytes = 64 * 1024;   // reserved at the start of every workspace (quasar.h)
 constexpr int64_t kMaxChannels = (int64_t)1 << 20;
@@ -117,22 +86,12 @@ int launch_smoothing_factors(const float* act_absmax, const __nv_bfloat16* w, in
   // entry k and overwrites it
   unsigned* colmax = reinterpret_cast<unsigned*>(s_out);
   QUASAR_CUDA_CHECK(cudaMemsetAsync(colmax, 0, (size_t)K * sizeof(unsigned), stream));
-  colmax_kernel<<<dim3((unsigned)((K + 255) / 256), (unsigned)((N + 63) / 64)), 256, 0, stream>>>(w, N, K, colmax);
+  if (K % 8 == 0)
+    colmax_kernel<<<dim3((unsigned)((K / 8 + 255) / 256), (unsigned)((N + 63) / 64)), 256, 0, stream>>>(w, N, K, colmax);
+  else
+    colmax_any_kernel<<<dim3((unsigned)((K + 255) / 256), (unsigned)((N + 63) / 64)), 256, 0, stream>>>(w, N, K, colmax);
   QUASAR_LAUNCH_CHECK();
   smooth_factor_kernel<<<(unsigned)((K + 255) / 256), 256, 0, stream>>>(act_absmax, colmax, K, (double)alpha, s_out);
-  QUASAR_LAUNCH_CHECK();
-  return QUASAR_OK;
-}
-
-int launch_quantize_smoothed(const __nv_bfloat16* v, const float* s, int mode, int64_t rows, int64_t K, int8_t* q,
-                             float* delta, cudaStream_t stream) {
-  if (rows == 0) return QUASAR_OK;
-  if (s == nullptr)
-    quantize_smoothed_kernel<kPlain><<<(unsigned)rows, kQuantThreads, 0, stream>>>(v, nullptr, K, q, delta);
-  else if (mode == kDivide)
-    quantize_smoothed_kernel<kDivide><<<(unsigned)rows, kQuantThreads, 0, stream>>>(v, s, K, q, delta);
-  else
-    quantize_smoothed_kernel<kMultiply><<<(unsigned)rows, kQuantThreads, 0, stream>>>(v, s, K, q, delta);
   QUASAR_LAUNCH_CHECK();
   return QUASAR_OK;
 }
@@ -158,7 +117,7 @@ int launch_linear_w8a8(const __nv_bfloat16* x, const float* smooth, const int8_t
   int8_t* xq = reinterpret_cast<int8_t*>(ws + kCounterBytes);
   float* dx = reinterpret_cast<float*>(ws + kCounterBytes + align256((size_t)M * K));
   // Eq. 9: fused smoothing + per-token quantisation of the activations
-  const int rc = launch_quantize_smoothed(x, smooth, kMultiply, M, K, xq, dx, stream);
+  const int rc = launch_quantize_smoothed(x, smooth, 2, M, K, xq, dx, stream);
   if (rc != QUASAR_OK) return rc;
   return launch_tc_linear_w8a8(xq, dx, w, delta_w, M, N, K, y, y_is_f32, residual, acc_out, nullptr, status, true, stream);
 }
