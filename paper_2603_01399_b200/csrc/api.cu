@@ -299,7 +299,7 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
       return launch_tc_linear_w8a8(op_q, op_scale, wq, delta, M, N, K, out, out_f32, res, nullptr, keys, status, true, stream);
     return launch_tc_linear_digits(op_q, op_scale, wq, delta, M, N, K, out, out_f32, res, keys, status, true, stream);
   };
-  const AttnList list{kv->seq_len, block_len, bi.valid, bi.anc, B, T_max, Hkv, Hq / Hkv, kv->s_max};
+  const AttnList list{kv->seq_len, block_len, bi.valid, bi.anc, B, T_max, Hkv, Hq / Hkv, kv->s_max, attn_nodes_per_tile(Hq / Hkv)};
   const AttnParts parts = tc_attention_parts(att, B, T_max, Hq, Hkv, D);
   auto norm_gain = [&](int l) {
     return reinterpret_cast<const __nv_bfloat16*>(l < c.n_layers ? m->layers[l].attn_norm : m->w.final_norm);

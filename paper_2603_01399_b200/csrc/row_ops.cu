@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(kMergeThreads) attention_merge_operand_kernel(
     int tiles, row_tiles;
     attn_shape(l, b, tiles, row_tiles);
     for (int hq = warp; hq < Hq; hq += kMergeThreads / 32) {
-      const int r = i * l.G + hq % l.G, s = (hq / l.G) * row_tiles + r / 128, row = r % 128;
+      const int s = (hq / l.G) * row_tiles + i / l.npt, row = (i % l.npt) * l.G + hq % l.G;
       const long long u0 = s_unit0 + (long long)s * tiles;
       const int c0 = (int)(((u0 + 1) * kAttnCtas - 1) / s_total), c1 = (int)(((u0 + tiles) * kAttnCtas - 1) / s_total);
       const int n = 2 * (c1 - c0 + 1);

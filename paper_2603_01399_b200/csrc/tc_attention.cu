@@ -9,7 +9,8 @@
 //   O += P V       P goes back to tensor memory as a bf16 high and low part (two MMAs: about 16 bits of the
 //                  probabilities) over S; V is read as it lies (keys x d, the MMA's transposed form)
 // Two groups of four softmax warps take the key tiles in turn, each with an S and an O of its own (4 x 128 columns, all of
-// the tensor memory), so that one group's softmax passes under the other's MMAs; nothing is exchanged between them.
+// the tensor memory), so that one group's softmax passes under the other's MMAs; nothing is exchanged between them.  The
+// query rows come by TMA too, two pieces of work deep, and the MMAs run on from piece to piece.
 // O is scaled only when a row's maximum grows by more than 2^8 over the one its sums stand against.
 //
 // Work split: the key tiles of all (sequence, kv head, row tile) segments form one list, and each of the 148 CTAs takes an
@@ -32,15 +33,15 @@ using namespace tc;
 
 constexpr int kKeys = 128;        // keys of a tile
 constexpr int kThreadsA = 320;    // TMA warp, MMA warp, two groups of four softmax warps
-constexpr int kStagesA = 3;
+constexpr int kSlots = 5;         // ring of K and V tiles in turn
 constexpr float kLog2eA = 1.4426950408889634f;
 constexpr float kGrow = 8.f;      // how far (in powers of two) a row's maximum may outgrow its reference
 
 struct TcAttnArgs {
-  const __nv_bfloat16* qkv;   // [B*T_max][(Hq+2Hkv)*D], q part already normalised + rotated
   AttnList list;
   float* o_part;              // [slots][2][128][D]
   float2* ml_part;            // [slots][2][128]
+  int q_rows;                 // query rows a box of map_q brings: G * npt
   int32_t* error;
 };
 
@@ -117,34 +118,35 @@ struct Walk {
 
 template <int D>
 __global__ void __launch_bounds__(kThreadsA, 1)
-tc_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v, const TcAttnArgs a) {
+tc_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
+                    const __grid_constant__ CUtensorMap map_v, const TcAttnArgs a) {
   constexpr int kSubs = D / 64;                     // 128-byte columns of a row
   constexpr int kSub = kKeys * 128;                 // bytes of one of them for a tile's keys (or the 128 query rows)
   constexpr int kTile = kSubs * kSub;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  unsigned char* q_s = smem;                        // then the ring: K tile, V tile
-  unsigned char* ring = smem + kTile;
-  uint64_t* full = reinterpret_cast<uint64_t*>(ring + (size_t)kStagesA * 2 * kTile);
-  uint64_t* empty = full + kStagesA;
-  uint64_t* q_ready = empty + kStagesA;             // the piece's query rows are in place
-  uint64_t* piece_done = q_ready + 1;               // every softmax warp is through with the piece
-  uint64_t* s_full = piece_done + 1;                // [2] S of a group's tile is complete
+  unsigned char* q_s = smem;                        // two pieces' query rows, then the ring
+  unsigned char* ring = smem + 2 * kTile;
+  uint64_t* full = reinterpret_cast<uint64_t*>(ring + (size_t)kSlots * kTile);
+  uint64_t* empty = full + kSlots;
+  uint64_t* q_full = empty + kSlots;                // [2] a piece's query rows have landed
+  uint64_t* q_empty = q_full + 2;                   // [2] its last S is complete
+  uint64_t* s_full = q_empty + 2;                   // [2] S of a group's tile is complete
   uint64_t* p_ready = s_full + 2;                   // [2] P lies over it
-  uint64_t* pv_done = p_ready + 2;                  // [2] O has its product
+  uint64_t* pv_done = p_ready + 2;                  // [2] O has the products of a group's part of a piece
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(pv_done + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     *abort_flag = 0;
-    for (int s = 0; s < kStagesA; ++s) {
+    for (int s = 0; s < kSlots; ++s) {
       mbar_init(full + s, 1);
       mbar_init(empty + s, 1);
     }
-    mbar_init(q_ready, 8);
-    mbar_init(piece_done, 8);
     for (int i = 0; i < 2; ++i) {
+      mbar_init(q_full + i, 1);
+      mbar_init(q_empty + i, 1);
       mbar_init(s_full + i, 1);
       mbar_init(p_ready + i, 4);
       mbar_init(pv_done + i, 1);
@@ -179,85 +181,115 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
   if (warp == 0) {
     // ---- TMA producer ----
     const uint64_t policy = l2_evict_first_policy();
-    int s = 0, issued = 0;
+    int s = 0, issued = 0, piece = 0;
     uint32_t ph = 0;
     bool ok = true;
     while (ok && w.next(a.list)) {
       const int row0 = (w.b * a.list.Hkv + w.hk) * a.list.s_max + w.t0 * kKeys;
-      for (int t = 0; t < w.nt; ++t) {
-        if (!(ok = mbar_wait(empty + s, ph ^ 1u, abort_flag, a.error))) break;
-        if (elect_one()) {
-          unsigned char* at = ring + (size_t)s * 2 * kTile;
-          mbar_expect_tx(full + s, 2 * kTile);
+      const int qb = piece & 1;
+      if (!(ok = mbar_wait(q_empty + qb, ((uint32_t)(piece >> 1) & 1u) ^ 1u, abort_flag, a.error))) break;
+      if (elect_one()) {
+        mbar_expect_tx(q_full + qb, (uint32_t)(kSubs * a.q_rows * 128));
 #pragma unroll
-          for (int c = 0; c < kSubs; ++c) {
-            tma_load_2d_hint(at + c * kSub, &map_k, c * 128, row0 + t * kKeys, full + s, policy);
-            tma_load_2d_hint(at + kTile + c * kSub, &map_v, c * 128, row0 + t * kKeys, full + s, policy);
+        for (int c = 0; c < kSubs; ++c)
+          tma_load_3d(q_s + qb * kTile + c * kSub, &map_q, c * 128, w.hk * a.list.G, w.b * a.list.T_max + w.rt * a.list.npt, q_full + qb);
+      }
+      __syncwarp();
+      ++piece;
+      for (int t = 0; t < w.nt && ok; ++t) {
+#pragma unroll 1
+        for (int kv = 0; kv < 2; ++kv) {
+          if (!(ok = mbar_wait(empty + s, ph ^ 1u, abort_flag, a.error))) break;
+          if (elect_one()) {
+            unsigned char* at = ring + (size_t)s * kTile;
+            mbar_expect_tx(full + s, kTile);
+#pragma unroll
+            for (int c = 0; c < kSubs; ++c)
+              tma_load_2d_hint(at + c * kSub, kv == 0 ? &map_k : &map_v, c * 128, row0 + t * kKeys, full + s, policy);
           }
+          __syncwarp();
+          ++issued;
+          if (++s == kSlots) { s = 0; ph ^= 1u; }
         }
-        __syncwarp();
-        ++issued;
-        if (++s == kStagesA) { s = 0; ph ^= 1u; }
       }
     }
     if (!ok) {   // given up: what is in flight lands (bounded) before the CTA leaves
-      for (int i = 0; i < min(kStagesA, issued); ++i) {
-        if (--s < 0) { s = kStagesA - 1; ph ^= 1u; }
+      for (int i = 0; i < min(kSlots, issued); ++i) {
+        if (--s < 0) { s = kSlots - 1; ph ^= 1u; }
         const unsigned long long t0 = gtime_ns();
         while (!mbar_try(full + s, ph) && gtime_ns() - t0 < 100000ull) {}
       }
-    }
-  } else if (warp == 1) {
-    // ---- MMA issuer: S of tile t, then O of tile t - 1 ----
-    const uint32_t id_s = idesc(1, 1, 128, kKeys);
-    const uint32_t id_o = idesc(1, 1, 128, D) | (1u << 16);   // B transposed
-    const uint64_t dq = desc_sw128(q_s), dk0 = desc_sw128(ring), dv0 = desc_v(ring + kTile);
-    uint32_t q_ph = 0, p_ph[2] = {0u, 0u};
-    int s = 0, s_pv = 0;
-    uint32_t ph = 0;
-    bool ok = true;
-    while (ok && w.next(a.list)) {
-      if (!(ok = mbar_wait(q_ready, q_ph, abort_flag, a.error))) break;
-      q_ph ^= 1u;
-      for (int t = 0; t <= w.nt; ++t) {
-        if (t < w.nt) {
-          if (!(ok = mbar_wait(full + s, ph, abort_flag, a.error))) break;
-          fence_after();
-          if (elect_one()) {
-            const uint64_t dk = dk0 + (uint64_t)((uint32_t)(s * 2 * kTile) >> 4);
-#pragma unroll
-            for (int j = 0; j < D / 16; ++j) {
-              const uint64_t off = (uint64_t)(((j >> 2) * kSub + (j & 3) * 32) >> 4);
-              mma_f16_ss(tmem + (uint32_t)((t & 1) * 128), dq + off, dk + off, id_s, j > 0 ? 1u : 0u);
-            }
-            commit(s_full + (t & 1));
-          }
-          __syncwarp();
-          if (++s == kStagesA) { s = 0; ph ^= 1u; }
-        }
-        if (t > 0) {
-          const int g = (t - 1) & 1;
-          if (!(ok = mbar_wait(p_ready + g, p_ph[g], abort_flag, a.error))) break;
-          p_ph[g] ^= 1u;
-          fence_after();
-          if (elect_one()) {
-            const uint64_t dv = dv0 + (uint64_t)((uint32_t)(s_pv * 2 * kTile) >> 4);
-            const uint32_t tp = tmem + (uint32_t)(g * 128), to = tmem + (uint32_t)(256 + g * 128);
-#pragma unroll
-            for (int kk = 0; kk < kKeys / 16; ++kk) {   // 16 keys: the high part of P, then the low part
-              const uint64_t dvk = dv + (uint64_t)((kk * 16 * 128) >> 4);
-              const uint32_t tpk = tp + (uint32_t)((kk >> 1) * 32 + (kk & 1) * 8);
-              mma_f16_ts(to, tpk, dvk, id_o, (t > 2 || kk > 0) ? 1u : 0u);
-              mma_f16_ts(to, tpk + 16u, dvk, id_o, 1u);
-            }
-            commit(empty + s_pv);
-            commit(pv_done + g);
-          }
-          __syncwarp();
-          if (++s_pv == kStagesA) s_pv = 0;
-        }
+      for (int i = 0; i < min(2, piece); ++i) {
+        const int p = piece - 1 - i;
+        const unsigned long long t0 = gtime_ns();
+        while (!mbar_try(q_full + (p & 1), (uint32_t)(p >> 1) & 1u) && gtime_ns() - t0 < 100000ull) {}
       }
     }
+  } else if (warp == 1) {
+    // ---- MMA issuer: S of tile i, then O of tile i - 1, on through the pieces.  (A commit covers every MMA before it, so the
+    //      s_full of tile i + 2 also says that P of tile i, which it overwrites, has been used.) ----
+    const uint32_t id_s = idesc(1, 1, 128, kKeys);
+    const uint32_t id_o = idesc(1, 1, 128, D) | (1u << 16);   // B transposed
+    uint32_t p_ph[2] = {0u, 0u};
+    int slot = 0, piece = 0, i = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    auto step_slot = [&]() { if (++slot == kSlots) { slot = 0; ph ^= 1u; } };
+    // the product of the tile before: its V slot, and whether it is its group's first of the piece / the last of it
+    bool pending = false, pend_first = false, pend_done = false;
+    int pend_slot = 0;
+    auto product = [&](int tile) {
+      const int g = tile & 1;
+      if (!(ok = mbar_wait(p_ready + g, p_ph[g], abort_flag, a.error))) return;
+      p_ph[g] ^= 1u;
+      fence_after();
+      if (elect_one()) {
+        const uint64_t dv = desc_v(ring + (size_t)pend_slot * kTile);
+        const uint32_t tp = tmem + (uint32_t)(g * 128), to = tmem + (uint32_t)(256 + g * 128);
+#pragma unroll
+        for (int kk = 0; kk < kKeys / 16; ++kk) {   // 16 keys: the high part of P, then the low part
+          const uint64_t dvk = dv + (uint64_t)((kk * 16 * 128) >> 4);
+          const uint32_t tpk = tp + (uint32_t)((kk >> 1) * 32 + (kk & 1) * 8);
+          mma_f16_ts(to, tpk, dvk, id_o, (!pend_first || kk > 0) ? 1u : 0u);
+          mma_f16_ts(to, tpk + 16u, dvk, id_o, 1u);
+        }
+        commit(empty + pend_slot);
+        if (pend_done) commit(pv_done + g);
+      }
+      __syncwarp();
+    };
+    while (ok && w.next(a.list)) {
+      const int qb = piece & 1;
+      if (!(ok = mbar_wait(q_full + qb, (uint32_t)(piece >> 1) & 1u, abort_flag, a.error))) break;
+      ++piece;
+      for (int t = 0; t < w.nt; ++t, ++i) {
+        if (!(ok = mbar_wait(full + slot, ph, abort_flag, a.error))) break;
+        fence_after();
+        if (elect_one()) {
+          const uint64_t dq = desc_sw128(q_s + qb * kTile), dk = desc_sw128(ring + (size_t)slot * kTile);
+#pragma unroll
+          for (int j = 0; j < D / 16; ++j) {
+            const uint64_t off = (uint64_t)(((j >> 2) * kSub + (j & 3) * 32) >> 4);
+            mma_f16_ss(tmem + (uint32_t)((i & 1) * 128), dq + off, dk + off, id_s, j > 0 ? 1u : 0u);
+          }
+          commit(s_full + (i & 1));
+          commit(empty + slot);
+          if (t == w.nt - 1) commit(q_empty + qb);
+        }
+        __syncwarp();
+        step_slot();
+        if (pending) product(i - 1);
+        if (!ok) break;
+        // (the softmax warps of this tile wait for its V themselves where they have to touch it)
+        if (!(ok = mbar_wait(full + slot, ph, abort_flag, a.error))) break;
+        pending = true;
+        pend_slot = slot;
+        pend_first = t < 2;
+        pend_done = t + 2 >= w.nt;
+        step_slot();
+      }
+    }
+    if (ok && pending) product(i - 1);
   } else {
     // ---- softmax: warps 2..9.  Group 0 the warps 2..5, group 1 the warps 6..9; a warp's tensor-memory lanes are 32 (warp % 4)
     //      .. + 31, lane = query row of the tile ----
@@ -266,36 +298,20 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16);
     const uint32_t ts = lane_base + (uint32_t)(g * 128), to = lane_base + (uint32_t)(256 + g * 128);
     const float scale_log2 = kLog2eA / sqrtf((float)D);
-    const int G = a.list.G, qkv_w = (a.list.Hkv * G + 2 * a.list.Hkv) * D;
-    uint32_t s_ph = 0, pv_ph = 0, piece_ph = 0;
-    int stage0 = 0;          // ring stage and use count of the piece's first tile
-    uint32_t uses0 = 0;
-    bool ok = true, first = true;
+    const int G = a.list.G;
+    uint32_t s_ph = 0, pv_ph = 0;
+    int done = 0;            // key tiles of the pieces before
+    bool ok = true;
     while (ok && w.next(a.list)) {
       const int T = a.list.block_len[w.b], P = a.list.seq_len[w.b], Lk = P + T;
-      const int rows = min(128, G * T - w.rt * 128);
-      if (!first) {   // the query rows of the piece before are no longer read
-        if (!(ok = __all_sync(0xffffffffu, mbar_wait(piece_done, piece_ph, abort_flag, a.error)))) break;
-        piece_ph ^= 1u;
-      }
-      first = false;
-      // the query rows, K-major with the 128-byte swizzle: 256 threads, a 16-byte piece each in turn
-      for (int i = (int)threadIdx.x - 64; i < rows * (D / 8); i += 256) {
-        const int r = i / (D / 8), c = i % (D / 8);
-        const int gr = w.rt * 128 + r, node = gr / G;
-        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(a.qkv + (size_t)(w.b * a.list.T_max + node) * qkv_w + (size_t)(w.hk * G + gr % G) * D) + c);
-        *reinterpret_cast<uint4*>(q_s + (c >> 3) * kSub + r * 128 + (((c & 7) ^ (r & 7)) << 4)) = v;
-      }
-      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-      __syncwarp();
-      if (lane == 0) mbar_arrive(q_ready);
-
+      const int node0 = w.rt * a.list.npt, rows = min(a.list.npt, T - node0) * G;
       const bool active = q * 32 < rows;   // (a warp without rows only keeps the hand-shakes going)
       const bool live = row < rows;
-      const unsigned long long anc = live ? a.list.anc[w.b * a.list.T_max + (w.rt * 128 + row) / G] : 0ull;
+      const unsigned long long anc = live ? a.list.anc[w.b * a.list.T_max + node0 + row / G] : 0ull;
       float m_ref = -INFINITY, sum = 0.f;
       const size_t slot = ((size_t)(blockIdx.x + w.seg) * 2 + g) * 128 + row;
-      for (int t = g; t < w.nt; t += 2) {
+      const int t_first = (done & 1) ^ g;   // this group's first tile of the piece
+      for (int t = t_first; t < w.nt; t += 2) {
         if (!(ok = __all_sync(0xffffffffu, mbar_wait(s_full + g, s_ph, abort_flag, a.error)))) break;
         s_ph ^= 1u;
         fence_after();
@@ -326,7 +342,7 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
           if (__any_sync(0xffffffffu, grow)) {
             const float m_new = grow ? mx : m_ref;
             const float f = grow ? (m_ref == -INFINITY ? 0.f : exp2f(m_ref - m_new)) : 1.f;
-            if (t > g) {   // (the product of this group's tile before has been waited for below)
+            if (t > t_first) {   // (this S is complete, so the product of this group's tile before is)
 #pragma unroll 1
               for (int c = 0; c < D / 32; ++c) {
                 float o[32];
@@ -364,29 +380,29 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
         }
         if (k0 + kKeys > Lk) {
           // rows of V beyond the end of the sequence are whatever lies there: zero, since P = 0 does not silence a NaN
-          const uint32_t n = uses0 + (uint32_t)(stage0 + t) / kStagesA;
-          const int st = (stage0 + t) % kStagesA;
-          if (!(ok = __all_sync(0xffffffffu, mbar_wait(full + st, n & 1u, abort_flag, a.error)))) break;
-          unsigned char* vt = ring + (size_t)st * 2 * kTile + kTile;
+          const int c = 2 * (done + t) + 1;   // this tile's V in the ring's order
+          if (!(ok = __all_sync(0xffffffffu, mbar_wait(full + c % kSlots, (uint32_t)(c / kSlots) & 1u, abort_flag, a.error)))) break;
+          unsigned char* vt = ring + (size_t)(c % kSlots) * kTile;
           const int from = Lk - k0;
           for (int i = from * 8 * kSubs + (q * 32 + lane); i < kKeys * 8 * kSubs; i += 128) {
-            const int r = i / (8 * kSubs), c = i % (8 * kSubs);
-            *reinterpret_cast<uint4*>(vt + (c >> 3) * kSub + r * 128 + ((c & 7) << 4)) = make_uint4(0, 0, 0, 0);
+            const int r = i / (8 * kSubs), pc = i % (8 * kSubs);
+            *reinterpret_cast<uint4*>(vt + (pc >> 3) * kSub + r * 128 + ((pc & 7) << 4)) = make_uint4(0, 0, 0, 0);
           }
           asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         }
         fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(p_ready + g);
-        // O has this tile's product before the next one may rescale it, or before it leaves
+      }
+      if (!ok) break;
+      if (w.nt > t_first) {   // the group's products are in O
         if (!(ok = __all_sync(0xffffffffu, mbar_wait(pv_done + g, pv_ph, abort_flag, a.error)))) break;
         pv_ph ^= 1u;
         fence_after();
       }
-      if (!ok) break;
       if (active) {   // the piece's partial result
         if (live) a.ml_part[slot] = make_float2(m_ref, sum);
-        if (w.nt > g) {
+        if (w.nt > t_first) {
 #pragma unroll
           for (int c = 0; c < D / 32; ++c) {
             float o[32];
@@ -398,13 +414,9 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
             }
           }
         }
+        fence_before();   // (the next piece's P, which follows in this warp's order, lets O be overwritten)
       }
-      stage0 += w.nt;
-      uses0 += (uint32_t)(stage0 / kStagesA);
-      stage0 %= kStagesA;
-      fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(piece_done);
+      done += w.nt;
     }
   }
   __syncwarp();
@@ -417,25 +429,25 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
 }
 
 template <int D>
-int launch_d(const CUtensorMap& mk, const CUtensorMap& mv, const TcAttnArgs& a, int ctas, cudaStream_t stream) {
-  constexpr size_t smem = (size_t)(1 + 2 * kStagesA) * (D / 64) * kKeys * 128 + 1024 + 512;
+int launch_d(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const TcAttnArgs& a, int ctas, cudaStream_t stream) {
+  constexpr size_t smem = (size_t)(2 + kSlots) * (D / 64) * kKeys * 128 + 1024 + 512;
   static bool configured = false;
   if (!configured) {
     QUASAR_CUDA_CHECK(cudaFuncSetAttribute(tc_attention_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     configured = true;
   }
-  return launch_dependent(tc_attention_kernel<D>, dim3((unsigned)ctas), dim3(kThreadsA), smem, true, stream, mk, mv, a);
+  return launch_dependent(tc_attention_kernel<D>, dim3((unsigned)ctas), dim3(kThreadsA), smem, true, stream, mq, mk, mv, a);
 }
 
 }  // namespace
 
 size_t tc_attention_workspace_bytes(int B, int T_max, int Hq, int Hkv, int D) {
-  const size_t slots = kAttnCtas + (size_t)B * Hkv * ((Hq / Hkv * T_max + 127) / 128);
+  const size_t slots = kAttnCtas + (size_t)B * Hkv * attn_row_tiles(Hq / Hkv, T_max);
   return slots * 2 * 128 * ((size_t)D * 4 + 8);
 }
 
 AttnParts tc_attention_parts(void* workspace, int B, int T_max, int Hq, int Hkv, int D) {
-  const size_t slots = kAttnCtas + (size_t)B * Hkv * ((Hq / Hkv * T_max + 127) / 128);
+  const size_t slots = kAttnCtas + (size_t)B * Hkv * attn_row_tiles(Hq / Hkv, T_max);
   AttnParts p;
   p.o = reinterpret_cast<float*>(workspace);
   p.ml = reinterpret_cast<float2*>(p.o + slots * 2 * 128 * D);
@@ -444,15 +456,18 @@ AttnParts tc_attention_parts(void* workspace, int B, int T_max, int Hq, int Hkv,
 
 int launch_tc_attention(const __nv_bfloat16* qkv, const __nv_bfloat16* k_cache_layer, const __nv_bfloat16* v_cache_layer,
                         const AttnList& list, int kv_batch, int D, const AttnParts& parts, int32_t* error, cudaStream_t stream) {
-  CUtensorMap mk, mv;
+  CUtensorMap mq, mk, mv;
   const uint64_t rows = (uint64_t)kv_batch * list.Hkv * list.s_max;
   int rc = make_map_sw128(&mk, k_cache_layer, rows, (uint64_t)D * 2, kKeys);
   if (rc != QUASAR_OK) return rc;
   rc = make_map_sw128(&mv, v_cache_layer, rows, (uint64_t)D * 2, kKeys);
   if (rc != QUASAR_OK) return rc;
+  rc = make_map3_sw128(&mq, qkv, (uint64_t)D * 2, (uint64_t)list.Hkv * (list.G + 2), (uint64_t)list.B * list.T_max,
+                       (uint32_t)list.G, (uint32_t)list.npt);
+  if (rc != QUASAR_OK) return rc;
   TcAttnArgs a;
-  a.qkv = qkv; a.list = list; a.o_part = parts.o; a.ml_part = parts.ml; a.error = error;
-  return D == 128 ? launch_d<128>(mk, mv, a, kAttnCtas, stream) : launch_d<64>(mk, mv, a, kAttnCtas, stream);
+  a.q_rows = list.G * list.npt; a.list = list; a.o_part = parts.o; a.ml_part = parts.ml; a.error = error;
+  return D == 128 ? launch_d<128>(mq, mk, mv, a, kAttnCtas, stream) : launch_d<64>(mq, mk, mv, a, kAttnCtas, stream);
 }
 
 }  // namespace quasar

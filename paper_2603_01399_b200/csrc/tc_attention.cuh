@@ -9,13 +9,17 @@ namespace quasar {
 constexpr int kAttnCtas = 148;    // one per SM
 constexpr int kShapes = 128;       // sequences whose shapes a CTA keeps in shared memory (more are looked up as they come)
 
-// Segments in order of sequence, kv head, row tile (128 of the G * T query rows of a kv head); a segment's units are its tiles
+// block rows whose query heads of one kv head make up a row tile of the 128-row MMAs
+constexpr int attn_nodes_per_tile(int G) { return 128 / G; }
+constexpr int attn_row_tiles(int G, int T) { return (T + attn_nodes_per_tile(G) - 1) / attn_nodes_per_tile(G); }
+
+// Segments in order of sequence, kv head, row tile (npt block rows x G query heads); a segment's units are its tiles
 // of 128 keys.  CTA c takes the units [c * total / ctas, (c + 1) * total / ctas), and its partial results for segment s
 // lie in slot c + s.
 struct AttnList {
   const int32_t *seq_len, *block_len, *valid;
   const uint64_t* anc;    // [B*T_max]
-  int B, T_max, Hkv, G, s_max;
+  int B, T_max, Hkv, G, s_max, npt;
 };
 
 struct AttnParts {
@@ -34,10 +38,9 @@ int launch_attention_merge(int op, const AttnList& list, const AttnParts& parts,
 #ifdef __CUDACC__
 // key tiles and row tiles of a sequence (none of a skipped one)
 __device__ __forceinline__ void attn_shape(const AttnList& l, int b, int& tiles, int& row_tiles) {
-  const bool ok = l.valid[b] != 0;
-  const int T = ok ? l.block_len[b] : 0, P = ok ? l.seq_len[b] : 0;
+  const int ok = l.valid[b], T = l.block_len[b], P = l.seq_len[b];   // (side by side: a skipped one's may be anything)
   tiles = ok ? (P + T + 127) / 128 : 0;
-  row_tiles = ok ? (l.G * T + 127) / 128 : 0;
+  row_tiles = ok ? (T + l.npt - 1) / l.npt : 0;
 }
 
 // units of all sequences (every lane of a converged warp gets the sum)

@@ -90,6 +90,13 @@ __device__ __forceinline__ void tma_load_2d_hint(void* smem_dst, const CUtensorM
       : "memory");
 }
 
+__device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];\n" ::"r"(
+          smem_u32(smem_dst)),
+      "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z)
+      : "memory");
+}
 // The same for one CTA of a pair whose MMAs read both CTAs' shared memory: `bar` is a barrier of the pair's leader
 // (a shared::cluster address), which counts the bytes of both.
 template <bool HINT>
@@ -232,6 +239,9 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 #endif
 
 // [rows][row_bytes] bytes, box = box_rows x 128 bytes with the 128-byte swizzle, zeros outside
+// the same for [planes][rows][row_bytes], box = box_planes x box_rows x 128 bytes
+int make_map3_sw128(CUtensorMap* map, const void* base, uint64_t row_bytes, uint64_t rows, uint64_t planes, uint32_t box_rows,
+                    uint32_t box_planes);
 int make_map_sw128(CUtensorMap* map, const void* base, uint64_t rows, uint64_t row_bytes, uint32_t box_rows);
 
 }  // namespace tc

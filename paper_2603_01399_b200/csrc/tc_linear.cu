@@ -49,25 +49,34 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-int make_map_sw128(CUtensorMap* map, const void* base, uint64_t rows, uint64_t row_bytes, uint32_t box_rows) {
+static int make_map(CUtensorMap* map, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box) {
   auto fn = encode_fn();
   if (fn == nullptr) {
     set_error("cuTensorMapEncodeTiled is not available from this driver");
     return QUASAR_ERR_CUDA;
   }
-  const cuuint64_t dims[2] = {row_bytes, rows};
-  const cuuint64_t strides[1] = {row_bytes};
-  const cuuint32_t box[2] = {128u, box_rows};
-  const cuuint32_t estr[2] = {1, 1};
-  const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr,
+  const cuuint32_t estr[3] = {1, 1, 1};
+  const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, estr,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
-    set_error("cuTensorMapEncodeTiled failed (%d) for %llu x %llu bytes", (int)r, (unsigned long long)rows,
-              (unsigned long long)row_bytes);
+    set_error("cuTensorMapEncodeTiled failed (%d) for %llu x %llu bytes", (int)r, (unsigned long long)dims[1], (unsigned long long)dims[0]);
     return QUASAR_ERR_CUDA;
   }
   return QUASAR_OK;
+}
+
+int make_map_sw128(CUtensorMap* map, const void* base, uint64_t rows, uint64_t row_bytes, uint32_t box_rows) {
+  const cuuint64_t dims[2] = {row_bytes, rows}, strides[1] = {row_bytes};
+  const cuuint32_t box[2] = {128u, box_rows};
+  return make_map(map, base, 2, dims, strides, box);
+}
+
+int make_map3_sw128(CUtensorMap* map, const void* base, uint64_t row_bytes, uint64_t rows, uint64_t planes, uint32_t box_rows,
+                    uint32_t box_planes) {
+  const cuuint64_t dims[3] = {row_bytes, rows, planes}, strides[2] = {row_bytes, row_bytes * rows};
+  const cuuint32_t box[3] = {128u, box_rows, box_planes};
+  return make_map(map, base, 3, dims, strides, box);
 }
 
 }  // namespace tc
