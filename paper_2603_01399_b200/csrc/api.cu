@@ -70,7 +70,7 @@ size_t align_up(size_t v, size_t a = 256) { return (v + a - 1) / a * a; }
 
 // Layout of the verify workspace; every offset is a multiple of 256 bytes.
 struct Workspace {
-  size_t x, h, qkv, attn, gu, act, attn16, act16, op, op_scale, keys, top1, anc, depth, valid, att, cand, ss_part, amax, attn_count, barrier, total;
+  size_t x, h, qkv, attn, gu, act, attn16, act16, op, op_scale, act_max, seq, keys, top1, anc, depth, valid, att, cand, ss_part, amax, attn_count, barrier, total;
   size_t att_bytes;
 };
 
@@ -94,6 +94,8 @@ Workspace layout(const quasar_config& c, int B, int T_max, int s_max) {
   const size_t widest = std::max(std::max((size_t)c.hidden, (size_t)c.n_q_heads * c.head_dim), (size_t)c.ffn);
   w.op = take(3 * M * widest);
   w.op_scale = take(M * 4);
+  w.seq = take((size_t)(B + 1) * sizeof(AttnSeq));
+  w.act_max = take((size_t)c.n_layers * M * 4);
   w.keys = take(M * 8);
   w.top1 = take(M * 4);
   w.anc = take(M * 8);
@@ -282,7 +284,8 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
   // the order of the norms' sums of squares: the W8A8 form keeps its two (a last bit there becomes quantisation steps)
   const int adders = form == kOperandBf16 || (a8 && (M > 72 || H > 8192 || F > 24576)) ? 256 : 1024;
   BlockArgs ba{tokens, parents, block_len, kv->seq_len, B, T_max, kv->s_max, c.vocab, bi,
-               reinterpret_cast<unsigned long long*>(wsp + ws.keys), status};
+               reinterpret_cast<unsigned long long*>(wsp + ws.keys), status, reinterpret_cast<AttnSeq*>(wsp + ws.seq), Hkv,
+               attn_nodes_per_tile(Hq / Hkv), reinterpret_cast<unsigned*>(wsp + ws.act_max), c.n_layers * M};
   int8_t* op_q = reinterpret_cast<int8_t*>(wsp + ws.op);
   float* op_scale = reinterpret_cast<float*>(wsp + ws.op_scale);
   // (the bf16 rows themselves are needed where they are the operand, and for a trace)
@@ -299,7 +302,8 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
       return launch_tc_linear_w8a8(op_q, op_scale, wq, delta, M, N, K, out, out_f32, res, nullptr, keys, status, true, stream);
     return launch_tc_linear_digits(op_q, op_scale, wq, delta, M, N, K, out, out_f32, res, keys, status, true, stream);
   };
-  const AttnList list{kv->seq_len, block_len, bi.valid, bi.anc, B, T_max, Hkv, Hq / Hkv, kv->s_max, attn_nodes_per_tile(Hq / Hkv)};
+  const bool fuse = !traced && tc_fusable(form, M);   // RoPE and SwiGLU in the epilogues of the layers before them
+  const AttnList list{kv->seq_len, block_len, bi.valid, ba.seq, bi.anc, B, T_max, Hkv, Hq / Hkv, kv->s_max, attn_nodes_per_tile(Hq / Hkv)};
   const AttnParts parts = tc_attention_parts(att, B, T_max, Hq, Hkv, D);
   auto norm_gain = [&](int l) {
     return reinterpret_cast<const __nv_bfloat16*>(l < c.n_layers ? m->layers[l].attn_norm : m->w.final_norm);
@@ -313,26 +317,40 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
     __nv_bfloat16* kc = reinterpret_cast<__nv_bfloat16*>(kv->k) + (size_t)l * layer_stride;
     __nv_bfloat16* vc = reinterpret_cast<__nv_bfloat16*>(kv->v) + (size_t)l * layer_stride;
     TRY(tr.put(h, (size_t)M * H * 2));
-    TRY(linear(h, L.qkv_w, L.qkv_delta, qkv_w, H, qkv, false, nullptr, nullptr));
-    TRY(tr.put(qkv, (size_t)M * qkv_w * 2));
-    TRY(launch_rope_append(qkv, reinterpret_cast<const __nv_bfloat16*>(c.qk_norm ? L.q_norm : nullptr),
-                           reinterpret_cast<const __nv_bfloat16*>(c.qk_norm ? L.k_norm : nullptr), m->rope_table,
-                           kv->seq_len, block_len, bi, B, T_max, Hq, Hkv, D, c.rms_eps, kc, vc, kv->s_max, stream));
-    TRY(tr.put(qkv, (size_t)M * qkv_w * 2));
-    if (a8 || Hq * D > 24576) {   // (longer rows do not fit the merge's shared memory)
+    const RopeArgs rope{qkv, reinterpret_cast<const __nv_bfloat16*>(c.qk_norm ? L.q_norm : nullptr),
+                        reinterpret_cast<const __nv_bfloat16*>(c.qk_norm ? L.k_norm : nullptr), m->rope_table, kv->seq_len, block_len,
+                        bi, kc, vc, T_max, Hq, Hkv, D, kv->s_max, c.rms_eps};
+    if (fuse) {
+      TRY(launch_tc_qkv_rope(form, form == kOperandBf16 ? (const void*)h : op_q, op_scale, L.qkv_w, L.qkv_delta, M, H, rope, status, stream));
+    } else {
+      TRY(linear(h, L.qkv_w, L.qkv_delta, qkv_w, H, qkv, false, nullptr, nullptr));
+      TRY(tr.put(qkv, (size_t)M * qkv_w * 2));
+      TRY(launch_rope_append(rope, B, stream));
+      TRY(tr.put(qkv, (size_t)M * qkv_w * 2));
+    }
+    const RowOperand attn_out{form == kOperandBf16 || traced ? attn : nullptr, op_q, op_scale, L.o_smooth};
+    if (a8) {
       // (the W8A8 form keeps the order of this kernel's sums: a last bit of the attention output becomes quantisation steps)
-      TRY(launch_attention(qkv, kc, vc, kv->seq_len, block_len, bi, B, T_max, Hq, Hkv, D, kv->s_max, attn, att, ws.att_bytes, stream));
-      TRY(launch_operand(form, attn, M, Hq * D, RowOperand{nullptr, op_q, op_scale, L.o_smooth}, stream));
+      AttnChunks chunks;
+      TRY(launch_attention(qkv, kc, vc, kv->seq_len, block_len, bi, B, T_max, Hq, Hkv, D, kv->s_max, att, ws.att_bytes, &chunks, stream));
+      TRY(launch_attention_merge(form, list, AttnParts{chunks.o, chunks.ml}, &chunks, M, D, attn_out, stream));
     } else {
       TRY(launch_tc_attention(qkv, kc, vc, list, kv->batch, D, parts, status, stream));
-      TRY(launch_attention_merge(form, list, parts, M, D, operand(attn, nullptr), stream));
+      TRY(launch_attention_merge(form, list, parts, nullptr, M, D, attn_out, stream));
     }
     TRY(tr.put(attn, (size_t)M * Hq * D * 2));
     TRY(linear(attn, L.o_w, L.o_delta, H, Hq * D, x, false, x, nullptr));
     TRY(tr.put(x, (size_t)M * H * 2));
     TRY(launch_norm(form, x, reinterpret_cast<const __nv_bfloat16*>(L.mlp_norm), M, H, c.rms_eps, adders, operand(h, L.gateup_smooth), stream));
-    TRY(linear(h, L.gateup_w, L.gateup_delta, 2 * (int64_t)F, H, gu, false, nullptr, nullptr));
-    TRY(launch_swiglu(form, gu, M, F, operand(act, L.down_smooth), stream));
+    if (fuse) {
+      unsigned* act_max = form == kOperandBf16 ? nullptr : reinterpret_cast<unsigned*>(wsp + ws.act_max) + (size_t)l * M;
+      TRY(launch_tc_gateup_swiglu(form, form == kOperandBf16 ? (const void*)h : op_q, op_scale, L.gateup_w, L.gateup_delta, M, F, H, act, act_max,
+                                  L.down_smooth, status, stream));
+      TRY(launch_operand(form, act, act_max, M, F, RowOperand{nullptr, op_q, op_scale, L.down_smooth}, stream));
+    } else {
+      TRY(linear(h, L.gateup_w, L.gateup_delta, 2 * (int64_t)F, H, gu, false, nullptr, nullptr));
+      TRY(launch_swiglu(form, gu, M, F, operand(act, L.down_smooth), stream));
+    }
     TRY(tr.put(act, (size_t)M * F * 2));
     TRY(linear(act, L.down_w, L.down_delta, H, F, x, false, x, nullptr));
     TRY(tr.put(x, (size_t)M * H * 2));

@@ -12,7 +12,7 @@
 // Parallelism: the key range of a sequence is cut into chunks of `chunk` positions; a CTA
 // handles one (sequence, kv head, chunk) with one warp per 16 query rows, all warps
 // sharing the K/V tiles staged in shared memory.  Each CTA leaves an un-normalised partial
-// (row max, row sum, O) and a second kernel merges the partials of a row in chunk order.
+// (row max, row sum, O) and a second kernel (row_ops.cu) merges the partials of a row in chunk order.
 // P is fed to the PV product as a bf16 high part plus a bf16 low part (two MMAs), which
 // keeps ~16 bits of the probabilities.
 #include <math.h>
@@ -37,7 +37,6 @@ struct AttnArgs {
   BlockInfo bi;
   float* o_part;             // [B][Hkv][nchunk][Rpad][D]
   float* ml_part;            // [B][Hkv][nchunk][Rpad][2]
-  __nv_bfloat16* out;        // [B*T_max][Hq*D]
   int B, T_max, Hq, Hkv, s_max, chunk, nchunk, Rpad, ngroups;
 };
 
@@ -285,70 +284,6 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 4) verify_attention_kernel(Att
   }
 }
 
-// One warp per (sequence, block row, query head): merge the chunk partials in chunk order.
-template <int D>
-__global__ void __launch_bounds__(128) attention_merge_kernel(AttnArgs a) {
-  tc::pdl_trigger();
-  tc::pdl_wait();
-  const int item = blockIdx.x * 4 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (item >= a.B * a.T_max * a.Hq) return;
-  const int hq = item % a.Hq;
-  const int m = item / a.Hq;
-  const int b = m / a.T_max, i = m % a.T_max;
-  __nv_bfloat16* dst = a.out + (size_t)m * a.Hq * D + (size_t)hq * D;
-  constexpr int kPer = D / 32;
-  if (!a.bi.valid[b] || i >= a.block_len[b]) {
-#pragma unroll
-    for (int e = 0; e < kPer; ++e) dst[lane * kPer + e] = __float2bfloat16_rn(0.f);
-    return;
-  }
-  const int G = a.Hq / a.Hkv;
-  const int hk = hq / G;
-  const int r = i * G + (hq % G);
-  const int Lk = a.seq_len[b] + a.block_len[b];
-  const int nch = (Lk + a.chunk - 1) / a.chunk;
-  const size_t slot0 = ((size_t)b * a.Hkv + hk) * a.nchunk * a.Rpad;
-  // the row's maximum over the chunks: the lanes take the chunks in turn
-  float mx = -INFINITY;
-  for (int c = lane; c < nch; c += 32) mx = fmaxf(mx, a.ml_part[(slot0 + (size_t)c * a.Rpad + r) * 2]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  float acc[kPer];
-#pragma unroll
-  for (int e = 0; e < kPer; ++e) acc[e] = 0.f;
-  float den = 0.f;
-  // chunks are added in chunk order, eight at a time so that their loads are in flight together
-  for (int c0 = 0; c0 < nch; c0 += 8) {
-    float2 ml[8];
-    float ov[8][kPer];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const bool in = c0 + j < nch;
-      const size_t s = slot0 + (size_t)(in ? c0 + j : c0) * a.Rpad + r;
-      ml[j] = in ? *reinterpret_cast<const float2*>(a.ml_part + s * 2) : make_float2(-INFINITY, 0.f);
-      if constexpr (kPer == 4) {
-        const float4 v = *reinterpret_cast<const float4*>(a.o_part + s * D + lane * kPer);
-        ov[j][0] = v.x; ov[j][1] = v.y; ov[j][2] = v.z; ov[j][3] = v.w;
-      } else {
-        const float2 v = *reinterpret_cast<const float2*>(a.o_part + s * D + lane * kPer);
-        ov[j][0] = v.x; ov[j][1] = v.y;
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if (ml[j].x == -INFINITY) continue;
-      const float w = exp2f(ml[j].x - mx);
-      den += w * ml[j].y;
-#pragma unroll
-      for (int e = 0; e < kPer; ++e) acc[e] += w * ov[j][e];
-    }
-  }
-  const float inv = 1.0f / den;
-#pragma unroll
-  for (int e = 0; e < kPer; ++e) dst[lane * kPer + e] = __float2bfloat16_rn(acc[e] * inv);
-}
-
 struct AttnPlan {
   int chunk, nchunk, Rpad, ngroups, warps;
 };
@@ -382,8 +317,7 @@ size_t attention_workspace_bytes(int B, int T_max, int Hq, int Hkv, int D, int s
 
 int launch_attention(const __nv_bfloat16* qkv, const __nv_bfloat16* k_cache_layer, const __nv_bfloat16* v_cache_layer,
                      const int32_t* seq_len, const int32_t* block_len, BlockInfo bi, int B, int T_max, int Hq, int Hkv,
-                     int D, int s_max, __nv_bfloat16* out, void* workspace, size_t workspace_bytes,
-                     cudaStream_t stream) {
+                     int D, int s_max, void* workspace, size_t workspace_bytes, AttnChunks* chunks, cudaStream_t stream) {
   const AttnPlan p = plan_attention(B, T_max, Hq, Hkv, s_max);
   if (workspace_bytes < attention_workspace_bytes(B, T_max, Hq, Hkv, D, s_max)) {
     set_error("attention: workspace too small");
@@ -394,11 +328,10 @@ int launch_attention(const __nv_bfloat16* qkv, const __nv_bfloat16* k_cache_laye
   const size_t rows = (size_t)B * Hkv * p.nchunk * p.Rpad;
   a.o_part = reinterpret_cast<float*>(workspace);
   a.ml_part = a.o_part + rows * D;
-  a.out = out;
   a.B = B; a.T_max = T_max; a.Hq = Hq; a.Hkv = Hkv; a.s_max = s_max;
   a.chunk = p.chunk; a.nchunk = p.nchunk; a.Rpad = p.Rpad; a.ngroups = p.ngroups;
+  *chunks = AttnChunks{p.chunk, p.nchunk, p.Rpad, a.o_part, reinterpret_cast<float2*>(a.ml_part)};
   dim3 grid(p.nchunk * p.ngroups, Hkv, B);
-  const int items = B * T_max * Hq;
   if (D == 128) {
     constexpr size_t smem128 = 4u * kKeyTile * (128 + 8) * sizeof(__nv_bfloat16);
     static bool configured128 = false;
@@ -407,18 +340,14 @@ int launch_attention(const __nv_bfloat16* qkv, const __nv_bfloat16* k_cache_laye
       QUASAR_CUDA_CHECK(cudaFuncSetAttribute(verify_attention_kernel<128>, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
       configured128 = true;
     }
-    const int rc = launch_dependent(verify_attention_kernel<128>, grid, dim3(p.warps * 32), smem128, true, stream, a);
-    if (rc != QUASAR_OK) return rc;
-    return launch_dependent(attention_merge_kernel<128>, dim3((items + 3) / 4), dim3(128), 0, true, stream, a);
-  } else if (D == 64) {
-    constexpr size_t smem64 = 4u * kKeyTile * (64 + 8) * sizeof(__nv_bfloat16);
-    const int rc = launch_dependent(verify_attention_kernel<64>, grid, dim3(p.warps * 32), smem64, true, stream, a);
-    if (rc != QUASAR_OK) return rc;
-    return launch_dependent(attention_merge_kernel<64>, dim3((items + 3) / 4), dim3(128), 0, true, stream, a);
-  } else {
-    set_error("head_dim %d not supported (64 or 128)", D);
-    return QUASAR_ERR_SHAPE;
+    return launch_dependent(verify_attention_kernel<128>, grid, dim3(p.warps * 32), smem128, true, stream, 1, a);
   }
+  if (D == 64) {
+    constexpr size_t smem64 = 4u * kKeyTile * (64 + 8) * sizeof(__nv_bfloat16);
+    return launch_dependent(verify_attention_kernel<64>, grid, dim3(p.warps * 32), smem64, true, stream, 1, a);
+  }
+  set_error("head_dim %d not supported (64 or 128)", D);
+  return QUASAR_ERR_SHAPE;
 }
 
 }  // namespace quasar

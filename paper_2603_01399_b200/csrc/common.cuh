@@ -34,20 +34,29 @@ void count_launch(int n = 1);
 static inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 #ifdef __CUDACC__
-// Launches a kernel that waits for the one in front of it on the stream by itself (griddepcontrol.wait); `pdl`: it may start
+// Launches a kernel (`cluster` neighbouring CTAs to a cluster) that waits for the one in front of it on the stream by itself (griddepcontrol.wait); `pdl`: it may start
 // before that one has finished.
 template <typename... P, typename... A>
-int launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, bool pdl, cudaStream_t stream, A&&... args) {
+int launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, bool pdl, cudaStream_t stream, int cluster, A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = pdl ? 1 : 0;
+  cudaLaunchAttribute attr[2];
+  unsigned n = 0;
+  if (pdl) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = (unsigned)cluster;
+    attr[n].val.clusterDim.y = 1;
+    attr[n++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = n;
   QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
   count_launch();
   return QUASAR_OK;
@@ -106,6 +115,12 @@ struct BlockInfo {
   int32_t* valid;   // [B] 1 if the sequence is processed (block fits, parents well formed)
 };
 
+// A sequence's place in the list that the tcgen05 attention deals out (tc_attention.cuh): its key tiles and row tiles (none if
+// it is skipped), the units and segments before it; entry B holds the totals.
+struct AttnSeq {
+  int tiles, row_tiles, unit0, seg0;
+};
+
 // What the kernels at either end of the pass need to know about the draft blocks.
 struct BlockArgs {
   const int32_t *tokens, *parents, *block_len, *seq_len;
@@ -113,6 +128,10 @@ struct BlockArgs {
   BlockInfo bi;
   unsigned long long* keys;   // [B*T_max] arg-max keys of the rows, cleared by the first kernel, or nullptr
   int32_t* status;
+  AttnSeq* seq;               // [B + 1]
+  int Hkv, npt;               // kv heads; block rows of a row tile
+  unsigned* clear;            // [n_clear] words that the first kernel sets to zero
+  int n_clear;
 };
 
 // ---- whole-row steps that leave the operand of the following linear layer (row_ops.cu) ----
@@ -128,21 +147,24 @@ int launch_embed_norm(int op, const BlockArgs& a, const __nv_bfloat16* embed, __
                       int adders, const RowOperand& out, cudaStream_t stream);
 int launch_norm(int op, const __nv_bfloat16* x, const __nv_bfloat16* g, int M, int H, float eps, int adders, const RowOperand& out, cudaStream_t stream);
 int launch_swiglu(int op, const __nv_bfloat16* gu, int M, int F, const RowOperand& out, cudaStream_t stream);
-int launch_operand(int op, const __nv_bfloat16* x, int M, int K, const RowOperand& out, cudaStream_t stream);
+int launch_operand(int op, const __nv_bfloat16* x, const unsigned* row_max, int M, int K, const RowOperand& out, cudaStream_t stream);
 int launch_accept(const BlockArgs& a, int32_t* accept_len, int32_t* bonus, int32_t* accept_path, cudaStream_t stream);
 
 // QK-RMSNorm + RoPE on the q and k heads of qkv (in place) and K/V append at slot seq_len[b] + row.
-int launch_rope_append(__nv_bfloat16* qkv, const __nv_bfloat16* q_norm, const __nv_bfloat16* k_norm,
-                       const float2* rope_table, const int32_t* seq_len, const int32_t* block_len, BlockInfo bi, int B,
-                       int T_max, int Hq, int Hkv, int D, float eps, __nv_bfloat16* k_cache_layer,
-                       __nv_bfloat16* v_cache_layer, int s_max, cudaStream_t stream);
+struct RopeArgs;
+int launch_rope_append(const RopeArgs& a, int B, cudaStream_t stream);
 
 size_t attention_workspace_bytes(int B, int T_max, int Hq, int Hkv, int D, int s_max);
+// Partial results over chunks of the keys: un-normalised outputs o [B][Hkv][nchunk][Rpad][D] and (row maximum, sum)
+// ml [B][Hkv][nchunk][Rpad], for launch_attention_merge
+struct AttnChunks {
+  int chunk, nchunk, Rpad;
+  float* o;
+  float2* ml;
+};
 int launch_attention(const __nv_bfloat16* qkv, const __nv_bfloat16* k_cache_layer, const __nv_bfloat16* v_cache_layer,
                      const int32_t* seq_len, const int32_t* block_len, BlockInfo bi, int B, int T_max, int Hq, int Hkv,
-                     int D, int s_max, __nv_bfloat16* out, void* workspace, size_t workspace_bytes,
-                     cudaStream_t stream);
-
+                     int D, int s_max, void* workspace, size_t workspace_bytes, AttnChunks* chunks, cudaStream_t stream);
 int launch_kv_commit(__nv_bfloat16* k_cache, __nv_bfloat16* v_cache, int32_t* seq_len, const int32_t* accept_len,
                      const int32_t* accept_path, int L, int B_cache, int B, int T_max, int Hkv, int D, int s_max,
                      cudaStream_t stream);

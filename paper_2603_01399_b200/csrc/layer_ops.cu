@@ -3,17 +3,12 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "rope.cuh"
 #include "tc_common.cuh"
 
 namespace quasar {
 
 namespace {
-
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 
 // ---- RoPE table: cos/sin(pos * theta^(-2i/D)) evaluated in fp64, stored as fp32 -------------
 __global__ void rope_table_kernel(float2* table, int max_pos, int D, double theta) {
@@ -29,61 +24,32 @@ __global__ void rope_table_kernel(float2* table, int max_pos, int D, double thet
 
 // ---- QK-RMSNorm + RoPE + KV append: one warp per (row, head) --------------------------------
 template <int D>
-__global__ void __launch_bounds__(128)
-rope_append_kernel(__nv_bfloat16* __restrict__ qkv, const __nv_bfloat16* __restrict__ q_norm,
-                   const __nv_bfloat16* __restrict__ k_norm, const float2* __restrict__ rope_table,
-                   const int32_t* __restrict__ seq_len, const int32_t* __restrict__ block_len, BlockInfo bi, int T_max,
-                   int Hq, int Hkv, float eps, __nv_bfloat16* __restrict__ k_cache, __nv_bfloat16* __restrict__ v_cache,
-                   int s_max, int n_items) {
+__global__ void __launch_bounds__(128) rope_append_kernel(const RopeArgs a, int n_items) {
   tc::pdl_trigger();
   tc::pdl_wait();
-  constexpr int kPairs = D / 64;  // rotation pairs (i, i + D/2) per lane
   const int item = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (item >= n_items) return;
   const int lane = threadIdx.x & 31;
-  const int heads = Hq + 2 * Hkv;
+  const int heads = a.Hq + 2 * a.Hkv;
   const int m = item / heads, head = item % heads;
-  const int b = m / T_max, i = m % T_max;
-  if (!bi.valid[b] || i >= block_len[b]) return;
-  const int P = seq_len[b];
-  __nv_bfloat16* src = qkv + (size_t)m * heads * D + (size_t)head * D;
-
-  if (head >= Hq + Hkv) {  // v head: copy into the cache
-    const int hk = head - Hq - Hkv;
-    __nv_bfloat16* dst = v_cache + (((size_t)b * Hkv + hk) * s_max + (P + i)) * D;
+  const int b = m / a.T_max, i = m % a.T_max;
+  if (!a.bi.valid[b] || i >= a.block_len[b]) return;
+  const int P = a.seq_len[b];
+  __nv_bfloat16* src = a.qkv + (size_t)m * heads * D + (size_t)head * D;
+  if (head >= a.Hq + a.Hkv) {  // v head: copy into the cache
+    __nv_bfloat16* dst = a.v_cache + (((size_t)b * a.Hkv + (head - a.Hq - a.Hkv)) * a.s_max + (P + i)) * D;
     if (lane < D / 8) reinterpret_cast<uint4*>(dst)[lane] = reinterpret_cast<const uint4*>(src)[lane];
     return;
   }
-  const bool is_q = head < Hq;
-  const __nv_bfloat16* gain = is_q ? q_norm : k_norm;
-  float lo[kPairs], hi[kPairs];
-  float ss = 0.f;
+  const bool is_q = head < a.Hq;
+  float lo[D / 64], hi[D / 64];
 #pragma unroll
-  for (int p = 0; p < kPairs; ++p) {
-    const int d = lane + 32 * p;
-    lo[p] = __bfloat162float(src[d]);
-    hi[p] = __bfloat162float(src[d + D / 2]);
-    ss += lo[p] * lo[p] + hi[p] * hi[p];
+  for (int p = 0; p < D / 64; ++p) {
+    lo[p] = __bfloat162float(src[lane + 32 * p]);
+    hi[p] = __bfloat162float(src[lane + 32 * p + D / 2]);
   }
-  if (gain != nullptr) {
-    ss = warp_sum(ss);
-    const float r = 1.0f / sqrtf(ss / (float)D + eps);
-#pragma unroll
-    for (int p = 0; p < kPairs; ++p) {
-      const int d = lane + 32 * p;
-      lo[p] = lo[p] * r * __bfloat162float(gain[d]);
-      hi[p] = hi[p] * r * __bfloat162float(gain[d + D / 2]);
-    }
-  }
-  const int pos = P + bi.depth[m];
-  __nv_bfloat16* dst = is_q ? src : k_cache + (((size_t)b * Hkv + (head - Hq)) * s_max + (P + i)) * D;
-#pragma unroll
-  for (int p = 0; p < kPairs; ++p) {
-    const int d = lane + 32 * p;
-    const float2 cs = rope_table[(size_t)pos * (D / 2) + d];
-    dst[d] = __float2bfloat16_rn(lo[p] * cs.x - hi[p] * cs.y);
-    dst[d + D / 2] = __float2bfloat16_rn(hi[p] * cs.x + lo[p] * cs.y);
-  }
+  __nv_bfloat16* dst = is_q ? src : a.k_cache + (((size_t)b * a.Hkv + (head - a.Hq)) * a.s_max + (P + i)) * D;
+  rope_head<D>(lo, hi, is_q ? a.q_norm : a.k_norm, a.table, P + a.bi.depth[m], a.eps, dst);
 }
 
 // ---- commit: (tree) move accepted rows into place, then bump seq_len --------------------------
@@ -135,22 +101,13 @@ int launch_rope_table(float2* table, int max_pos, int D, float theta, cudaStream
   return QUASAR_OK;
 }
 
-int launch_rope_append(__nv_bfloat16* qkv, const __nv_bfloat16* q_norm, const __nv_bfloat16* k_norm,
-                       const float2* rope_table, const int32_t* seq_len, const int32_t* block_len, BlockInfo bi, int B,
-                       int T_max, int Hq, int Hkv, int D, float eps, __nv_bfloat16* k_cache_layer,
-                       __nv_bfloat16* v_cache_layer, int s_max, cudaStream_t stream) {
-  const int n_items = B * T_max * (Hq + 2 * Hkv);
-  const int grid = (n_items + 3) / 4;
-  if (D == 128) {
-    return launch_dependent(rope_append_kernel<128>, dim3(grid), dim3(128), 0, true, stream, qkv, q_norm, k_norm, rope_table, seq_len, block_len, bi, T_max,
-                                                       Hq, Hkv, eps, k_cache_layer, v_cache_layer, s_max, n_items);
-  } else if (D == 64) {
-    return launch_dependent(rope_append_kernel<64>, dim3(grid), dim3(128), 0, true, stream, qkv, q_norm, k_norm, rope_table, seq_len, block_len, bi, T_max,
-                                                      Hq, Hkv, eps, k_cache_layer, v_cache_layer, s_max, n_items);
-  } else {
-    set_error("head_dim %d not supported (64 or 128)", D);
-    return QUASAR_ERR_SHAPE;
-  }
+int launch_rope_append(const RopeArgs& a, int B, cudaStream_t stream) {
+  const int n_items = B * a.T_max * (a.Hq + 2 * a.Hkv);
+  const dim3 grid((unsigned)((n_items + 3) / 4));
+  if (a.D == 128) return launch_dependent(rope_append_kernel<128>, grid, dim3(128), 0, true, stream, 1, a, n_items);
+  if (a.D == 64) return launch_dependent(rope_append_kernel<64>, grid, dim3(128), 0, true, stream, 1, a, n_items);
+  set_error("head_dim %d not supported (64 or 128)", a.D);
+  return QUASAR_ERR_SHAPE;
 }
 
 int launch_kv_commit(__nv_bfloat16* k_cache, __nv_bfloat16* v_cache, int32_t* seq_len, const int32_t* accept_len,

@@ -46,7 +46,7 @@ __device__ __forceinline__ uint4 round8(float (&f)[8]) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-template <bool MAX, int THREADS = kRowThreads>
+template <bool MAX>
 __device__ __forceinline__ float block_reduce(float v, float* s_buf) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -57,7 +57,7 @@ __device__ __forceinline__ float block_reduce(float v, float* s_buf) {
   __syncthreads();
   v = s_buf[0];
 #pragma unroll
-  for (int i = 1; i < THREADS / 32; ++i) v = MAX ? fmaxf(v, s_buf[i]) : v + s_buf[i];   // warps in order
+  for (int i = 1; i < kRowThreads / 32; ++i) v = MAX ? fmaxf(v, s_buf[i]) : v + s_buf[i];   // warps in order
   return v;
 }
 
@@ -72,17 +72,28 @@ __device__ __forceinline__ void load_smooth8(const float* smooth, int i, float (
   s[0] = a.x; s[1] = a.y; s[2] = a.z; s[3] = a.w; s[4] = b.x; s[5] = b.y; s[6] = b.z; s[7] = b.w;
 }
 
+// Eq. 9 for eight elements: codes of the smoothed values
+__device__ __forceinline__ uint2 smoothed_codes8(const float (&f)[8], const float (&s)[8], float scale) {
+  uint32_t p[2] = {0u, 0u};
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const int q = max(-127, min(127, __float2int_rn(__fdiv_rn(__fmul_rn(f[e], s[e]), scale))));
+    p[e >> 2] |= (uint32_t)(q & 0xff) << (8 * (e & 3));
+  }
+  return make_uint2(p[0], p[1]);
+}
+
 // The row's values (eight of vector i by value(i, j, f); j is the turn) as the operand.
-template <int OP, int V, int THREADS = kRowThreads, typename F>
+template <int OP, int V, typename F>
 __device__ __forceinline__ void write_operand(F&& value, int nvec, int m, const RowOperand& out, float* s_buf) {
   if (OP == kOperandBf16) {   // (the values have been stored as they were made)
     float f[8];
     if (V > 0) {
 #pragma unroll
       for (int j = 0; j < (V > 0 ? V : 1); ++j)
-        if ((int)threadIdx.x + j * THREADS < nvec) value((int)threadIdx.x + j * THREADS, j, f);
+        if ((int)threadIdx.x + j * kRowThreads < nvec) value((int)threadIdx.x + j * kRowThreads, j, f);
     } else {
-      for (int i = threadIdx.x; i < nvec; i += THREADS) value(i, 0, f);
+      for (int i = threadIdx.x; i < nvec; i += kRowThreads) value(i, 0, f);
     }
     return;
   }
@@ -92,7 +103,7 @@ __device__ __forceinline__ void write_operand(F&& value, int nvec, int m, const 
   if (V > 0) {
 #pragma unroll
     for (int j = 0; j < (V > 0 ? V : 1); ++j) {
-      const int i = (int)threadIdx.x + j * THREADS;
+      const int i = (int)threadIdx.x + j * kRowThreads;
       if (i < nvec) {
         value(i, j, f[j]);
 #pragma unroll
@@ -100,13 +111,13 @@ __device__ __forceinline__ void write_operand(F&& value, int nvec, int m, const 
       }
     }
   } else {
-    for (int i = threadIdx.x; i < nvec; i += THREADS) {
+    for (int i = threadIdx.x; i < nvec; i += kRowThreads) {
       value(i, 0, f[0]);
 #pragma unroll
       for (int e = 0; e < 8; ++e) amax = fmaxf(amax, fabsf(f[0][e]));
     }
   }
-  amax = block_reduce<true, THREADS>(amax, s_buf);
+  amax = block_reduce<true>(amax, s_buf);
   float up = 1.f, scale = 1.f;
   if (OP == kOperandDigits) digit_scale(amax, up, scale);
   else scale = amax == 0.f ? 1.0f : __fdiv_rn(amax, 127.0f);
@@ -127,9 +138,9 @@ __device__ __forceinline__ void write_operand(F&& value, int nvec, int m, const 
   if (V > 0) {
 #pragma unroll
     for (int j = 0; j < (V > 0 ? V : 1); ++j)
-      if ((int)threadIdx.x + j * THREADS < nvec) put((int)threadIdx.x + j * THREADS, f[j]);
+      if ((int)threadIdx.x + j * kRowThreads < nvec) put((int)threadIdx.x + j * kRowThreads, f[j]);
   } else {
-    for (int i = threadIdx.x; i < nvec; i += THREADS) {
+    for (int i = threadIdx.x; i < nvec; i += kRowThreads) {
       value(i, 0, f[0]);
       put(i, f[0]);
     }
@@ -263,132 +274,190 @@ swiglu_kernel(const __nv_bfloat16* gu, int nvec, RowOperand out) {
       nvec, m, out, s_buf);
 }
 
-template <int OP, int V>
-__global__ void __launch_bounds__(kRowThreads) operand_kernel(const __nv_bfloat16* x, int nvec, RowOperand out) {
-  __shared__ float s_buf[32];
+// The operand of rows whose largest magnitude is known (its bits in row_max, gathered by the kernel that wrote the rows): every
+// element for itself.
+constexpr int kElemThreads = 128;
+template <int OP>
+__global__ void __launch_bounds__(kElemThreads)
+operand_kernel(const __nv_bfloat16* x, const unsigned* row_max, int nvec, RowOperand out) {
   pdl_trigger();
+  const int m = blockIdx.y, i = blockIdx.x * kElemThreads + threadIdx.x;
+  float s[8];
+  if (OP == kOperandCodes && i < nvec) load_smooth8(out.smooth, i, s);
   pdl_wait();
-  const int m = blockIdx.x;
-  const uint4* row = reinterpret_cast<const uint4*>(x + (size_t)m * nvec * 8);
-  write_operand<OP, V>(
-      [&](int i, int j, float (&f)[8]) {
-        unpack8(row[i], f);
-        if (OP == kOperandCodes) {
-          float s[8];
-          load_smooth8(out.smooth, i, s);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) f[e] = __fmul_rn(f[e], s[e]);
-        }
-      },
-      nvec, m, out, s_buf);
+  const float amax = __uint_as_float(row_max[m]);
+  float up = 1.f, scale = 1.f;
+  if (OP == kOperandDigits) digit_scale(amax, up, scale);
+  else scale = amax == 0.f ? 1.0f : __fdiv_rn(amax, 127.0f);
+  if (blockIdx.x == 0 && threadIdx.x == 0) out.scale[m] = scale;
+  if (i >= nvec) return;
+  float f[8];
+  unpack8(reinterpret_cast<const uint4*>(x + (size_t)m * nvec * 8)[i], f);
+  const int64_t width = (int64_t)nvec * 8;
+  if (OP == kOperandDigits) {
+    write_digits8(f, up, out.q + 3 * (int64_t)m * width, width, (int64_t)i * 8);
+  } else {
+    *reinterpret_cast<uint2*>(out.q + (int64_t)m * width + (int64_t)i * 8) = smoothed_codes8(f, s, scale);
+  }
 }
 
-// Puts the partial results of the tcgen05 attention together (tc_attention.cuh says where they lie): one CTA per block row, a
-// warp per query head in turn.  A head's parts are the two groups of every CTA whose run of the list touched its segment,
-// added in list order; the finished row goes through shared memory into the operand of the o projection.
-constexpr int kMergeThreads = 1024;   // a warp for each of 32 heads
+// Puts an attention's partial results together and leaves the o projection's operand: a cluster of four CTAs per block row,
+// each a quarter of the query heads, a warp per head.  A head's parts lie `stride` entries apart and are added in their order
+// (tcgen05 form: the two groups of every CTA whose run of the list touched the head's segment, see tc_attention.cuh; the other
+// form: the chunks of the keys); the copies of 8 or 16 parts are in flight together.  Latency-bound; 6 rows of 32 heads and 18 or 34
+// parts took 10-17 us with one CTA per row or eight parts at a time and another kernel for the operand.
+constexpr int kMergeCtas = 4, kMergeWarps = 16;
 
-template <int OP, int V, int D>
-__global__ void __launch_bounds__(kMergeThreads) attention_merge_operand_kernel(AttnList l, AttnParts parts, int nvec, RowOperand out) {
-  __shared__ float s_buf[kMergeThreads / 32];
-  __shared__ long long s_total, s_unit0;
-  __shared__ int s_seg0;
-  extern __shared__ __align__(16) unsigned char s_row[];   // [Hq * D] bf16
+template <int OP, int D, bool LIST>
+__global__ void __launch_bounds__(kMergeWarps * 32)
+attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, RowOperand out) {
+  __shared__ float s_buf[kMergeWarps];
+  __shared__ float s_amax;
+  extern __shared__ __align__(16) unsigned char s_row[];   // this CTA's heads, bf16; then each warp's parts of a batch
   pdl_trigger();
   pdl_wait();
-  const int m = blockIdx.x, b = m / l.T_max, i = m % l.T_max;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const bool live = l.valid[b] != 0 && i < l.block_len[b];
+  const int rank = blockIdx.x % kMergeCtas, m = blockIdx.x / kMergeCtas, b = m / l.T_max, i = m % l.T_max;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+  const int Hq = l.Hkv * l.G, h0 = rank * Hq / kMergeCtas, h1 = (rank + 1) * Hq / kMergeCtas;
   constexpr int kPer = D / 32;
-  const int Hq = l.Hkv * l.G;
-  if (live) {
-    if (warp == 0) {   // units and segments of the sequences before this one
-      long long units = 0, before = 0;
-      int segs = 0;
-      for (int x = lane; x < l.B; x += 32) {
-        int t, r;
-        attn_shape(l, x, t, r);
-        units += (long long)t * r * l.Hkv;
-        if (x < b) { before += (long long)t * r * l.Hkv; segs += r * l.Hkv; }
-      }
+  __shared__ float4 s_part[kMergeWarps][32];   // per warp: the non-empty parts' (index, weight, sum)
+  bool live;
+  int n0 = 0, stride, tiles = 0, row_tiles = 0, unit0 = 0, seg0 = 0, row0;
+  unsigned total = 1, ctas = 1;
+  if (LIST) {
+    const AttnSeq q = l.seq[b];
+    total = (unsigned)l.seq[l.B].unit0;
+    tiles = q.tiles; row_tiles = q.row_tiles; unit0 = q.unit0; seg0 = q.seg0;
+    live = tiles > 0 && i < l.block_len[b];
+    ctas = attn_ctas(total);
+    const int t = i / l.npt;
+    unit0 += t * tiles;    // of head 0's row tile that holds this row
+    seg0 += t;
+    row0 = (i - t * l.npt) * l.G;
+    stride = 128;
+  } else {
+    const int T = l.block_len[b];
+    live = l.valid[b] != 0 && i < T;
+    n0 = (l.seq_len[b] + T + ch.chunk - 1) / ch.chunk;
+    stride = ch.Rpad;
+    row0 = i * l.G;
+  }
+  float* s_o = reinterpret_cast<float*>(s_row + (size_t)((Hq + kMergeCtas - 1) / kMergeCtas) * D * 2) + (size_t)warp * batch * D;
+  for (int hq = h0 + warp; hq < h1; hq += warps) {
+    uint32_t pk[kPer / 2];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        units += __shfl_xor_sync(0xffffffffu, units, o);
-        before += __shfl_xor_sync(0xffffffffu, before, o);
-        segs += __shfl_xor_sync(0xffffffffu, segs, o);
+    for (int e = 0; e < kPer / 2; ++e) pk[e] = 0u;
+    if (live) {
+      const int hk = hq / l.G, row = row0 + hq - hk * l.G;
+      size_t at0;
+      int n = n0;
+      if (LIST) {   // CTA c takes the units [c * total / ctas, (c + 1) * total / ctas): the ones that share u0 .. u1 - 1
+        const int u0 = unit0 + hk * row_tiles * tiles, u1 = u0 + tiles, s = seg0 + hk * row_tiles;
+        int c0, c1;
+        if (total < (1u << 24)) {
+          c0 = (int)(((unsigned)(u0 + 1) * ctas - 1u) / total);
+          c1 = (int)(((unsigned)u1 * ctas - 1u) / total);
+        } else {
+          c0 = (int)(((unsigned long long)(u0 + 1) * ctas - 1) / total);
+          c1 = (int)(((unsigned long long)u1 * ctas - 1) / total);
+        }
+        n = 2 * (c1 - c0 + 1);
+        at0 = (size_t)(c0 + s) * 256 + row;
+      } else {
+        at0 = ((size_t)b * l.Hkv + hk) * ch.nchunk * ch.Rpad + row;
       }
-      if (lane == 0) { s_total = units; s_unit0 = before; s_seg0 = segs; }
-    }
-    __syncthreads();
-    int tiles, row_tiles;
-    attn_shape(l, b, tiles, row_tiles);
-    for (int hq = warp; hq < Hq; hq += kMergeThreads / 32) {
-      const int s = (hq / l.G) * row_tiles + i / l.npt, row = (i % l.npt) * l.G + hq % l.G;
-      const long long u0 = s_unit0 + (long long)s * tiles;
-      const int c0 = (int)(((u0 + 1) * kAttnCtas - 1) / s_total), c1 = (int)(((u0 + tiles) * kAttnCtas - 1) / s_total);
-      const int n = 2 * (c1 - c0 + 1);
-      const size_t at0 = ((size_t)(c0 + s_seg0 + s) * 2) * 128 + row;   // part p: 128 entries further
-      float mx = -INFINITY;
-      for (int p = lane; p < n; p += 32) mx = fmaxf(mx, __ldcg(&parts.ml[at0 + (size_t)p * 128].x));
+      float2 ml = lane < n ? __ldcg(&parts.ml[at0 + (size_t)lane * stride]) : make_float2(-INFINITY, 0.f);
+      float mx = ml.x;
+      for (int p = lane + 32; p < n; p += 32) mx = fmaxf(mx, __ldcg(&parts.ml[at0 + (size_t)p * stride].x));
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       float acc[kPer], den = 0.f;
 #pragma unroll
       for (int e = 0; e < kPer; ++e) acc[e] = 0.f;
       for (int p0 = 0; p0 < n; p0 += 32) {
-        float2 ml = p0 + lane < n ? __ldcg(&parts.ml[at0 + (size_t)(p0 + lane) * 128]) : make_float2(-INFINITY, 0.f);
+        if (p0 > 0) ml = p0 + lane < n ? __ldcg(&parts.ml[at0 + (size_t)(p0 + lane) * stride]) : make_float2(-INFINITY, 0.f);
         const float w = ml.x == -INFINITY ? 0.f : exp2f(ml.x - mx);
-        float wl = w * ml.y;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) wl += __shfl_xor_sync(0xffffffffu, wl, o);
-        den += wl;
-        for (int q0 = 0; q0 < 32 && p0 + q0 < n; q0 += 8) {   // eight parts' loads at a time
-          float v[8][kPer], wq[8];
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            wq[q] = __shfl_sync(0xffffffffu, w, q0 + q);
-            const float* src = parts.o + (at0 + (size_t)(p0 + q0 + q) * 128) * D + lane * kPer;
-            if (wq[q] != 0.f) {   // (a part without a visible key may never have been written)
-              if constexpr (kPer == 4) {
-                const float4 t = __ldcg(reinterpret_cast<const float4*>(src));
-                v[q][0] = t.x; v[q][1] = t.y; v[q][2] = t.z; v[q][3] = t.w;
-              } else {
-                const float2 t = __ldcg(reinterpret_cast<const float2*>(src));
-                v[q][0] = t.x; v[q][1] = t.y;
-              }
-            } else {
-#pragma unroll
-              for (int e = 0; e < kPer; ++e) v[q][e] = 0.f;
-            }
+        // the non-empty parts in a row (one without a visible key may never have been written)
+        const unsigned some = __ballot_sync(0xffffffffu, w != 0.f);
+        const int cnt = __popc(some);
+        __syncwarp();
+        if (w != 0.f) s_part[warp][__popc(some & ((1u << lane) - 1u))] = make_float4(__int_as_float(p0 + lane), w, ml.y, 0.f);
+        __syncwarp();
+        for (int j0 = 0; j0 < cnt; j0 += batch) {
+          // the batch's copies in flight together (as loads into registers the compiler spreads them over their uses)
+          const int nb = min(batch, cnt - j0);
+          for (int q = 0; q < nb; ++q) {
+            const float* src = parts.o + (at0 + (size_t)__float_as_int(s_part[warp][j0 + q].x) * stride) * D + lane * kPer;
+            asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(tc::smem_u32(s_o + (q * 32 + lane) * kPer)), "l"(src),
+                         "n"(kPer * 4)
+                         : "memory");
           }
+          asm volatile("cp.async.wait_all;\n" ::: "memory");   // (each lane reads only what it copied)
+          for (int q = 0; q < nb; ++q) {
+            const float4 part = s_part[warp][j0 + q];
+            den += part.y * part.z;
 #pragma unroll
-          for (int q = 0; q < 8; ++q)
-#pragma unroll
-            for (int e = 0; e < kPer; ++e) acc[e] += wq[q] * v[q][e];
+            for (int e = 0; e < kPer; ++e) acc[e] += part.y * s_o[(q * 32 + lane) * kPer + e];
+          }
         }
       }
       const float inv = 1.0f / den;
-      uint32_t pk[kPer / 2];
 #pragma unroll
       for (int e = 0; e < kPer / 2; ++e) {
         const __nv_bfloat162 t = __floats2bfloat162_rn(acc[2 * e] * inv, acc[2 * e + 1] * inv);
         pk[e] = *reinterpret_cast<const uint32_t*>(&t);
       }
-      uint32_t* dst = reinterpret_cast<uint32_t*>(s_row) + hq * (D / 2) + lane * (kPer / 2);
-#pragma unroll
-      for (int e = 0; e < kPer / 2; ++e) dst[e] = pk[e];
     }
-  } else {
-    for (int v = threadIdx.x; v < nvec; v += kMergeThreads) reinterpret_cast<uint4*>(s_row)[v] = make_uint4(0, 0, 0, 0);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(s_row) + (hq - h0) * (D / 2) + lane * (kPer / 2);
+#pragma unroll
+    for (int e = 0; e < kPer / 2; ++e) dst[e] = pk[e];
   }
   __syncthreads();
-  write_operand<OP, V, kMergeThreads>(
-      [&](int v, int j, float (&f)[8]) {
-        const uint4 y = reinterpret_cast<const uint4*>(s_row)[v];
-        if (out.y != nullptr) reinterpret_cast<uint4*>(out.y + (size_t)m * nvec * 8)[v] = y;
-        unpack8(y, f);
-      },
-      nvec, m, out, s_buf);
+  const int nvec = (h1 - h0) * (D / 8), first = h0 * (D / 8);   // this CTA's 16-byte pieces of the row
+  const int64_t width = (int64_t)Hq * D;
+  float amax = 0.f, f[8], s[8];
+  for (int v = threadIdx.x; v < nvec; v += blockDim.x) {
+    const uint4 y = reinterpret_cast<const uint4*>(s_row)[v];
+    if (out.y != nullptr) reinterpret_cast<uint4*>(out.y + (size_t)m * width)[first + v] = y;
+    unpack8(y, f);
+    if (OP == kOperandCodes) {
+      load_smooth8(out.smooth, first + v, s);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) f[e] = __fmul_rn(f[e], s[e]);
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) amax = fmaxf(amax, fabsf(f[e]));
+  }
+  if (OP == kOperandBf16) return;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+  if (lane == 0) s_buf[warp] = amax;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < warps; ++w) amax = fmaxf(amax, s_buf[w]);
+    s_amax = amax;
+  }
+  __syncwarp();
+  tc::cluster_arrive();
+  tc::cluster_wait();
+  amax = 0.f;
+#pragma unroll
+  for (int c = 0; c < kMergeCtas; ++c) amax = fmaxf(amax, tc::ld_cluster_f32(tc::cluster_map(tc::smem_u32(&s_amax), (uint32_t)c)));
+  float up = 1.f, scale = 1.f;
+  if (OP == kOperandDigits) digit_scale(amax, up, scale);
+  else scale = amax == 0.f ? 1.0f : __fdiv_rn(amax, 127.0f);
+  if (rank == 0 && threadIdx.x == 0) out.scale[m] = scale;
+  for (int v = threadIdx.x; v < nvec; v += blockDim.x) {
+    unpack8(reinterpret_cast<const uint4*>(s_row)[v], f);
+    if (OP == kOperandDigits) {
+      write_digits8(f, up, out.q + 3 * (int64_t)m * width, width, (int64_t)(first + v) * 8);
+    } else {
+      load_smooth8(out.smooth, first + v, s);
+      *reinterpret_cast<uint2*>(out.q + (int64_t)m * width + (int64_t)(first + v) * 8) = smoothed_codes8(f, s, scale);
+    }
+  }
+  tc::cluster_arrive();   // (nobody's maximum goes away while another CTA may read it)
+  tc::cluster_wait();
 }
 
 // One warp checks a sequence's tokens / parents / capacity and derives ancestor bit masks and depths.  A chain's are known
@@ -438,19 +507,54 @@ __device__ void prepare_sequence(const BlockArgs& a, int b, int* s_parent, unsig
   }
 }
 
-// The pass's first kernel: CTA m < M gathers the embedding of row m into the residual stream and normalises it; CTA M + b
-// does the bookkeeping of sequence b.
+// Every sequence's place in the attention's list (AttnSeq): a warp, 32 sequences at a time, a running total behind the last.
+__device__ void lay_out_list(const BlockArgs& a) {
+  const int lane = threadIdx.x & 31;
+  int units = 0, segs = 0;
+  for (int b0 = 0; b0 < a.B; b0 += 32) {
+    const int b = b0 + lane;
+    AttnSeq q = {0, 0, 0, 0};
+    if (b < a.B && a.bi.valid[b] != 0) {
+      const int T = a.block_len[b];
+      q.tiles = (a.seq_len[b] + T + 127) / 128;
+      q.row_tiles = (T + a.npt - 1) / a.npt;
+    }
+    int u = q.tiles * q.row_tiles * a.Hkv, s = q.row_tiles * a.Hkv;
+    const int own_u = u, own_s = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int pu = __shfl_up_sync(0xffffffffu, u, o), ps = __shfl_up_sync(0xffffffffu, s, o);
+      if (lane >= o) { u += pu; s += ps; }
+    }
+    q.unit0 = units + u - own_u;
+    q.seg0 = segs + s - own_s;
+    if (b < a.B) a.seq[b] = q;
+    units += __shfl_sync(0xffffffffu, u, 31);
+    segs += __shfl_sync(0xffffffffu, s, 31);
+  }
+  if (lane == 0) a.seq[a.B] = AttnSeq{0, 0, units, segs};
+}
+
+// The pass's first kernel: CTA m < M gathers the embedding of row m into the residual stream and normalises it; CTA M does
+// the bookkeeping, a warp per sequence in turn.
 template <int OP, int V>
 __global__ void __launch_bounds__(kRowThreads)
 embed_norm_kernel(BlockArgs a, int M, const __nv_bfloat16* __restrict__ embed, __nv_bfloat16* x, const __nv_bfloat16* __restrict__ g,
                   int nvec, float eps, int adders, RowOperand out) {
   __shared__ float s_buf[64];
-  __shared__ int s_parent[QUASAR_MAX_BLOCK], s_depth[QUASAR_MAX_BLOCK];
-  __shared__ unsigned long long s_anc[QUASAR_MAX_BLOCK];
   pdl_trigger();
   const int m = blockIdx.x;
   if (m >= M) {
-    if (threadIdx.x < 32) prepare_sequence(a, m - M, s_parent, s_anc, s_depth);
+    __shared__ int s_parent[kRowThreads / 32][QUASAR_MAX_BLOCK], s_depth[kRowThreads / 32][QUASAR_MAX_BLOCK];
+    __shared__ unsigned long long s_anc[kRowThreads / 32][QUASAR_MAX_BLOCK];
+    const int warp = threadIdx.x >> 5;
+    for (int k = threadIdx.x; k < a.n_clear; k += kRowThreads) a.clear[k] = 0u;
+    for (int b = warp; b < a.B; b += kRowThreads / 32) {
+      prepare_sequence(a, b, s_parent[warp], s_anc[warp], s_depth[warp]);
+      __syncwarp();
+    }
+    __syncthreads();
+    if (warp == 0) lay_out_list(a);
     return;
   }
   uint4 gain[V > 0 ? V : 1];
@@ -526,7 +630,7 @@ int turns_of(int nvec) {
 
 template <typename... P, typename... A>
 int launch_row(void (*kernel)(P...), int grid, size_t smem, bool pdl, cudaStream_t stream, A&&... args) {
-  return launch_dependent(kernel, dim3((unsigned)grid), dim3(kRowThreads), smem, pdl, stream, static_cast<A&&>(args)...);
+  return launch_dependent(kernel, dim3((unsigned)grid), dim3(kRowThreads), smem, pdl, stream, 1, static_cast<A&&>(args)...);
 }
 
 // shared memory of a norm: the pairs' sums of a row that stays in registers (at most 48 KB)
@@ -552,7 +656,7 @@ size_t norm_smem(int nvec) { return turns_of(nvec) > 0 ? (size_t)nvec * 16 : 0; 
 int launch_embed_norm(int op, const BlockArgs& a, const __nv_bfloat16* embed, __nv_bfloat16* x, const __nv_bfloat16* g, int H, float eps,
                       int adders, const RowOperand& out, cudaStream_t stream) {
   const int nvec = H / 8, M = a.B * a.T_max;
-  ROW_DISPATCH(embed_norm_kernel, M + a.B, norm_smem(nvec), false, stream, a, M, embed, x, g, nvec, eps, adders, out)
+  ROW_DISPATCH(embed_norm_kernel, M + 1, norm_smem(nvec), false, stream, a, M, embed, x, g, nvec, eps, adders, out)
 }
 
 int launch_norm(int op, const __nv_bfloat16* x, const __nv_bfloat16* g, int M, int H, float eps, int adders, const RowOperand& out, cudaStream_t stream) {
@@ -565,33 +669,52 @@ int launch_swiglu(int op, const __nv_bfloat16* gu, int M, int F, const RowOperan
   ROW_DISPATCH(swiglu_kernel, M, 0, true, stream, gu, nvec, out)
 }
 
-int launch_operand(int op, const __nv_bfloat16* x, int M, int K, const RowOperand& out, cudaStream_t stream) {
+int launch_operand(int op, const __nv_bfloat16* x, const unsigned* row_max, int M, int K, const RowOperand& out, cudaStream_t stream) {
   if (op == kOperandBf16) return QUASAR_OK;   // the row itself is the operand
   const int nvec = K / 8;
-  ROW_DISPATCH(operand_kernel, M, 0, true, stream, x, nvec, out)
+  const dim3 grid((unsigned)((nvec + kElemThreads - 1) / kElemThreads), (unsigned)M);
+  if (op == kOperandDigits) return launch_dependent(operand_kernel<kOperandDigits>, grid, dim3(kElemThreads), 0, true, stream, 1, x, row_max, nvec, out);
+  return launch_dependent(operand_kernel<kOperandCodes>, grid, dim3(kElemThreads), 0, true, stream, 1, x, row_max, nvec, out);
 }
 
-int launch_attention_merge(int op, const AttnList& list, const AttnParts& parts, int M, int D, const RowOperand& out, cudaStream_t stream) {
-  const int K = list.Hkv * list.G * D, nvec = K / 8;
-  const size_t smem = (size_t)K * 2;
-  if (smem > 48 * 1024) { set_error("attention merge: rows of %d elements (at most 24576)", K); return QUASAR_ERR_SHAPE; }
-#define MERGE(OP, V, DD)                                                                                                    \
-  return launch_dependent(attention_merge_operand_kernel<OP, V, DD>, dim3((unsigned)M), dim3(kMergeThreads), smem, true, stream, \
-                          list, parts, nvec, out)
-  const bool digits = op == kOperandDigits, wide = nvec > kMergeThreads;   // more than a turn of 8 elements a thread
-  if (D == 128) {
-    if (wide) { if (digits) MERGE(kOperandDigits, 3, 128); MERGE(kOperandBf16, 3, 128); }
-    if (digits) MERGE(kOperandDigits, 1, 128);
-    MERGE(kOperandBf16, 1, 128);
-  }
-  if (wide) { if (digits) MERGE(kOperandDigits, 3, 64); MERGE(kOperandBf16, 3, 64); }
-  if (digits) MERGE(kOperandDigits, 1, 64);
-  MERGE(kOperandBf16, 1, 64);
+namespace {
+constexpr size_t kMergeMaxSmem = 216 * 1024;
+template <int OP, int D, bool LIST>
+int launch_merge(int warps, size_t smem, const AttnList& list, const AttnParts& parts, const AttnChunks& ch, int batch, int M,
+                 const RowOperand& out, cudaStream_t stream) {
+  static const cudaError_t set_up =
+      cudaFuncSetAttribute(attention_merge_kernel<OP, D, LIST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMergeMaxSmem);
+  QUASAR_CUDA_CHECK(set_up);
+  return launch_dependent(attention_merge_kernel<OP, D, LIST>, dim3((unsigned)(M * kMergeCtas)), dim3((unsigned)warps * 32), smem, true, stream,
+                          kMergeCtas, list, parts, ch, batch, out);
+}
+}  // namespace
+
+int launch_attention_merge(int op, const AttnList& list, const AttnParts& parts, const AttnChunks* chunks, int M, int D,
+                           const RowOperand& out, cudaStream_t stream) {
+  const int heads = (list.Hkv * list.G + kMergeCtas - 1) / kMergeCtas;   // of a CTA
+  const int warps = heads < kMergeWarps ? heads : kMergeWarps;
+  const int batch = M <= 16 ? 16 : 8;   // few rows: round trips count; many: CTAs on an SM do
+  const size_t smem = (size_t)heads * D * 2 + (size_t)warps * batch * D * 4;
+  if (smem > kMergeMaxSmem) { set_error("attention merge: %d query heads of %d", list.Hkv * list.G, D); return QUASAR_ERR_SHAPE; }
+  const AttnChunks ch = chunks ? *chunks : AttnChunks{};
+#define MERGE_AS(OP, DD, LIST) return launch_merge<OP, DD, LIST>(warps, smem, list, parts, ch, batch, M, out, stream)
+#define MERGE(OP)                                     \
+  if (D == 128) {                                     \
+    if (chunks) MERGE_AS(OP, 128, false);             \
+    MERGE_AS(OP, 128, true);                          \
+  }                                                   \
+  if (chunks) MERGE_AS(OP, 64, false);                \
+  MERGE_AS(OP, 64, true);
+  if (op == kOperandDigits) { MERGE(kOperandDigits) }
+  if (op == kOperandCodes) { MERGE(kOperandCodes) }
+  MERGE(kOperandBf16)
+#undef MERGE_AS
 #undef MERGE
 }
 
 int launch_accept(const BlockArgs& a, int32_t* accept_len, int32_t* bonus, int32_t* accept_path, cudaStream_t stream) {
-  return launch_dependent(accept_kernel, dim3((unsigned)a.B), dim3(32), 0, true, stream, a, accept_len, bonus, accept_path);
+  return launch_dependent(accept_kernel, dim3((unsigned)a.B), dim3(32), 0, true, stream, 1, a, accept_len, bonus, accept_path);
 }
 
 }  // namespace quasar

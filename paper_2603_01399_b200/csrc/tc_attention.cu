@@ -92,25 +92,25 @@ __device__ __forceinline__ uint64_t desc_v(const void* smem_tile) {
 // A CTA's run through the list: piece by piece (a piece = its tiles of one segment).
 struct Walk {
   AttnCursor cur;
-  long long u, end;
+  const AttnSeq* known;
+  int u, end;
   int b, hk, rt, t0, nt, seg;   // the piece: sequence, kv head, row tile, first key tile, key tiles, ordinal of the segment
-  const int2* shapes;
-  __device__ Walk(const AttnList& l, const int2* sh, long long total, int cta, int ncta) : shapes(sh) {
-    u = (long long)cta * total / ncta;
-    end = (long long)(cta + 1) * total / ncta;
-    cur.start(l, shapes);
+  __device__ Walk(const AttnList& l, const AttnSeq* k, int total, int cta) : known(k) {
+    const int ctas = (int)attn_ctas((unsigned)total);
+    u = cta < ctas ? (int)((long long)cta * total / ctas) : 0;
+    end = cta < ctas ? (int)((long long)(cta + 1) * total / ctas) : 0;
+    cur.start(l, known);
   }
   __device__ bool next(const AttnList& l) {
     if (u >= end) return false;
-    cur.seek(l, shapes, u);
+    cur.seek(l, known, u);
     b = cur.b;
-    const long long in = u - cur.unit0;
-    const int s = (int)(in / cur.tiles);
-    t0 = (int)(in - (long long)s * cur.tiles);
-    nt = (int)min((long long)(cur.tiles - t0), end - u);
-    hk = s / cur.row_tiles;
-    rt = s - hk * cur.row_tiles;
-    seg = cur.seg0 + s;
+    const int in = u - cur.q.unit0, s = in / cur.q.tiles;
+    t0 = in - s * cur.q.tiles;
+    nt = min(cur.q.tiles - t0, end - u);
+    hk = s / cur.q.row_tiles;
+    rt = s - hk * cur.q.row_tiles;
+    seg = cur.q.seg0 + s;
     u += nt;
     return true;
   }
@@ -163,21 +163,14 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   const uint32_t tmem = *tmem_slot;   // columns: S (then P) of group 0, of group 1, O of group 0, of group 1
   if (threadIdx.x == 0) pdl_trigger();
   pdl_wait();
-  // the sequences' shapes, fetched once and side by side (each role walks them on its own)
-  __shared__ int2 s_shape[kShapes];
-  __shared__ long long s_total;
-  for (int b = (int)threadIdx.x; b < min(a.list.B, kShapes); b += kThreadsA) {
-    int t, r;
-    attn_shape(a.list, b, t, r);
-    s_shape[b] = make_int2(t, r);
-  }
-  if (warp == 2) {
-    const long long total = attn_total(a.list);
-    if (lane == 0) s_total = total;
-  }
+  // the sequences' places, fetched once and side by side (each role walks them on its own)
+  __shared__ AttnSeq s_seq[kShapes];
+  __shared__ int s_total;
+  for (int b = (int)threadIdx.x; b < min(a.list.B, kShapes); b += kThreadsA) s_seq[b] = a.list.seq[b];
+  if (threadIdx.x == kThreadsA - 1) s_total = a.list.seq[a.list.B].unit0;
   __syncthreads();
 
-  Walk w(a.list, s_shape, s_total, (int)blockIdx.x, (int)gridDim.x);
+  Walk w(a.list, s_seq, s_total, (int)blockIdx.x);
   if (warp == 0) {
     // ---- TMA producer ----
     const uint64_t policy = l2_evict_first_policy();
@@ -436,7 +429,7 @@ int launch_d(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv
     QUASAR_CUDA_CHECK(cudaFuncSetAttribute(tc_attention_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     configured = true;
   }
-  return launch_dependent(tc_attention_kernel<D>, dim3((unsigned)ctas), dim3(kThreadsA), smem, true, stream, mq, mk, mv, a);
+  return launch_dependent(tc_attention_kernel<D>, dim3((unsigned)ctas), dim3(kThreadsA), smem, true, stream, 1, mq, mk, mv, a);
 }
 
 }  // namespace

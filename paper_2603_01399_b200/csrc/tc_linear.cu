@@ -29,6 +29,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "rope.cuh"
 #include "tc_common.cuh"
 #include "tc_linear.cuh"
 
@@ -95,6 +96,11 @@ constexpr int kTmemCols = 256;           // two CTAs share an SM's 512 columns: 
 constexpr size_t kMaxSmem = 227 * 1024;
 constexpr size_t kSmemSlack = 1024 + 256;       // alignment of the ring, barriers
 
+// What tc_linear_kernel does with a tile's finished sums: stores them; makes them q, k and v - QK-norm, RoPE, cache append
+// (a tile of 128 channels is one head of 128 or two of 64); or multiplies silu(gate) by up (a tile is `chan / 2` gate channels
+// and the matching up channels).
+enum TcEpilogue { kStore = 0, kRope = 1, kSwiglu = 2 };
+
 struct TcArgs {
   const float* dx;             // [M] step sizes of the int8 activations
   const float* dw;             // [N] step sizes of the int8 weights
@@ -108,6 +114,10 @@ struct TcArgs {
   int rows, brows;             // activation rows of a row tile; rows of operand B (three per activation row for digits), padded to 16
   int row_tiles, nsplit, stages;
   int y_is_f32;
+  RopeArgs rope;               // kRope
+  __nv_bfloat16* act;          // kSwiglu: [M][N / 2]
+  unsigned* act_max;           // [M] bits of the largest magnitude of a row of act (times smooth), or nullptr
+  const float* smooth;         // [N / 2] or nullptr
   int early_weights;           // the weights may be asked for before the kernel in front has finished
 };
 
@@ -173,6 +183,81 @@ __device__ __forceinline__ void store4(const TcArgs& a, const uint32_t (&v)[4], 
   }
 }
 
+// one row of a 128-channel tile, four channels a lane: q and k heads normalised, rotated and put in their places, v heads copied
+template <int KIND, int D>
+__device__ __forceinline__ void store_rope(const TcArgs& a, const uint32_t (&v)[4], int m, int n0, float dx) {
+  const RopeArgs& r = a.rope;
+  const int lane = threadIdx.x & 31, n = n0 + lane * 4;
+  float f[4];   // as the linear layer's bf16 output
+#pragma unroll
+  for (int e = 0; e < 4; ++e)
+    f[e] = __bfloat162float(__float2bfloat16_rn(finish<KIND>(v[e], dx, (KIND != kBf16 && n + e < a.N) ? __ldg(a.dw + n + e) : 1.f)));
+  const int b = m / r.T_max, i = m % r.T_max;
+  if (!r.bi.valid[b] || i >= r.block_len[b]) return;
+  const int P = r.seq_len[b], pos = P + r.bi.depth[m];
+#pragma unroll
+  for (int h = 0; h < 128 / D; ++h) {
+    const int head = n0 / D + h;
+    // lane l takes the channels l + 32 k of the head, which lane (l + 32 k) / 4 holds
+    float x[D / 32];
+#pragma unroll
+    for (int k = 0; k < D / 32; ++k) {
+      const int from = (h * D + 32 * k + lane) >> 2;
+      x[k] = 0.f;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float t = __shfl_sync(0xffffffffu, f[e], from);
+        if ((lane & 3) == e) x[k] = t;
+      }
+    }
+    if (head >= r.Hq + 2 * r.Hkv) continue;
+    if (head >= r.Hq + r.Hkv) {
+      __nv_bfloat16* dst = r.v_cache + (((size_t)b * r.Hkv + (head - r.Hq - r.Hkv)) * r.s_max + (P + i)) * D;
+#pragma unroll
+      for (int k = 0; k < D / 32; ++k) dst[lane + 32 * k] = __float2bfloat16_rn(x[k]);
+      continue;
+    }
+    const bool is_q = head < r.Hq;
+    float lo[D / 64], hi[D / 64];
+#pragma unroll
+    for (int p = 0; p < D / 64; ++p) { lo[p] = x[p]; hi[p] = x[p + D / 64]; }
+    __nv_bfloat16* dst = is_q ? r.qkv + (size_t)m * a.N + (size_t)head * D
+                              : r.k_cache + (((size_t)b * r.Hkv + (head - r.Hq)) * r.s_max + (P + i)) * D;
+    rope_head<D>(lo, hi, is_q ? r.q_norm : r.k_norm, r.table, pos, r.eps, dst);
+  }
+}
+
+// one row, four units from u on: silu(gate) * up, both rounded to bf16 first (they are tensors of the layer)
+template <int KIND>
+__device__ __forceinline__ float store_swiglu(const TcArgs& a, const uint32_t (&g)[4], const uint32_t (&up)[4], int m, int u, float dx) {
+  const int F = a.N / 2;   // a multiple of 16: four units from a multiple of four on are inside or outside together
+  float4 dg = make_float4(1.f, 1.f, 1.f, 1.f), du = dg;
+  if (KIND != kBf16) {
+    dg = __ldg(reinterpret_cast<const float4*>(a.dw + u));
+    du = __ldg(reinterpret_cast<const float4*>(a.dw + F + u));
+  }
+  const float dgv[4] = {dg.x, dg.y, dg.z, dg.w}, duv[4] = {du.x, du.y, du.z, du.w};
+  float f[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const float gt = __bfloat162float(__float2bfloat16_rn(finish<KIND>(g[e], dx, dgv[e])));
+    const float uv = __bfloat162float(__float2bfloat16_rn(finish<KIND>(up[e], dx, duv[e])));
+    f[e] = gt / (1.0f + expf(-gt)) * uv;
+  }
+  const __nv_bfloat162 lo = __floats2bfloat162_rn(f[0], f[1]), hi = __floats2bfloat162_rn(f[2], f[3]);
+  const uint32_t w0 = *reinterpret_cast<const uint32_t*>(&lo), w1 = *reinterpret_cast<const uint32_t*>(&hi);
+  *reinterpret_cast<uint2*>(a.act + (size_t)m * F + u) = make_uint2(w0, w1);
+  float s[4] = {1.f, 1.f, 1.f, 1.f};
+  if (a.smooth != nullptr) {
+    const float4 t = __ldg(reinterpret_cast<const float4*>(a.smooth + u));
+    s[0] = t.x; s[1] = t.y; s[2] = t.z; s[3] = t.w;
+  }
+  float amax = fmaxf(0.f, fabsf(__fmul_rn(__uint_as_float(w0 << 16), s[0])));
+  amax = fmaxf(amax, fabsf(__fmul_rn(__uint_as_float(w0 & 0xffff0000u), s[1])));
+  amax = fmaxf(amax, fabsf(__fmul_rn(__uint_as_float(w1 << 16), s[2])));
+  return fmaxf(amax, fabsf(__fmul_rn(__uint_as_float(w1 & 0xffff0000u), s[3])));
+}
+
 // The MMAs of one stage: four steps of 32 bytes along the rows of both operands
 template <int KIND, bool PAIR>
 __device__ __forceinline__ void issue_stage(uint32_t d, uint64_t da, uint64_t db, uint32_t id, bool accumulate) {
@@ -192,7 +277,7 @@ __device__ __forceinline__ void issue_stage(uint32_t d, uint64_t da, uint64_t db
 
 // PAIR: CTAs 2 i and 2 i + 1 of a cluster work as one on two neighbouring channel tiles.  Each brings its own weights and HALF
 // of the activation rows; the leader's MMAs (256 rows) read both CTAs' shared memory.
-template <int KIND, bool PAIR>
+template <int KIND, bool PAIR, int EPI>
 __global__ void __launch_bounds__(kThreadsTc, 2)
 tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const TcArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -259,8 +344,13 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
       };
       auto load_w = [&](int i, int kb) {
         unsigned char* at = smem + (size_t)i * stage_bytes;
-        if (PAIR) tma_load_2d_pair<true>(at, &map_w, kb * 128, n0, cluster_map(smem_u32(full + i), leader), policy);
-        else tma_load_2d_hint(at, &map_w, kb * 128, n0, full + i, policy);
+#pragma unroll
+        for (int h = 0; h < (EPI == kSwiglu ? 2 : 1); ++h) {   // gate rows, then the matching up rows
+          const int y = EPI == kSwiglu ? h * (a.N / 2) + n0 / 2 : n0;
+          unsigned char* dst = EPI == kSwiglu ? at + h * (a.chan / 2) * 128 : at;
+          if (PAIR) tma_load_2d_pair<true>(dst, &map_w, kb * 128, y, cluster_map(smem_u32(full + i), leader), policy);
+          else tma_load_2d_hint(dst, &map_w, kb * 128, y, full + i, policy);
+        }
       };
       auto load_x = [&](int i, int kb) {
         unsigned char* at = smem + (size_t)i * stage_bytes + kAStage;
@@ -377,43 +467,74 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     const int rows = min(a.rows, a.M - m0);
     const int per = (rows + a.nsplit - 1) / a.nsplit;
     const int r_begin = split * per, r_end = min(rows, r_begin + per);
-    const int n = n0 + lane * 4;
-    const bool live = lane * 4 < a.chan && n < a.N;
     const uint32_t red_addr = smem_u32(smem);
-    for (int m = r_begin + warp; m < r_end; m += kThreadsTc / 32) {
-      unsigned long long best = 0;
-      if (live) {
-      const uint32_t off = (uint32_t)(m * kTileN + lane * 4) * 4;
-      uint32_t sum[4];
+    // the sums of row m (of the tile) over the ranges, four channels from c on
+    auto sums = [&](int m, int c, uint32_t (&sum)[4]) {
+      const uint32_t off = (uint32_t)(m * kTileN + c) * 4;
       if (a.nsplit == 1) {
         const uint4 p = *reinterpret_cast<const uint4*>(smem + off);
         sum[0] = p.x; sum[1] = p.y; sum[2] = p.z; sum[3] = p.w;
-      } else {
-        uint4 p[8];
+        return;
+      }
+      uint4 p[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
-          if (k < a.nsplit) p[k] = ld_cluster_v4(cluster_map(red_addr + off, (uint32_t)(PAIR ? 2 * k + pair_x : k)));
+      for (int k = 0; k < 8; ++k)
+        if (k < a.nsplit) p[k] = ld_cluster_v4(cluster_map(red_addr + off, (uint32_t)(PAIR ? 2 * k + pair_x : k)));
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          if (k >= a.nsplit) break;
-          const uint32_t w[4] = {p[k].x, p[k].y, p[k].z, p[k].w};
+      for (int k = 0; k < 8; ++k) {
+        if (k >= a.nsplit) break;
+        const uint32_t w[4] = {p[k].x, p[k].y, p[k].z, p[k].w};
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            if (k == 0) sum[e] = w[e];
-            else if (KIND == kCodes) sum[e] += w[e];
-            else sum[e] = __float_as_uint(__uint_as_float(sum[e]) + __uint_as_float(w[e]));
+        for (int e = 0; e < 4; ++e) {
+          if (k == 0) sum[e] = w[e];
+          else if (KIND == kCodes) sum[e] += w[e];
+          else sum[e] = __float_as_uint(__uint_as_float(sum[e]) + __uint_as_float(w[e]));
+        }
+      }
+    };
+    uint32_t sum[4];
+    if (EPI == kSwiglu) {   // 16 lanes a row
+      const int half = a.chan / 2, c = (lane & 15) * 4, u = n0 / 2 + c;
+      const bool live = c < half && u < a.N / 2;
+      for (int mb = r_begin + warp * 2; mb < r_end; mb += kThreadsTc / 32 * 2) {
+        const int m = mb + (lane >> 4);
+        float amax = 0.f;
+        if (live && m < r_end) {
+          uint32_t up[4];
+          sums(m, c, sum);
+          sums(m, half + c, up);
+          amax = store_swiglu<KIND>(a, sum, up, m0 + m, u, KIND != kBf16 ? a.dx[m0 + m] : 1.f);
+        }
+        if (a.act_max != nullptr) {
+#pragma unroll
+          for (int o = 8; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+          if ((lane & 15) == 0 && m < r_end && amax > 0.f) atomicMax(a.act_max + m0 + m, __float_as_uint(amax));
+        }
+      }
+    } else {
+      const int n = n0 + lane * 4;
+      const bool live = lane * 4 < a.chan && n < a.N;
+      for (int m = r_begin + warp; m < r_end; m += kThreadsTc / 32) {
+        const float dx = KIND != kBf16 ? a.dx[m0 + m] : 1.f;
+        if (EPI == kRope) {   // (all 128 channels; ones beyond the matrix are zero)
+          sums(m, lane * 4, sum);
+          if (a.rope.D == 128) store_rope<KIND, 128>(a, sum, m0 + m, n0, dx);
+          else store_rope<KIND, 64>(a, sum, m0 + m, n0, dx);
+          continue;
+        }
+        unsigned long long best = 0;
+        if (live) {
+          sums(m, lane * 4, sum);
+          store4<KIND>(a, sum, m0 + m, n, dx, best);
+        }
+        if (a.keys != nullptr) {
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
+            best = other > best ? other : best;
           }
+          if (lane == 0 && best != 0) atomicMax(a.keys + m0 + m, best);
         }
-      }
-      store4<KIND>(a, sum, m0 + m, n, KIND != kBf16 ? a.dx[m0 + m] : 1.f, best);
-      }
-      if (a.keys != nullptr) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
-          best = other > best ? other : best;
-        }
-        if (lane == 0 && best != 0) atomicMax(a.keys + m0 + m, best);
       }
     }
   }
@@ -722,7 +843,7 @@ TcPlan plan_base(int64_t M, int64_t K, int kind, bool pair) {
 }
 
 // one tile or k-range of a tile per CTA, all of them at once
-TcPlan plan_tiles(int64_t M, int64_t N, int64_t K, int kind, bool pair, const void* kernel) {
+TcPlan plan_tiles(int64_t M, int64_t N, int64_t K, int kind, bool pair, int epi, const void* kernel) {
   TcPlan p = plan_base(M, K, kind, pair);
   p.stream = 0;
   const int b_bytes = p.brows * (pair ? 64 : 128), stage = kAStage + b_bytes;
@@ -738,7 +859,7 @@ TcPlan plan_tiles(int64_t M, int64_t N, int64_t K, int kind, bool pair, const vo
     // (two CTAs of a cluster can share an SM)
     const int cs = s * group;
     const long long fit = per_sm == 1 ? max_clusters(kernel, cs) : std::max(2 * max_clusters(kernel, cs), max_clusters(kernel, (cs + 1) / 2));
-    for (int c = 128; c >= 64; c -= 8) {
+    for (int c = 128; c >= (epi == kRope ? 128 : 64); c -= epi == kSwiglu ? 16 : 8) {   // (whole heads; whole swizzle patterns of each half)
       const long long tiles = ((N + c - 1) / c + group - 1) / group * group;
       const long long clusters = tiles / group * p.row_tiles;
       const long long waves = (clusters + fit - 1) / fit;
@@ -782,7 +903,7 @@ TcPlan plan_stream(int64_t M, int64_t N, int64_t K, int kind, bool pair) {
   return p;
 }
 
-template <int KIND, bool PAIR>
+template <int KIND, bool PAIR, int EPI>
 int launch_kind(const CUtensorMap& map_w, const CUtensorMap& map_x, const TcArgs& a, const TcPlan& p, bool pdl, cudaStream_t stream) {
   const size_t smem = (size_t)p.stages * (kAStage + p.brows * (PAIR ? 64 : 128)) + kSmemSlack + (p.stream ? 2048 : 0);
   cudaLaunchConfig_t cfg = {};
@@ -809,56 +930,94 @@ int launch_kind(const CUtensorMap& map_w, const CUtensorMap& map_x, const TcArgs
   if (p.stream)
     QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_stream_kernel<KIND, PAIR>, map_w, map_x, a, p.tiles / (PAIR ? 2 : 1) * p.row_tiles));
   else
-    QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_linear_kernel<KIND, PAIR>, map_w, map_x, a));
+    QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_linear_kernel<KIND, PAIR, EPI>, map_w, map_x, a));
   count_launch();
   return QUASAR_OK;
 }
 
+struct Kernels { const void* tiles[2][3]; const void* stream[2]; };   // [pair][epilogue]
+template <int KIND>
+constexpr Kernels kernels_of() {
+  return {{{(const void*)tc_linear_kernel<KIND, false, kStore>, (const void*)tc_linear_kernel<KIND, false, kRope>,
+            (const void*)tc_linear_kernel<KIND, false, kSwiglu>},
+           {(const void*)tc_linear_kernel<KIND, true, kStore>, (const void*)tc_linear_kernel<KIND, true, kRope>,
+            (const void*)tc_linear_kernel<KIND, true, kSwiglu>}},
+          {(const void*)tc_stream_kernel<KIND, false>, (const void*)tc_stream_kernel<KIND, true>}};
+}
+
+// The plan of a layer: the quickest by estimate; a fused epilogue has the tiled form only.
+int plan_layer(int64_t M, int64_t N, int64_t K, int kind, int epi, TcPlan* out) {
+  static const Kernels kernels[3] = {kernels_of<kDigits>(), kernels_of<kBf16>(), kernels_of<kCodes>()};
+  static std::once_flag once;
+  static cudaError_t set_up = cudaSuccess;
+  std::call_once(once, [] {
+    auto allow = [](const void* k) {
+      if (set_up == cudaSuccess) set_up = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+      if (set_up == cudaSuccess) set_up = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    };
+    for (auto& k : kernels)
+      for (int p = 0; p < 2; ++p) {
+        for (const void* t : k.tiles[p]) allow(t);
+        allow(k.stream[p]);
+      }
+  });
+  QUASAR_CUDA_CHECK(set_up);
+  // A pair of CTAs halves what the activations add to an SM's intake; narrow blocks have too few of them for that to matter.
+  TcPlan p = plan_tiles(M, N, K, kind, false, epi, kernels[kind].tiles[0][epi]);
+  auto consider = [&](const TcPlan& q) { if (q.cost < p.cost) p = q; };
+  if (epi == kStore) consider(plan_stream(M, N, K, kind, false));
+  if (p.brows >= 64) {
+    consider(plan_tiles(M, N, K, kind, true, epi, kernels[kind].tiles[1][epi]));
+    if (epi == kStore) consider(plan_stream(M, N, K, kind, true));
+  }
+  *out = p;
+  return QUASAR_OK;
+}
+
+struct Operand {   // activations in the form the kind takes, and the weights
+  const void* x;
+  const float* dx;
+  const void* w;
+  const float* dw;
+  int64_t M, N, K;
+};
+
+int launch_layer(int kind, int epi, const Operand& o, TcArgs a, bool pdl, cudaStream_t stream) {
+  TcPlan p;
+  int rc = plan_layer(o.M, o.N, o.K, kind, epi, &p);
+  if (rc != QUASAR_OK) return rc;
+  CUtensorMap map_w, map_x;
+  rc = make_map_sw128(&map_w, o.w, (uint64_t)o.N, (uint64_t)o.K * (kind == kBf16 ? 2 : 1), (uint32_t)(epi == kSwiglu ? p.chan / 2 : p.chan));
+  if (rc != QUASAR_OK) return rc;
+  rc = make_map_sw128(&map_x, o.x, (uint64_t)o.M * (kind == kDigits ? 3 : 1), (uint64_t)o.K * (kind == kBf16 ? 2 : 1),
+                      (uint32_t)(p.pair ? p.brows / 2 : p.brows));
+  if (rc != QUASAR_OK) return rc;
+  a.dx = o.dx; a.dw = o.dw;
+  a.M = (int)o.M; a.N = (int)o.N; a.kblocks = p.kblocks; a.chan = p.chan; a.rows = p.rows; a.brows = p.brows;
+  a.row_tiles = p.row_tiles; a.nsplit = p.nsplit; a.stages = p.stages;
+  a.early_weights = pdl ? 1 : 0;
+#define LAUNCH_LAYER(KIND, EPI) return p.pair ? launch_kind<KIND, true, EPI>(map_w, map_x, a, p, pdl, stream) : launch_kind<KIND, false, EPI>(map_w, map_x, a, p, pdl, stream)
+#define LAUNCH_KIND(EPI)                          \
+  switch (kind) {                                 \
+    case kDigits: LAUNCH_LAYER(kDigits, EPI);     \
+    case kBf16: LAUNCH_LAYER(kBf16, EPI);         \
+    default: LAUNCH_LAYER(kCodes, EPI);           \
+  }
+  if (epi == kRope) LAUNCH_KIND(kRope)
+  if (epi == kSwiglu) LAUNCH_KIND(kSwiglu)
+  LAUNCH_KIND(kStore)
+#undef LAUNCH_KIND
+#undef LAUNCH_LAYER
+}
+
 int launch_any(int kind, const void* x, const float* dx, const void* w, const float* dw, int64_t M, int64_t N, int64_t K, void* y,
                bool y_is_f32, const __nv_bfloat16* residual, int32_t* acc_out, unsigned long long* keys, int32_t* error, bool pdl, cudaStream_t stream) {
-  static const void* const kernels[3][4] = {
-      {(const void*)tc_linear_kernel<kDigits, false>, (const void*)tc_linear_kernel<kDigits, true>,
-       (const void*)tc_stream_kernel<kDigits, false>, (const void*)tc_stream_kernel<kDigits, true>},
-      {(const void*)tc_linear_kernel<kBf16, false>, (const void*)tc_linear_kernel<kBf16, true>,
-       (const void*)tc_stream_kernel<kBf16, false>, (const void*)tc_stream_kernel<kBf16, true>},
-      {(const void*)tc_linear_kernel<kCodes, false>, (const void*)tc_linear_kernel<kCodes, true>,
-       (const void*)tc_stream_kernel<kCodes, false>, (const void*)tc_stream_kernel<kCodes, true>}};
-  static bool configured = false;
-  if (!configured) {
-    for (auto& row : kernels)
-      for (const void* k : row) {
-        QUASAR_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
-        QUASAR_CUDA_CHECK(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-      }
-    configured = true;
-  }
-  // A pair of CTAs halves what the activations add to an SM's intake; narrow blocks have too few of them for that to matter.
-  TcPlan p = plan_tiles(M, N, K, kind, false, kernels[kind][0]);
-  auto consider = [&](const TcPlan& q) { if (q.cost < p.cost) p = q; };
-  consider(plan_stream(M, N, K, kind, false));
-  if (p.brows >= 64) {
-    consider(plan_tiles(M, N, K, kind, true, kernels[kind][1]));
-    consider(plan_stream(M, N, K, kind, true));
-  }
-  CUtensorMap map_w, map_x;
-  int rc = make_map_sw128(&map_w, w, (uint64_t)N, (uint64_t)K * (kind == kBf16 ? 2 : 1), (uint32_t)p.chan);
-  if (rc != QUASAR_OK) return rc;
-  rc = make_map_sw128(&map_x, x, (uint64_t)M * (kind == kDigits ? 3 : 1), (uint64_t)K * (kind == kBf16 ? 2 : 1), (uint32_t)(p.pair ? p.brows / 2 : p.brows));
-  if (rc != QUASAR_OK) return rc;
-  TcArgs a;
-  a.dx = dx; a.dw = dw; a.y = y; a.res = residual; a.acc_out = acc_out; a.keys = keys; a.error = error;
-  a.M = (int)M; a.N = (int)N; a.kblocks = p.kblocks; a.chan = p.chan; a.rows = p.rows; a.brows = p.brows;
-  a.row_tiles = p.row_tiles; a.nsplit = p.nsplit; a.stages = p.stages; a.y_is_f32 = y_is_f32 ? 1 : 0;
-  a.early_weights = pdl ? 1 : 0;
-  switch (kind * 2 + p.pair) {
-    case kDigits * 2: return launch_kind<kDigits, false>(map_w, map_x, a, p, pdl, stream);
-    case kDigits * 2 + 1: return launch_kind<kDigits, true>(map_w, map_x, a, p, pdl, stream);
-    case kBf16 * 2: return launch_kind<kBf16, false>(map_w, map_x, a, p, pdl, stream);
-    case kBf16 * 2 + 1: return launch_kind<kBf16, true>(map_w, map_x, a, p, pdl, stream);
-    case kCodes * 2: return launch_kind<kCodes, false>(map_w, map_x, a, p, pdl, stream);
-    default: return launch_kind<kCodes, true>(map_w, map_x, a, p, pdl, stream);
-  }
+  TcArgs a = {};
+  a.y = y; a.res = residual; a.acc_out = acc_out; a.keys = keys; a.error = error; a.y_is_f32 = y_is_f32 ? 1 : 0;
+  return launch_layer(kind, kStore, Operand{x, dx, w, dw, M, N, K}, a, pdl, stream);
 }
+
+int kind_of(int form) { return form == kOperandDigits ? kDigits : form == kOperandCodes ? kCodes : kBf16; }
 
 }  // namespace
 
@@ -916,6 +1075,23 @@ int launch_tc_linear_w8a8(const int8_t* xq, const float* dx, const int8_t* w, co
                           void* y, bool y_is_f32, const __nv_bfloat16* residual, int32_t* acc_out, unsigned long long* keys,
                           int32_t* error, bool pdl, cudaStream_t stream) {
   return launch_any(kCodes, xq, dx, w, dw, M, N, K, y, y_is_f32, residual, acc_out, keys, error, pdl, stream);
+}
+
+// A fused epilogue needs a block of one row tile: wider ones stream their tiles, which the plain epilogue does.
+bool tc_fusable(int form, int64_t M) { return M <= (form == kOperandDigits ? 80 : 128); }
+
+int launch_tc_qkv_rope(int form, const void* x, const float* dx, const void* w, const float* dw, int64_t M, int64_t K, const RopeArgs& rope,
+                       int32_t* error, cudaStream_t stream) {
+  TcArgs a = {};
+  a.rope = rope; a.error = error;
+  return launch_layer(kind_of(form), kRope, Operand{x, dx, w, dw, M, (int64_t)(rope.Hq + 2 * rope.Hkv) * rope.D, K}, a, true, stream);
+}
+
+int launch_tc_gateup_swiglu(int form, const void* x, const float* dx, const void* w, const float* dw, int64_t M, int64_t F, int64_t K,
+                            __nv_bfloat16* act, unsigned* act_max, const float* smooth, int32_t* error, cudaStream_t stream) {
+  TcArgs a = {};
+  a.act = act; a.act_max = act_max; a.smooth = smooth; a.error = error;
+  return launch_layer(kind_of(form), kSwiglu, Operand{x, dx, w, dw, M, 2 * F, K}, a, true, stream);
 }
 
 }  // namespace quasar

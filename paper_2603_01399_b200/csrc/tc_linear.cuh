@@ -2,6 +2,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "rope.cuh"
 
 namespace quasar {
 
@@ -25,6 +26,17 @@ int launch_tc_linear_digits(const int8_t* xd, const float* row_scale, const int8
 int launch_tc_linear_w8a8(const int8_t* xq, const float* dx, const int8_t* w, const float* dw, int64_t M, int64_t N, int64_t K,
                           void* y, bool y_is_f32, const __nv_bfloat16* residual, int32_t* acc_out, unsigned long long* keys, int32_t* error, bool pdl,
                           cudaStream_t stream);
+
+// Layers of the pass with the step that follows in their epilogue (form: OperandForm, which the operand is in; always
+// dependent launches), for blocks that tc_fusable accepts.
+// qkv projection: QK-norm, RoPE and KV append; writes q (into rope.qkv) and the cache rows.
+bool tc_fusable(int form, int64_t M);
+int launch_tc_qkv_rope(int form, const void* x, const float* dx, const void* w, const float* dw, int64_t M, int64_t K, const RopeArgs& rope,
+                       int32_t* error, cudaStream_t stream);
+// gate+up projection: act = silu(gate) * up, [M][F] bf16; act_max [M] (zero before): bits of each row's largest magnitude,
+// times the smoothing factors of the down projection's input if there are any
+int launch_tc_gateup_swiglu(int form, const void* x, const float* dx, const void* w, const float* dw, int64_t M, int64_t F, int64_t K,
+                            __nv_bfloat16* act, unsigned* act_max, const float* smooth, int32_t* error, cudaStream_t stream);
 
 #ifdef __CUDACC__
 // Order-preserving key of a value and its index: the larger key is the larger value and, among equals, the lower index.
