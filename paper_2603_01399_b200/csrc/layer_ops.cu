@@ -49,7 +49,9 @@ __global__ void __launch_bounds__(128) rope_append_kernel(const RopeArgs a, int 
     hi[p] = __bfloat162float(src[lane + 32 * p + D / 2]);
   }
   __nv_bfloat16* dst = is_q ? src : a.k_cache + (((size_t)b * a.Hkv + (head - a.Hq)) * a.s_max + (P + i)) * D;
-  rope_head<D>(lo, hi, is_q ? a.q_norm : a.k_norm, a.table, P + a.bi.depth[m], a.eps, dst);
+  RopeLane<D> rl;
+  rope_load<D>(rl, is_q ? a.q_norm : a.k_norm, a.table, P + a.bi.depth[m]);
+  rope_head<D>(lo, hi, rl, a.eps, dst);
 }
 
 // ---- commit: (tree) move accepted rows into place, then bump seq_len --------------------------

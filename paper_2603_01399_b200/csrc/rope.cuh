@@ -18,13 +18,31 @@ struct RopeArgs {
 };
 
 #ifdef __CUDACC__
-// Lane l holds the rotation pairs (d, d + D/2), d = l + 32 p, in lo[p], hi[p]; they are normalised (gain not null), rotated to
-// position `pos` and stored to dst.
+// What a lane needs to rotate its pairs (d, d + D/2), d = lane + 32 p, of a head vector; loaded apart, so that the loads can be
+// under way before the vector is there.
 template <int D>
-__device__ __forceinline__ void rope_head(float (&lo)[D / 64], float (&hi)[D / 64], const __nv_bfloat16* gain, const float2* table,
-                                          int pos, float eps, __nv_bfloat16* dst) {
+struct RopeLane {
+  float2 cs[D / 64];
+  float glo[D / 64], ghi[D / 64];
+  bool normed;
+};
+template <int D>
+__device__ __forceinline__ void rope_load(RopeLane<D>& r, const __nv_bfloat16* gain, const float2* table, int pos) {
   const int lane = threadIdx.x & 31;
-  if (gain != nullptr) {
+  r.normed = gain != nullptr;
+#pragma unroll
+  for (int p = 0; p < D / 64; ++p) {
+    const int d = lane + 32 * p;
+    r.cs[p] = table[(size_t)pos * (D / 2) + d];
+    r.glo[p] = r.normed ? __bfloat162float(gain[d]) : 1.f;
+    r.ghi[p] = r.normed ? __bfloat162float(gain[d + D / 2]) : 1.f;
+  }
+}
+// the pairs lo[p], hi[p] normalised (if the model does), rotated and stored to dst
+template <int D>
+__device__ __forceinline__ void rope_head(float (&lo)[D / 64], float (&hi)[D / 64], const RopeLane<D>& rl, float eps, __nv_bfloat16* dst) {
+  const int lane = threadIdx.x & 31;
+  if (rl.normed) {
     float ss = 0.f;
 #pragma unroll
     for (int p = 0; p < D / 64; ++p) ss += lo[p] * lo[p] + hi[p] * hi[p];
@@ -33,17 +51,15 @@ __device__ __forceinline__ void rope_head(float (&lo)[D / 64], float (&hi)[D / 6
     const float r = 1.0f / sqrtf(ss / (float)D + eps);
 #pragma unroll
     for (int p = 0; p < D / 64; ++p) {
-      const int d = lane + 32 * p;
-      lo[p] = lo[p] * r * __bfloat162float(gain[d]);
-      hi[p] = hi[p] * r * __bfloat162float(gain[d + D / 2]);
+      lo[p] = lo[p] * r * rl.glo[p];
+      hi[p] = hi[p] * r * rl.ghi[p];
     }
   }
 #pragma unroll
   for (int p = 0; p < D / 64; ++p) {
     const int d = lane + 32 * p;
-    const float2 cs = table[(size_t)pos * (D / 2) + d];
-    dst[d] = __float2bfloat16_rn(lo[p] * cs.x - hi[p] * cs.y);
-    dst[d + D / 2] = __float2bfloat16_rn(hi[p] * cs.x + lo[p] * cs.y);
+    dst[d] = __float2bfloat16_rn(lo[p] * rl.cs[p].x - hi[p] * rl.cs[p].y);
+    dst[d + D / 2] = __float2bfloat16_rn(hi[p] * rl.cs[p].x + lo[p] * rl.cs[p].y);
   }
 }
 #endif

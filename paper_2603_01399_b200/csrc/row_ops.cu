@@ -312,9 +312,10 @@ template <int OP, int D, bool LIST>
 __global__ void __launch_bounds__(kMergeWarps * 32)
 attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, RowOperand out) {
   __shared__ float s_buf[kMergeWarps];
-  __shared__ float s_amax;
+  __shared__ float s_amax[kMergeCtas];   // of every CTA of the cluster
   extern __shared__ __align__(16) unsigned char s_row[];   // this CTA's heads, bf16; then each warp's parts of a batch
   pdl_trigger();
+  if (OP != kOperandBf16) tc::cluster_arrive();   // (every CTA of the cluster has started before one writes into another's memory)
   pdl_wait();
   const int rank = blockIdx.x % kMergeCtas, m = blockIdx.x / kMergeCtas, b = m / l.T_max, i = m % l.T_max;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
@@ -386,6 +387,7 @@ attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, Ro
         for (int j0 = 0; j0 < cnt; j0 += batch) {
           // the batch's copies in flight together (as loads into registers the compiler spreads them over their uses)
           const int nb = min(batch, cnt - j0);
+#pragma unroll 4
           for (int q = 0; q < nb; ++q) {
             const float* src = parts.o + (at0 + (size_t)__float_as_int(s_part[warp][j0 + q].x) * stride) * D + lane * kPer;
             asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(tc::smem_u32(s_o + (q * 32 + lane) * kPer)), "l"(src),
@@ -393,6 +395,7 @@ attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, Ro
                          : "memory");
           }
           asm volatile("cp.async.wait_all;\n" ::: "memory");   // (each lane reads only what it copied)
+#pragma unroll 4
           for (int q = 0; q < nb; ++q) {
             const float4 part = s_part[warp][j0 + q];
             den += part.y * part.z;
@@ -435,14 +438,16 @@ attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, Ro
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < warps; ++w) amax = fmaxf(amax, s_buf[w]);
-    s_amax = amax;
   }
+  tc::cluster_wait();
+  amax = __shfl_sync(0xffffffffu, amax, 0);
+  if (threadIdx.x < kMergeCtas) tc::st_cluster_f32(tc::cluster_map(tc::smem_u32(s_amax + rank), threadIdx.x), amax);   // (warp 0 holds it)
   __syncwarp();
   tc::cluster_arrive();
   tc::cluster_wait();
   amax = 0.f;
 #pragma unroll
-  for (int c = 0; c < kMergeCtas; ++c) amax = fmaxf(amax, tc::ld_cluster_f32(tc::cluster_map(tc::smem_u32(&s_amax), (uint32_t)c)));
+  for (int c = 0; c < kMergeCtas; ++c) amax = fmaxf(amax, s_amax[c]);
   float up = 1.f, scale = 1.f;
   if (OP == kOperandDigits) digit_scale(amax, up, scale);
   else scale = amax == 0.f ? 1.0f : __fdiv_rn(amax, 127.0f);
@@ -456,8 +461,6 @@ attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, Ro
       *reinterpret_cast<uint2*>(out.q + (int64_t)m * width + (int64_t)(first + v) * 8) = smoothed_codes8(f, s, scale);
     }
   }
-  tc::cluster_arrive();   // (nobody's maximum goes away while another CTA may read it)
-  tc::cluster_wait();
 }
 
 // One warp checks a sequence's tokens / parents / capacity and derives ancestor bit masks and depths.  A chain's are known

@@ -128,21 +128,64 @@ __device__ __forceinline__ float finish(uint32_t bits, float dx, float dw) {
   return __uint_as_float(bits);
 }
 
-// one row, four channels from n on; `best`: the row's arg-max key so far
-template <int KIND>
-__device__ __forceinline__ void store4(const TcArgs& a, const uint32_t (&v)[4], int m, int n, float dx, unsigned long long& best) {
-  const size_t idx = (size_t)m * a.N + n;
-  const bool vec = (a.N & 3) == 0;   // then n + 3 < N, and every address below is aligned
-  float f[4];
-  if (vec) {
-    float4 dw = make_float4(1.f, 1.f, 1.f, 1.f);
-    if (KIND != kBf16) dw = __ldg(reinterpret_cast<const float4*>(a.dw + n));
-    f[0] = finish<KIND>(v[0], dx, dw.x); f[1] = finish<KIND>(v[1], dx, dw.y);
-    f[2] = finish<KIND>(v[2], dx, dw.z); f[3] = finish<KIND>(v[3], dx, dw.w);
+// What finishing four channels of a row needs besides their sums.  Loaded apart: the first row's loads are under way while the
+// sums are still being made (fetched behind them they cost a round trip or, with RoPE, three: 1-2 us a launch).
+template <int KIND, int EPI>
+struct RowPre {
+  float dx;
+  float4 dw, dw2, smooth;   // step sizes (SwiGLU: gate, up), smoothing factors
+  uint2 res;
+  RopeLane<128> r128;
+  RopeLane<64> r64[2];
+  int slot;                 // RoPE: the row's cache position, or -1: a row that takes no part
+};
+
+template <int KIND, int EPI>
+__device__ __forceinline__ void load_pre(RowPre<KIND, EPI>& p, const TcArgs& a, int m, int n, int n0) {
+  p.dx = KIND != kBf16 ? a.dx[m] : 1.f;
+  if (EPI == kSwiglu) {   // n: the unit
+    const int F = a.N / 2;
+    const bool in = n < F;
+    if (KIND != kBf16) {
+      p.dw = in ? __ldg(reinterpret_cast<const float4*>(a.dw + n)) : make_float4(1.f, 1.f, 1.f, 1.f);
+      p.dw2 = in ? __ldg(reinterpret_cast<const float4*>(a.dw + F + n)) : make_float4(1.f, 1.f, 1.f, 1.f);
+    }
+    p.smooth = in && a.smooth != nullptr ? __ldg(reinterpret_cast<const float4*>(a.smooth + n)) : make_float4(1.f, 1.f, 1.f, 1.f);
+    return;
+  }
+  if (KIND != kBf16) {
+    if ((a.N & 3) == 0) {   // (then four channels from a multiple of four on are inside or outside together)
+      p.dw = n < a.N ? __ldg(reinterpret_cast<const float4*>(a.dw + n)) : make_float4(1.f, 1.f, 1.f, 1.f);
+    } else {
+      p.dw = make_float4(n < a.N ? a.dw[n] : 1.f, n + 1 < a.N ? a.dw[n + 1] : 1.f, n + 2 < a.N ? a.dw[n + 2] : 1.f, n + 3 < a.N ? a.dw[n + 3] : 1.f);
+    }
+  }
+  if (EPI == kStore) {
+    if (a.res != nullptr && (a.N & 3) == 0 && n < a.N) p.res = *reinterpret_cast<const uint2*>(a.res + (size_t)m * a.N + n);
+    return;
+  }
+  const RopeArgs& r = a.rope;
+  const int b = m / r.T_max, i = m - b * r.T_max;
+  const int valid = r.bi.valid[b], len = r.block_len[b], P = r.seq_len[b], depth = r.bi.depth[m];
+  p.slot = valid != 0 && i < len ? P + i : -1;
+  const int pos = p.slot < 0 ? 0 : P + depth;
+  if (r.D == 128) {
+    const int head = n0 / 128;
+    rope_load<128>(p.r128, head < r.Hq ? r.q_norm : r.k_norm, r.table, pos);
   } else {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) f[e] = finish<KIND>(v[e], dx, (KIND != kBf16 && n + e < a.N) ? a.dw[n + e] : 1.f);
+    for (int h = 0; h < 2; ++h) rope_load<64>(p.r64[h], n0 / 64 + h < r.Hq ? r.q_norm : r.k_norm, r.table, pos);
   }
+}
+
+// one row, four channels from n on; `best`: the row's arg-max key so far
+template <int KIND>
+__device__ __forceinline__ void store4(const TcArgs& a, const uint32_t (&v)[4], int m, int n, const RowPre<KIND, kStore>& p, unsigned long long& best) {
+  const size_t idx = (size_t)m * a.N + n;
+  const bool vec = (a.N & 3) == 0;   // then n + 3 < N, and every address below is aligned
+  const float f0[4] = {finish<KIND>(v[0], p.dx, p.dw.x), finish<KIND>(v[1], p.dx, p.dw.y), finish<KIND>(v[2], p.dx, p.dw.z),
+                       finish<KIND>(v[3], p.dx, p.dw.w)};
+  float f[4] = {f0[0], f0[1], f0[2], f0[3]};
   if (a.keys != nullptr) {
 #pragma unroll
     for (int e = 0; e < 4; ++e)
@@ -156,8 +199,7 @@ __device__ __forceinline__ void store4(const TcArgs& a, const uint32_t (&v)[4], 
     if (KIND == kCodes && a.acc_out != nullptr)
       *reinterpret_cast<int4*>(a.acc_out + idx) = make_int4((int)v[0], (int)v[1], (int)v[2], (int)v[3]);
     if (a.res != nullptr) {
-      const uint2 r = *reinterpret_cast<const uint2*>(a.res + idx);
-      const uint32_t rr[2] = {r.x, r.y};
+      const uint32_t rr[2] = {p.res.x, p.res.y};
 #pragma unroll
       for (int e = 0; e < 4; ++e)
         f[e] = __bfloat162float(__float2bfloat16_rn(f[e])) +
@@ -185,16 +227,15 @@ __device__ __forceinline__ void store4(const TcArgs& a, const uint32_t (&v)[4], 
 
 // one row of a 128-channel tile, four channels a lane: q and k heads normalised, rotated and put in their places, v heads copied
 template <int KIND, int D>
-__device__ __forceinline__ void store_rope(const TcArgs& a, const uint32_t (&v)[4], int m, int n0, float dx) {
+__device__ __forceinline__ void store_rope(const TcArgs& a, const uint32_t (&v)[4], int m, int n0, const RowPre<KIND, kRope>& p) {
   const RopeArgs& r = a.rope;
-  const int lane = threadIdx.x & 31, n = n0 + lane * 4;
+  const int lane = threadIdx.x & 31;
+  const float dw[4] = {p.dw.x, p.dw.y, p.dw.z, p.dw.w};
   float f[4];   // as the linear layer's bf16 output
 #pragma unroll
-  for (int e = 0; e < 4; ++e)
-    f[e] = __bfloat162float(__float2bfloat16_rn(finish<KIND>(v[e], dx, (KIND != kBf16 && n + e < a.N) ? __ldg(a.dw + n + e) : 1.f)));
-  const int b = m / r.T_max, i = m % r.T_max;
-  if (!r.bi.valid[b] || i >= r.block_len[b]) return;
-  const int P = r.seq_len[b], pos = P + r.bi.depth[m];
+  for (int e = 0; e < 4; ++e) f[e] = __bfloat162float(__float2bfloat16_rn(finish<KIND>(v[e], p.dx, dw[e])));
+  if (p.slot < 0) return;
+  const int b = m / r.T_max;
 #pragma unroll
   for (int h = 0; h < 128 / D; ++h) {
     const int head = n0 / D + h;
@@ -212,31 +253,29 @@ __device__ __forceinline__ void store_rope(const TcArgs& a, const uint32_t (&v)[
     }
     if (head >= r.Hq + 2 * r.Hkv) continue;
     if (head >= r.Hq + r.Hkv) {
-      __nv_bfloat16* dst = r.v_cache + (((size_t)b * r.Hkv + (head - r.Hq - r.Hkv)) * r.s_max + (P + i)) * D;
+      __nv_bfloat16* dst = r.v_cache + (((size_t)b * r.Hkv + (head - r.Hq - r.Hkv)) * r.s_max + p.slot) * D;
 #pragma unroll
       for (int k = 0; k < D / 32; ++k) dst[lane + 32 * k] = __float2bfloat16_rn(x[k]);
       continue;
     }
-    const bool is_q = head < r.Hq;
     float lo[D / 64], hi[D / 64];
 #pragma unroll
-    for (int p = 0; p < D / 64; ++p) { lo[p] = x[p]; hi[p] = x[p + D / 64]; }
-    __nv_bfloat16* dst = is_q ? r.qkv + (size_t)m * a.N + (size_t)head * D
-                              : r.k_cache + (((size_t)b * r.Hkv + (head - r.Hq)) * r.s_max + (P + i)) * D;
-    rope_head<D>(lo, hi, is_q ? r.q_norm : r.k_norm, r.table, pos, r.eps, dst);
+    for (int q = 0; q < D / 64; ++q) { lo[q] = x[q]; hi[q] = x[q + D / 64]; }
+    __nv_bfloat16* dst = head < r.Hq ? r.qkv + (size_t)m * a.N + (size_t)head * D
+                                     : r.k_cache + (((size_t)b * r.Hkv + (head - r.Hq)) * r.s_max + p.slot) * D;
+    if constexpr (D == 128) rope_head<128>(lo, hi, p.r128, r.eps, dst);
+    else rope_head<64>(lo, hi, p.r64[h], r.eps, dst);
   }
 }
 
 // one row, four units from u on: silu(gate) * up, both rounded to bf16 first (they are tensors of the layer)
 template <int KIND>
-__device__ __forceinline__ float store_swiglu(const TcArgs& a, const uint32_t (&g)[4], const uint32_t (&up)[4], int m, int u, float dx) {
+__device__ __forceinline__ float store_swiglu(const TcArgs& a, const uint32_t (&g)[4], const uint32_t (&up)[4], int m, int u,
+                                              const RowPre<KIND, kSwiglu>& p) {
   const int F = a.N / 2;   // a multiple of 16: four units from a multiple of four on are inside or outside together
-  float4 dg = make_float4(1.f, 1.f, 1.f, 1.f), du = dg;
-  if (KIND != kBf16) {
-    dg = __ldg(reinterpret_cast<const float4*>(a.dw + u));
-    du = __ldg(reinterpret_cast<const float4*>(a.dw + F + u));
-  }
-  const float dgv[4] = {dg.x, dg.y, dg.z, dg.w}, duv[4] = {du.x, du.y, du.z, du.w};
+  const float dgv[4] = {p.dw.x, p.dw.y, p.dw.z, p.dw.w}, duv[4] = {p.dw2.x, p.dw2.y, p.dw2.z, p.dw2.w};
+  const float s[4] = {p.smooth.x, p.smooth.y, p.smooth.z, p.smooth.w};
+  const float dx = p.dx;
   float f[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
@@ -247,11 +286,6 @@ __device__ __forceinline__ float store_swiglu(const TcArgs& a, const uint32_t (&
   const __nv_bfloat162 lo = __floats2bfloat162_rn(f[0], f[1]), hi = __floats2bfloat162_rn(f[2], f[3]);
   const uint32_t w0 = *reinterpret_cast<const uint32_t*>(&lo), w1 = *reinterpret_cast<const uint32_t*>(&hi);
   *reinterpret_cast<uint2*>(a.act + (size_t)m * F + u) = make_uint2(w0, w1);
-  float s[4] = {1.f, 1.f, 1.f, 1.f};
-  if (a.smooth != nullptr) {
-    const float4 t = __ldg(reinterpret_cast<const float4*>(a.smooth + u));
-    s[0] = t.x; s[1] = t.y; s[2] = t.z; s[3] = t.w;
-  }
   float amax = fmaxf(0.f, fabsf(__fmul_rn(__uint_as_float(w0 << 16), s[0])));
   amax = fmaxf(amax, fabsf(__fmul_rn(__uint_as_float(w0 & 0xffff0000u), s[1])));
   amax = fmaxf(amax, fabsf(__fmul_rn(__uint_as_float(w1 << 16), s[2])));
@@ -334,6 +368,17 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
   // Only now may the kernel behind this one start: a tcgen05 kernel further down the stream waits for this one while it
   // holds tensor memory, so every CTA here must have its own first.
   if (threadIdx.x == 0) pdl_trigger();
+
+  // this CTA's share of the tile's rows: 32 threads a row and four channels a thread (SwiGLU: 16 threads a row, four units), the
+  // warps that do nothing else first
+  const int rows = min(a.rows, a.M - m0);
+  const int per = (rows + a.nsplit - 1) / a.nsplit;
+  const int r_begin = split * per, r_end = min(rows, r_begin + per);
+  constexpr int kRowsPerWarp = EPI == kSwiglu ? 2 : 1;
+  const int turn = (warp + 8) % 10;
+  int pre_m = r_begin + turn * kRowsPerWarp + (EPI == kSwiglu ? lane >> 4 : 0);
+  const int pre_n = EPI == kSwiglu ? n0 / 2 + (lane & 15) * 4 : n0 + lane * 4;
+  RowPre<KIND, EPI> pre;
 
   if (warp == 0) {
     {   // ---- TMA producer ----
@@ -425,6 +470,8 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     const int q = warp & 3, half = (warp - 2) >> 2;
     const int r = q * 32 + lane;
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
+    pdl_wait();   // (what a row's finishing needs may come from the kernel in front)
+    if (pre_m < r_end) load_pre<KIND, EPI>(pre, a, m0 + pre_m, pre_n, n0);
     if (__all_sync(0xffffffffu, mbar_wait(accum_done, 0, abort_flag, a.error))) {
       fence_after();
       uint32_t* red = reinterpret_cast<uint32_t*>(smem);
@@ -463,10 +510,6 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
   }
   pdl_wait();   // every thread: the residual below may come from the kernel in front
   if (*abort_flag == 0) {
-    // this CTA's share of the tile's rows, 32 threads a row, four channels a thread; the ranges in ascending order
-    const int rows = min(a.rows, a.M - m0);
-    const int per = (rows + a.nsplit - 1) / a.nsplit;
-    const int r_begin = split * per, r_end = min(rows, r_begin + per);
     const uint32_t red_addr = smem_u32(smem);
     // the sums of row m (of the tile) over the ranges, four channels from c on
     auto sums = [&](int m, int c, uint32_t (&sum)[4]) {
@@ -493,18 +536,20 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
       }
     };
     uint32_t sum[4];
-    if (EPI == kSwiglu) {   // 16 lanes a row
-      const int half = a.chan / 2, c = (lane & 15) * 4, u = n0 / 2 + c;
-      const bool live = c < half && u < a.N / 2;
-      for (int mb = r_begin + warp * 2; mb < r_end; mb += kThreadsTc / 32 * 2) {
-        const int m = mb + (lane >> 4);
+    bool loaded = warp >= 2;
+    if (EPI == kSwiglu) {
+      const int half = a.chan / 2, c = (lane & 15) * 4;
+      const bool live = c < half && pre_n < a.N / 2;
+      for (int m = pre_m; m - (lane >> 4) < r_end; m += kThreadsTc / 32 * 2) {
         float amax = 0.f;
         if (live && m < r_end) {
+          if (!loaded) load_pre<KIND, EPI>(pre, a, m0 + m, pre_n, n0);
           uint32_t up[4];
           sums(m, c, sum);
           sums(m, half + c, up);
-          amax = store_swiglu<KIND>(a, sum, up, m0 + m, u, KIND != kBf16 ? a.dx[m0 + m] : 1.f);
+          if constexpr (EPI == kSwiglu) amax = store_swiglu<KIND>(a, sum, up, m0 + m, pre_n, pre);
         }
+        loaded = false;
         if (a.act_max != nullptr) {
 #pragma unroll
           for (int o = 8; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
@@ -512,20 +557,22 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         }
       }
     } else {
-      const int n = n0 + lane * 4;
-      const bool live = lane * 4 < a.chan && n < a.N;
-      for (int m = r_begin + warp; m < r_end; m += kThreadsTc / 32) {
-        const float dx = KIND != kBf16 ? a.dx[m0 + m] : 1.f;
-        if (EPI == kRope) {   // (all 128 channels; ones beyond the matrix are zero)
+      const bool live = lane * 4 < a.chan && pre_n < a.N;
+      for (int m = pre_m; m < r_end; m += kThreadsTc / 32) {
+        if (!loaded) load_pre<KIND, EPI>(pre, a, m0 + m, pre_n, n0);
+        loaded = false;
+        if constexpr (EPI == kRope) {   // (all 128 channels; ones beyond the matrix are zero)
           sums(m, lane * 4, sum);
-          if (a.rope.D == 128) store_rope<KIND, 128>(a, sum, m0 + m, n0, dx);
-          else store_rope<KIND, 64>(a, sum, m0 + m, n0, dx);
+          if (a.rope.D == 128) store_rope<KIND, 128>(a, sum, m0 + m, n0, pre);
+          else store_rope<KIND, 64>(a, sum, m0 + m, n0, pre);
           continue;
         }
         unsigned long long best = 0;
-        if (live) {
-          sums(m, lane * 4, sum);
-          store4<KIND>(a, sum, m0 + m, n, dx, best);
+        if constexpr (EPI == kStore) {
+          if (live) {
+            sums(m, lane * 4, sum);
+            store4<KIND>(a, sum, m0 + m, pre_n, pre, best);
+          }
         }
         if (a.keys != nullptr) {
 #pragma unroll
