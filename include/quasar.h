@@ -27,6 +27,8 @@
  *    stream has been synchronised.  quasar_plan_create is the supported way to freeze a
  *    pass for replay: it captures the kernel-per-step form into a CUDA graph itself and
  *    keeps the persistent single-kernel form (a cooperative launch) as a plain launch.
+ *    quasar_verify itself captures a call that keeps coming back with the same pointers
+ *    and sizes, at its third appearance, and replays that (eight argument sets a model).
  *  - Argument errors that the host can see are reported before anything is
  *    launched.  Errors only the device can see (a token id out of range, a
  *    malformed parent array, a sequence that would overflow its cache) set the
@@ -201,8 +203,8 @@ typedef struct quasar_config {
   int32_t max_seq;      /* cache capacity S_max (positions) the RoPE table covers */
   int32_t act_dtype;    /* QUASAR_A_BF16, or QUASAR_A_INT8 (needs weight_dtype QUASAR_W_INT8; the
                            weights must then be Q(W diag(s)^-1) for the smoothing vectors below) */
-  int32_t weights_in_place; /* 0: the model borrows the weight matrices and keeps a second, permuted copy for
-                           the persistent single-kernel pass (twice the weight bytes).  1: the caller hands
+  int32_t weights_in_place; /* 0: the model borrows the weight matrices; a second, permuted copy is made
+                           only if quasar_set_path asks for the persistent single-kernel pass.  1: the caller hands
                            the matrices over: quasar_model_create permutes each of them WHERE IT LIES into the
                            order the persistent kernel streams it (their contents are no longer row-major
                            afterwards) and keeps no copy, so the model occupies the weight bytes once - the
@@ -374,9 +376,9 @@ int quasar_plan_run_host(quasar_plan* p, const int32_t* tokens_host, const int32
 int quasar_trace_bytes(const quasar_model* m, int32_t B, int32_t T_max, size_t* bytes_out /* host */);
 int quasar_set_trace(quasar_model* m, void* trace_buf, size_t bytes);
 
-/* Which implementation quasar_verify uses: 0 = automatic (the persistent single-kernel pass
- * when the block has at most 8 rows in total, else one kernel per step), 1 = always one kernel
- * per step, 2 = require the persistent kernel (QUASAR_ERR_SHAPE if the call does not fit it).
+/* Which implementation quasar_verify uses: 0 = automatic (one kernel per step, the faster form
+ * at every size), 1 = one kernel per step, 2 = require the persistent kernel (at most 8 block rows in
+ * total; QUASAR_ERR_SHAPE if the call does not fit it).  The first 2 makes that kernel's copy of the weights.
  * Both compute the same pass (Section 3.1, 3.3); they differ in summation order only. */
 int quasar_set_path(quasar_model* m, int32_t path);
 

@@ -339,7 +339,7 @@ class Model:
         _check(lib().quasar_set_trace(self.handle, _ptr(buf), 0 if buf is None else buf.numel() * buf.element_size()))
 
     def set_path(self, path: int) -> None:
-        """0 automatic, 1 one kernel per step, 2 persistent single-kernel pass."""
+        """0 automatic (one kernel per step), 1 one kernel per step, 2 persistent single-kernel pass."""
         _check(lib().quasar_set_path(self.handle, path))
 
     def launch_kind(self, batch: int, t_max: int) -> str:

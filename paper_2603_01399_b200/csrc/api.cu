@@ -7,6 +7,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -19,6 +20,7 @@ namespace quasar {
 
 static thread_local char g_err[512] = "";
 static std::atomic<long long> g_launches{0};
+static thread_local long long t_launches = 0;   // those of this thread: what a capture of its own holds
 
 void set_error(const char* fmt, ...) {
   va_list ap;
@@ -27,11 +29,32 @@ void set_error(const char* fmt, ...) {
   va_end(ap);
 }
 
-void count_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
+void count_launch(int n) {
+  g_launches.fetch_add(n, std::memory_order_relaxed);
+  t_launches += n;
+}
 
 }  // namespace quasar
 
 using namespace quasar;
+
+// A pass that is called again and again with the same buffers, as a graph (see replay_call).
+struct CallGraph {
+  const void* args[12];             // every pointer of the call
+  size_t workspace_bytes;
+  int32_t B, T_max, kv_batch, s_max;
+  int calls;                        // eager calls seen with these arguments
+  unsigned long long used;          // the model's call counter at the last one
+  cudaGraphExec_t exec;
+  int kernels;
+
+  bool same(const CallGraph& o) const {
+    return memcmp(args, o.args, sizeof(args)) == 0 && workspace_bytes == o.workspace_bytes && B == o.B && T_max == o.T_max &&
+           kv_batch == o.kv_batch && s_max == o.s_max;
+  }
+};
+
+constexpr int kCallGraphs = 8;
 
 struct quasar_model {
   quasar_config cfg;
@@ -45,13 +68,16 @@ struct quasar_model {
   MegaLayer* mega_layers = nullptr; // device
   unsigned char* mega_weights = nullptr;  // device: every matrix again, permuted for the persistent kernel
   int mega_ncta = 0;                // 0: not available on this device
-  int path = 0;                     // 0 auto, 1 one kernel per step, 2 persistent kernel
+  int path = 0;                     // 0 and 1 one kernel per step, 2 persistent kernel
   unsigned long long wait_budget_ns = 2000000000ull;   // bound of every device-side wait of the persistent kernel
   unsigned barrier_extra = 0;       // test of the failure path only (quasar_set_wait_budget)
+  // graphs of calls without a plan
+  std::mutex calls_lock;
+  CallGraph calls[kCallGraphs] = {};
+  unsigned long long call_clock = 0, builds = 0, replays = 0;
 };
 
 struct quasar_plan {
-  cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;   // null: the pass is a single persistent kernel, launched directly
   quasar_model* model = nullptr;
   quasar_kv kv;
@@ -180,7 +206,7 @@ struct TraceCursor {
 
 bool uses_persistent_kernel(const quasar_model* m, int B, int T_max) {
   const quasar_config& c = m->cfg;
-  return m->path != 1 && m->mega_ncta > 0 && m->mega_ncta <= kMaxGrid && m->trace_buf == nullptr &&
+  return m->path == 2 && m->mega_ncta > 0 && m->trace_buf == nullptr &&
          mega_supported(B * T_max, T_max, c.n_q_heads, c.n_kv_heads, c.head_dim);
 }
 
@@ -242,13 +268,12 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
   const size_t layer_stride = (size_t)kv->batch * Hkv * (size_t)kv->s_max * D;
   TraceCursor tr{reinterpret_cast<unsigned char*>(m->trace_buf), 0, m->trace_bytes, stream};
 
-  const bool can_mega = m->mega_ncta > 0 && m->mega_ncta <= kMaxGrid && m->trace_buf == nullptr &&
-                        mega_supported(M, T_max, Hq, Hkv, D);
-  if (m->path == 2 && !can_mega) {
+  const bool persistent = uses_persistent_kernel(m, B, T_max);
+  if (m->path == 2 && !persistent) {
     set_error("verify: the persistent kernel handles at most 8 block rows in total and no trace");
     return QUASAR_ERR_SHAPE;
   }
-  if (can_mega && m->path != 1) {
+  if (persistent) {
     MegaParams p;
     p.jobs = m->mega_jobs; p.layers = m->mega_layers; p.n_jobs = 4 * c.n_layers + 1; p.L = c.n_layers;
     p.B = B; p.T_max = T_max; p.M = M; p.H = H; p.Hq = Hq; p.Hkv = Hkv; p.vocab = c.vocab; p.s_max = kv->s_max;
@@ -360,6 +385,218 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
   // (the LM head finds the rows' top choices as it goes and writes logits only for a caller who wants them)
   TRY(linear(h, m->w.lm_w, m->w.lm_delta, c.vocab, H, logits_out, true, nullptr, ba.keys));
   return launch_accept(ba, accept_len, bonus, accept_path, stream);
+}
+
+// Captures one pass on a stream of its own.  The capture is thread-local, so other threads go on as they are; the kernels' attributes
+// have been set by an earlier eager pass of the same sizes.
+int capture_pass(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, const int32_t* parents, const int32_t* block_len, int32_t B,
+                 int32_t T_max, float* logits_out, int32_t* accept_len, int32_t* bonus, int32_t* accept_path, void* workspace,
+                 size_t workspace_bytes, int32_t* status, cudaStream_t s, cudaGraphExec_t* exec, int* kernels) {
+  cudaGraph_t graph = nullptr;
+  const long long before = t_launches;
+  cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
+  if (e != cudaSuccess) { set_error("begin capture: %s", cudaGetErrorString(e)); return QUASAR_ERR_CUDA; }
+  int rc = verify_impl(m, kv, tokens, parents, block_len, B, T_max, logits_out, accept_len, bonus, accept_path, workspace,
+                       workspace_bytes, status, s);
+  e = cudaStreamEndCapture(s, &graph);
+  *kernels = (int)(t_launches - before);
+  count_launch(-*kernels);  // captured launches did not run
+  if (rc == QUASAR_OK && e != cudaSuccess) { set_error("end capture: %s", cudaGetErrorString(e)); rc = QUASAR_ERR_CUDA; }
+  if (rc == QUASAR_OK) {
+    e = cudaGraphInstantiate(exec, graph, 0);
+    if (e != cudaSuccess) { set_error("instantiate: %s", cudaGetErrorString(e)); rc = QUASAR_ERR_CUDA; }
+  }
+  if (graph) cudaGraphDestroy(graph);
+  return rc;
+}
+
+void drop_call_graphs(quasar_model* m) {
+  std::lock_guard<std::mutex> hold(m->calls_lock);
+  for (CallGraph& g : m->calls) {
+    if (g.exec) cudaGraphExecDestroy(g.exec);
+    g = CallGraph{};
+  }
+}
+
+// A pass is some eight launches a layer, 58 us of host time for the two layers of a tiny decoder and 2.1 ms for 36 layers, and
+// between eager launches the device waits a little longer than between the nodes of a graph (tiny chain of 5 rows: 75.1 us a
+// call, 65.5 us as a graph; 8B, 6 rows: 2475 and 2283 us).  So a call that comes back with the same pointers and sizes, as those
+// of a decoding loop do, is captured at its third appearance and replayed from then on: what is kept is the list of launches, all
+// the work is done on every call.  Eight argument sets are remembered, the one used longest ago makes room, and capturing stops
+// while it has not been paid back (a capture costs the host about two eager passes; 16 replays for each).  false: run it eagerly.
+bool replay_call(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, const int32_t* parents, const int32_t* block_len, int32_t B,
+                 int32_t T_max, float* logits_out, int32_t* accept_len, int32_t* bonus, int32_t* accept_path, void* workspace,
+                 size_t workspace_bytes, int32_t* status, cudaStream_t stream, int* rc) {
+  if (m == nullptr || kv == nullptr || m->trace_buf != nullptr || m->path == 2) return false;
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess || capturing != cudaStreamCaptureStatusNone) return false;
+  const CallGraph want{{kv->k, kv->v, kv->seq_len, tokens, parents, block_len, logits_out, accept_len, bonus, accept_path, workspace, status},
+                       workspace_bytes, B, T_max, kv->batch, kv->s_max, 0, 0, nullptr, 0};
+  std::lock_guard<std::mutex> hold(m->calls_lock);
+  ++m->call_clock;
+  CallGraph* g = nullptr;
+  CallGraph* oldest = m->calls;
+  for (CallGraph& c : m->calls) {
+    if (c.used != 0 && c.same(want)) g = &c;
+    if (c.used < oldest->used) oldest = &c;
+  }
+  if (g == nullptr) {
+    if (oldest->exec) cudaGraphExecDestroy(oldest->exec);
+    *oldest = want;
+    oldest->used = m->call_clock;
+    oldest->calls = 1;
+    return false;
+  }
+  g->used = m->call_clock;
+  if (g->exec == nullptr) {
+    if (++g->calls < 3 || m->builds > 4 + m->replays / 16) return false;
+    // (relaxed for the while: another thread may be capturing a stream of its own in the global mode)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) { cudaGetLastError(); return false; }
+    cudaStream_t s;
+    int built = QUASAR_ERR_CUDA;
+    if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess) {
+      built = capture_pass(m, kv, tokens, parents, block_len, B, T_max, logits_out, accept_len, bonus, accept_path, workspace,
+                           workspace_bytes, status, s, &g->exec, &g->kernels);
+      cudaStreamDestroy(s);
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (built != QUASAR_OK) {   // (the eager pass reports what is wrong with the call, if it is the call)
+      cudaGetLastError();
+      *g = CallGraph{};
+      return false;
+    }
+    ++m->builds;
+  }
+  ++m->replays;
+  *rc = QUASAR_OK;
+  const cudaError_t e = cudaGraphLaunch(g->exec, stream);
+  if (e != cudaSuccess) {
+    set_error("verify: graph launch: %s", cudaGetErrorString(e));
+    *rc = QUASAR_ERR_CUDA;
+  } else {
+    count_launch(g->kernels);
+  }
+  return true;
+}
+
+void drop_persistent(quasar_model* m) {
+  if (m->mega_weights) cudaFree(m->mega_weights);
+  if (m->mega_jobs) cudaFree(m->mega_jobs);
+  if (m->mega_layers) cudaFree(m->mega_layers);
+  m->mega_weights = nullptr;
+  m->mega_jobs = nullptr;
+  m->mega_layers = nullptr;
+}
+
+// What the persistent kernel needs: its grid, the matrices in the order each CTA streams them (a copy, or permuted where they
+// lie), and the table of the GEMMs of the pass in execution order.  Made once, for a model that is to run it; where the kernel
+// cannot run, mega_ncta stays 0 and nothing is made.
+int build_persistent(quasar_model* m) {
+  const quasar_config& c = m->cfg;
+  const bool q = c.weight_dtype == QUASAR_W_INT8;
+  int ncta = 0;
+  if (c.act_dtype != QUASAR_A_BF16 || mega_grid_size(c.weight_dtype, c.head_dim, &ncta) != QUASAR_OK || ncta <= 0 || ncta > kMaxGrid)
+    return QUASAR_OK;
+  std::vector<MegaJob> jobs;
+  std::vector<MegaLayer> mls;
+  std::vector<const void*> src;
+  const int qkv_w = (c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim;
+  for (int l = 0; l < c.n_layers; ++l) {
+    const quasar_layer_weights& L = m->layers[l];
+    jobs.push_back({nullptr, q ? L.qkv_delta : nullptr, reinterpret_cast<const __nv_bfloat16*>(L.attn_norm), qkv_w,
+                    c.hidden, kJobQkv, 1.f});
+    src.push_back(L.qkv_w);
+    jobs.push_back({nullptr, q ? L.o_delta : nullptr, nullptr, c.hidden, c.n_q_heads * c.head_dim, kJobO, 1.f});
+    src.push_back(L.o_w);
+    jobs.push_back({nullptr, q ? L.gateup_delta : nullptr, reinterpret_cast<const __nv_bfloat16*>(L.mlp_norm),
+                    2 * c.ffn, c.hidden, kJobGateUp, 1.f});
+    src.push_back(L.gateup_w);
+    jobs.push_back({nullptr, q ? L.down_delta : nullptr, nullptr, c.hidden, c.ffn, kJobDown, 1.f});
+    src.push_back(L.down_w);
+    mls.push_back({reinterpret_cast<const __nv_bfloat16*>(c.qk_norm ? L.q_norm : nullptr),
+                   reinterpret_cast<const __nv_bfloat16*>(c.qk_norm ? L.k_norm : nullptr)});
+  }
+  jobs.push_back({nullptr, q ? m->w.lm_delta : nullptr, reinterpret_cast<const __nv_bfloat16*>(m->w.final_norm),
+                  c.vocab, c.hidden, kJobLm, 1.f});
+  src.push_back(m->w.lm_w);
+  if (mls.empty()) mls.push_back({nullptr, nullptr});
+  // Normed GEMMs feed h = x * r * gain with |x r| <= sqrt(K): a static power-of-two scale keeps h
+  // inside the fp16 range whatever the activations are (1 unless a gain is in the hundreds).
+  {
+    std::vector<uint16_t> gh;
+    for (auto& j : jobs) {
+      if (j.gain == nullptr) continue;
+      gh.resize(j.K);
+      if (cudaMemcpy(gh.data(), j.gain, (size_t)j.K * 2, cudaMemcpyDeviceToHost) != cudaSuccess) {
+        set_error("persistent kernel: reading a norm gain failed: %s", cudaGetErrorString(cudaGetLastError()));
+        return QUASAR_ERR_CUDA;
+      }
+      float gmax = 0.f;
+      for (int k = 0; k < j.K; ++k) {
+        const uint32_t bits = (uint32_t)gh[k] << 16;
+        float f;
+        memcpy(&f, &bits, 4);
+        f = f < 0 ? -f : f;
+        if (f > gmax) gmax = f;
+      }
+      const float bound = gmax * sqrtf((float)j.K) * 1.01f;
+      if (bound > 32768.f && bound < 3.0e38f) {
+        int e;
+        (void)frexpf(bound, &e);
+        j.xscale = ldexpf(1.f, 15 - e);
+      }
+    }
+  }
+  const size_t esz = q ? 1 : 2;
+  size_t total = 0;
+  std::vector<size_t> offs;
+  for (auto& j : jobs) {
+    offs.push_back(total);
+    total += align_up((size_t)j.N * j.K * esz);
+  }
+  // weights_in_place: the caller hands the weight buffers over to the persistent kernel - every matrix is
+  // permuted where it lies (through one scratch buffer of the largest matrix, freed again), no second copy is
+  // kept, and the kernel-per-step form, which reads the row-major layout, is switched off for this model.
+  const bool in_place = c.weights_in_place != 0;
+  cudaError_t e2 = cudaSuccess;
+  unsigned char* scratch = nullptr;
+  if (in_place) {
+    size_t largest = 0;
+    for (auto& j : jobs) largest = std::max(largest, align_up((size_t)j.N * j.K * esz));
+    e2 = cudaMalloc(&scratch, largest);
+  } else {
+    e2 = cudaMalloc(&m->mega_weights, total);
+  }
+  if (e2 == cudaSuccess) e2 = cudaMalloc(&m->mega_jobs, jobs.size() * sizeof(MegaJob));
+  if (e2 == cudaSuccess) e2 = cudaMalloc(&m->mega_layers, mls.size() * sizeof(MegaLayer));
+  int rc2 = QUASAR_OK;
+  if (e2 == cudaSuccess) {
+    for (size_t i = 0; i < jobs.size() && rc2 == QUASAR_OK; ++i) {
+      if (in_place) {
+        void* w = const_cast<void*>(src[i]);
+        jobs[i].wp = w;
+        rc2 = launch_repack(src[i], scratch, jobs[i].N, jobs[i].K, jobs[i].kind, c.weight_dtype, ncta, 0);
+        if (rc2 == QUASAR_OK)
+          e2 = cudaMemcpyAsync(w, scratch, (size_t)jobs[i].N * jobs[i].K * esz, cudaMemcpyDeviceToDevice, 0);
+        if (e2 != cudaSuccess) break;
+      } else {
+        jobs[i].wp = m->mega_weights + offs[i];
+        rc2 = launch_repack(src[i], m->mega_weights + offs[i], jobs[i].N, jobs[i].K, jobs[i].kind, c.weight_dtype, ncta, 0);
+      }
+    }
+    if (rc2 == QUASAR_OK && e2 == cudaSuccess) e2 = cudaMemcpy(m->mega_jobs, jobs.data(), jobs.size() * sizeof(MegaJob), cudaMemcpyHostToDevice);
+    if (rc2 == QUASAR_OK && e2 == cudaSuccess) e2 = cudaMemcpy(m->mega_layers, mls.data(), mls.size() * sizeof(MegaLayer), cudaMemcpyHostToDevice);
+    if (rc2 == QUASAR_OK && e2 == cudaSuccess) e2 = cudaStreamSynchronize(0);
+  }
+  if (scratch) cudaFree(scratch);
+  if (e2 != cudaSuccess || rc2 != QUASAR_OK) {
+    if (e2 != cudaSuccess) set_error("tables of the persistent kernel (%zu bytes): %s", total, cudaGetErrorString(e2));
+    drop_persistent(m);
+    return e2 != cudaSuccess ? QUASAR_ERR_CUDA : rc2;
+  }
+  m->mega_ncta = ncta;
+  return QUASAR_OK;
 }
 
 int plan_replay(quasar_plan* p, cudaStream_t stream) {
@@ -557,111 +794,14 @@ int quasar_model_create(const quasar_config* cfg, const quasar_weights* w, quasa
     delete m;
     return rc;
   }
-  // The persistent kernel: its grid, a permuted copy of every matrix in the order each CTA streams it,
-  // and the table of the GEMMs of the pass in execution order.
-  int ncta = 0;
-  if (cfg->act_dtype == QUASAR_A_BF16 && mega_grid_size(cfg->weight_dtype, cfg->head_dim, &ncta) == QUASAR_OK && ncta > 0 &&
-      ncta <= kMaxGrid) {
-    std::vector<MegaJob> jobs;
-    std::vector<MegaLayer> mls;
-    std::vector<const void*> src;
-    const int qkv_w = (cfg->n_q_heads + 2 * cfg->n_kv_heads) * cfg->head_dim;
-    for (int l = 0; l < cfg->n_layers; ++l) {
-      const quasar_layer_weights& L = m->layers[l];
-      jobs.push_back({nullptr, q ? L.qkv_delta : nullptr, reinterpret_cast<const __nv_bfloat16*>(L.attn_norm), qkv_w,
-                      cfg->hidden, kJobQkv, 1.f});
-      src.push_back(L.qkv_w);
-      jobs.push_back({nullptr, q ? L.o_delta : nullptr, nullptr, cfg->hidden, cfg->n_q_heads * cfg->head_dim, kJobO, 1.f});
-      src.push_back(L.o_w);
-      jobs.push_back({nullptr, q ? L.gateup_delta : nullptr, reinterpret_cast<const __nv_bfloat16*>(L.mlp_norm),
-                      2 * cfg->ffn, cfg->hidden, kJobGateUp, 1.f});
-      src.push_back(L.gateup_w);
-      jobs.push_back({nullptr, q ? L.down_delta : nullptr, nullptr, cfg->hidden, cfg->ffn, kJobDown, 1.f});
-      src.push_back(L.down_w);
-      mls.push_back({reinterpret_cast<const __nv_bfloat16*>(cfg->qk_norm ? L.q_norm : nullptr),
-                     reinterpret_cast<const __nv_bfloat16*>(cfg->qk_norm ? L.k_norm : nullptr)});
-    }
-    jobs.push_back({nullptr, q ? w->lm_delta : nullptr, reinterpret_cast<const __nv_bfloat16*>(w->final_norm),
-                    cfg->vocab, cfg->hidden, kJobLm, 1.f});
-    src.push_back(w->lm_w);
-    if (mls.empty()) mls.push_back({nullptr, nullptr});
-    // Normed GEMMs feed h = x * r * gain with |x r| <= sqrt(K): a static power-of-two scale keeps h
-    // inside the fp16 range whatever the activations are (1 unless a gain is in the hundreds).
-    {
-      std::vector<uint16_t> gh;
-      for (auto& j : jobs) {
-        if (j.gain == nullptr) continue;
-        gh.resize(j.K);
-        if (cudaMemcpy(gh.data(), j.gain, (size_t)j.K * 2, cudaMemcpyDeviceToHost) != cudaSuccess) {
-          set_error("model_create: reading a norm gain failed: %s", cudaGetErrorString(cudaGetLastError()));
-          quasar_model_destroy(m);
-          return QUASAR_ERR_CUDA;
-        }
-        float gmax = 0.f;
-        for (int k = 0; k < j.K; ++k) {
-          const uint32_t bits = (uint32_t)gh[k] << 16;
-          float f;
-          memcpy(&f, &bits, 4);
-          f = f < 0 ? -f : f;
-          if (f > gmax) gmax = f;
-        }
-        const float bound = gmax * sqrtf((float)j.K) * 1.01f;
-        if (bound > 32768.f && bound < 3.0e38f) {
-          int e;
-          (void)frexpf(bound, &e);
-          j.xscale = ldexpf(1.f, 15 - e);
-        }
-      }
-    }
-    const size_t esz = q ? 1 : 2;
-    size_t total = 0;
-    std::vector<size_t> offs;
-    for (auto& j : jobs) {
-      offs.push_back(total);
-      total += align_up((size_t)j.N * j.K * esz);
-    }
-    // weights_in_place: the caller hands the weight buffers over to the persistent kernel - every matrix is
-    // permuted where it lies (through one scratch buffer of the largest matrix, freed again), no second copy is
-    // kept, and the kernel-per-step form, which reads the row-major layout, is switched off for this model.
-    const bool in_place = cfg->weights_in_place != 0;
-    cudaError_t e2 = cudaSuccess;
-    unsigned char* scratch = nullptr;
-    if (in_place) {
-      size_t largest = 0;
-      for (auto& j : jobs) largest = std::max(largest, align_up((size_t)j.N * j.K * esz));
-      e2 = cudaMalloc(&scratch, largest);
-    } else {
-      e2 = cudaMalloc(&m->mega_weights, total);
-    }
-    if (e2 == cudaSuccess) e2 = cudaMalloc(&m->mega_jobs, jobs.size() * sizeof(MegaJob));
-    if (e2 == cudaSuccess) e2 = cudaMalloc(&m->mega_layers, mls.size() * sizeof(MegaLayer));
-    int rc2 = QUASAR_OK;
-    if (e2 == cudaSuccess) {
-      for (size_t i = 0; i < jobs.size() && rc2 == QUASAR_OK; ++i) {
-        if (in_place) {
-          void* w = const_cast<void*>(src[i]);
-          jobs[i].wp = w;
-          rc2 = launch_repack(src[i], scratch, jobs[i].N, jobs[i].K, jobs[i].kind, cfg->weight_dtype, ncta, 0);
-          if (rc2 == QUASAR_OK)
-            e2 = cudaMemcpyAsync(w, scratch, (size_t)jobs[i].N * jobs[i].K * esz, cudaMemcpyDeviceToDevice, 0);
-          if (e2 != cudaSuccess) break;
-        } else {
-          jobs[i].wp = m->mega_weights + offs[i];
-          rc2 = launch_repack(src[i], m->mega_weights + offs[i], jobs[i].N, jobs[i].K, jobs[i].kind, cfg->weight_dtype, ncta, 0);
-        }
-      }
-      if (rc2 == QUASAR_OK && e2 == cudaSuccess) e2 = cudaMemcpy(m->mega_jobs, jobs.data(), jobs.size() * sizeof(MegaJob), cudaMemcpyHostToDevice);
-      if (rc2 == QUASAR_OK && e2 == cudaSuccess) e2 = cudaMemcpy(m->mega_layers, mls.data(), mls.size() * sizeof(MegaLayer), cudaMemcpyHostToDevice);
-      if (rc2 == QUASAR_OK && e2 == cudaSuccess) e2 = cudaStreamSynchronize(0);
-    }
-    if (scratch) cudaFree(scratch);
-    if (in_place && e2 == cudaSuccess && rc2 == QUASAR_OK) m->path = 2;
-    if (e2 != cudaSuccess || rc2 != QUASAR_OK) {
-      if (e2 != cudaSuccess) set_error("model_create: tables of the persistent kernel (%zu bytes): %s", total, cudaGetErrorString(e2));
+  // (weights_in_place: the matrices are permuted for the persistent kernel now; other models get its copy when it is asked for)
+  if (cfg->weights_in_place) {
+    rc = build_persistent(m);
+    if (rc != QUASAR_OK) {
       quasar_model_destroy(m);
-      return e2 != cudaSuccess ? QUASAR_ERR_CUDA : rc2;
+      return rc;
     }
-    m->mega_ncta = ncta;
+    if (m->mega_ncta > 0) m->path = 2;
   }
   *out = m;
   return QUASAR_OK;
@@ -673,6 +813,7 @@ int quasar_set_path(quasar_model* m, int32_t path) {
     set_error("set_path: this model's weights were permuted in place for the persistent kernel; only path 2 exists");
     return QUASAR_ERR_INVALID_ARG;
   }
+  if (path == 2 && m->mega_ncta == 0) TRY(build_persistent(m));
   m->path = path;
   return QUASAR_OK;
 }
@@ -694,9 +835,8 @@ int quasar_set_wait_budget(quasar_model* m, uint64_t budget_ns, int32_t test_ext
 
 int quasar_model_destroy(quasar_model* m) {
   if (m == nullptr) return QUASAR_OK;
-  if (m->mega_weights) cudaFree(m->mega_weights);
-  if (m->mega_jobs) cudaFree(m->mega_jobs);
-  if (m->mega_layers) cudaFree(m->mega_layers);
+  drop_call_graphs(m);
+  drop_persistent(m);
   if (m->rope_table) cudaFree(m->rope_table);
   delete m;
   return QUASAR_OK;
@@ -729,6 +869,10 @@ int quasar_verify(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, c
                   const int32_t* block_len, int32_t B, int32_t T_max, float* logits_out, int32_t* accept_len,
                   int32_t* bonus, int32_t* accept_path, void* workspace, size_t workspace_bytes, int32_t* status,
                   void* stream) {
+  int rc = QUASAR_OK;
+  if (replay_call(m, kv, tokens, parents, block_len, B, T_max, logits_out, accept_len, bonus, accept_path, workspace,
+                  workspace_bytes, status, (cudaStream_t)stream, &rc))
+    return rc;
   return verify_impl(m, kv, tokens, parents, block_len, B, T_max, logits_out, accept_len, bonus, accept_path, workspace,
                      workspace_bytes, status, (cudaStream_t)stream);
 }
@@ -802,26 +946,12 @@ int quasar_plan_create(quasar_model* m, const quasar_kv* kv, const int32_t* toke
                        workspace, workspace_bytes, status, s);
   if (rc == QUASAR_OK && cudaStreamSynchronize(s) != cudaSuccess) { set_error("plan_create: eager pass failed: %s", cudaGetErrorString(cudaGetLastError())); rc = QUASAR_ERR_CUDA; }
   if (rc == QUASAR_OK && !uses_persistent_kernel(m, B, T_max)) {
-    const long long before = quasar_kernel_launches();
-    cudaError_t e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
-    if (e != cudaSuccess) { set_error("plan_create: begin capture: %s", cudaGetErrorString(e)); rc = QUASAR_ERR_CUDA; }
-    if (rc == QUASAR_OK) {
-      rc = verify_impl(m, kv, tokens, parents, block_len, B, T_max, logits_out, accept_len, bonus, accept_path,
-                       workspace, workspace_bytes, status, s);
-      e = cudaStreamEndCapture(s, &p->graph);
-      if (rc == QUASAR_OK && e != cudaSuccess) { set_error("plan_create: end capture: %s", cudaGetErrorString(e)); rc = QUASAR_ERR_CUDA; }
-    }
-    p->kernels = (int)(quasar_kernel_launches() - before);
-    count_launch(-p->kernels);  // captured launches did not run
-    if (rc == QUASAR_OK) {
-      e = cudaGraphInstantiate(&p->exec, p->graph, 0);
-      if (e != cudaSuccess) { set_error("plan_create: instantiate: %s", cudaGetErrorString(e)); rc = QUASAR_ERR_CUDA; }
-    }
+    rc = capture_pass(m, kv, tokens, parents, block_len, B, T_max, logits_out, accept_len, bonus, accept_path, workspace,
+                      workspace_bytes, status, s, &p->exec, &p->kernels);
   }
   cudaStreamDestroy(s);
   if (rc != QUASAR_OK) {
     if (p->exec) cudaGraphExecDestroy(p->exec);
-    if (p->graph) cudaGraphDestroy(p->graph);
     delete p;
     return rc;
   }
@@ -841,7 +971,6 @@ int quasar_plan_launch(quasar_plan* p, void* stream) {
 int quasar_plan_destroy(quasar_plan* p) {
   if (p == nullptr) return QUASAR_OK;
   if (p->exec) cudaGraphExecDestroy(p->exec);
-  if (p->graph) cudaGraphDestroy(p->graph);
   delete p;
   return QUASAR_OK;
 }

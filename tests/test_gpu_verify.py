@@ -459,3 +459,28 @@ def test_full_product_tree_of_28_nodes(world):
     kv, buf, _ = _run_gpu(shape, gm, okv, tokens, parents, bl)
     assert int(buf.status[0]) == 0
     _check_against_oracle(shape, r, buf, bl)
+
+
+@pytest.mark.parametrize("rows", [1, 5, 64])
+def test_calls_that_come_back_are_replayed_and_still_read_their_inputs(world, rows):
+    """The third call with the same buffers is captured and replayed (the block is 1 row, a draft, the largest).  What the buffers
+    hold changes from call to call, and every call gives what a fresh set of buffers, run eagerly, gives; a tenth set of buffers
+    takes the place of the first, which then starts again; two streams may take turns."""
+    shape, om, gm, okv, root = world
+    gm.set_path(0)
+    rng = np.random.default_rng(rows)
+    kv = _kv_to_gpu(shape, okv, 1)
+    bufs = [binding.VerifyBuffers(gm, 1, rows) for _ in range(10)]
+    side = torch.cuda.Stream()
+    for turn in range(5):
+        for i, buf in enumerate(bufs if turn == 4 else bufs[:1]):
+            tokens = rng.integers(0, shape.vocab, (1, rows)).astype(np.int32)
+            _, want, _ = _run_gpu(shape, gm, okv, tokens, None, np.array([rows], np.int32))
+            buf.tokens.copy_(torch.from_numpy(tokens))
+            torch.cuda.synchronize()
+            with torch.cuda.stream(side if turn % 2 else torch.cuda.current_stream()):
+                binding.quasar_verify(gm, kv, buf)
+            torch.cuda.synchronize()
+            assert int(buf.status[0]) == 0
+            assert torch.equal(buf.logits, want.logits)
+            assert torch.equal(buf.accept_len, want.accept_len) and torch.equal(buf.bonus, want.bonus)
