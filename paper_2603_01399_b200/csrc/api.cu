@@ -15,6 +15,7 @@
 #include "megakernel.cuh"
 #include "tc_attention.cuh"
 #include "tc_linear.cuh"
+#include "tc_wide.cuh"
 
 namespace quasar {
 
@@ -304,7 +305,8 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
 
   // ---- one kernel per step.  Every kernel but the first is a dependent launch: it starts under the one in front of it (the
   //      linear layers ask for their first weights then) and waits by itself for what that one writes. ----
-  const OperandForm form = a8 ? kOperandCodes : wd == QUASAR_W_INT8 ? kOperandDigits : kOperandBf16;
+  const bool wide = wd == QUASAR_W_INT8 && !a8 && tc_wide_better(M);
+  const OperandForm form = a8 ? kOperandCodes : wd == QUASAR_W_INT8 && !wide ? kOperandDigits : kOperandBf16;
   const bool traced = m->trace_buf != nullptr;
   // the order of the norms' sums of squares: the W8A8 form keeps its two (a last bit there becomes quantisation steps)
   const int adders = form == kOperandBf16 || (a8 && (M > 72 || H > 8192 || F > 24576)) ? 256 : 1024;
@@ -320,6 +322,8 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
   // one linear layer of the pass on the operand its producer left: weight-only (Eq. 8) or the paper's W8A8 form (Eq. 9-10)
   auto linear = [&](const __nv_bfloat16* in, const void* w, const float* delta, int64_t N, int64_t K, void* out, bool out_f32,
                     const __nv_bfloat16* res, unsigned long long* keys) -> int {
+    if (wide)
+      return launch_tc_wide(in, reinterpret_cast<const int8_t*>(w), delta, M, N, K, out, out_f32, res, keys, status, true, stream);
     if (form == kOperandBf16)
       return launch_tc_linear_bf16(in, reinterpret_cast<const __nv_bfloat16*>(w), M, N, K, out, out_f32, res, keys, status, true, stream);
     const int8_t* wq = reinterpret_cast<const int8_t*>(w);
@@ -327,7 +331,7 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
       return launch_tc_linear_w8a8(op_q, op_scale, wq, delta, M, N, K, out, out_f32, res, nullptr, keys, status, true, stream);
     return launch_tc_linear_digits(op_q, op_scale, wq, delta, M, N, K, out, out_f32, res, keys, status, true, stream);
   };
-  const bool fuse = !traced && tc_fusable(form, M);   // RoPE and SwiGLU in the epilogues of the layers before them
+  const bool fuse = !traced && !wide && tc_fusable(form, M);   // RoPE and SwiGLU in the epilogues of the layers before them
   const AttnList list{kv->seq_len, block_len, bi.valid, ba.seq, bi.anc, B, T_max, Hkv, Hq / Hkv, kv->s_max, attn_nodes_per_tile(Hq / Hkv)};
   const AttnParts parts = tc_attention_parts(att, B, T_max, Hq, Hkv, D);
   auto norm_gain = [&](int l) {
@@ -372,6 +376,8 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
       TRY(launch_tc_gateup_swiglu(form, form == kOperandBf16 ? (const void*)h : op_q, op_scale, L.gateup_w, L.gateup_delta, M, F, H, act, act_max,
                                   L.down_smooth, status, stream));
       TRY(launch_operand(form, act, act_max, M, F, RowOperand{nullptr, op_q, op_scale, L.down_smooth}, stream));
+    } else if (wide && !traced) {
+      TRY(launch_tc_wide_swiglu(h, reinterpret_cast<const int8_t*>(L.gateup_w), L.gateup_delta, M, F, H, act, status, true, stream));
     } else {
       TRY(linear(h, L.gateup_w, L.gateup_delta, 2 * (int64_t)F, H, gu, false, nullptr, nullptr));
       TRY(launch_swiglu(form, gu, M, F, operand(act, L.down_smooth), stream));

@@ -12,6 +12,7 @@
 
 #include "common.cuh"
 #include "tc_linear.cuh"
+#include "tc_wide.cuh"
 
 namespace quasar {
 
@@ -188,11 +189,12 @@ int launch_linear(const __nv_bfloat16* x, const void* w, const float* delta, int
     return launch_tc_linear_bf16(x, reinterpret_cast<const __nv_bfloat16*>(w), M, N, K, y, y_is_f32, residual, nullptr, status, false,
                                  stream);
   const int8_t* wq = reinterpret_cast<const int8_t*>(w);
+  if (tc_wide_better(M)) return launch_tc_wide(x, wq, delta, M, N, K, y, y_is_f32, residual, nullptr, status, false, stream);
   const size_t ybytes = y_is_f32 ? 4 : 2;
   // rows whose digits fit behind the reserved start of the workspace: all of them, unless the workspace is smaller than
   // linear_workspace_bytes reports (the built-in one of linear_static)
-  const int64_t room = (int64_t)(workspace_bytes - kCounterBytes) - 512;
-  const int64_t fit = room > 0 ? room / (3 * K + 4) : 0;
+  const int64_t room = (int64_t)(workspace_bytes - kCounterBytes);
+  const int64_t fit = (int64_t)digit_bytes(M, K) <= room ? M : room > 512 ? (room - 512) / (3 * K + 4) : 0;
   if ((M <= 8 && K <= kSub) || fit < 1) {
     for (int64_t m0 = 0; m0 < M; m0 += 8) {
       GemmArgs a;

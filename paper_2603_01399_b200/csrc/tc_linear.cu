@@ -613,8 +613,8 @@ tc_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
   uint64_t* empty = full + S;
   uint64_t* acc_full = empty + S;        // [2] a tile's sums are complete
   uint64_t* acc_empty = acc_full + 2;    // [2] they have been read out
-  unsigned long long* s_best = reinterpret_cast<unsigned long long*>(acc_empty + 2);   // [256] arg-max keys of the row tile's rows
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_best + 256);
+  unsigned long long* s_best = reinterpret_cast<unsigned long long*>(acc_empty + 2);   // [4][256] arg-max keys of the row tile's rows, by quarter
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_best + 1024);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp: uniform)
@@ -636,7 +636,7 @@ tc_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     }
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-  if (threadIdx.x < 256) s_best[threadIdx.x] = 0ull;
+  for (int i = threadIdx.x; i < 1024; i += kThreadsTc) s_best[i] = 0ull;
   if (PAIR) {
     __syncwarp();
     cluster_arrive();
@@ -782,26 +782,34 @@ tc_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         } else {
           tmem_ld16(t0 + (uint32_t)r0, v);
         }
+        const int count = rows - r0;
+        float f[16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const int m = m0 + r0 + j;
-          if (r0 + j >= rows) break;
-          float f = finish<KIND>(v[j], KIND != kBf16 ? __ldg(a.dx + m) : 1.f, dw);
-          if (a.keys != nullptr) {   // the warp's largest value, its lowest channel on ties (NaNs never enter)
-            const bool in = live && f == f;
-            const uint32_t key = in ? (uint32_t)(argmax_key(f, 0) >> 32) : 0u;
-            const uint32_t top = __reduce_max_sync(0xffffffffu, key);
-            const unsigned who = __ballot_sync(0xffffffffu, in && key == top);
-            if (lane == 0 && who != 0u)
-              atomicMax(one_row_tile ? s_best + r0 + j : a.keys + m, ((unsigned long long)top << 32) | (unsigned long long)(0xffffffffu - (uint32_t)(n + __ffs(who) - 1)));
-          }
-          if (!live || a.y == nullptr) continue;
-          const size_t idx = (size_t)m * a.N + n;
-          if (KIND == kCodes && a.acc_out != nullptr) a.acc_out[idx] = (int)v[j];
-          if (a.res != nullptr) f = __bfloat162float(__float2bfloat16_rn(f)) + __bfloat162float(a.res[idx]);
-          if (a.y_is_f32) reinterpret_cast<float*>(a.y)[idx] = f;
-          else reinterpret_cast<__nv_bfloat16*>(a.y)[idx] = __float2bfloat16_rn(f);
+        for (int j = 0; j < 16; ++j) f[j] = finish<KIND>(v[j], KIND != kBf16 && j < count ? __ldg(a.dx + m0 + r0 + j) : 1.f, dw);
+        if (a.keys != nullptr) best16(f, live, n, count, s_best + q * 256 + r0);
+        if (a.y == nullptr) continue;
+        if (KIND == kCodes && a.acc_out != nullptr && live) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            if (j < count) a.acc_out[(size_t)(m0 + r0 + j) * a.N + n] = (int)v[j];
         }
+        uint16_t res[16];
+        if (a.res != nullptr) load_res16(res, a.res, live, (size_t)(m0 + r0), n, a.N, count);
+        store16(f, live, (size_t)(m0 + r0), n, a.N, count, a.y, a.y_is_f32 != 0, a.res != nullptr, res);
+      }
+      if (a.keys != nullptr && (!one_row_tile || u + step >= units)) {   // the row tile changes, or this was the last
+        asm volatile("bar.sync 1, 256;\n" ::: "memory");
+        const int t = (int)threadIdx.x - 64;
+        if (t < rows) {
+          unsigned long long k = 0;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            k = s_best[i * 256 + t] > k ? s_best[i * 256 + t] : k;
+            s_best[i * 256 + t] = 0;
+          }
+          if (k != 0) atomicMax(a.keys + m0 + t, k);
+        }
+        asm volatile("bar.sync 1, 256;\n" ::: "memory");
       }
       fence_before();
       __syncwarp();
@@ -810,11 +818,6 @@ tc_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         else mbar_arrive(acc_empty + buf);
       }
       if ((buf ^= 1) == 0) bph ^= 1u;
-    }
-    if (a.keys != nullptr && one_row_tile && first < units) {
-      asm volatile("bar.sync 1, 256;\n" ::: "memory");
-      const int t = (int)threadIdx.x - 64, m0 = row_of(first);
-      if (t < min(a.rows, a.M - m0) && s_best[t] != 0ull) atomicMax(a.keys + m0 + t, s_best[t]);
     }
   }
   __syncwarp();
@@ -928,7 +931,7 @@ TcPlan plan_stream(int64_t M, int64_t N, int64_t K, int kind, bool pair) {
   TcPlan p = plan_base(M, K, kind, pair);
   p.stream = 1;
   const int b_bytes = p.brows * (pair ? 64 : 128), stage = kAStage + b_bytes;
-  const int st = (int)((kMaxSmem - kSmemSlack - 2048) / stage);
+  const int st = (int)((kMaxSmem - kSmemSlack - 8192) / stage);
   p.stages = st > 10 ? 10 : st;
   const int group = pair ? 2 : 1, lanes = 148 / group;
   for (int c = 128; c >= 64; c -= 8) {
@@ -952,7 +955,7 @@ TcPlan plan_stream(int64_t M, int64_t N, int64_t K, int kind, bool pair) {
 
 template <int KIND, bool PAIR, int EPI>
 int launch_kind(const CUtensorMap& map_w, const CUtensorMap& map_x, const TcArgs& a, const TcPlan& p, bool pdl, cudaStream_t stream) {
-  const size_t smem = (size_t)p.stages * (kAStage + p.brows * (PAIR ? 64 : 128)) + kSmemSlack + (p.stream ? 2048 : 0);
+  const size_t smem = (size_t)p.stages * (kAStage + p.brows * (PAIR ? 64 : 128)) + kSmemSlack + (p.stream ? 8192 : 0);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = p.stream ? dim3((unsigned)p.ctas) : dim3((unsigned)(p.tiles * p.row_tiles), (unsigned)p.nsplit);
   cfg.blockDim = dim3(kThreadsTc);
@@ -1067,10 +1070,6 @@ int launch_any(int kind, const void* x, const float* dx, const void* w, const fl
 int kind_of(int form) { return form == kOperandDigits ? kDigits : form == kOperandCodes ? kCodes : kBf16; }
 
 }  // namespace
-
-bool tc_linear_usable(int64_t M, int64_t N, int64_t K) {
-  return M >= 1 && N >= 1 && K >= 16 && K % 16 == 0 && M <= (1 << 20) && N <= (1 << 30) && K <= (1 << 28);
-}
 
 // ---- activations as digit rows: row m of x becomes the rows 3 m .. 3 m + 2 of xd -------------------------------------
 __global__ void __launch_bounds__(kDigitThreads)

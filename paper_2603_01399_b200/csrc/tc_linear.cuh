@@ -6,8 +6,6 @@
 
 namespace quasar {
 
-bool tc_linear_usable(int64_t M, int64_t N, int64_t K);
-
 // The launchers below take `pdl`: launched as a dependent of the kernel in front of it on the stream, whose results are waited
 // for before the activations, the residual or y are touched; the WEIGHTS may be read before that, so a caller sets it only
 // where the kernel in front does not write them and was itself launched behind whatever did.
@@ -45,6 +43,54 @@ __device__ __forceinline__ unsigned long long argmax_key(float x, int idx) {
   uint32_t u = __float_as_uint(x);
   u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
   return ((unsigned long long)u << 32) | (unsigned long long)(0xffffffffu - (uint32_t)idx);
+}
+
+// Sixteen rows of a tile whose lanes are 32 neighbouring channels: rows r0 .. r0 + 15 of f, one channel (n) a lane.
+
+// The rows' arg-max over the warp's channels joins what the warp has seen of them so far: best [16] for the rows r0 .. (lane j
+// looks after row j, so nothing here is atomic).  NaNs never enter; of equal values the lowest channel does.
+__device__ __forceinline__ void best16(const float (&f)[16], bool live, int n, int count, unsigned long long* best) {
+  const int lane = threadIdx.x & 31;
+  uint32_t mine = 0u, at = 0u;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const uint32_t key = live && f[j] == f[j] ? (uint32_t)(argmax_key(f[j], 0) >> 32) : 0u;
+    const uint32_t top = __reduce_max_sync(0xffffffffu, key);
+    const unsigned who = __ballot_sync(0xffffffffu, key == top);
+    if (lane == j) { mine = top; at = (uint32_t)__ffs(who) - 1u; }
+  }
+  if (lane < count && mine != 0u) {   // (no value has the key 0: that of a negative NaN)
+    const unsigned long long k = ((unsigned long long)mine << 32) | (unsigned long long)(0xffffffffu - ((uint32_t)(n - lane) + at));
+    if (k > best[lane]) best[lane] = k;
+  }
+}
+
+// The rows to their places, y [.][N] from row m on.  (Rows, residual and type are told apart outside the loops: inside, a row
+// took a warp 175 cycles of one instruction waiting for another.)
+__device__ __forceinline__ void store16(float (&f)[16], bool live, size_t m, int n, int N, int count, void* y, bool f32, bool with_res,
+                                        const uint16_t (&res)[16]) {
+  if (!live) return;
+  if (with_res) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) f[j] = __bfloat162float(__float2bfloat16_rn(f[j])) + __uint_as_float((uint32_t)res[j] << 16);
+  }
+  if (f32) {
+    float* p = reinterpret_cast<float*>(y) + m * N + n;
+#pragma unroll
+    for (int j = 0; j < 16; ++j, p += N)
+      if (j < count) *p = f[j];
+  } else {
+    __nv_bfloat16* p = reinterpret_cast<__nv_bfloat16*>(y) + m * N + n;
+#pragma unroll
+    for (int j = 0; j < 16; ++j, p += N)
+      if (j < count) *p = __float2bfloat16_rn(f[j]);
+  }
+}
+
+__device__ __forceinline__ void load_res16(uint16_t (&r)[16], const __nv_bfloat16* res, bool live, size_t m, int n, int N, int count) {
+  const uint16_t* p = reinterpret_cast<const uint16_t*>(res) + m * N + n;
+#pragma unroll
+  for (int j = 0; j < 16; ++j, p += N) r[j] = live && j < count ? *p : (uint16_t)0;
 }
 
 constexpr int kDigitThreads = 256;

@@ -1,0 +1,95 @@
+"""Every kernel variant at the sizes where its split of the work can go wrong: one row and one channel more than a tile,
+remainders of the contraction, k-ranges, pairs of thread blocks, row tiles (needs a GPU)."""
+import pytest
+import torch
+
+from paper_2603_01399_b200 import binding, synth
+from tests.common import gpu_model
+
+pytestmark = pytest.mark.gpu
+
+
+def _within(y, x, w, scale, res=None):
+    """y against the float64 product.  fp32 accumulation: K products are added in K / 16 steps that may truncate, at most
+    2^-23 of the sum of magnitudes each, and the sums of up to 8 ranges join; a bf16 output rounds twice (2^-9 each) where a
+    residual is added."""
+    xd, wd = x.double(), w.double()
+    t = (xd @ wd.T) * scale
+    mag = (xd.abs() @ wd.abs().T) * scale.abs()
+    bound = mag * ((x.shape[1] / 16 + 24) * 2.0 ** -23)
+    if res is not None:
+        bound = bound + t.abs() * 2.0 ** -8
+        t = t + res.double()
+    if y.dtype == torch.bfloat16:
+        bound = bound + t.abs() * 2.0 ** -8
+    assert bool(((y.double() - t).abs() <= bound + 1e-30).all()), ((y.double() - t).abs() - bound).max()
+
+
+# rows: one tile of digit rows, its edge (80), wide blocks of one and more row tiles; channels: part of a tile, an odd count,
+# a tile and a bit, more tiles than SMs; contraction: one block with a tail, ranges, long
+SIZES = [(1, 129, 1040), (8, 40, 512), (9, 257, 16), (16, 4096, 4096), (17, 1000, 528), (72, 4104, 2064), (80, 24576, 256), (81, 333, 2064),
+         (81, 128, 16), (96, 4096, 4096), (128, 257, 1040), (176, 20480, 272), (193, 512, 4096), (256, 1001, 2048), (257, 4096, 1040), (512, 600, 4112)]
+
+
+@pytest.mark.parametrize("weights", ["int8", "bf16"])
+@pytest.mark.parametrize("m,n,k", SIZES)
+def test_linear_forms(m, n, k, weights):
+    x = synth.normal_bf16((m, k), 1.0, seed=m + n, device="cuda")
+    x[m // 2] *= 2.0 ** 60                     # a row of its own range
+    w = synth.normal_bf16((n, k), 0.02, seed=n + k, device="cuda")
+    scale = torch.ones(n, dtype=torch.float64, device="cuda")
+    q, d = w, None
+    if weights == "int8":
+        q, d = binding.quasar_quantize(w)
+        scale = d.double()
+    res = synth.normal_bf16((m, n), 1.0, seed=7, device="cuda")
+    _within(binding.quasar_linear(x, q, d, out_f32=True), x, q, scale)
+    _within(binding.quasar_linear(x, q, d, residual=res), x, q, scale, res)
+
+
+@pytest.mark.parametrize("m,n,k", [s for s in SIZES if s[0] <= 256])
+def test_w8a8_forms(m, n, k):
+    x = synth.normal_bf16((m, k), 1.0, seed=m + n, device="cuda")
+    q, d = binding.quasar_quantize(synth.normal_bf16((n, k), 0.02, seed=n + k, device="cuda"))
+    codes, dx = binding.quasar_quantize_activations(x, None)
+    y, acc = binding.quasar_linear_w8a8(x, None, q, d, out_f32=True, want_acc=True)
+    want = (codes.double() @ q.double().T)     # exact: below 2^53
+    assert torch.equal(acc.double(), want)
+    assert torch.equal(y, want.float() * (d[None, :] * dx[:, None]))
+
+
+@pytest.mark.parametrize("kind", ["int8", "bf16"])
+@pytest.mark.parametrize("name,rows", [("tiny", 10), ("tiny", 11), ("tiny_qknorm", 16), ("tiny_qknorm", 17), ("tiny", 64)])
+def test_a_batch_gives_what_its_sequences_give_alone(name, rows, kind):
+    """8 x rows block rows take other forms of the linear layers than rows do (fused epilogues up to 80 rows of digits and 128
+    otherwise, wide blocks beyond); the attention deals out more pieces than one.  Sums in another order: bf16 roundings,
+    1e-2 of the logits, as between the two forms of the pass."""
+    shape = synth.SHAPES[name]
+    s_max, B = 448, 8
+    m = gpu_model(shape, seed=0, int8=kind == "int8", max_seq=s_max)
+    lens = [0, 1, 127, 128, 129, 200, 300, 384]
+    kk, vv = synth.kv_prefix(shape, B, s_max, seed=3, device="cuda")
+    tokens = synth.uniform_tokens((B, rows), shape.vocab, 5).to(torch.int32)
+    block = [max(1, rows - 3 * b) for b in range(B)]
+
+    def run(which):
+        kv = binding.KVCache(shape, len(which), s_max, k=kk[:, which].contiguous(), v=vv[:, which].contiguous(),
+                             seq_len=torch.tensor([lens[b] for b in which], dtype=torch.int32, device="cuda"))
+        buf = binding.VerifyBuffers(m, len(which), rows)
+        buf.tokens.copy_(tokens[which])
+        buf.block_len.copy_(torch.tensor([block[b] for b in which], dtype=torch.int32))
+        binding.quasar_verify(m, kv, buf)
+        torch.cuda.synchronize()
+        assert int(buf.status[0]) == 0
+        return buf, kv
+
+    every, kv = run(list(range(B)))
+    for b in range(B):
+        alone, kv1 = run([b])
+        a, e = alone.logits[0, :block[b]].double(), every.logits[b, :block[b]].double()
+        assert float((a - e).norm() / a.norm()) <= 1e-2, b
+        p = lens[b]
+        for x, y in ((kv1.k, kv.k), (kv1.v, kv.v)):
+            u, v = x[:, 0, :, p:p + block[b]].double(), y[:, b, :, p:p + block[b]].double()
+            assert float((u - v).norm() / u.norm()) <= 1e-2, b
+            assert torch.equal(x[:, 0, :, :p], y[:, b, :, :p])
