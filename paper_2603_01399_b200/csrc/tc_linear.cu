@@ -797,19 +797,15 @@ tc_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         if (a.res != nullptr) load_res16(res, a.res, live, (size_t)(m0 + r0), n, a.N, count);
         store16(f, live, (size_t)(m0 + r0), n, a.N, count, a.y, a.y_is_f32 != 0, a.res != nullptr, res);
       }
-      if (a.keys != nullptr && (!one_row_tile || u + step >= units)) {   // the row tile changes, or this was the last
-        asm volatile("bar.sync 1, 256;\n" ::: "memory");
-        const int t = (int)threadIdx.x - 64;
-        if (t < rows) {
-          unsigned long long k = 0;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            k = s_best[i * 256 + t] > k ? s_best[i * 256 + t] : k;
-            s_best[i * 256 + t] = 0;
+      if (a.keys != nullptr && !one_row_tile) {   // the next tile is of other rows: the warp hands on what it has
+        __syncwarp();
+        for (int r0 = half * 16; r0 < rows; r0 += 32) {
+          unsigned long long& k = s_best[q * 256 + r0 + lane % 16];
+          if (lane < 16 && r0 + lane < rows && k != 0) {
+            atomicMax(a.keys + m0 + r0 + lane, k);
+            k = 0;
           }
-          if (k != 0) atomicMax(a.keys + m0 + t, k);
         }
-        asm volatile("bar.sync 1, 256;\n" ::: "memory");
       }
       fence_before();
       __syncwarp();
@@ -818,6 +814,16 @@ tc_stream_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
         else mbar_arrive(acc_empty + buf);
       }
       if ((buf ^= 1) == 0) bph ^= 1u;
+    }
+    if (a.keys != nullptr && one_row_tile && first < units) {
+      asm volatile("bar.sync 1, 256;\n" ::: "memory");   // (every epilogue warp comes here, one that has given up too)
+      const int t = (int)threadIdx.x - 64, m0 = row_of(first);
+      if (t < min(a.rows, a.M - m0)) {
+        unsigned long long k = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) k = s_best[i * 256 + t] > k ? s_best[i * 256 + t] : k;
+        if (k != 0) atomicMax(a.keys + m0 + t, k);
+      }
     }
   }
   __syncwarp();

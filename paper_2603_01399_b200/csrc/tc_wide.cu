@@ -323,23 +323,30 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
           if (a.y != nullptr) store16(f, live, (size_t)(m0 + r0), n, a.N, count, a.y, a.y_is_f32 != 0, a.res != nullptr, res);
         }
       }
-      if (a.keys != nullptr && (!one_row_tile || u + step >= a.units)) {   // the tile's rows change, or this was the last
-        asm volatile("bar.sync 1, 128;\n" ::: "memory");
-        for (int t = (int)threadIdx.x - 576; t < rows; t += 128) {
-          unsigned long long k = 0;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            k = s_best[i * 256 + t] > k ? s_best[i * 256 + t] : k;
-            s_best[i * 256 + t] = 0;
+      if (a.keys != nullptr && !one_row_tile) {   // the next tile is of other rows: the warp hands on what it has
+        __syncwarp();
+        for (int r0 = 0; r0 < rows; r0 += 16) {
+          unsigned long long& k = s_best[q * 256 + r0 + lane % 16];
+          if (lane < 16 && r0 + lane < rows && k != 0) {
+            atomicMax(a.keys + m0 + r0 + lane, k);
+            k = 0;
           }
-          if (k != 0) atomicMax(a.keys + m0 + t, k);
         }
-        asm volatile("bar.sync 1, 128;\n" ::: "memory");
       }
       fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(cluster_map(smem_u32(acc_empty + buf), leader));
       if (++buf == a.accs) { buf = 0; bph ^= 1u; }
+    }
+    if (a.keys != nullptr && one_row_tile && first < a.units) {
+      asm volatile("bar.sync 1, 128;\n" ::: "memory");   // (every epilogue warp comes here, one that has given up too)
+      const int m0 = row_of(first);
+      for (int t = (int)threadIdx.x - 576; t < min(a.rows, a.M - m0); t += 128) {
+        unsigned long long k = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) k = s_best[i * 256 + t] > k ? s_best[i * 256 + t] : k;
+        if (k != 0) atomicMax(a.keys + m0 + t, k);
+      }
     }
   }
   if (SPLIT && warp >= 2) {
