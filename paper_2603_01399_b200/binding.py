@@ -204,7 +204,7 @@ def quasar_linear_w8a8(x: torch.Tensor, s: Optional[torch.Tensor], w: torch.Tens
     acc = torch.empty((m, n), dtype=torch.int32, device=x.device) if want_acc else None
     nbytes = _sz(0)
     _check(lib().quasar_linear_w8a8_workspace_bytes(m, n, k, C.byref(nbytes)))
-    ws = torch.zeros(int(nbytes.value), dtype=torch.uint8, device=x.device)
+    ws = torch.empty(int(nbytes.value), dtype=torch.uint8, device=x.device)
     _check(lib().quasar_linear_w8a8(_ptr(x), _ptr(s), _ptr(w), _ptr(delta_w), m, n, k, _ptr(y), 1 if out_f32 else 0,
                                     _ptr(residual), _ptr(acc), _ptr(ws), ws.numel(), _stream()))
     return (y, acc) if want_acc else y

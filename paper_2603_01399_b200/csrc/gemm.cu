@@ -209,6 +209,9 @@ int launch_linear(const __nv_bfloat16* x, const void* w, const float* delta, int
     }
     return QUASAR_OK;
   }
+  bool done = false;
+  const int rc = launch_tc_linear_direct(x, wq, delta, M, N, K, y, y_is_f32, residual, status, &done, stream);
+  if (rc != QUASAR_OK || done) return rc;
   const int64_t step = fit < M ? fit : M;
   for (int64_t m0 = 0; m0 < M; m0 += step) {
     const int64_t rows = (M - m0) < step ? (M - m0) : step;

@@ -101,7 +101,13 @@ constexpr size_t kSmemSlack = 1024 + 256;       // alignment of the ring, barrie
 // and the matching up channels).
 enum TcEpilogue { kStore = 0, kRope = 1, kSwiglu = 2 };
 
+// DIRECT (digits, narrow blocks): the activations come as bf16, and every CTA makes the digit rows of its own k-range in its
+// shared memory while its weights are on their way, against the rows' maxima within the range.
+constexpr int kDirectRows = 6, kDirectBlocks = 16;   // rows of a block, and 128 of K each of a range, at most (8 rows: 10.3 us against 9.0)
+
 struct TcArgs {
+  const __nv_bfloat16* x;      // DIRECT: [M][K]
+  int K;
   const float* dx;             // [M] step sizes of the int8 activations
   const float* dw;             // [N] step sizes of the int8 weights
   void* y;                     // [M][N] bf16 or fp32, or nullptr: only the arg-max is wanted
@@ -142,7 +148,7 @@ struct RowPre {
 
 template <int KIND, int EPI>
 __device__ __forceinline__ void load_pre(RowPre<KIND, EPI>& p, const TcArgs& a, int m, int n, int n0) {
-  p.dx = KIND != kBf16 ? a.dx[m] : 1.f;
+  p.dx = KIND != kBf16 && a.dx != nullptr ? a.dx[m] : 1.f;   // (DIRECT: in the sums already)
   if (EPI == kSwiglu) {   // n: the unit
     const int F = a.N / 2;
     const bool in = n < F;
@@ -311,19 +317,22 @@ __device__ __forceinline__ void issue_stage(uint32_t d, uint64_t da, uint64_t db
 
 // PAIR: CTAs 2 i and 2 i + 1 of a cluster work as one on two neighbouring channel tiles.  Each brings its own weights and HALF
 // of the activation rows; the leader's MMAs (256 rows) read both CTAs' shared memory.
-template <int KIND, bool PAIR, int EPI>
+template <int KIND, bool PAIR, int EPI, bool DIRECT = false>
 __global__ void __launch_bounds__(kThreadsTc, 2)
 tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const TcArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // the swizzle repeats every 1024 bytes
   const int b_rows = PAIR ? a.brows / 2 : a.brows;   // of this CTA
   const int b_bytes = b_rows * 128;
-  const int stage_bytes = kAStage + b_bytes;
+  const int stage_bytes = kAStage + (DIRECT ? 0 : b_bytes);
   const int S = a.stages;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)S * stage_bytes);   // the stage's bytes have landed
+  unsigned char* x_s = smem + (size_t)S * stage_bytes;                            // DIRECT: the digit rows of the whole range
+  uint64_t* full = reinterpret_cast<uint64_t*>(x_s + (DIRECT ? (size_t)((a.kblocks + a.nsplit - 1) / a.nsplit) * b_bytes : 0));   // the stage's bytes have landed
   uint64_t* empty = full + S;             // its MMAs have read it
   uint64_t* accum_done = empty + S;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(accum_done + 1);
+  uint64_t* x_ready = accum_done + 1;     // DIRECT
+  float* s_dx = reinterpret_cast<float*>(x_ready + 1);   // DIRECT: powers of two of the rows
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_dx + kDirectRows);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp: uniform)
@@ -333,7 +342,7 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
   const int split = blockIdx.y;
   const int n0 = tile * a.chan, m0 = row_tile * a.rows;
   const int kb0 = (int)((long long)split * a.kblocks / a.nsplit), kb1 = (int)((long long)(split + 1) * a.kblocks / a.nsplit);
-  const uint32_t tx = (uint32_t)(a.chan * 128 + b_bytes);
+  const uint32_t tx = (uint32_t)(a.chan * 128 + (DIRECT ? 0 : b_bytes));
 
   if (threadIdx.x == 0) {
     *abort_flag = 0;
@@ -342,6 +351,7 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
       mbar_init(empty + s, 1);
     }
     mbar_init(accum_done, 1);
+    if (DIRECT) mbar_init(x_ready, 8);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   if (PAIR) {   // (also: the leader's barriers exist before the other CTA's loads arrive at them)
@@ -425,7 +435,7 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
             arm(s);
             load_w(s, kb);
           }
-          load_x(s, kb);
+          if (!DIRECT) load_x(s, kb);
         }
         __syncwarp();
         if (++s == S) { s = 0; ph ^= 1u; }
@@ -442,16 +452,17 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     if (pair_x == 0) {   // ---- MMA issuer ----
       const uint16_t mask = (uint16_t)(3u << (2 * split));
       const uint32_t id = idesc(KIND == kBf16 ? 1 : 2, 1, PAIR ? 2 * kTileN : kTileN, a.brows);
-      const uint64_t da0 = desc_sw128(smem), db0 = desc_sw128(smem + kAStage);
+      const uint64_t da0 = desc_sw128(smem), db0 = desc_sw128(DIRECT ? x_s : smem + kAStage);
       int s = 0;
       uint32_t ph = 0;
-      bool ok = true;
-      for (int kb = kb0; kb < kb1; ++kb) {
+      bool ok = !DIRECT || mbar_wait(x_ready, 0, abort_flag, a.error);
+      for (int kb = kb0; kb < kb1 && ok; ++kb) {
         if (!(ok = mbar_wait(full + s, ph, abort_flag, a.error))) break;
         fence_after();
         const uint64_t off = (uint64_t)((uint32_t)(s * stage_bytes) >> 4);
+        const uint64_t off_x = DIRECT ? (uint64_t)((uint32_t)((kb - kb0) * b_bytes) >> 4) : off;
         if (elect_one()) {
-          issue_stage<KIND, PAIR>(tmem_base, da0 + off, db0 + off, id, kb > kb0);
+          issue_stage<KIND, PAIR>(tmem_base, da0 + off, db0 + off_x, id, kb > kb0);
           if (PAIR) commit_pair(empty + s, mask);
           else commit(empty + s);
         }
@@ -471,6 +482,52 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     const int r = q * 32 + lane;
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
     pdl_wait();   // (what a row's finishing needs may come from the kernel in front)
+    if (DIRECT) {   // a warp a row: its part of the range in registers, the maximum, the digits
+      for (int m = warp - 2; m < min(a.rows, a.M - m0); m += 8) {
+        const uint4* row = reinterpret_cast<const uint4*>(a.x + (size_t)(m0 + m) * a.K + (size_t)kb0 * 128);
+        const int nvec = (min(a.K, kb1 * 128) - kb0 * 128) / 8, span = (kb1 - kb0) * 16;
+        uint4 v[kDirectBlocks / 2];
+#pragma unroll
+        for (int i = 0; i < kDirectBlocks / 2; ++i) v[i] = i * 32 + lane < nvec ? row[i * 32 + lane] : make_uint4(0, 0, 0, 0);
+        float amax = 0.f;
+#pragma unroll
+        for (int i = 0; i < kDirectBlocks / 2; ++i) {
+          const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) amax = fmaxf(amax, fmaxf(fabsf(__uint_as_float(w[e] << 16)), fabsf(__uint_as_float(w[e] & 0xffff0000u))));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+        float up, down;
+        digit_scale(amax, up, down);
+        bool bad = false;   // (fmaxf passes over NaNs)
+#pragma unroll
+        for (int i = 0; i < kDirectBlocks / 2; ++i) {
+          const int at = i * 32 + lane;   // eight elements: 16-byte chunk at / 2 of the range, its half at & 1
+          if (at >= span) break;
+          const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+          float f[8];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) { f[2 * e] = __uint_as_float(w[e] << 16); f[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u); }
+#pragma unroll
+          for (int e = 0; e < 8; ++e) bad |= f[e] != f[e];
+          uint2 d[3];
+          digits8(f, up, d);
+          unsigned char* block = x_s + (size_t)(at >> 4) * b_bytes;
+#pragma unroll
+          for (int p = 0; p < 3; ++p) {
+            const int r = 3 * m + p;
+            *reinterpret_cast<uint2*>(block + r * 128 + ((((at >> 1) & 7) ^ (r & 7)) << 4) + (at & 1) * 8) = d[p];
+          }
+        }
+        if (__any_sync(0xffffffffu, bad)) down = __int_as_float(0x7fc00000);
+        if (lane == 0) s_dx[m] = down;
+      }
+      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(x_ready);
+      asm volatile("bar.sync 1, 256;\n" ::: "memory");   // (s_dx)
+    }
     if (pre_m < r_end) load_pre<KIND, EPI>(pre, a, m0 + pre_m, pre_n, n0);
     if (__all_sync(0xffffffffu, mbar_wait(accum_done, 0, abort_flag, a.error))) {
       fence_after();
@@ -484,7 +541,7 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
             const long long total = ((long long)(int)d[3 * j + 2] << 16) + ((long long)(int)d[3 * j + 1] << 8) + (long long)(int)d[3 * j];
-            v[j] = __float_as_uint((float)total);
+            v[j] = __float_as_uint(DIRECT ? (float)total * (r0 + j < a.rows ? s_dx[r0 + j] : 0.f) : (float)total);
           }
         } else {
           tmem_ld16(lane_addr + (uint32_t)r0, v);
@@ -932,6 +989,36 @@ TcPlan plan_tiles(int64_t M, int64_t N, int64_t K, int kind, bool pair, int epi,
   return p;
 }
 
+// DIRECT: every tile or range at once, its digit rows beside the ring; false where they do not fit so
+bool plan_direct(int64_t M, int64_t N, int64_t K, const void* kernel, TcPlan* out) {
+  TcPlan p = plan_base(M, K, kDigits, false);
+  p.stream = 0;
+  if (M > kDirectRows) return false;
+  for (int s = 1; s <= 8 && s <= p.kblocks; ++s) {
+    const int kb = (p.kblocks + s - 1) / s;
+    if (kb > kDirectBlocks) continue;
+    const size_t rows_bytes = (size_t)kb * p.brows * 128, half = kMaxSmem / 2 - 1024 - kSmemSlack;
+    const int per_sm = half >= rows_bytes + 3 * kAStage ? 2 : 1;
+    const int st = (int)(((per_sm == 2 ? half : kMaxSmem - kSmemSlack) - rows_bytes) / kAStage);
+    const long long fit = per_sm == 1 ? max_clusters(kernel, s) : std::max(2 * max_clusters(kernel, s), max_clusters(kernel, (s + 1) / 2));
+    for (int c = 128; c >= 64; c -= 8) {
+      const long long tiles = (N + c - 1) / c;
+      if (tiles > fit) break;
+      const double ctas = (double)tiles * s;
+      const double cost = 4.0 + stages_us(p, kb, ctas > 148 ? ctas / 148 : 1.0, ctas, c, 0) + 0.15 * s;
+      if (p.nsplit == 0 || cost < p.cost * 0.99) {
+        p.cost = cost;
+        p.nsplit = s;
+        p.chan = c;
+        p.tiles = (int)tiles;
+        p.stages = st > 8 ? 8 : st;
+      }
+    }
+  }
+  *out = p;
+  return p.nsplit > 0;
+}
+
 // tiles in turn on one CTA (or pair) per SM
 TcPlan plan_stream(int64_t M, int64_t N, int64_t K, int kind, bool pair) {
   TcPlan p = plan_base(M, K, kind, pair);
@@ -959,9 +1046,10 @@ TcPlan plan_stream(int64_t M, int64_t N, int64_t K, int kind, bool pair) {
   return p;
 }
 
-template <int KIND, bool PAIR, int EPI>
+template <int KIND, bool PAIR, int EPI, bool DIRECT = false>
 int launch_kind(const CUtensorMap& map_w, const CUtensorMap& map_x, const TcArgs& a, const TcPlan& p, bool pdl, cudaStream_t stream) {
-  const size_t smem = (size_t)p.stages * (kAStage + p.brows * (PAIR ? 64 : 128)) + kSmemSlack + (p.stream ? 8192 : 0);
+  const size_t smem = (DIRECT ? (size_t)p.stages * kAStage + (size_t)((p.kblocks + p.nsplit - 1) / p.nsplit) * p.brows * 128
+                             : (size_t)p.stages * (kAStage + p.brows * (PAIR ? 64 : 128))) + kSmemSlack + (p.stream ? 8192 : 0);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = p.stream ? dim3((unsigned)p.ctas) : dim3((unsigned)(p.tiles * p.row_tiles), (unsigned)p.nsplit);
   cfg.blockDim = dim3(kThreadsTc);
@@ -986,7 +1074,7 @@ int launch_kind(const CUtensorMap& map_w, const CUtensorMap& map_x, const TcArgs
   if (p.stream)
     QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_stream_kernel<KIND, PAIR>, map_w, map_x, a, p.tiles / (PAIR ? 2 : 1) * p.row_tiles));
   else
-    QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_linear_kernel<KIND, PAIR, EPI>, map_w, map_x, a));
+    QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_linear_kernel<KIND, PAIR, EPI, DIRECT>, map_w, map_x, a));
   count_launch();
   return QUASAR_OK;
 }
@@ -1001,8 +1089,28 @@ constexpr Kernels kernels_of() {
           {(const void*)tc_stream_kernel<KIND, false>, (const void*)tc_stream_kernel<KIND, true>}};
 }
 
-// The plan of a layer: the quickest by estimate; a fused epilogue has the tiled form only.
+constexpr int kDirectPlan = 3;   // beside the epilogues, for plan_layer
+
+// The plan of a layer: the quickest by estimate; a fused epilogue has the tiled form only.  (A hundred estimates, 2 us of host
+// time, more than the launch: a thread keeps the plans of the last sizes it met.)
+int find_plan(int64_t M, int64_t N, int64_t K, int kind, int epi, TcPlan* out);
 int plan_layer(int64_t M, int64_t N, int64_t K, int kind, int epi, TcPlan* out) {
+  struct Kept { int64_t M, N, K; int kind, epi; TcPlan plan; };
+  static thread_local Kept kept[64] = {};
+  const uint64_t h = ((uint64_t)M * 0x9e3779b97f4a7c15ull) ^ ((uint64_t)N * 0xc2b2ae3d27d4eb4full) ^ ((uint64_t)K * 0x165667b19e3779f9ull) ^
+                     (uint64_t)(kind * 4 + epi) * 0xff51afd7ed558ccdull;
+  Kept& k = kept[h >> 58];
+  if (k.M != M || k.N != N || k.K != K || k.kind != kind || k.epi != epi) {
+    k.M = 0;
+    const int rc = find_plan(M, N, K, kind, epi, &k.plan);
+    if (rc != QUASAR_OK) return rc;
+    k.M = M; k.N = N; k.K = K; k.kind = kind; k.epi = epi;
+  }
+  *out = k.plan;
+  return QUASAR_OK;
+}
+
+int find_plan(int64_t M, int64_t N, int64_t K, int kind, int epi, TcPlan* out) {
   static const Kernels kernels[3] = {kernels_of<kDigits>(), kernels_of<kBf16>(), kernels_of<kCodes>()};
   static std::once_flag once;
   static cudaError_t set_up = cudaSuccess;
@@ -1016,8 +1124,13 @@ int plan_layer(int64_t M, int64_t N, int64_t K, int kind, int epi, TcPlan* out) 
         for (const void* t : k.tiles[p]) allow(t);
         allow(k.stream[p]);
       }
+    allow((const void*)tc_linear_kernel<kDigits, false, kStore, true>);
   });
   QUASAR_CUDA_CHECK(set_up);
+  if (epi == kDirectPlan) {
+    if (!plan_direct(M, N, K, (const void*)tc_linear_kernel<kDigits, false, kStore, true>, out)) out->nsplit = 0;
+    return QUASAR_OK;
+  }
   // A pair of CTAs halves what the activations add to an SM's intake; narrow blocks have too few of them for that to matter.
   TcPlan p = plan_tiles(M, N, K, kind, false, epi, kernels[kind].tiles[0][epi]);
   auto consider = [&](const TcPlan& q) { if (q.cost < p.cost) p = q; };
@@ -1073,6 +1186,16 @@ int launch_any(int kind, const void* x, const float* dx, const void* w, const fl
   return launch_layer(kind, kStore, Operand{x, dx, w, dw, M, N, K}, a, pdl, stream);
 }
 
+int launch_direct(const Operand& o, TcArgs a, const TcPlan& p, cudaStream_t stream) {
+  CUtensorMap map_w;
+  const int rc = make_map_sw128(&map_w, o.w, (uint64_t)o.N, (uint64_t)o.K, (uint32_t)p.chan);
+  if (rc != QUASAR_OK) return rc;
+  a.x = reinterpret_cast<const __nv_bfloat16*>(o.x); a.K = (int)o.K; a.dw = o.dw;
+  a.M = (int)o.M; a.N = (int)o.N; a.kblocks = p.kblocks; a.chan = p.chan; a.rows = p.rows; a.brows = p.brows;
+  a.row_tiles = p.row_tiles; a.nsplit = p.nsplit; a.stages = p.stages;
+  return launch_kind<kDigits, false, kStore, true>(map_w, map_w, a, p, false, stream);
+}
+
 int kind_of(int form) { return form == kOperandDigits ? kDigits : form == kOperandCodes ? kCodes : kBf16; }
 
 }  // namespace
@@ -1121,6 +1244,19 @@ int launch_tc_linear_digits(const int8_t* xd, const float* row_scale, const int8
                             int64_t K, void* y, bool y_is_f32, const __nv_bfloat16* residual, unsigned long long* keys,
                             int32_t* error, bool pdl, cudaStream_t stream) {
   return launch_any(kDigits, xd, row_scale, w, dw, M, N, K, y, y_is_f32, residual, nullptr, keys, error, pdl, stream);
+}
+
+int launch_tc_linear_direct(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t N, int64_t K, void* y, bool y_is_f32,
+                            const __nv_bfloat16* residual, int32_t* error, bool* done, cudaStream_t stream) {
+  *done = false;
+  if (M > kDirectRows) return QUASAR_OK;
+  TcPlan p;
+  const int rc = plan_layer(M, N, K, kDigits, kDirectPlan, &p);
+  if (rc != QUASAR_OK || p.nsplit == 0) return rc;
+  TcArgs a = {};
+  a.y = y; a.res = residual; a.error = error; a.y_is_f32 = y_is_f32 ? 1 : 0;
+  *done = true;
+  return launch_direct(Operand{x, nullptr, w, dw, M, N, K}, a, p, stream);
 }
 
 int launch_tc_linear_w8a8(const int8_t* xq, const float* dx, const int8_t* w, const float* dw, int64_t M, int64_t N, int64_t K,

@@ -20,6 +20,10 @@ int launch_tc_linear_digits(const int8_t* xd, const float* row_scale, const int8
                             int64_t K, void* y, bool y_is_f32, const __nv_bfloat16* residual, unsigned long long* keys, int32_t* error, bool pdl,
                             cudaStream_t stream);
 
+// the same on the bf16 rows themselves, in one launch, for blocks of up to 6 rows; *done false: not for this matrix, nothing launched
+int launch_tc_linear_direct(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t N, int64_t K, void* y, bool y_is_f32,
+                            const __nv_bfloat16* residual, int32_t* error, bool* done, cudaStream_t stream);
+
 // int8 weights, int8 activations with their step sizes (Eq. 8, Eq. 10); acc_out: the raw sums, or nullptr
 int launch_tc_linear_w8a8(const int8_t* xq, const float* dx, const int8_t* w, const float* dw, int64_t M, int64_t N, int64_t K,
                           void* y, bool y_is_f32, const __nv_bfloat16* residual, int32_t* acc_out, unsigned long long* keys, int32_t* error, bool pdl,
@@ -122,8 +126,8 @@ __device__ __forceinline__ void digit_scale(float amax, float& up, float& down) 
   }
 }
 
-// q as three balanced base-256 digits, q = d0 + 256 d1 + 65536 d2, each an int8: eight elements from k on, plane d at d * K
-__device__ __forceinline__ void write_digits8(const float (&f)[8], float up, int8_t* dst, int64_t K, int64_t k) {
+// q as three balanced base-256 digits, q = d0 + 256 d1 + 65536 d2, each an int8: eight elements, digit by digit
+__device__ __forceinline__ void digits8(const float (&f)[8], float up, uint2 (&out)[3]) {
   uint32_t p[3][2] = {{0u, 0u}, {0u, 0u}, {0u, 0u}};
 #pragma unroll
   for (int e = 0; e < 8; ++e) {
@@ -138,7 +142,14 @@ __device__ __forceinline__ void write_digits8(const float (&f)[8], float up, int
     p[2][e >> 2] |= (uint32_t)(a2 & 0xff) << (8 * (e & 3));
   }
 #pragma unroll
-  for (int d = 0; d < 3; ++d) *reinterpret_cast<uint2*>(dst + d * K + k) = make_uint2(p[d][0], p[d][1]);
+  for (int d = 0; d < 3; ++d) out[d] = make_uint2(p[d][0], p[d][1]);
+}
+// eight elements from k on, plane d at d * K
+__device__ __forceinline__ void write_digits8(const float (&f)[8], float up, int8_t* dst, int64_t K, int64_t k) {
+  uint2 p[3];
+  digits8(f, up, p);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) *reinterpret_cast<uint2*>(dst + d * K + k) = p[d];
 }
 #endif
 

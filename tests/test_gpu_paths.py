@@ -27,7 +27,7 @@ def _within(y, x, w, scale, res=None):
 
 # rows: one tile of digit rows, its edge (80), wide blocks of one and more row tiles; channels: part of a tile, an odd count,
 # a tile and a bit, more tiles than SMs; contraction: one block with a tail, ranges, long
-SIZES = [(1, 129, 1040), (8, 40, 512), (9, 257, 16), (16, 4096, 4096), (17, 1000, 528), (72, 4104, 2064), (80, 24576, 256), (81, 333, 2064),
+SIZES = [(1, 129, 1040), (1, 64, 528), (5, 4096, 4096), (6, 4096, 12288), (15, 1001, 2064), (8, 40, 512), (9, 257, 16), (16, 4096, 4096), (17, 1000, 528), (72, 4104, 2064), (80, 24576, 256), (81, 333, 2064),
          (81, 128, 16), (96, 4096, 4096), (128, 257, 1040), (176, 20480, 272), (193, 512, 4096), (256, 1001, 2048), (257, 4096, 1040), (512, 600, 4112)]
 
 
