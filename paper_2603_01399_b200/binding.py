@@ -7,6 +7,7 @@ the library has not been built, `lib()` raises.
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
 from typing import Dict, List, Optional
 
@@ -130,6 +131,14 @@ def _stream() -> int:
     return torch.cuda.current_stream().cuda_stream
 
 
+@functools.lru_cache(maxsize=512)
+def _bytes(query: str, *sizes: int) -> int:
+    """A workspace size, which depends on nothing but the sizes asked about."""
+    out = _sz(0)
+    _check(getattr(lib(), query)(*sizes, C.byref(out)))
+    return int(out.value)
+
+
 def kernel_launches() -> int:
     return int(lib().quasar_kernel_launches())
 
@@ -139,8 +148,8 @@ def quasar_quantize(w_bf16: torch.Tensor):
     """bf16 [N][K] on the device -> (int8 [N][K], fp32 [N])."""
     assert w_bf16.is_cuda and w_bf16.dtype == torch.bfloat16 and w_bf16.is_contiguous() and w_bf16.dim() == 2
     n, k = w_bf16.shape
-    q = torch.empty((n, k), dtype=torch.int8, device=w_bf16.device)
-    d = torch.empty((n,), dtype=torch.float32, device=w_bf16.device)
+    q = torch.empty(n, k, dtype=torch.int8, device=w_bf16.device)
+    d = torch.empty(n, dtype=torch.float32, device=w_bf16.device)
     _check(lib().quasar_quantize(_ptr(w_bf16), n, k, _ptr(q), _ptr(d), _stream()))
     return q, d
 
@@ -159,7 +168,7 @@ def quasar_linear(x: torch.Tensor, w: torch.Tensor, delta: Optional[torch.Tensor
     n = w.shape[0]
     wd = QUASAR_W_INT8 if w.dtype == torch.int8 else QUASAR_W_BF16
     if out is None:
-        out = torch.empty((m, n), dtype=torch.float32 if out_f32 else torch.bfloat16, device=x.device)
+        out = torch.empty(m, n, dtype=torch.float32 if out_f32 else torch.bfloat16, device=x.device)
     if workspace is None:
         workspace = torch.zeros(max(quasar_linear_workspace_bytes(m, n, k), 16), dtype=torch.uint8, device=x.device)
     _check(lib().quasar_linear(_ptr(x), _ptr(w), _ptr(delta), wd, m, n, k, _ptr(out), 1 if out_f32 else 0,
@@ -179,8 +188,8 @@ def quasar_smoothing_factors(act_absmax: torch.Tensor, w_bf16: torch.Tensor, alp
 def quasar_quantize_weights_smoothed(w_bf16: torch.Tensor, s: Optional[torch.Tensor]):
     """Q(W diag(s)^-1, delta_w): bf16 [N][K] (+ fp32 [K]) -> (int8 [N][K], fp32 [N])."""
     n, k = w_bf16.shape
-    q = torch.empty((n, k), dtype=torch.int8, device=w_bf16.device)
-    d = torch.empty((n,), dtype=torch.float32, device=w_bf16.device)
+    q = torch.empty(n, k, dtype=torch.int8, device=w_bf16.device)
+    d = torch.empty(n, dtype=torch.float32, device=w_bf16.device)
     _check(lib().quasar_quantize_weights_smoothed(_ptr(w_bf16), _ptr(s), n, k, _ptr(q), _ptr(d), _stream()))
     return q, d
 
@@ -188,8 +197,8 @@ def quasar_quantize_weights_smoothed(w_bf16: torch.Tensor, s: Optional[torch.Ten
 def quasar_quantize_activations(x_bf16: torch.Tensor, s: Optional[torch.Tensor]):
     """Q(X * s, delta_x) per token: bf16 [M][K] (+ fp32 [K]) -> (int8 [M][K], fp32 [M])."""
     m, k = x_bf16.shape
-    q = torch.empty((m, k), dtype=torch.int8, device=x_bf16.device)
-    d = torch.empty((m,), dtype=torch.float32, device=x_bf16.device)
+    q = torch.empty(m, k, dtype=torch.int8, device=x_bf16.device)
+    d = torch.empty(m, dtype=torch.float32, device=x_bf16.device)
     _check(lib().quasar_quantize_activations(_ptr(x_bf16), _ptr(s), m, k, _ptr(q), _ptr(d), _stream()))
     return q, d
 
@@ -200,11 +209,9 @@ def quasar_linear_w8a8(x: torch.Tensor, s: Optional[torch.Tensor], w: torch.Tens
     accumulators when want_acc)."""
     m, k = x.shape
     n = w.shape[0]
-    y = torch.empty((m, n), dtype=torch.float32 if out_f32 else torch.bfloat16, device=x.device)
-    acc = torch.empty((m, n), dtype=torch.int32, device=x.device) if want_acc else None
-    nbytes = _sz(0)
-    _check(lib().quasar_linear_w8a8_workspace_bytes(m, n, k, C.byref(nbytes)))
-    ws = torch.empty(int(nbytes.value), dtype=torch.uint8, device=x.device)
+    y = torch.empty(m, n, dtype=torch.float32 if out_f32 else torch.bfloat16, device=x.device)
+    acc = torch.empty(m, n, dtype=torch.int32, device=x.device) if want_acc else None
+    ws = torch.empty(_bytes("quasar_linear_w8a8_workspace_bytes", m, n, k), dtype=torch.uint8, device=x.device)
     _check(lib().quasar_linear_w8a8(_ptr(x), _ptr(s), _ptr(w), _ptr(delta_w), m, n, k, _ptr(y), 1 if out_f32 else 0,
                                     _ptr(residual), _ptr(acc), _ptr(ws), ws.numel(), _stream()))
     return (y, acc) if want_acc else y
@@ -213,8 +220,8 @@ def quasar_linear_w8a8(x: torch.Tensor, s: Optional[torch.Tensor], w: torch.Tens
 def quasar_quantize_int4(w_bf16: torch.Tensor):
     """bf16 [N][K] (K a multiple of 128) -> (packed uint8 [N][K/2], delta fp32 [N][K/128])."""
     n, k = w_bf16.shape
-    packed = torch.empty((n, k // 2), dtype=torch.uint8, device=w_bf16.device)
-    delta = torch.empty((n, k // 128), dtype=torch.float32, device=w_bf16.device)
+    packed = torch.empty(n, k // 2, dtype=torch.uint8, device=w_bf16.device)
+    delta = torch.empty(n, k // 128, dtype=torch.float32, device=w_bf16.device)
     _check(lib().quasar_quantize_int4(_ptr(w_bf16), n, k, _ptr(packed), _ptr(delta), _stream()))
     return packed, delta
 
@@ -224,13 +231,11 @@ def quasar_linear_w4(x: torch.Tensor, packed: torch.Tensor, delta: torch.Tensor,
     m, k = x.shape
     n = packed.shape[0]
     if out is None:
-        out = torch.empty((m, n), dtype=torch.float32 if out_f32 else torch.bfloat16, device=x.device)
-    if workspace is None:
-        nbytes = _sz(0)
-        _check(lib().quasar_linear_w4_workspace_bytes(m, n, k, C.byref(nbytes)))
-        workspace = torch.empty(max(int(nbytes.value), 16), dtype=torch.uint8, device=x.device)
+        out = torch.empty(m, n, dtype=torch.float32 if out_f32 else torch.bfloat16, device=x.device)
+    # (the call wants 16 bytes and keeps nothing there: without a workspace it is shown the output's address)
+    ws, ws_bytes = (out, 16) if workspace is None else (workspace, workspace.numel())
     _check(lib().quasar_linear_w4(_ptr(x), _ptr(packed), _ptr(delta), m, n, k, _ptr(out), 1 if out.dtype == torch.float32 else 0,
-                                  _ptr(residual), _ptr(workspace), workspace.numel(), _stream()))
+                                  _ptr(residual), _ptr(ws), ws_bytes, _stream()))
     return out
 
 
@@ -416,7 +421,7 @@ def quasar_kv_commit(model: Model, kv: KVCache, buf: VerifyBuffers, tree: bool =
 def quasar_ngram_draft(history: torch.Tensor, hist_len: torch.Tensor, gamma: int, k_min: int, k_max: int):
     """history int32 [B][S], hist_len int32 [B] -> (draft int32 [B][gamma], draft_len int32 [B])."""
     b, s = history.shape
-    draft = torch.empty((b, gamma), dtype=torch.int32, device=history.device)
+    draft = torch.empty(b, gamma, dtype=torch.int32, device=history.device)
     dlen = torch.empty(b, dtype=torch.int32, device=history.device)
     _check(lib().quasar_ngram_draft(_ptr(history), _ptr(hist_len), b, s, gamma, k_min, k_max, _ptr(draft), _ptr(dlen), _stream()))
     return draft, dlen
@@ -429,9 +434,7 @@ def quasar_accept_stochastic(logits: torch.Tensor, tokens: torch.Tensor, block_l
     b, t, v = logits.shape
     accept_len = torch.empty(b, dtype=torch.int32, device=logits.device)
     nxt = torch.empty(b, dtype=torch.int32, device=logits.device)
-    nbytes = _sz(0)
-    _check(lib().quasar_accept_stochastic_workspace_bytes(b, t, C.byref(nbytes)))
-    ws = torch.empty(int(nbytes.value), dtype=torch.uint8, device=logits.device)
+    ws = torch.empty(_bytes("quasar_accept_stochastic_workspace_bytes", b, t), dtype=torch.uint8, device=logits.device)
     _check(lib().quasar_accept_stochastic(_ptr(logits), _ptr(tokens), _ptr(block_len), _ptr(q_probs), b, t, v, temperature,
                                           _ptr(r_accept), _ptr(r_sample), _ptr(accept_len), _ptr(nxt), _ptr(ws), ws.numel(),
                                           _stream()))

@@ -14,6 +14,7 @@
 // accumulation per group, folded into the running sum with the group's step size.  The ranges of a channel block form a
 // cluster and add their sums through distributed shared memory in the order of the ranges.
 #include <algorithm>
+#include <mutex>
 
 #include "common.cuh"
 #include "quant.cuh"
@@ -80,11 +81,10 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1
 
 // eight packed codes -> four bf16 pairs (code i, code i + 4), i = 0..3
 __device__ __forceinline__ void nib8_to_bf16(uint32_t w, uint32_t (&out)[4]) {
-  const uint32_t u = w ^ 0x88888888u;                 // code + 8 in every nibble
   const __nv_bfloat162 bias = __floats2bfloat162_rn(136.f, 136.f);
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const uint32_t v = ((u >> (4 * i)) & 0x000F000Fu) | 0x43004300u;     // bf16 128 + (code + 8)
+    const uint32_t v = ((w >> (4 * i)) & 0x000F000Fu) ^ 0x43084308u;     // bf16 128 + (code + 8): code + 8 is the nibble with its top bit turned
     const __nv_bfloat162 r = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&v), bias);
     out[i] = *reinterpret_cast<const uint32_t*>(&r);
   }
@@ -237,27 +237,59 @@ __global__ void __launch_bounds__(kW4Threads) w4_gemm_kernel(W4Args a) {
   }
 }
 
+// Clusters of s CTAs with this much shared memory that the device holds at once (they lie within a group of SMs, so long ones
+// leave SMs unused).
+template <int NT>
+int w4_clusters(int s, int chunk, size_t smem) {
+  static std::mutex mu;
+  static int seen[9][64] = {};
+  std::lock_guard<std::mutex> lock(mu);
+  int& n = seen[s][chunk];
+  if (n == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1, (unsigned)s);
+    cfg.blockDim = dim3(kW4Threads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 1;
+    attr.val.clusterDim.y = (unsigned)s;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, w4_gemm_kernel<NT>, &cfg) != cudaSuccess) cudaGetLastError();
+    if (n < 1) n = 1;
+  }
+  return n;
+}
+
 template <int NT>
 int launch_w4_nt(W4Args a, cudaStream_t stream) {
+  static const cudaError_t set_up = cudaFuncSetAttribute(w4_gemm_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+  QUASAR_CUDA_CHECK(set_up);
   const int nblocks = (a.N + kW4BlockN - 1) / kW4BlockN, ngroups = a.K / kGroup;
-  // Ranges: two CTAs on an SM (296 at once); a launch takes waves * (groups of a range + what a range costs besides, about
-  // two groups).  No range shorter than three groups.
+  // Ranges: a launch takes the waves of clusters that the device holds at once - where they do not all fit, half a one more, as
+  // CTAs follow one another - times the groups of a range and what a range costs besides, about three groups.  No range shorter
+  // than three groups.  (us at 1 row by ranges 1 / 2 / 3 / 4 / 5 / 6 / 8: 24,576 x 4096 30 / 28 / 33 / 31 / 33 / 38 / 38; 6144 x 4096
+  // 21 / 15 / 15 / 13 / 12 / 15 / 15; 151,936 x 4096 111 / 121 / 146; at 64 rows, one CTA on an SM: 4096 x 4096 52 / 32 / 25 / 19 / 31.)
+  constexpr int kGroupBytes = NT * 8 * 256;
   double best = 0;
+  size_t smem = 0;
   a.nsplit = 0;
   for (int s = 1; s <= 8 && (s == 1 || ngroups / s >= 3); ++s) {
-    const double cost = (double)(((long long)nblocks * s + 295) / 296) * ((ngroups + s - 1) / s + 2);
-    if (a.nsplit == 0 || cost < best) { best = cost; a.nsplit = s; }
-  }
-  constexpr int kGroupBytes = NT * 8 * 256;
-  const int per = (ngroups + a.nsplit - 1) / a.nsplit;
-  int chunk = (96 * 1024) / kGroupBytes;
-  if (chunk > kW4Ahead) chunk = chunk / kW4Ahead * kW4Ahead;
-  a.chunk = std::min(chunk, per);
-  const size_t smem = std::max((size_t)a.chunk * kGroupBytes, (size_t)NT * 8 * kW4BlockN * 4);
-  static bool configured = false;
-  if (!configured) {
-    QUASAR_CUDA_CHECK(cudaFuncSetAttribute(w4_gemm_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
-    configured = true;
+    const int per = (ngroups + s - 1) / s;
+    int chunk = (96 * 1024) / kGroupBytes;
+    if (chunk > kW4Ahead) chunk = chunk / kW4Ahead * kW4Ahead;
+    chunk = std::min(chunk, per);
+    const size_t need = std::max((size_t)chunk * kGroupBytes, (size_t)NT * 8 * kW4BlockN * 4);
+    const double waves = (double)nblocks / w4_clusters<NT>(s, chunk, need);
+    const double cost = (waves > 1 ? waves + 0.5 : 1.0) * (per + 3);
+    if (a.nsplit == 0 || cost < best) {
+      best = cost;
+      a.nsplit = s;
+      a.chunk = chunk;
+      smem = need;
+    }
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)nblocks, (unsigned)a.nsplit);
