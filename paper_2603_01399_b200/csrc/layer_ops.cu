@@ -25,8 +25,8 @@ __global__ void rope_table_kernel(float2* table, int max_pos, int D, double thet
 // ---- QK-RMSNorm + RoPE + KV append: one warp per (row, head) --------------------------------
 template <int D>
 __global__ void __launch_bounds__(128) rope_append_kernel(const RopeArgs a, int n_items) {
-  tc::pdl_trigger();
   tc::pdl_wait();
+  tc::pdl_trigger();   // (only now: the attention reads before its own wait what the kernels in front of this one's predecessor left)
   const int item = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (item >= n_items) return;
   const int lane = threadIdx.x & 31;

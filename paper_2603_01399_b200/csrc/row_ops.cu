@@ -316,7 +316,7 @@ attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, Ro
   extern __shared__ __align__(16) unsigned char s_row[];   // this CTA's heads, bf16; then each warp's parts of a batch
   pdl_trigger();
   if (OP != kOperandBf16) tc::cluster_arrive();   // (every CTA of the cluster has started before one writes into another's memory)
-  pdl_wait();
+  if (!LIST) pdl_wait();   // (the list's description is older than the kernel in front, see tc_attention_kernel)
   const int rank = blockIdx.x % kMergeCtas, m = blockIdx.x / kMergeCtas, b = m / l.T_max, i = m % l.T_max;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
   const int Hq = l.Hkv * l.G, h0 = rank * Hq / kMergeCtas, h1 = (rank + 1) * Hq / kMergeCtas;
@@ -343,6 +343,7 @@ attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, Ro
     stride = ch.Rpad;
     row0 = i * l.G;
   }
+  if (LIST) pdl_wait();
   float* s_o = reinterpret_cast<float*>(s_row + (size_t)((Hq + kMergeCtas - 1) / kMergeCtas) * D * 2) + (size_t)warp * batch * D;
   for (int hq = h0 + warp; hq < h1; hq += warps) {
     uint32_t pk[kPer / 2];

@@ -161,9 +161,8 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;   // columns: S (then P) of group 0, of group 1, O of group 0, of group 1
-  if (threadIdx.x == 0) pdl_trigger();
-  pdl_wait();
-  // the sequences' places, fetched once and side by side (each role walks them on its own)
+  // The sequences' places, fetched once and side by side (each role walks them on its own).  They come from the pass's first
+  // kernel, which is complete: the kernel in front lets this one start only once it has waited for all before it.
   __shared__ AttnSeq s_seq[kShapes];
   __shared__ int s_total;
   for (int b = (int)threadIdx.x; b < min(a.list.B, kShapes); b += kThreadsA) s_seq[b] = a.list.seq[b];
@@ -171,13 +170,32 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   __syncthreads();
 
   Walk w(a.list, s_seq, s_total, (int)blockIdx.x);
+  if (warp != 0) pdl_wait();
   if (warp == 0) {
     // ---- TMA producer ----
     const uint64_t policy = l2_evict_first_policy();
     int s = 0, issued = 0, piece = 0;
     uint32_t ph = 0;
     bool ok = true;
-    while (ok && w.next(a.list)) {
+    auto load_kv = [&](int i, int row, bool v) {
+      unsigned char* at = ring + (size_t)i * kTile;
+      mbar_expect_tx(full + i, kTile);
+#pragma unroll
+      for (int c = 0; c < kSubs; ++c) tma_load_2d_hint(at + c * kSub, v ? &map_v : &map_k, c * 128, row, full + i, policy);
+    };
+    // the first piece's tiles that lie in the cached context do not depend on the kernel in front
+    bool more = w.next(a.list);
+    int early = 0;
+    if (more) {
+      const int P = a.list.seq_len[w.b], row0 = (w.b * a.list.Hkv + w.hk) * a.list.s_max + w.t0 * kKeys;
+      for (; early < min(2 * w.nt, kSlots) && (w.t0 + (early >> 1) + 1) * kKeys <= P; ++early) {
+        if (elect_one()) load_kv(early, row0 + (early >> 1) * kKeys, (early & 1) != 0);
+        __syncwarp();
+      }
+    }
+    pdl_wait();
+    if (lane == 0) pdl_trigger();
+    for (; ok && more; more = w.next(a.list)) {
       const int row0 = (w.b * a.list.Hkv + w.hk) * a.list.s_max + w.t0 * kKeys;
       const int qb = piece & 1;
       if (!(ok = mbar_wait(q_empty + qb, ((uint32_t)(piece >> 1) & 1u) ^ 1u, abort_flag, a.error))) break;
@@ -192,21 +210,19 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       for (int t = 0; t < w.nt && ok; ++t) {
 #pragma unroll 1
         for (int kv = 0; kv < 2; ++kv) {
-          if (!(ok = mbar_wait(empty + s, ph ^ 1u, abort_flag, a.error))) break;
-          if (elect_one()) {
-            unsigned char* at = ring + (size_t)s * kTile;
-            mbar_expect_tx(full + s, kTile);
-#pragma unroll
-            for (int c = 0; c < kSubs; ++c)
-              tma_load_2d_hint(at + c * kSub, kv == 0 ? &map_k : &map_v, c * 128, row0 + t * kKeys, full + s, policy);
+          if (issued >= early) {
+            if (!(ok = mbar_wait(empty + s, ph ^ 1u, abort_flag, a.error))) break;
+            if (elect_one()) load_kv(s, row0 + t * kKeys, kv != 0);
+            __syncwarp();
           }
-          __syncwarp();
           ++issued;
           if (++s == kSlots) { s = 0; ph ^= 1u; }
         }
       }
     }
     if (!ok) {   // given up: what is in flight lands (bounded) before the CTA leaves
+      for (; issued < early; ++issued)
+        if (++s == kSlots) { s = 0; ph ^= 1u; }
       for (int i = 0; i < min(kSlots, issued); ++i) {
         if (--s < 0) { s = kSlots - 1; ph ^= 1u; }
         const unsigned long long t0 = gtime_ns();

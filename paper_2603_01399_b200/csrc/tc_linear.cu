@@ -377,7 +377,8 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
   const uint32_t tmem_base = *tmem_slot;
   // Only now may the kernel behind this one start: a tcgen05 kernel further down the stream waits for this one while it
   // holds tensor memory, so every CTA here must have its own first.
-  if (threadIdx.x == 0) pdl_trigger();
+  // (With RoPE it is the attention, which counts on everything in front of THIS kernel being complete: see below.)
+  if (EPI != kRope && threadIdx.x == 0) pdl_trigger();
 
   // this CTA's share of the tile's rows: 32 threads a row and four channels a thread (SwiGLU: 16 threads a row, four units), the
   // warps that do nothing else first
@@ -482,6 +483,7 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constan
     const int r = q * 32 + lane;
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
     pdl_wait();   // (what a row's finishing needs may come from the kernel in front)
+    if (EPI == kRope && threadIdx.x == 64) pdl_trigger();
     if (DIRECT) {   // a warp a row: its part of the range in registers, the maximum, the digits
       for (int m = warp - 2; m < min(a.rows, a.M - m0); m += 8) {
         const uint4* row = reinterpret_cast<const uint4*>(a.x + (size_t)(m0 + m) * a.K + (size_t)kb0 * 128);
