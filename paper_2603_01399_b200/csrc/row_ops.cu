@@ -321,7 +321,7 @@ attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, Ro
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
   const int Hq = l.Hkv * l.G, h0 = rank * Hq / kMergeCtas, h1 = (rank + 1) * Hq / kMergeCtas;
   constexpr int kPer = D / 32;
-  __shared__ float4 s_part[kMergeWarps][32];   // per warp: the non-empty parts' (index, weight, sum)
+  __shared__ float4 s_part[kMergeWarps][64];   // per warp: the non-empty parts' (index, weight, sum)
   bool live;
   int n0 = 0, stride, tiles = 0, row_tiles = 0, unit0 = 0, seg0 = 0, row0;
   unsigned total = 1, ctas = 1;
@@ -368,22 +368,27 @@ attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, Ro
       } else {
         at0 = ((size_t)b * l.Hkv + hk) * ch.nchunk * ch.Rpad + row;
       }
-      float2 ml = lane < n ? __ldcg(&parts.ml[at0 + (size_t)lane * stride]) : make_float2(-INFINITY, 0.f);
-      float mx = ml.x;
-      for (int p = lane + 32; p < n; p += 32) mx = fmaxf(mx, __ldcg(&parts.ml[at0 + (size_t)p * stride].x));
+      auto part_ml = [&](int p) { return p < n ? __ldcg(&parts.ml[at0 + (size_t)p * stride]) : make_float2(-INFINITY, 0.f); };
+      float2 ml[2] = {part_ml(lane), part_ml(lane + 32)};   // (64 parts in one round trip: more are rare)
+      float mx = fmaxf(ml[0].x, ml[1].x);
+      for (int p = lane + 64; p < n; p += 32) mx = fmaxf(mx, __ldcg(&parts.ml[at0 + (size_t)p * stride].x));
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       float acc[kPer], den = 0.f;
 #pragma unroll
       for (int e = 0; e < kPer; ++e) acc[e] = 0.f;
-      for (int p0 = 0; p0 < n; p0 += 32) {
-        if (p0 > 0) ml = p0 + lane < n ? __ldcg(&parts.ml[at0 + (size_t)(p0 + lane) * stride]) : make_float2(-INFINITY, 0.f);
-        const float w = ml.x == -INFINITY ? 0.f : exp2f(ml.x - mx);
+      for (int p0 = 0; p0 < n; p0 += 64) {
+        if (p0 > 0) { ml[0] = part_ml(p0 + lane); ml[1] = part_ml(p0 + 32 + lane); }
         // the non-empty parts in a row (one without a visible key may never have been written)
-        const unsigned some = __ballot_sync(0xffffffffu, w != 0.f);
-        const int cnt = __popc(some);
+        int cnt = 0;
         __syncwarp();
-        if (w != 0.f) s_part[warp][__popc(some & ((1u << lane) - 1u))] = make_float4(__int_as_float(p0 + lane), w, ml.y, 0.f);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float w = ml[h].x == -INFINITY ? 0.f : exp2f(ml[h].x - mx);
+          const unsigned some = __ballot_sync(0xffffffffu, w != 0.f);
+          if (w != 0.f) s_part[warp][cnt + __popc(some & ((1u << lane) - 1u))] = make_float4(__int_as_float(p0 + 32 * h + lane), w, ml[h].y, 0.f);
+          cnt += __popc(some);
+        }
         __syncwarp();
         for (int j0 = 0; j0 < cnt; j0 += batch) {
           // the batch's copies in flight together (as loads into registers the compiler spreads them over their uses)
@@ -682,7 +687,7 @@ int launch_operand(int op, const __nv_bfloat16* x, const unsigned* row_max, int 
 }
 
 namespace {
-constexpr size_t kMergeMaxSmem = 216 * 1024;
+constexpr size_t kMergeMaxSmem = 208 * 1024;
 template <int OP, int D, bool LIST>
 int launch_merge(int warps, size_t smem, const AttnList& list, const AttnParts& parts, const AttnChunks& ch, int batch, int M,
                  const RowOperand& out, cudaStream_t stream) {
@@ -698,8 +703,11 @@ int launch_attention_merge(int op, const AttnList& list, const AttnParts& parts,
                            const RowOperand& out, cudaStream_t stream) {
   const int heads = (list.Hkv * list.G + kMergeCtas - 1) / kMergeCtas;   // of a CTA
   const int warps = heads < kMergeWarps ? heads : kMergeWarps;
-  const int batch = M <= 16 ? 16 : 8;   // few rows: round trips count; many: CTAs on an SM do
-  const size_t smem = (size_t)heads * D * 2 + (size_t)warps * batch * D * 4;
+  // few rows: round trips count (6 rows, 34 chunks of the W8A8 form: all at once), many: CTAs on an SM do
+  int batch = M > 16 ? 8 : chunks == nullptr ? 16 : std::min(40, std::max(16, chunks->nchunk));
+  auto bytes = [&] { return (size_t)heads * D * 2 + (size_t)warps * batch * D * 4; };
+  while (bytes() > kMergeMaxSmem && batch > 1) batch /= 2;
+  const size_t smem = bytes();
   if (smem > kMergeMaxSmem) { set_error("attention merge: %d query heads of %d", list.Hkv * list.G, D); return QUASAR_ERR_SHAPE; }
   const AttnChunks ch = chunks ? *chunks : AttnChunks{};
 #define MERGE_AS(OP, DD, LIST) return launch_merge<OP, DD, LIST>(warps, smem, list, parts, ch, batch, M, out, stream)
