@@ -90,14 +90,17 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 4) verify_attention_kernel(Att
   const int c = blockIdx.x / a.ngroups, group = blockIdx.x % a.ngroups;
   const int hk = blockIdx.y, b = blockIdx.z;
   tc::pdl_trigger();
-  tc::pdl_wait();
-  if (!a.bi.valid[b]) return;
+  // The kernel in front lets this one start once it has waited for all before it, so the blocks' description is there, and a chunk
+  // whose first keys all lie in the cached context can ask for them now; only the query rows and the block's keys are waited for.
   const int T = a.block_len[b];
   const int P = a.seq_len[b];
   const int Lk = P + T;
   const int key_begin = c * a.chunk;
   const int key_end = min(Lk, key_begin + a.chunk);
-  if (key_begin >= key_end) return;
+  if (!a.bi.valid[b] || key_begin >= key_end) {
+    tc::pdl_wait();   // (nobody's end may say that the kernels in front have ended)
+    return;
+  }
 
   const int G = a.Hq / a.Hkv;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -105,25 +108,6 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 4) verify_attention_kernel(Att
   const int g = lane >> 2, t = lane & 3;
   const int row_tile = group * nwarps + warp;
   const int qkv_w = (a.Hq + 2 * a.Hkv) * D;
-
-  // the two query rows of this thread: r = node * G + head-in-group
-  int node[2];
-  uint64_t anc[2];
-  uint32_t qf[kDSteps][4];
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int r = row_tile * 16 + g + 8 * h;
-    node[h] = r / G;
-    const bool ok = node[h] < T;
-    anc[h] = ok ? a.bi.anc[b * a.T_max + node[h]] : 0ull;
-    const __nv_bfloat16* qrow =
-        a.qkv + (size_t)(b * a.T_max + (ok ? node[h] : 0)) * qkv_w + (size_t)(hk * G + (r % G)) * D;
-#pragma unroll
-    for (int kd = 0; kd < kDSteps; ++kd) {
-      qf[kd][h] = ok ? *reinterpret_cast<const uint32_t*>(qrow + kd * 16 + 2 * t) : 0u;
-      qf[kd][h + 2] = ok ? *reinterpret_cast<const uint32_t*>(qrow + kd * 16 + 8 + 2 * t) : 0u;
-    }
-  }
 
   float o[D / 8][4];
 #pragma unroll
@@ -155,7 +139,28 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 4) verify_attention_kernel(Att
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
   };
-  stage_tile(0, key_begin);
+  const bool early = min(key_end, key_begin + kKeyTile) <= P;
+  if (early) stage_tile(0, key_begin);
+  tc::pdl_wait();
+  if (!early) stage_tile(0, key_begin);
+  // the two query rows of this thread: r = node * G + head-in-group
+  int node[2];
+  uint64_t anc[2];
+  uint32_t qf[kDSteps][4];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int r = row_tile * 16 + g + 8 * h;
+    node[h] = r / G;
+    const bool ok = node[h] < T;
+    anc[h] = ok ? a.bi.anc[b * a.T_max + node[h]] : 0ull;
+    const __nv_bfloat16* qrow =
+        a.qkv + (size_t)(b * a.T_max + (ok ? node[h] : 0)) * qkv_w + (size_t)(hk * G + (r % G)) * D;
+#pragma unroll
+    for (int kd = 0; kd < kDSteps; ++kd) {
+      qf[kd][h] = ok ? *reinterpret_cast<const uint32_t*>(qrow + kd * 16 + 2 * t) : 0u;
+      qf[kd][h + 2] = ok ? *reinterpret_cast<const uint32_t*>(qrow + kd * 16 + 8 + 2 * t) : 0u;
+    }
+  }
   int buf = 0;
   for (int k0 = key_begin; k0 < key_end; k0 += kKeyTile, buf ^= 1) {
     if (k0 + kKeyTile < key_end) {
