@@ -84,18 +84,15 @@ int quasar_quantize(const void* w_bf16, int64_t N, int64_t K, int8_t* q_out, flo
  * (QUASAR_W_BF16, delta ignored and may be NULL).  y: [M][N], bf16 or fp32
  * (y_is_f32).  residual: [M][N] bf16 or NULL; with a residual the product is
  * first rounded to bf16, then added, then rounded again (the order the decoder
- * layer uses).  y may alias residual.  M >= 1 (rows are processed in groups of
- * at most 72), K % 16 == 0, 1 <= N <= 1048576 (QUASAR_ERR_SHAPE beyond).
- * workspace: at least quasar_linear_workspace_bytes(M, N, K) bytes; its first
- * use must find its first 64 KiB zero-filled, and every call leaves it reusable by the next call of
- * any shape (the split-K arrival counters live in those 64 KiB and reset themselves).
- * Accumulation is fp32, or better: int8 weights with more than 8 rows run on the tcgen05 tensor
- * cores (fp16 operands - exact for bf16 rows scaled by a power of two - fp32 sums in tensor
- * memory); int8 weights with at most 8 rows on a matrix of at least 128 MiB run as an exact
- * integer contraction (the activation row as 21-bit fixed point against a power of two above its
- * largest magnitude).  Which kernel runs depends only on the shape and on whether the workspace
- * has the size quasar_linear_workspace_bytes reports (a smaller one that still fits the fp32
- * kernel is accepted); the kernels agree to fp32 accumulation accuracy, not bit for bit.
+ * layer uses).  y may alias residual.  M >= 1, K % 16 == 0, 1 <= N <= 1048576 (QUASAR_ERR_SHAPE beyond).
+ * workspace: at least quasar_linear_workspace_bytes(M, N, K) bytes; every call leaves it reusable by
+ * the next call of any shape.  (Its first 64 KiB are kept free, as before; nothing in it has to be zero.)
+ * Accumulation is fp32, or better.  int8 weights: up to 80 rows run as an exact integer contraction (the
+ * activation row as 21-bit fixed point against a power of two above its largest magnitude - of the row,
+ * or, up to 6 rows, of the part of the row that a thread block contracts), more as bf16 x bf16 with the
+ * weights converted exactly; up to 8 rows with K <= 512, or where the workspace has no room for the
+ * fixed-point rows, on the warp-level tensor cores.  Which kernel runs depends only on the shape and on
+ * the size of the workspace; the kernels agree to fp32 accumulation accuracy, not bit for bit.
  * ---------------------------------------------------------------------- */
 int quasar_linear_workspace_bytes(int64_t M, int64_t N, int64_t K, size_t* bytes_out /* host */);
 int quasar_linear(const void* x, const void* w, const float* delta, int32_t weight_dtype, int64_t M, int64_t N,
@@ -119,8 +116,8 @@ int quasar_linear(const void* x, const void* w, const float* delta, int32_t weig
  * quasar_linear_w8a8 (Eq. 8, Eq. 10): quantises x as above into the workspace, then
  *     Y_int32 = W_int8 x X_int8 (exact), Y = Y_int32 * (delta_w[n] * delta_x[m]) in fp32
  *     (+ residual as in quasar_linear).  acc_out: int32 [M][N] or NULL - the raw accumulators,
- *     for callers that want to check them.  K % 16 == 0; workspace as for quasar_linear
- *     (first 64 KiB zero on first use), size from quasar_linear_w8a8_workspace_bytes.
+ *     for callers that want to check them.  K % 16 == 0; workspace as for quasar_linear,
+ *     size from quasar_linear_w8a8_workspace_bytes.
  * All bit-exact in the integer codes and accumulators; K % 8 == 0 for the quantisers.
  * ---------------------------------------------------------------------- */
 int quasar_smoothing_factors(const float* act_absmax, const void* w_bf16, int64_t N, int64_t K, float alpha,
