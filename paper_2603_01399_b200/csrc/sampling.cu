@@ -19,6 +19,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "tc_common.cuh"
 
 namespace quasar {
 
@@ -82,6 +83,7 @@ __global__ void __launch_bounds__(kSegThreads)
 softmax_segment_kernel(const float* __restrict__ logits, const int32_t* __restrict__ block_len, int T_max, int V, int nseg,
                        int chunks, float inv_t, float2* __restrict__ part, unsigned* __restrict__ arrivals) {
   __shared__ float2 sh[kSegThreads / 32];
+  tc::pdl_trigger();
   const int s = blockIdx.x, i = blockIdx.y, b = blockIdx.z;
   if (s == 0 && i == 0 && threadIdx.x == 0) arrivals[b] = 0;
   if (i >= block_len[b]) return;
@@ -177,6 +179,7 @@ __global__ void __launch_bounds__(kSegThreads) draw_segment_kernel(DrawArgs a) {
     s_q[t_row] = q;
     s_r[t_row] = r;
   }
+  tc::pdl_wait();   // (what was fetched so far is older than the kernel in front)
   for (int i = threadIdx.x >> 4; i < (T + 1) / 2 * 2; i += kSegThreads / 16) {   // (both halves of a warp take every turn)
     const float2* p = a.part + ((size_t)b * a.T_max + i) * a.nseg;
     float2 v[kMaxSegments / 16];
@@ -380,9 +383,7 @@ int launch_accept_stochastic(const float* logits, const int32_t* tokens, const i
   softmax_segment_kernel<<<dim3(p.nseg, T_max, B), kSegThreads, 0, stream>>>(logits, block_len, T_max, V, p.nseg, p.chunks, a.inv_t,
                                                                              part, a.arrivals);
   QUASAR_LAUNCH_CHECK();
-  draw_segment_kernel<<<dim3(p.nseg, B), kSegThreads, 0, stream>>>(a);
-  QUASAR_LAUNCH_CHECK();
-  return QUASAR_OK;
+  return launch_dependent(draw_segment_kernel, dim3(p.nseg, B), dim3(kSegThreads), 0, true, stream, 1, a);
 }
 
 }  // namespace quasar
