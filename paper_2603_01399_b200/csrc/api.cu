@@ -308,8 +308,8 @@ int verify_impl(quasar_model* m, const quasar_kv* kv, const int32_t* tokens, con
   const bool wide = wd == QUASAR_W_INT8 && !a8 && tc_wide_better(M);
   const OperandForm form = a8 ? kOperandCodes : wd == QUASAR_W_INT8 && !wide ? kOperandDigits : kOperandBf16;
   const bool traced = m->trace_buf != nullptr;
-  // the order of the norms' sums of squares: the W8A8 form keeps its two (a last bit there becomes quantisation steps)
-  const int adders = form == kOperandBf16 || (a8 && (M > 72 || H > 8192 || F > 24576)) ? 256 : 1024;
+  // the order of the norms' sums of squares, for the W8A8 form: it keeps its two (a last bit there becomes quantisation steps)
+  const int adders = M > 72 || H > 8192 || F > 24576 ? 256 : 1024;
   BlockArgs ba{tokens, parents, block_len, kv->seq_len, B, T_max, kv->s_max, c.vocab, bi,
                reinterpret_cast<unsigned long long*>(wsp + ws.keys), status, reinterpret_cast<AttnSeq*>(wsp + ws.seq), Hkv,
                attn_nodes_per_tile(Hq / Hkv), reinterpret_cast<unsigned*>(wsp + ws.act_max), c.n_layers * M};
