@@ -397,6 +397,7 @@ attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, Ro
   }
   if (LIST) pdl_wait();
   float* s_o = reinterpret_cast<float*>(s_row + (size_t)((Hq + kMergeCtas - 1) / kMergeCtas) * D * 2) + (size_t)warp * batch * D;
+  float amax = 0.f;   // of the operand's values, head by head as they are made
   for (int hq = h0 + warp; hq < h1; hq += warps) {
     uint32_t pk[kPer / 2];
 #pragma unroll
@@ -472,34 +473,41 @@ attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, Ro
     uint32_t* dst = reinterpret_cast<uint32_t*>(s_row) + (hq - h0) * (D / 2) + lane * (kPer / 2);
 #pragma unroll
     for (int e = 0; e < kPer / 2; ++e) dst[e] = pk[e];
+    if (OP != kOperandBf16) {
+#pragma unroll
+      for (int e = 0; e < kPer / 2; ++e) {
+        float lo = __uint_as_float(pk[e] << 16), hi = __uint_as_float(pk[e] & 0xffff0000u);
+        if (OP == kOperandCodes && out.smooth != nullptr) {
+          const float2 f = __ldg(reinterpret_cast<const float2*>(out.smooth + hq * D + lane * kPer) + e);
+          lo = __fmul_rn(lo, f.x);
+          hi = __fmul_rn(hi, f.y);
+        }
+        amax = fmaxf(amax, fmaxf(fabsf(lo), fabsf(hi)));
+      }
+    }
+  }
+  if (OP != kOperandBf16) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+    if (lane == 0) s_buf[warp] = amax;
   }
   __syncthreads();
   const int nvec = (h1 - h0) * (D / 8), first = h0 * (D / 8);   // this CTA's 16-byte pieces of the row
   const int64_t width = (int64_t)Hq * D;
-  float amax = 0.f, f[8], s[8];
-  for (int v = threadIdx.x; v < nvec; v += blockDim.x) {
-    const uint4 y = reinterpret_cast<const uint4*>(s_row)[v];
-    if (out.y != nullptr) reinterpret_cast<uint4*>(out.y + (size_t)m * width)[first + v] = y;
-    unpack8(y, f);
-    if (OP == kOperandCodes) {
-      load_smooth8(out.smooth, first + v, s);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) f[e] = __fmul_rn(f[e], s[e]);
-    }
-#pragma unroll
-    for (int e = 0; e < 8; ++e) amax = fmaxf(amax, fabsf(f[e]));
+  float f[8], s[8];
+  if (out.y != nullptr) {
+    for (int v = threadIdx.x; v < nvec; v += blockDim.x)
+      reinterpret_cast<uint4*>(out.y + (size_t)m * width)[first + v] = reinterpret_cast<const uint4*>(s_row)[v];
   }
   if (OP == kOperandBf16) return;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-  if (lane == 0) s_buf[warp] = amax;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < warps; ++w) amax = fmaxf(amax, s_buf[w]);
-  }
   tc::cluster_wait();
-  amax = __shfl_sync(0xffffffffu, amax, 0);
-  if (threadIdx.x < kMergeCtas) tc::st_cluster_f32(tc::cluster_map(tc::smem_u32(s_amax + rank), threadIdx.x), amax);   // (warp 0 holds it)
+  if (warp == 0) {
+    amax = lane < warps ? s_buf[lane] : 0.f;
+#pragma unroll
+    for (int o = kMergeWarps / 2; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+    amax = __shfl_sync(0xffffffffu, amax, 0);
+    if (lane < kMergeCtas) tc::st_cluster_f32(tc::cluster_map(tc::smem_u32(s_amax + rank), (uint32_t)lane), amax);
+  }
   __syncwarp();
   tc::cluster_arrive();
   tc::cluster_wait();
