@@ -620,12 +620,12 @@ __device__ void lay_out_list(const BlockArgs& a) {
   if (lane == 0) a.seq[a.B] = AttnSeq{0, 0, units, segs};
 }
 
-// The pass's first kernel: CTA m < M gathers the embedding of row m into the residual stream and normalises it - or, with
-// ss_out [M], leaves its sum of squares -; CTA M does the bookkeeping, a warp per sequence in turn.
+// The pass's first kernel: CTA m < M gathers the embedding of row m into the residual stream and normalises it; CTA M does
+// the bookkeeping, a warp per sequence in turn.
 template <int OP, int V>
 __global__ void __launch_bounds__(kRowThreads)
 embed_norm_kernel(BlockArgs a, int M, const __nv_bfloat16* __restrict__ embed, __nv_bfloat16* x, const __nv_bfloat16* __restrict__ g,
-                  int nvec, float eps, int adders, RowOperand out, float* ss_out) {
+                  int nvec, float eps, int adders, RowOperand out) {
   __shared__ float s_buf[64];
   pdl_trigger();
   const int m = blockIdx.x;
@@ -649,20 +649,6 @@ embed_norm_kernel(BlockArgs a, int M, const __nv_bfloat16* __restrict__ embed, _
   const bool ok = tok >= 0 && tok < a.vocab;
   const uint4* src = reinterpret_cast<const uint4*>(embed) + (size_t)(ok ? tok : 0) * nvec;
   uint4* dst = reinterpret_cast<uint4*>(x) + (size_t)m * nvec;
-  if (ss_out != nullptr) {   // the layer behind normalises the row itself
-    float ss = 0.f;
-    for (int i = threadIdx.x; i < nvec; i += kRowThreads) {
-      const uint4 v = ok ? __ldg(src + i) : make_uint4(0, 0, 0, 0);
-      dst[i] = v;
-      float f[8];
-      unpack8(v, f);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) ss += f[e] * f[e];
-    }
-    ss = block_sum(ss, s_buf);
-    if (threadIdx.x == 0) ss_out[m] = ss;
-    return;
-  }
   norm_row<OP, V>(
       [&](int i, float (&f)[8]) {
         const uint4 v = ok ? __ldg(src + i) : make_uint4(0, 0, 0, 0);
@@ -756,7 +742,7 @@ size_t norm_smem(int nvec) { return turns_of(nvec) > 0 ? (size_t)nvec * 16 : 0; 
 }  // namespace
 
 int launch_embed_norm(int op, const BlockArgs& a, const __nv_bfloat16* embed, __nv_bfloat16* x, const __nv_bfloat16* g, int H, float eps,
-                      int adders, const RowOperand& out, float* ss_out, cudaStream_t stream) {
+                      int adders, const RowOperand& out, cudaStream_t stream) {
   const int nvec = H / 8, M = a.B * a.T_max;
   if (op == kOperandCodes) {
     static DeviceOnce once;
@@ -765,7 +751,7 @@ int launch_embed_norm(int op, const BlockArgs& a, const __nv_bfloat16* embed, __
                                         (const void*)embed_norm_kernel<kOperandCodes, 3>, (const void*)embed_norm_kernel<kOperandCodes, 6>});
     if (rc != QUASAR_OK) return rc;
   }
-  ROW_DISPATCH(embed_norm_kernel, M + 1, op == kOperandCodes ? norm_smem(nvec) : 0, false, stream, a, M, embed, x, g, nvec, eps, adders, out, ss_out)
+  ROW_DISPATCH(embed_norm_kernel, M + 1, op == kOperandCodes ? norm_smem(nvec) : 0, false, stream, a, M, embed, x, g, nvec, eps, adders, out)
 }
 
 int launch_norm(int op, const __nv_bfloat16* x, const __nv_bfloat16* g, int M, int H, float eps, int adders, const RowOperand& out, cudaStream_t stream) {

@@ -22,18 +22,9 @@ int launch_tc_linear_digits(const int8_t* xd, const float* row_scale, const int8
                             int64_t K, void* y, bool y_is_f32, const __nv_bfloat16* residual, unsigned long long* keys, int32_t* error, bool pdl,
                             cudaStream_t stream);
 
-// the same on the bf16 rows themselves, in one launch, for blocks of up to 8 rows; *done false: not for this matrix, nothing launched
+// the same on the bf16 rows themselves, in one launch, for blocks of up to 6 rows; *done false: not for this matrix, nothing launched
 int launch_tc_linear_direct(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t N, int64_t K, void* y, bool y_is_f32,
                             const __nv_bfloat16* residual, int32_t* error, bool* done, cudaStream_t stream);
-
-// The pass's layers of narrow blocks in that form (always dependent launches), for sizes that tc_direct_fits accepts: the layer
-// plain with its residual, leaving the sums of squares of the rows of y in `tiles` parts a row (ss_out [M][tiles], or nullptr);
-// and the qkv projection behind its RMSNorm - of rows whose sums of squares lie in ss [M][ss_parts] - with RoPE and cache append.
-bool tc_direct_fits(int64_t M, int64_t N, int64_t K, bool rope, int* tiles);
-int launch_tc_direct_layer(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t N, int64_t K, __nv_bfloat16* y,
-                           const __nv_bfloat16* residual, float* ss_out, int32_t* error, cudaStream_t stream);
-int launch_tc_direct_qkv_rope(const __nv_bfloat16* x, const __nv_bfloat16* gain, const float* ss, int ss_parts, float eps, const int8_t* w,
-                              const float* dw, int64_t M, int64_t K, const RopeArgs& rope, int32_t* error, cudaStream_t stream);
 
 // int8 weights, int8 activations with their step sizes (Eq. 8, Eq. 10); acc_out: the raw sums, or nullptr
 int launch_tc_linear_w8a8(const int8_t* xq, const float* dx, const int8_t* w, const float* dw, int64_t M, int64_t N, int64_t K,
