@@ -20,23 +20,13 @@ __device__ __forceinline__ QuantStep quant_step(float delta, bool has_nan) {
 }
 
 // f[e]: a float whose low mantissa bits hold round_half_even(v[e] / delta) in two's complement.
-// With the rounded reciprocal y of delta, v y is within 1.2e-5 of the rounded quotient (of up to 127.5: 2^-24 of it from y, 2^-24 of
-// it from the quotient's own rounding), so where v y is 2e-5 or more away from the middle between two integers, its nearest integer is
-// the quotient's.  Where one of the eight is nearer to a middle (one in 3,000 groups of eight of spread-out values; rows whose
-// maximum has the mantissa 254 / 256 meet exact middles all along), all eight take the correctly rounded quotient by Markstein's theorem (IBM J. Res. Dev. 34, 1990): with y the rounded reciprocal
+// The quotient is the correctly rounded one by Markstein's theorem (IBM J. Res. Dev. 34, 1990): with y the rounded reciprocal
 // of b, q an approximation of a / b within one unit in the last place and r = a - b q, exact by a fused multiply-add,
 // q + r y rounded once is a / b rounded.  The first step brings a y (within three units) to q, the second is the theorem's.
 // |v| <= limit * delta up to a rounding, so the integer needs no clamp.
 __device__ __forceinline__ void quantize8(const float (&v)[8], const QuantStep& s, int limit, float (&f)[8]) {
   constexpr float kMagic = 12582912.f;   // 1.5 * 2^23: adding it leaves the nearest integer, ties to even, in the low bits
   if (s.quick) {
-    float off = 0.f;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      f[e] = __fmaf_rn(v[e], s.inv, kMagic);
-      off = fmaxf(off, fabsf(__fmaf_rn(v[e], s.inv, -__fadd_rn(f[e], -kMagic))));
-    }
-    if (off <= 0.49998f) return;
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       float q = __fmul_rn(v[e], s.inv);

@@ -5,8 +5,6 @@
 // codes, 1 to 8 warps a row so that a lane holds up to 4 (12 on the longest rows) 16-byte pieces, all of them in flight at
 // once, and the quotients are rounded without a division (quant.cuh).  A CTA per row that read it twice and divided took
 // 88 us for 24,576 x 4096; the memory needs 47.
-#include <algorithm>
-
 #include "common.cuh"
 #include "quant.cuh"
 #include "tc_common.cuh"
@@ -19,9 +17,6 @@ constexpr int kQuantThreads = 256;
 constexpr int kQuantWarps = kQuantThreads / 32;
 
 enum SmoothMode { kPlain = 0, kDivide = 1, kMultiply = 2 };
-
-// CTAs of a kernel on an SM (what their registers allow): the grid is no larger
-constexpr int quant_ctas(int mode, int v) { return mode == kPlain ? (v <= 4 ? 4 : v <= 8 ? 2 : 1) : v <= 2 ? 4 : v <= 4 ? 2 : 1; }
 
 // the eight values of vector i, smoothed
 template <int MODE>
@@ -42,82 +37,71 @@ __device__ __forceinline__ void take_packed(__nv_bfloat162& m, const uint4& v) {
 
 __device__ __forceinline__ float step_of(float amax) { return amax == 0.f ? 1.0f : __fdiv_rn(amax, 127.0f); }
 
-// V pieces of 8 elements per lane, `wpr` warps per row (V * 32 * wpr pieces >= the row's).  A CTA takes its rows in turn and asks for
-// the next ones before it works on those it has.
+// V pieces of 8 elements per lane, `wpr` warps per row (V * 32 * wpr pieces >= the row's)
 template <int MODE, int V>
-__global__ void __launch_bounds__(kQuantThreads, quant_ctas(MODE, V))
+__global__ void __launch_bounds__(kQuantThreads)
 quantize_rows_kernel(const __nv_bfloat16* __restrict__ w, const float* __restrict__ s, int64_t N, int nvec, int wpr,
                      int8_t* __restrict__ q, float* __restrict__ delta) {
   tc::pdl_trigger();   // (the contraction that follows in quasar_linear_w8a8 asks for its weights meanwhile)
-  __shared__ uint2 s_max[2][kQuantWarps];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rows = kQuantWarps / wpr;   // rows of the CTA at a time
+  __shared__ uint2 s_max[kQuantWarps];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t n = (int64_t)blockIdx.x * (kQuantWarps / wpr) + warp / wpr;
+  const bool live = n < N;
   const int first = (warp % wpr) * 32 + lane, step = 32 * wpr;
+  const uint4* row = reinterpret_cast<const uint4*>(w) + (live ? n : 0) * nvec;
   uint4 raw[V];
-  auto fetch = [&](int64_t n) {
-    const uint4* row = reinterpret_cast<const uint4*>(w) + n * nvec;
 #pragma unroll
-    for (int j = 0; j < V; ++j) raw[j] = (n < N && first + j * step < nvec) ? __ldg(row + first + j * step) : make_uint4(0, 0, 0, 0);
-  };
-  int64_t n = (int64_t)blockIdx.x * rows + warp / wpr;
-  fetch(n);
-  int turn = 0;
-  const int64_t ahead = (int64_t)gridDim.x * rows;
-  for (int64_t n0 = (int64_t)blockIdx.x * rows; n0 < N; n0 += ahead, n += ahead, turn ^= 1) {
-    uint4 cur[V];
+  for (int j = 0; j < V; ++j) raw[j] = (live && first + j * step < nvec) ? __ldg(row + first + j * step) : make_uint4(0, 0, 0, 0);
+  float f[MODE == kPlain ? 1 : V][8];
+  AbsMax m;
+  if (MODE == kPlain) {
+    __nv_bfloat162 pm = __floats2bfloat162_rn(0.f, 0.f);
 #pragma unroll
-    for (int j = 0; j < V; ++j) cur[j] = raw[j];
-    if (n0 + ahead < N) fetch(n + ahead);
-    float f[MODE == kPlain ? 1 : V][8];
-    AbsMax m;
-    if (MODE == kPlain) {
-      __nv_bfloat162 pm = __floats2bfloat162_rn(0.f, 0.f);
-#pragma unroll
-      for (int j = 0; j < V; ++j) take_packed(pm, cur[j]);
-      m.take(__low2float(pm));
-      m.take(__high2float(pm));
-      if (m.has_nan()) {   // the largest of the numbers among them
-#pragma unroll
-        for (int j = 0; j < V; ++j) {
-          unpack_bf16x8(cur[j], f[0]);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) m.take(f[0][e]);
-        }
-      }
-    } else {
+    for (int j = 0; j < V; ++j) take_packed(pm, raw[j]);
+    m.take(__low2float(pm));
+    m.take(__high2float(pm));
+    if (m.has_nan()) {   // the largest of the numbers among them
 #pragma unroll
       for (int j = 0; j < V; ++j) {
-        float (&x)[8] = f[MODE == kPlain ? 0 : j];
-        unpack_bf16x8(cur[j], x);
-        if (first + j * step < nvec) smooth8<MODE>(x, s, first + j * step);
+        unpack_bf16x8(raw[j], f[0]);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) m.take(x[e]);
+        for (int e = 0; e < 8; ++e) m.take(f[0][e]);
       }
     }
-    m.num = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m.num)));   // (magnitudes order like their bits)
-    m.bits = __reduce_max_sync(0xffffffffu, m.bits);
-    if (wpr > 1) {   // (two sets in turn: one meeting of the CTA a turn)
-      if (lane == 0) s_max[turn][warp] = make_uint2(__float_as_uint(m.num), m.bits);
-      __syncthreads();
-      for (int i = 0; i < wpr; ++i) {
-        const uint2 o = s_max[turn][warp / wpr * wpr + i];
-        m.num = fmaxf(m.num, __uint_as_float(o.x));
-        m.bits = max(m.bits, o.y);
-      }
-    }
-    const QuantStep st = quant_step(step_of(m.num), m.has_nan());
-    if (n >= N) continue;
-    if (first == 0) delta[n] = st.delta;
-    uint2* qrow = reinterpret_cast<uint2*>(q) + n * nvec;
+  } else {
 #pragma unroll
     for (int j = 0; j < V; ++j) {
-      const int i = first + j * step;
-      if (i >= nvec) continue;
       float (&x)[8] = f[MODE == kPlain ? 0 : j];
-      if (MODE == kPlain) unpack_bf16x8(cur[j], x);
-      float c[8];
-      quantize8(x, st, 127, c);
-      qrow[i] = pack_codes8(c);
+      unpack_bf16x8(raw[j], x);
+      if (first + j * step < nvec) smooth8<MODE>(x, s, first + j * step);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) m.take(x[e]);
     }
+  }
+  m.num = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m.num)));   // (magnitudes order like their bits)
+  m.bits = __reduce_max_sync(0xffffffffu, m.bits);
+  if (wpr > 1) {
+    if (lane == 0) s_max[warp] = make_uint2(__float_as_uint(m.num), m.bits);
+    __syncthreads();
+    for (int i = 0; i < wpr; ++i) {
+      const uint2 o = s_max[warp / wpr * wpr + i];
+      m.num = fmaxf(m.num, __uint_as_float(o.x));
+      m.bits = max(m.bits, o.y);
+    }
+  }
+  const QuantStep st = quant_step(step_of(m.num), m.has_nan());
+  if (!live) return;
+  if (first == 0) delta[n] = st.delta;
+  uint2* qrow = reinterpret_cast<uint2*>(q) + n * nvec;
+#pragma unroll
+  for (int j = 0; j < V; ++j) {
+    const int i = first + j * step;
+    if (i >= nvec) continue;
+    float (&x)[8] = f[MODE == kPlain ? 0 : j];
+    if (MODE == kPlain) unpack_bf16x8(raw[j], x);
+    float c[8];
+    quantize8(x, st, 127, c);
+    qrow[i] = pack_codes8(c);
   }
 }
 
@@ -163,16 +147,15 @@ int launch_mode(const __nv_bfloat16* w, const float* s, int64_t N, int64_t K, in
   const int64_t nvec = K / 8;
   int wpr = 1;
   while (wpr < 8 && nvec > (int64_t)4 * 32 * wpr) wpr *= 2;
-  const int64_t ctas = (N + kQuantWarps / wpr - 1) / (kQuantWarps / wpr);
-  auto grid = [&](int v) { return (unsigned)std::min(ctas, (int64_t)148 * quant_ctas(MODE, v)); };
+  const unsigned grid = (unsigned)((N + kQuantWarps / wpr - 1) / (kQuantWarps / wpr));
   if (nvec <= (int64_t)2 * 32 * wpr)
-    quantize_rows_kernel<MODE, 2><<<grid(2), kQuantThreads, 0, stream>>>(w, s, N, (int)nvec, wpr, q, delta);
+    quantize_rows_kernel<MODE, 2><<<grid, kQuantThreads, 0, stream>>>(w, s, N, (int)nvec, wpr, q, delta);
   else if (nvec <= (int64_t)4 * 32 * wpr)
-    quantize_rows_kernel<MODE, 4><<<grid(4), kQuantThreads, 0, stream>>>(w, s, N, (int)nvec, wpr, q, delta);
+    quantize_rows_kernel<MODE, 4><<<grid, kQuantThreads, 0, stream>>>(w, s, N, (int)nvec, wpr, q, delta);
   else if (nvec <= (int64_t)8 * 32 * wpr)
-    quantize_rows_kernel<MODE, 8><<<grid(8), kQuantThreads, 0, stream>>>(w, s, N, (int)nvec, wpr, q, delta);
+    quantize_rows_kernel<MODE, 8><<<grid, kQuantThreads, 0, stream>>>(w, s, N, (int)nvec, wpr, q, delta);
   else if (nvec <= (int64_t)12 * 32 * wpr)
-    quantize_rows_kernel<MODE, 12><<<grid(12), kQuantThreads, 0, stream>>>(w, s, N, (int)nvec, wpr, q, delta);
+    quantize_rows_kernel<MODE, 12><<<grid, kQuantThreads, 0, stream>>>(w, s, N, (int)nvec, wpr, q, delta);
   else
     quantize_long_rows_kernel<MODE><<<(unsigned)N, kQuantThreads, 0, stream>>>(w, s, nvec, q, delta);
   QUASAR_LAUNCH_CHECK();
