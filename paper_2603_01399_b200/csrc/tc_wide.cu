@@ -18,11 +18,11 @@
 // LM head 675 -> 474 us (1.35); prompt chunks of 8 x 64 rows through the 8B model 12.5 -> 9.5 ms.  Tensor memory: accumulators of `brows` columns - two where that leaves room, so that a tile leaves
 // for memory under the next one's MMAs - and a ring of 32-column pieces of operand A.
 // Work split: units of 256 channels x one row tile.  Either in turn on one pair per SM pair; or, for matrices of few units, k-ranges
-// of a unit in the pairs of one cluster, added through distributed shared memory in the order of the ranges.  Where the units in turn
-// leave a last turn that few pairs take part in and the caller has memory for it, its units are shared instead, ahead of the whole
-// ones: cut along k into equal shares of stages, one a pair.  A share leaves its sums in global memory (L2); of a unit's sharers
-// the CTA that finishes last adds them, in the order of k, and finishes the rows, while its next unit is multiplied.  Nobody waits
-// for another CTA, and the result does not depend on which one is last.
+// of a unit in the pairs of one cluster, added through distributed shared memory in the order of the ranges; or, where the caller
+// has memory for it, shared: the units that make up no whole turn of all pairs - for a small matrix all there are - are cut along k
+// into equal shares of stages, one a pair.  A share leaves its sums in global memory (L2), and the CTA that finishes last of a
+// unit's sharers adds them, in the order of k, and finishes the rows: nobody waits for another CTA, and the result does not depend
+// on which one is last.
 //
 // Every wait is bounded (2 s): on expiry the CTA raises an error word, stops waiting everywhere, releases its tensor
 // memory and returns.
@@ -68,10 +68,10 @@ struct WideArgs {
 };
 
 // What is done with a unit's finished sums: stored; multiplied as gate and up units; or made q, k and v (QK-norm, RoPE, cache
-// append: only behind ranges, whose exchange leaves whole rows of a head to a warp)
+// append: only where all units are shared, for it takes whole rows of a head)
 enum WideEpilogue { kWideStore = 0, kWideSwiglu = 1, kWideRope = 2 };
 
-// A pair's way through its work: its share of the last turn, at most two pieces of units, then its whole units.
+// A pair's way through its work: its share of the rest, at most two pieces of units, then its whole units.
 struct WidePiece {
   int u, k0, k1;   // unit, stages
   int share;       // which piece of the share (0, 1), or -1: a whole unit (or the range of one)
@@ -147,52 +147,68 @@ __device__ __forceinline__ int channel_of(int n0, int r, int N) {
   return (r & 16) ? N / 2 + u : u;
 }
 
-// A shared unit's parts added and its rows finished, by the four epilogue warps (warp of 0 .. 3): two rows a warp at a time, four
-// channels a lane, four parts of each row asked for at once.
+// A shared unit's parts added and its rows finished, by all warps of the CTA: two rows a warp at a time, four channels a lane, four
+// parts of each row asked for at once.
 template <int EPI>
-__device__ __forceinline__ void finish_shared(const WideArgs& a, int u, int pair_x, int m0, int n0, int warp) {
-  constexpr int kRows = 2, kParts = 4;
-  const int lane = threadIdx.x & 31;
+__device__ __forceinline__ void finish_shared(const WideArgs& a, int u, int pair_x, int m0, int n0) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rows = min(a.rows, a.M - m0), F = a.N / 2;
   int p0, p1;
   wide_sharers(a, u, p0, p1);
-  const int parts = p1 - p0 + 1;
   const float* part0 = part_slot(a, p0, u, pair_x) + lane * 4;
   const size_t part_step = (size_t)2 * a.rows * 128;
   const int n = EPI == kWideSwiglu ? channel_of<true>(n0, lane * 4, a.N) : n0 + lane * 4;   // four neighbours either way
   const int unit = n0 / 2 + (lane >> 3) * 16 + (lane & 3) * 4;
-  const bool quad = (a.N & 3) == 0;   // (then four channels are inside or outside together, and aligned)
+  const bool up_lane = (lane & 4) != 0;
   float dw[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) dw[e] = (EPI == kWideSwiglu ? unit + e < F : n + e < a.N) ? __ldg(a.dw + n + e) : 1.f;
-#pragma unroll 1
-  for (int r0 = kRows * warp; r0 < rows; r0 += kRows * 4) {
-    float f[kRows][4];
+  constexpr int kTwo = EPI == kWideRope ? 1 : 2;
+  for (int r0 = kTwo * warp; r0 < rows; r0 += kTwo * (kThreadsW / 32)) {
+    float f[kTwo][4];
+    RopeRow rope;
+    if constexpr (EPI == kWideRope) rope_row_load(rope, a.rope, m0 + r0, n0);
+    uint2 res[kTwo];
+    const bool quad = (a.N & 3) == 0;   // (then four channels are inside or outside together, and aligned)
+    if (EPI == kWideStore && a.res != nullptr && quad) {
 #pragma unroll
-    for (int h = 0; h < kRows; ++h) f[h][0] = f[h][1] = f[h][2] = f[h][3] = 0.f;
-#pragma unroll 1
-    for (int q0 = 0; q0 < parts; q0 += kParts) {
-      float4 v[kParts][kRows];
+      for (int h = 0; h < kTwo; ++h)
+        if (r0 + h < rows && n < a.N) res[h] = *reinterpret_cast<const uint2*>(a.res + (size_t)(m0 + r0 + h) * a.N + n);
+    }
 #pragma unroll
-      for (int q = 0; q < kParts; ++q)
+    for (int h = 0; h < kTwo; ++h) f[h][0] = f[h][1] = f[h][2] = f[h][3] = 0.f;
+    for (int q0 = 0; q0 <= p1 - p0; q0 += 4) {
+      float4 v[4][kTwo];
 #pragma unroll
-        for (int h = 0; h < kRows; ++h)
-          v[q][h] = q0 + q < parts && r0 + h < rows ? __ldcg(reinterpret_cast<const float4*>(part0 + (q0 + q) * part_step + (size_t)(r0 + h) * 128))
-                                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int q = 0; q < 4; ++q)
 #pragma unroll
-      for (int q = 0; q < kParts; ++q)
+        for (int h = 0; h < kTwo; ++h)
+          if (q0 + q <= p1 - p0 && r0 + h < rows)
+            v[q][h] = __ldcg(reinterpret_cast<const float4*>(part0 + (q0 + q) * part_step + (size_t)(r0 + h) * 128));
 #pragma unroll
-        for (int h = 0; h < kRows; ++h) {
-          if (q0 + q >= parts) continue;
-          f[h][0] += v[q][h].x; f[h][1] += v[q][h].y; f[h][2] += v[q][h].z; f[h][3] += v[q][h].w;
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int h = 0; h < kTwo; ++h) {
+          if (q0 + q > p1 - p0 || r0 + h >= rows) continue;
+          const float w[4] = {v[q][h].x, v[q][h].y, v[q][h].z, v[q][h].w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) f[h][e] = q0 + q == 0 ? w[e] : f[h][e] + w[e];
         }
     }
 #pragma unroll
-    for (int h = 0; h < kRows; ++h) {
+    for (int h = 0; h < kTwo; ++h) {
       const int m = m0 + r0 + h;
       if (r0 + h >= rows) break;
 #pragma unroll
       for (int e = 0; e < 4; ++e) f[h][e] *= dw[e];
+      if constexpr (EPI == kWideRope) {
+        float b[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) b[e] = round_bf16(f[h][e]);
+        if (a.rope.D == 128) rope_row_store<128>(a.rope, b, m, n0, rope);
+        else rope_row_store<64>(a.rope, b, m, n0, rope);
+        continue;
+      }
       if constexpr (EPI == kWideSwiglu) {
         float o[4];
 #pragma unroll
@@ -200,7 +216,7 @@ __device__ __forceinline__ void finish_shared(const WideArgs& a, int u, int pair
           const float t = round_bf16(f[h][e]), other = __shfl_xor_sync(0xffffffffu, t, 4);
           o[e] = t / (1.0f + expf(-t)) * other;
         }
-        if ((lane & 4) == 0 && unit < F) {   // (gate lanes; F is a multiple of 16)
+        if (!up_lane && unit < F) {   // (F is a multiple of 16)
           const __nv_bfloat162 lo = __floats2bfloat162_rn(o[0], o[1]), hi = __floats2bfloat162_rn(o[2], o[3]);
           *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.y) + (size_t)m * F + unit) =
               make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
@@ -224,8 +240,14 @@ __device__ __forceinline__ void finish_shared(const WideArgs& a, int u, int pair
         if (lane == 0 && best != 0) atomicMax(a.keys + m, best);
       }
       if (a.y == nullptr) continue;
-      if (quad && a.res == nullptr) {
+      if (quad) {
         if (n >= a.N) continue;
+        if (a.res != nullptr) {
+          f[h][0] = round_bf16(f[h][0]) + __uint_as_float(res[h].x << 16);
+          f[h][1] = round_bf16(f[h][1]) + __uint_as_float(res[h].x & 0xffff0000u);
+          f[h][2] = round_bf16(f[h][2]) + __uint_as_float(res[h].y << 16);
+          f[h][3] = round_bf16(f[h][3]) + __uint_as_float(res[h].y & 0xffff0000u);
+        }
         if (a.y_is_f32) {
           *reinterpret_cast<float4*>(reinterpret_cast<float*>(a.y) + idx) = make_float4(f[h][0], f[h][1], f[h][2], f[h][3]);
         } else {
@@ -247,7 +269,7 @@ __device__ __forceinline__ void finish_shared(const WideArgs& a, int u, int pair
   }
 }
 
-// SPLIT: k-ranges in a cluster (not SwiGLU)
+// SPLIT: k-ranges in a cluster (kWideStore only)
 template <bool SPLIT, int EPI>
 __global__ void __launch_bounds__(kThreadsW, 1)
 tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const WideArgs a) {
@@ -270,7 +292,7 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_best + 1024);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   int* s_out = reinterpret_cast<int*>(tmem_slot + 2);   // [2] of the share's first, second piece: warps whose sums are out;
-  volatile int* s_finish = s_out + 2;                   // [2] 2 where this CTA is its unit's last, 1 where it is not
+  volatile int* s_finish = s_out + 2;                   // [2] whether this CTA is its unit's last
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp: uniform)
   const int pair_x = (int)blockIdx.x & 1;
@@ -457,6 +479,7 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     // ---- epilogue: a thread one channel, 16 rows at a time ----
     const int q = warp & 3, r = q * 32 + lane;
     pdl_wait();   // the residual comes from a kernel in front
+    if (EPI == kWideRope && threadIdx.x == 576) pdl_trigger();
     const bool one_row_tile = step % a.row_tiles == 0;
     int buf = 0;
     uint32_t bph = 0;
@@ -482,7 +505,7 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         }
         __threadfence();
       }
-      for (int r0 = 0; p.share < 0 && r0 < rows; r0 += 16) {
+      for (int r0 = 0; EPI != kWideRope && p.share < 0 && r0 < rows; r0 += 16) {
         uint32_t v[16];
         tmem_ld16_async(t0 + (uint32_t)r0, v);
         const int count = rows - r0;
@@ -523,21 +546,15 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(cluster_map(smem_u32(acc_empty + buf), leader));
       if (++buf == a.accs) { buf = 0; bph ^= 1u; }
-      if (p.share >= 0) {
-        if (lane == 0 && atomicAdd(s_out + p.share, 1) == 3) {   // the four warps' sums are out
-          __threadfence();
-          int p0, p1;
-          wide_sharers(a, u, p0, p1);
-          unsigned* count = a.arrived + 2 * (u - a.whole) + pair_x;
-          const bool last = p0 == p1 || (int)atomicAdd(count, 1u) == p1 - p0;
-          if (last && p0 != p1) *count = 0u;
-          __threadfence();
-          s_finish[p.share] = last ? 2 : 1;
-        }
-        int state = 0;
-        const unsigned long long t0 = gtime_ns();
-        while ((state = s_finish[p.share]) == 0 && *abort_flag == 0 && gtime_ns() - t0 < kBudgetNs) {}   // (another warp is on its way there)
-        if (__all_sync(0xffffffffu, state == 2)) finish_shared<EPI>(a, u, pair_x, m0, n0, warp - 18);
+      if (p.share >= 0 && lane == 0 && atomicAdd(s_out + p.share, 1) == 3) {   // the four warps' sums are out
+        __threadfence();
+        int p0, p1;
+        wide_sharers(a, u, p0, p1);
+        unsigned* count = a.arrived + 2 * (u - a.whole) + pair_x;
+        const bool last = p0 == p1 || (int)atomicAdd(count, 1u) == p1 - p0;
+        if (last && p0 != p1) *count = 0u;
+        __threadfence();
+        s_finish[p.share] = last ? 1 : 0;
       }
     }
     if (a.keys != nullptr && one_row_tile && first < a.whole) {
@@ -550,10 +567,6 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         if (k != 0) atomicMax(a.keys + m0 + t, k);
       }
     }
-  }
-  if (SPLIT && EPI == kWideRope && warp == 18) {   // (see the trigger above)
-    pdl_wait();
-    if (lane == 0) pdl_trigger();
   }
   if (SPLIT && warp >= 2) {
     // ---- this range's sums to shared memory, [row][channel] (the ring is idle then: every load has landed and every MMA read it) ----
@@ -589,8 +602,6 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
 #pragma unroll
       for (int e = 0; e < 4; ++e) dw[e] = n + e < a.N ? __ldg(a.dw + n + e) : 1.f;
       for (int m = split * per + warp; m < r_end; m += kThreadsW / 32) {
-        RopeRow rope;
-        if constexpr (EPI == kWideRope) rope_row_load(rope, a.rope, m0 + m, chan_of(first));
         uint4 p[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k)
@@ -602,13 +613,6 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
           const uint32_t v[4] = {p[k].x, p[k].y, p[k].z, p[k].w};
 #pragma unroll
           for (int e = 0; e < 4; ++e) f[e] = k == 0 ? __uint_as_float(v[e]) : f[e] + __uint_as_float(v[e]);
-        }
-        if constexpr (EPI == kWideRope) {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) f[e] = round_bf16(f[e] * dw[e]);
-          if (a.rope.D == 128) rope_row_store<128>(a.rope, f, m0 + m, chan_of(first), rope);
-          else rope_row_store<64>(a.rope, f, m0 + m, chan_of(first), rope);
-          continue;
         }
         unsigned long long best = 0;
         const size_t idx = (size_t)(m0 + m) * a.N + n;
@@ -659,6 +663,16 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     cluster_arrive();   // nobody's shared memory goes away while another CTA may read it
     cluster_wait();
   }
+  if (!SPLIT && *abort_flag == 0 && (s_finish[0] | s_finish[1]) != 0) {
+    pdl_wait();   // (every thread: the residual comes from a kernel in front)
+    WideWalk walk(a, first, kb0, kb1);
+    WidePiece p;
+#pragma unroll 1
+    for (int i = 0; i < 2; ++i) {
+      if (!walk.next(a, step, p) || p.share != i) break;
+      if (s_finish[i] != 0) finish_shared<EPI>(a, p.u, pair_x, row_of(p.u), chan_of(p.u));
+    }
+  }
 }
 
 struct WidePlan {
@@ -696,8 +710,8 @@ constexpr int kLeastShare = 3;    // stages
 
 // Row tiles, k-ranges and shares by an estimate of the time in us.  A stage (128 of K) takes its MMAs (7.0e6 multiply-adds per us on an
 // SM), or its way into the SM, or 0.41 us of the hand-overs from load to conversion to MMA.  Sharing (room: bytes there are for the parts)
-// is for a last turn behind whole ones only, whose MMAs hide the way of the parts through L2: small matrices that shared all their
-// units, 6144, 4096 and 4096 x 12288 channels at 72 rows, took 6 us longer each than ranges, and their sums are longer than a range's.
+// costs its parts' way through L2 and a few round trips; it never makes the sums of a product longer, and with them less exact, than they
+// are without it.
 WidePlan plan_wide(int64_t M, int64_t N, int64_t K, int epi, bool keys, size_t room) {
   WidePlan best = {}, shared = {};
   const bool swiglu = epi == kWideSwiglu;
@@ -735,17 +749,17 @@ WidePlan plan_wide(int64_t M, int64_t N, int64_t K, int epi, bool keys, size_t r
         // the rest of the last turn shared
         const int full = keys && kPairs / t > 0 ? kPairs / t * t : kPairs, rest = units % full;
         const long long stages = (long long)rest * kblocks, fits = (long long)(room / ((size_t)p.rows * 1024)) - rest;
-        const int sharers = (int)std::min(std::min((long long)full, std::max(stages / kLeastShare, 1LL)), fits);
-        if (rest > 0 && units > full && sharers > rest && stages <= 0x7fffffffLL && epi != kWideRope) {
+        const int sharers = (int)std::min(std::min((long long)(units > full ? full : kPairs), std::max(stages / kLeastShare, 1LL)), fits);
+        if (rest > 0 && sharers >= rest && stages <= 0x7fffffffLL && (epi != kWideRope || units < full)) {
           WidePlan q = p;
           q.nsplit = 1;
           q.whole = units - rest;
           q.sharers = sharers;
-          q.ctas = 2 * full;
+          q.ctas = 2 * (q.whole > 0 ? full : sharers);
           const int per = (int)((stages + sharers - 1) / sharers);
-          q.longest = kblocks;
+          q.longest = q.whole > 0 ? kblocks : per;
           q.cost = 4.0 + (units / full + 1) * (p.accs == 1 ? drain : 0.2) + (p.accs == 2 ? drain : 0.0) + ((double)(units / full) * kblocks + per) * a +
-                   1.0 + 0.006 * p.brows;
+                   2.0 + 0.004 * p.brows * ((double)sharers / rest + 1.0);
           q.cost = std::max(q.cost, (double)N * K / 6.3e6);
           if (shared.sharers == 0 || q.cost < shared.cost * 0.99) shared = q;
         }
@@ -761,7 +775,7 @@ WidePlan plan_wide(int64_t M, int64_t N, int64_t K, int epi, bool keys, size_t r
       if (best.nsplit == 0 || p.cost < best.cost * 0.99) best = p;
     }
   }
-  if (shared.sharers > 0 && shared.longest <= best.longest && shared.cost < best.cost) return shared;
+  if (shared.sharers > 0 && shared.longest <= best.longest && (epi == kWideRope || shared.cost < best.cost)) return shared;
   return best;
 }
 
@@ -769,7 +783,7 @@ int launch_wide(int epi, const __nv_bfloat16* x, const int8_t* w, int64_t M, int
                 cudaStream_t stream) {
   static DeviceOnce once;
   int rc = allow_shared_memory(once, kSmemW, true, {(const void*)tc_wide_kernel<true, kWideStore>, (const void*)tc_wide_kernel<false, kWideStore>,
-                                                    (const void*)tc_wide_kernel<false, kWideSwiglu>, (const void*)tc_wide_kernel<true, kWideRope>});
+                                                    (const void*)tc_wide_kernel<false, kWideSwiglu>, (const void*)tc_wide_kernel<false, kWideRope>});
   if (rc != QUASAR_OK) return rc;
   const WidePlan p = plan_wide(M, N, K, epi, a.keys != nullptr, scratch.parts_bytes);
   CUtensorMap map_w, map_x;
@@ -797,7 +811,7 @@ int launch_wide(int epi, const __nv_bfloat16* x, const int8_t* w, int64_t M, int
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 2u : 1u;
   if (epi == kWideSwiglu) QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<false, kWideSwiglu>, map_w, map_x, a));
-  else if (epi == kWideRope) QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<true, kWideRope>, map_w, map_x, a));
+  else if (epi == kWideRope) QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<false, kWideRope>, map_w, map_x, a));
   else if (p.nsplit > 1) QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<true, kWideStore>, map_w, map_x, a));
   else QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<false, kWideStore>, map_w, map_x, a));
   count_launch();
@@ -830,13 +844,15 @@ int launch_tc_wide_swiglu(const __nv_bfloat16* x, const int8_t* w, const float* 
   return launch_wide(kWideSwiglu, x, w, M, 2 * F, K, scratch, a, pdl, stream);
 }
 
-bool tc_wide_rope_fits(int64_t M, int64_t N, int64_t K) { return plan_wide(M, N, K, kWideRope, false, 0).nsplit > 1; }
+bool tc_wide_rope_fits(int64_t M, int64_t N, int64_t K, const WideScratch& scratch) {
+  return plan_wide(M, N, K, kWideRope, false, scratch.parts_bytes).sharers > 0;
+}
 
 int launch_tc_wide_qkv_rope(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t K, const RopeArgs& rope,
-                            int32_t* error, cudaStream_t stream) {
+                            const WideScratch& scratch, int32_t* error, cudaStream_t stream) {
   WideArgs a = {};
   a.dw = dw; a.error = error; a.rope = rope;
-  return launch_wide(kWideRope, x, w, M, (int64_t)(rope.Hq + 2 * rope.Hkv) * rope.D, K, WideScratch{}, a, true, stream);
+  return launch_wide(kWideRope, x, w, M, (int64_t)(rope.Hq + 2 * rope.Hkv) * rope.D, K, scratch, a, true, stream);
 }
 
 }  // namespace quasar

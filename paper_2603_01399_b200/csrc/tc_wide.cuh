@@ -26,8 +26,8 @@ int launch_tc_wide(const __nv_bfloat16* x, const int8_t* w, const float* dw, int
 int launch_tc_wide_swiglu(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t F, int64_t K, __nv_bfloat16* act,
                           const WideScratch& scratch, int32_t* error, bool pdl, cudaStream_t stream);
 // qkv projection with QK-norm, RoPE and KV append, for sizes that tc_wide_rope_fits accepts; writes q (into rope.qkv) and the cache rows
-bool tc_wide_rope_fits(int64_t M, int64_t N, int64_t K);
+bool tc_wide_rope_fits(int64_t M, int64_t N, int64_t K, const WideScratch& scratch);
 int launch_tc_wide_qkv_rope(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t K, const RopeArgs& rope,
-                            int32_t* error, cudaStream_t stream);
+                            const WideScratch& scratch, int32_t* error, cudaStream_t stream);
 
 }  // namespace quasar
