@@ -368,7 +368,7 @@ operand_kernel(const __nv_bfloat16* x, const unsigned* row_max, int nvec, RowOpe
 
 // Puts an attention's partial results together and leaves the o projection's operand: a cluster of four CTAs per block row,
 // each a quarter of the query heads, a warp per head.  A head's parts lie `stride` entries apart and are added in their order
-// (tcgen05 form: the CTAs that share the head's segment, see tc_attention.cuh - one that had it to itself has left the rows -; the other
+// (tcgen05 form: the two groups of every CTA whose run of the list touched the head's segment, see tc_attention.cuh; the other
 // form: the chunks of the keys); the copies of 8 or 16 parts are in flight together.  Latency-bound; 6 rows of 32 heads and 18 or 34
 // parts took 10-17 us with one CTA per row or eight parts at a time and another kernel for the operand.
 constexpr int kMergeCtas = 4, kMergeWarps = 16;
@@ -397,7 +397,7 @@ attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, Ro
     live = tiles > 0 && i < l.block_len[b];
     ctas = attn_ctas(total);
     const int t = i / l.npt;
-    unit0 += t * attn_span(tiles) + kAttnPad;    // of head 0's row tile that holds this row: its first key tile
+    unit0 += t * tiles;    // of head 0's row tile that holds this row
     seg0 += t;
     row0 = (i - t * l.npt) * l.G;
     stride = 128;
@@ -420,7 +420,7 @@ attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, Ro
       size_t at0;
       int n = n0;
       if (LIST) {   // CTA c takes the units [c * total / ctas, (c + 1) * total / ctas): the ones that share u0 .. u1 - 1
-        const int u0 = unit0 + hk * row_tiles * attn_span(tiles), u1 = u0 + tiles, s = seg0 + hk * row_tiles;
+        const int u0 = unit0 + hk * row_tiles * tiles, u1 = u0 + tiles, s = seg0 + hk * row_tiles;
         int c0, c1;
         if (total < (1u << 24)) {
           c0 = (int)(((unsigned)(u0 + 1) * ctas - 1u) / total);
@@ -429,16 +429,10 @@ attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, Ro
           c0 = (int)(((unsigned long long)(u0 + 1) * ctas - 1) / total);
           c1 = (int)(((unsigned long long)u1 * ctas - 1) / total);
         }
-        n = c1 - c0 + 1;
-        at0 = (size_t)(c0 + s) * 128 + row;
+        n = 2 * (c1 - c0 + 1);
+        at0 = (size_t)(c0 + s) * 256 + row;
       } else {
         at0 = ((size_t)b * l.Hkv + hk) * ch.nchunk * ch.Rpad + row;
-      }
-      if (LIST && n == 1) {
-        const uint32_t* done = reinterpret_cast<const uint32_t*>(parts.rows + ((size_t)m * Hq + hq) * D) + lane * (kPer / 2);
-#pragma unroll
-        for (int e = 0; e < kPer / 2; ++e) pk[e] = __ldcg(done + e);
-        n = 0;
       }
       auto part_ml = [&](int p) { return p < n ? __ldcg(&parts.ml[at0 + (size_t)p * stride]) : make_float2(-INFINITY, 0.f); };
       float2 ml[2] = {part_ml(lane), part_ml(lane + 32)};   // (64 parts in one round trip: more are rare)
@@ -486,7 +480,7 @@ attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, Ro
 #pragma unroll
       for (int e = 0; e < kPer / 2; ++e) {
         const __nv_bfloat162 t = __floats2bfloat162_rn(acc[2 * e] * inv, acc[2 * e + 1] * inv);
-        if (n > 0) pk[e] = *reinterpret_cast<const uint32_t*>(&t);
+        pk[e] = *reinterpret_cast<const uint32_t*>(&t);
       }
     }
     uint32_t* dst = reinterpret_cast<uint32_t*>(s_row) + (hq - h0) * (D / 2) + lane * (kPer / 2);
@@ -604,7 +598,7 @@ __device__ void lay_out_list(const BlockArgs& a) {
       q.tiles = (a.seq_len[b] + T + 127) / 128;
       q.row_tiles = (T + a.npt - 1) / a.npt;
     }
-    int u = attn_span(q.tiles) * q.row_tiles * a.Hkv, s = q.row_tiles * a.Hkv;
+    int u = q.tiles * q.row_tiles * a.Hkv, s = q.row_tiles * a.Hkv;
     const int own_u = u, own_s = s;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {

@@ -14,9 +14,8 @@
 // O is scaled only when a row's maximum grows by more than 2^8 over the one its sums stand against.
 //
 // Work split: the key tiles of all (sequence, kv head, row tile) segments form one list, and each of the 148 CTAs takes an
-// equal run of it, whatever the lengths of the sequences.  At the end of a run's part of a segment the groups put their results
-// together, each half of the columns (a warp reads the other group's O in its own tensor-memory lanes); a whole segment's rows are
-// finished there, a part leaves a partial result (row maxima, sums, O), which attention_merge (row_ops.cu) adds in list order.
+// equal run of it, whatever the lengths of the sequences; a run's part of a segment leaves two partial results (one per
+// group: row maxima, sums, O), which attention_merge (row_ops.cu) adds in list order.
 //
 // What bounds it: HBM on long prefixes.  Per 128 keys (64 KB) an SM spends about 1540 cycles of MMAs, 1030 issue slots of
 // softmax and 2900 cycles of its share of the memory's bandwidth.
@@ -40,9 +39,8 @@ constexpr float kGrow = 8.f;      // how far (in powers of two) a row's maximum 
 
 struct TcAttnArgs {
   AttnList list;
-  float* o_part;              // [slots][128][D]
-  float2* ml_part;            // [slots][128]
-  __nv_bfloat16* out;         // [B*T_max][Hkv*G*D] rows of segments that one CTA has to itself
+  float* o_part;              // [slots][2][128][D]
+  float2* ml_part;            // [slots][2][128]
   int q_rows;                 // query rows a box of map_q brings: G * npt
   int32_t* error;
 };
@@ -97,7 +95,6 @@ struct Walk {
   const AttnSeq* known;
   int u, end;
   int b, hk, rt, t0, nt, seg;   // the piece: sequence, kv head, row tile, first key tile, key tiles, ordinal of the segment
-  bool whole;                   // all of the segment's key tiles
   __device__ Walk(const AttnList& l, const AttnSeq* k, int total, int cta) : known(k) {
     const int ctas = (int)attn_ctas((unsigned)total);
     u = cta < ctas ? (int)((long long)cta * total / ctas) : 0;
@@ -105,21 +102,17 @@ struct Walk {
     cur.start(l, known);
   }
   __device__ bool next(const AttnList& l) {
-    while (u < end) {
-      cur.seek(l, known, u);
-      const int span = attn_span(cur.q.tiles), in = u - cur.q.unit0, s = in / span, at = in - s * span, n = min(span - at, end - u);
-      t0 = max(at - kAttnPad, 0);
-      nt = min(at + n - kAttnPad, cur.q.tiles) - t0;
-      u += n;
-      if (nt <= 0) continue;   // (nothing but idle units)
-      b = cur.b;
-      hk = s / cur.q.row_tiles;
-      rt = s - hk * cur.q.row_tiles;
-      seg = cur.q.seg0 + s;
-      whole = nt == cur.q.tiles;
-      return true;
-    }
-    return false;
+    if (u >= end) return false;
+    cur.seek(l, known, u);
+    b = cur.b;
+    const int in = u - cur.q.unit0, s = in / cur.q.tiles;
+    t0 = in - s * cur.q.tiles;
+    nt = min(cur.q.tiles - t0, end - u);
+    hk = s / cur.q.row_tiles;
+    rt = s - hk * cur.q.row_tiles;
+    seg = cur.q.seg0 + s;
+    u += nt;
+    return true;
   }
 };
 
@@ -141,10 +134,7 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
   uint64_t* s_full = q_empty + 2;                   // [2] S of a group's tile is complete
   uint64_t* p_ready = s_full + 2;                   // [2] P lies over it
   uint64_t* pv_done = p_ready + 2;                  // [2] O has the products of a group's part of a piece
-  uint64_t* o_ready = pv_done + 2;                  // [2] group 1's O of a piece is there, and its rows' maxima and sums; group 0's likewise
-  uint64_t* o_free = o_ready + 2;                   // both groups have read both O
-  float2* s_ml = reinterpret_cast<float2*>(o_free + 1);   // [128] group 1's, then, once a row of group 0 has taken it, group 0's
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_ml + 128);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(pv_done + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
@@ -160,9 +150,7 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
       mbar_init(s_full + i, 1);
       mbar_init(p_ready + i, 4);
       mbar_init(pv_done + i, 1);
-      mbar_init(o_ready + i, 4);
     }
-    mbar_init(o_free, 8);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   if (warp == 1) {
@@ -322,16 +310,15 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
     const int G = a.list.G;
     uint32_t s_ph = 0, pv_ph = 0;
     int done = 0;            // key tiles of the pieces before
-    int piece = 0;
     bool ok = true;
-    for (; ok && w.next(a.list); ++piece) {
+    while (ok && w.next(a.list)) {
       const int T = a.list.block_len[w.b], P = a.list.seq_len[w.b], Lk = P + T;
       const int node0 = w.rt * a.list.npt, rows = min(a.list.npt, T - node0) * G;
       const bool active = q * 32 < rows;   // (a warp without rows only keeps the hand-shakes going)
       const bool live = row < rows;
       const unsigned long long anc = live ? a.list.anc[w.b * a.list.T_max + node0 + row / G] : 0ull;
       float m_ref = -INFINITY, sum = 0.f;
-      const size_t slot = (size_t)(blockIdx.x + w.seg) * 128 + row;
+      const size_t slot = ((size_t)(blockIdx.x + w.seg) * 2 + g) * 128 + row;
       const int t_first = (done & 1) ^ g;   // this group's first tile of the piece
       for (int t = t_first; t < w.nt; t += 2) {
         if (!(ok = __all_sync(0xffffffffu, mbar_wait(s_full + g, s_ph, abort_flag, a.error)))) break;
@@ -412,8 +399,6 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
           }
           asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         }
-        // (the products of this tile overwrite O: both groups have read it by then)
-        if (t == t_first && piece > 0 && !(ok = __all_sync(0xffffffffu, mbar_wait(o_free, (uint32_t)(piece - 1) & 1u, abort_flag, a.error)))) break;
         fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(p_ready + g);
@@ -424,71 +409,22 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
         pv_ph ^= 1u;
         fence_after();
       }
-      float2 ml0 = make_float2(m_ref, sum), ml1 = ml0;
-      fence_before();
-      if (g == 1) {
-        s_ml[row] = ml1;
-        __syncwarp();
-        if (lane == 0) mbar_arrive(o_ready);
-        if (!(ok = __all_sync(0xffffffffu, mbar_wait(o_ready + 1, (uint32_t)piece & 1u, abort_flag, a.error)))) break;
-        ml0 = s_ml[row];
-      } else {
-        if (!(ok = __all_sync(0xffffffffu, mbar_wait(o_ready, (uint32_t)piece & 1u, abort_flag, a.error)))) break;
-        ml1 = s_ml[row];
-        s_ml[row] = ml0;
-        __syncwarp();
-        if (lane == 0) mbar_arrive(o_ready + 1);
-      }
-      fence_after();
-      if (active) {   // the piece's result, this group half of its columns
-        const float m = fmaxf(ml0.x, ml1.x);
-        const float f0 = ml0.x == -INFINITY ? 0.f : exp2f(ml0.x - m), f1 = ml1.x == -INFINITY ? 0.f : exp2f(ml1.x - m);
-        const float total = f0 * ml0.y + f1 * ml1.y;
-        const bool two = w.nt > 1;                        // (one tile: one group's, that of its parity)
-        const bool from0 = two || (done & 1) == 0, from1 = two || (done & 1) == 1;
-        const float inv = w.whole ? 1.0f / total : 1.0f;
-        if (!w.whole && g == 0 && live) a.ml_part[slot] = make_float2(m, total);
-        const int node = node0 + row / G, head = w.hk * G + row % G;
-        __nv_bfloat16* dst_row = a.out + ((size_t)(w.b * a.list.T_max + node) * (a.list.Hkv * G) + head) * D + g * (D / 2);
-#pragma unroll 1
-        for (int c = 0; c < D / 64; ++c) {
-          float o[32];
-          const uint32_t col = (uint32_t)(g * (D / 2) + c * 32);
-          if (from0) {
-            tmem_ld32(lane_base + 256u + col, o);
+      if (active) {   // the piece's partial result
+        if (live) a.ml_part[slot] = make_float2(m_ref, sum);
+        if (w.nt > t_first) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) o[j] = f0 != 0.f ? o[j] * f0 : 0.f;
-          } else {
+          for (int c = 0; c < D / 32; ++c) {
+            float o[32];
+            tmem_ld32(to + (uint32_t)(c * 32), o);
+            if (live) {
+              float4* dst = reinterpret_cast<float4*>(a.o_part + slot * D + c * 32);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) o[j] = 0.f;
-          }
-          if (from1) {
-            float o1[32];
-            tmem_ld32(lane_base + 384u + col, o1);
-#pragma unroll
-            for (int j = 0; j < 32; ++j) o[j] += f1 != 0.f ? o1[j] * f1 : 0.f;
-          }
-          if (live && w.whole) {
-            uint32_t p[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const __nv_bfloat162 t = __floats2bfloat162_rn(o[2 * j] * inv, o[2 * j + 1] * inv);
-              p[j] = *reinterpret_cast<const uint32_t*>(&t);
+              for (int j = 0; j < 8; ++j) dst[j] = make_float4(o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
             }
-            uint4* dst = reinterpret_cast<uint4*>(dst_row + c * 32);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) dst[j] = make_uint4(p[4 * j], p[4 * j + 1], p[4 * j + 2], p[4 * j + 3]);
-          } else if (live) {
-            float4* dst = reinterpret_cast<float4*>(a.o_part + slot * D + g * (D / 2) + c * 32);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) dst[j] = make_float4(o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
           }
-          __syncwarp();
         }
-        fence_before();
+        fence_before();   // (the next piece's P, which follows in this warp's order, lets O be overwritten)
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(o_free);
       done += w.nt;
     }
   }
@@ -503,7 +439,7 @@ tc_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_cons
 
 template <int D>
 int launch_d(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const TcAttnArgs& a, int ctas, cudaStream_t stream) {
-  constexpr size_t smem = (size_t)(2 + kSlots) * (D / 64) * kKeys * 128 + 1024 + 1216;   // (barriers; maxima and sums)
+  constexpr size_t smem = (size_t)(2 + kSlots) * (D / 64) * kKeys * 128 + 1024 + 512;
   static DeviceOnce once;
   const int rc = allow_shared_memory(once, smem, false, {(const void*)tc_attention_kernel<D>});
   if (rc != QUASAR_OK) return rc;
@@ -517,12 +453,11 @@ size_t tc_attention_workspace_bytes(int B, int T_max, int Hq, int Hkv, int D) {
   return slots * 2 * 128 * ((size_t)D * 4 + 8);
 }
 
-AttnParts tc_attention_parts(void* workspace, __nv_bfloat16* rows, int B, int T_max, int Hq, int Hkv, int D) {
+AttnParts tc_attention_parts(void* workspace, int B, int T_max, int Hq, int Hkv, int D) {
   const size_t slots = kAttnCtas + (size_t)B * Hkv * attn_row_tiles(Hq / Hkv, T_max);
   AttnParts p;
   p.o = reinterpret_cast<float*>(workspace);
-  p.ml = reinterpret_cast<float2*>(p.o + slots * 128 * D);
-  p.rows = rows;
+  p.ml = reinterpret_cast<float2*>(p.o + slots * 2 * 128 * D);
   return p;
 }
 
@@ -538,7 +473,7 @@ int launch_tc_attention(const __nv_bfloat16* qkv, const __nv_bfloat16* k_cache_l
                        (uint32_t)list.G, (uint32_t)list.npt);
   if (rc != QUASAR_OK) return rc;
   TcAttnArgs a;
-  a.q_rows = list.G * list.npt; a.list = list; a.o_part = parts.o; a.ml_part = parts.ml; a.out = parts.rows; a.error = error;
+  a.q_rows = list.G * list.npt; a.list = list; a.o_part = parts.o; a.ml_part = parts.ml; a.error = error;
   return D == 128 ? launch_d<128>(mq, mk, mv, a, kAttnCtas, stream) : launch_d<64>(mq, mk, mv, a, kAttnCtas, stream);
 }
 

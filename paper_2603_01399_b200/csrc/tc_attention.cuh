@@ -7,17 +7,15 @@
 namespace quasar {
 
 constexpr int kAttnCtas = 148;    // one per SM
-constexpr int kShapes = 48;       // sequences whose places a CTA keeps in shared memory (more are looked up as they come)
+constexpr int kShapes = 64;       // sequences whose places a CTA keeps in shared memory (more are looked up as they come)
 
 // block rows whose query heads of one kv head make up a row tile of the 128-row MMAs
 constexpr int attn_nodes_per_tile(int G) { return 128 / G; }
 constexpr int attn_row_tiles(int G, int T) { return (T + attn_nodes_per_tile(G) - 1) / attn_nodes_per_tile(G); }
 
 // Segments in order of sequence, kv head, row tile (npt block rows x G query heads); a segment's units are its tiles
-// of 128 keys, with kAttnPad idle ones on either side that stand for what a piece costs besides its tiles.  CTA c < ctas = min(148, total)
-// takes the units [c * total / ctas, (c + 1) * total / ctas) - one at least -, and its partial results for segment s
-// lie in slot c + s.  A segment whose tiles all fall to one CTA has no partial results.
-constexpr int kAttnPad = 1;
+// of 128 keys.  CTA c < ctas = min(148, total) takes the units [c * total / ctas, (c + 1) * total / ctas) - one at least -, and its partial results for segment s
+// lie in slot c + s.
 struct AttnList {
   const int32_t *seq_len, *block_len, *valid;
   const AttnSeq* seq;     // [B + 1]
@@ -26,13 +24,12 @@ struct AttnList {
 };
 
 struct AttnParts {
-  float* o;      // [slots][128 rows][D] un-normalised outputs
-  float2* ml;    // [slots][128] row maximum (power of two), sum
-  __nv_bfloat16* rows;   // [B*T_max][Hkv*G*D] the rows of segments without partial results
+  float* o;      // [slots][2 groups][128 rows][D] un-normalised outputs
+  float2* ml;    // [slots][2][128] row maximum (power of two), sum
 };
 
 size_t tc_attention_workspace_bytes(int B, int T_max, int Hq, int Hkv, int D);
-AttnParts tc_attention_parts(void* workspace, __nv_bfloat16* rows, int B, int T_max, int Hq, int Hkv, int D);
+AttnParts tc_attention_parts(void* workspace, int B, int T_max, int Hq, int Hkv, int D);
 int launch_tc_attention(const __nv_bfloat16* qkv, const __nv_bfloat16* k_cache_layer, const __nv_bfloat16* v_cache_layer,
                         const AttnList& list, int kv_batch, int D, const AttnParts& parts, int32_t* error, cudaStream_t stream);
 
@@ -42,7 +39,6 @@ int launch_attention_merge(int op, const AttnList& list, const AttnParts& parts,
                            const RowOperand& out, cudaStream_t stream);
 
 #ifdef __CUDACC__
-__device__ __forceinline__ int attn_span(int tiles) { return tiles + 2 * kAttnPad; }   // units of a segment
 __device__ __forceinline__ unsigned attn_ctas(unsigned total) { return total < (unsigned)kAttnCtas ? total : (unsigned)kAttnCtas; }
 
 // Walks the sequences in order, to the one that holds a unit.
@@ -55,7 +51,7 @@ struct AttnCursor {
     load(l, known);
   }
   __device__ __forceinline__ void seek(const AttnList& l, const AttnSeq* known, int u) {
-    while (b + 1 < l.B && u >= q.unit0 + attn_span(q.tiles) * q.row_tiles * l.Hkv) {
+    while (b + 1 < l.B && u >= q.unit0 + q.tiles * q.row_tiles * l.Hkv) {
       ++b;
       load(l, known);
     }
