@@ -190,7 +190,7 @@ int launch_linear(const __nv_bfloat16* x, const void* w, const float* delta, int
     return launch_tc_linear_bf16(x, reinterpret_cast<const __nv_bfloat16*>(w), M, N, K, y, y_is_f32, residual, nullptr, status, false,
                                  stream);
   const int8_t* wq = reinterpret_cast<const int8_t*>(w);
-  if (tc_wide_better(M, K)) return launch_tc_wide(x, wq, delta, M, N, K, y, y_is_f32, residual, nullptr, WideScratch{}, status, false, stream);
+  if (tc_wide_better(M, K)) return launch_tc_wide(x, wq, delta, M, N, K, y, y_is_f32, residual, nullptr, status, false, stream);
   const size_t ybytes = y_is_f32 ? 4 : 2;
   // rows whose digits fit behind the reserved start of the workspace: all of them, unless the workspace is smaller than
   // linear_workspace_bytes reports (the built-in one of linear_static)

@@ -628,7 +628,6 @@ embed_norm_kernel(BlockArgs a, int M, const __nv_bfloat16* __restrict__ embed, _
     __shared__ unsigned long long s_anc[kRowThreads / 32][QUASAR_MAX_BLOCK];
     const int warp = threadIdx.x >> 5;
     for (int k = threadIdx.x; k < a.n_clear; k += kRowThreads) a.clear[k] = 0u;
-    for (int k = threadIdx.x; k < a.n_clear2; k += kRowThreads) a.clear2[k] = 0u;
     for (int b = warp; b < a.B; b += kRowThreads / 32) {
       prepare_sequence(a, b, s_parent[warp], s_anc[warp], s_depth[warp]);
       __syncwarp();

@@ -17,12 +17,8 @@
 // the conversion, beyond that the tensor cores: 24,576 x 4096 at 512 rows 118 us as digit rows, 82 here (1.25 PFLOP/s),
 // LM head 675 -> 474 us (1.35); prompt chunks of 8 x 64 rows through the 8B model 12.5 -> 9.5 ms.  Tensor memory: accumulators of `brows` columns - two where that leaves room, so that a tile leaves
 // for memory under the next one's MMAs - and a ring of 32-column pieces of operand A.
-// Work split: units of 256 channels x one row tile.  Either in turn on one pair per SM pair; or, for matrices of few units, k-ranges
-// of a unit in the pairs of one cluster, added through distributed shared memory in the order of the ranges; or, where the caller
-// has memory for it, shared: the units that make up no whole turn of all pairs - for a small matrix all there are - are cut along k
-// into equal shares of stages, one a pair.  A share leaves its sums in global memory (L2), and the CTA that finishes last of a
-// unit's sharers adds them, in the order of k, and finishes the rows: nobody waits for another CTA, and the result does not depend
-// on which one is last.
+// Two forms: tiles in turn on one pair per SM pair; or, for matrices of few tiles, k-ranges of a tile in the pairs of one
+// cluster, added through distributed shared memory in the order of the ranges.
 //
 // Every wait is bounded (2 s): on expiry the CTA raises an error word, stops waiting everywhere, releases its tensor
 // memory and returns.
@@ -31,7 +27,6 @@
 #include <algorithm>
 #include <mutex>
 
-#include "rope.cuh"
 #include "tc_common.cuh"
 #include "tc_linear.cuh"
 #include "tc_wide.cuh"
@@ -59,62 +54,9 @@ struct WideArgs {
   int rows, brows, row_tiles, nsplit, stages;
   int accs, pieces;            // accumulators; pieces of operand A in the ring
   int acc_cols;                // columns from one accumulator to the next
-  int units, whole;            // units; those dealt out in whole turns, `whole` first ones
-  int sharers;                 // pairs that share the stages of the rest
-  float* parts;                // [sharers + rest][2][rows][128] sums of the shares, see part_slot
-  unsigned* arrived;           // [rest][2] shares that have left their sums; zero before and after
+  int units;
   int y_is_f32, early_weights;
-  RopeArgs rope;               // kWideRope
 };
-
-// What is done with a unit's finished sums: stored; multiplied as gate and up units; or made q, k and v (QK-norm, RoPE, cache
-// append: only where all units are shared, for it takes whole rows of a head)
-enum WideEpilogue { kWideStore = 0, kWideSwiglu = 1, kWideRope = 2 };
-
-// A pair's way through its work: its share of the rest, at most two pieces of units, then its whole units.
-struct WidePiece {
-  int u, k0, k1;   // unit, stages
-  int share;       // which piece of the share (0, 1), or -1: a whole unit (or the range of one)
-};
-struct WideWalk {
-  int pos, end, next_share, u;
-  int k0, k1;
-  __device__ __forceinline__ WideWalk(const WideArgs& a, int pair, int k0_, int k1_) : k0(k0_), k1(k1_) {
-    const long long rest = (long long)(a.units - a.whole) * a.kblocks;
-    pos = pair < a.sharers ? (int)(rest * pair / a.sharers) : 0;
-    end = pair < a.sharers ? (int)(rest * (pair + 1) / a.sharers) : 0;
-    next_share = 0;
-    u = pair;
-  }
-  __device__ __forceinline__ bool next(const WideArgs& a, int step, WidePiece& p) {
-    if (pos < end) {
-      const int r = pos / a.kblocks;
-      p.u = a.whole + r;
-      p.k0 = pos - r * a.kblocks;
-      p.k1 = min(a.kblocks, p.k0 + end - pos);
-      p.share = next_share++;
-      pos += p.k1 - p.k0;
-      return true;
-    }
-    if (u >= a.whole) return false;
-    p.u = u;
-    p.k0 = k0;
-    p.k1 = k1;
-    p.share = -1;
-    u += step;
-    return true;
-  }
-};
-// The pairs that share unit u: stage i of the rest belongs to pair ((i + 1) * sharers - 1) / stages.  Part of pair p: slot
-// p + (u - whole), since every pair's and every unit's first part is one further.
-__device__ __forceinline__ void wide_sharers(const WideArgs& a, int u, int& p0, int& p1) {
-  const long long rest = (long long)(a.units - a.whole) * a.kblocks, i0 = (long long)(u - a.whole) * a.kblocks, i1 = i0 + a.kblocks;
-  p0 = (int)(((i0 + 1) * a.sharers - 1) / rest);
-  p1 = (int)((i1 * a.sharers - 1) / rest);
-}
-__device__ __forceinline__ float* part_slot(const WideArgs& a, int pair, int u, int pair_x) {
-  return a.parts + ((size_t)(pair + u - a.whole) * 2 + pair_x) * ((size_t)a.rows * 128);
-}
 
 // four int8 -> four bf16, exactly: 0x43bb is 128 + bb for the low seven bits, and the sign bit asks for 256 instead of 128 to go
 __device__ __forceinline__ void bf16x4(uint32_t w, uint32_t& lo, uint32_t& hi) {
@@ -147,133 +89,9 @@ __device__ __forceinline__ int channel_of(int n0, int r, int N) {
   return (r & 16) ? N / 2 + u : u;
 }
 
-// A shared unit's parts added and its rows finished, by all warps of the CTA: two rows a warp at a time, four channels a lane, four
-// parts of each row asked for at once.
-template <int EPI>
-__device__ __forceinline__ void finish_shared(const WideArgs& a, int u, int pair_x, int m0, int n0) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rows = min(a.rows, a.M - m0), F = a.N / 2;
-  int p0, p1;
-  wide_sharers(a, u, p0, p1);
-  const float* part0 = part_slot(a, p0, u, pair_x) + lane * 4;
-  const size_t part_step = (size_t)2 * a.rows * 128;
-  const int n = EPI == kWideSwiglu ? channel_of<true>(n0, lane * 4, a.N) : n0 + lane * 4;   // four neighbours either way
-  const int unit = n0 / 2 + (lane >> 3) * 16 + (lane & 3) * 4;
-  const bool up_lane = (lane & 4) != 0;
-  float dw[4];
-#pragma unroll
-  for (int e = 0; e < 4; ++e) dw[e] = (EPI == kWideSwiglu ? unit + e < F : n + e < a.N) ? __ldg(a.dw + n + e) : 1.f;
-  constexpr int kTwo = EPI == kWideRope ? 1 : 2;
-  for (int r0 = kTwo * warp; r0 < rows; r0 += kTwo * (kThreadsW / 32)) {
-    float f[kTwo][4];
-    RopeRow rope;
-    if constexpr (EPI == kWideRope) rope_row_load(rope, a.rope, m0 + r0, n0);
-    uint2 res[kTwo];
-    const bool quad = (a.N & 3) == 0;   // (then four channels are inside or outside together, and aligned)
-    if (EPI == kWideStore && a.res != nullptr && quad) {
-#pragma unroll
-      for (int h = 0; h < kTwo; ++h)
-        if (r0 + h < rows && n < a.N) res[h] = *reinterpret_cast<const uint2*>(a.res + (size_t)(m0 + r0 + h) * a.N + n);
-    }
-#pragma unroll
-    for (int h = 0; h < kTwo; ++h) f[h][0] = f[h][1] = f[h][2] = f[h][3] = 0.f;
-    for (int q0 = 0; q0 <= p1 - p0; q0 += 4) {
-      float4 v[4][kTwo];
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int h = 0; h < kTwo; ++h)
-          if (q0 + q <= p1 - p0 && r0 + h < rows)
-            v[q][h] = __ldcg(reinterpret_cast<const float4*>(part0 + (q0 + q) * part_step + (size_t)(r0 + h) * 128));
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int h = 0; h < kTwo; ++h) {
-          if (q0 + q > p1 - p0 || r0 + h >= rows) continue;
-          const float w[4] = {v[q][h].x, v[q][h].y, v[q][h].z, v[q][h].w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) f[h][e] = q0 + q == 0 ? w[e] : f[h][e] + w[e];
-        }
-    }
-#pragma unroll
-    for (int h = 0; h < kTwo; ++h) {
-      const int m = m0 + r0 + h;
-      if (r0 + h >= rows) break;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) f[h][e] *= dw[e];
-      if constexpr (EPI == kWideRope) {
-        float b[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) b[e] = round_bf16(f[h][e]);
-        if (a.rope.D == 128) rope_row_store<128>(a.rope, b, m, n0, rope);
-        else rope_row_store<64>(a.rope, b, m, n0, rope);
-        continue;
-      }
-      if constexpr (EPI == kWideSwiglu) {
-        float o[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float t = round_bf16(f[h][e]), other = __shfl_xor_sync(0xffffffffu, t, 4);
-          o[e] = t / (1.0f + expf(-t)) * other;
-        }
-        if (!up_lane && unit < F) {   // (F is a multiple of 16)
-          const __nv_bfloat162 lo = __floats2bfloat162_rn(o[0], o[1]), hi = __floats2bfloat162_rn(o[2], o[3]);
-          *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.y) + (size_t)m * F + unit) =
-              make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
-        }
-        continue;
-      }
-      const size_t idx = (size_t)m * a.N + n;
-      if (a.keys != nullptr) {
-        unsigned long long best = 0;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          if (n + e >= a.N || f[h][e] != f[h][e]) continue;   // NaNs never enter
-          const unsigned long long k = argmax_key(f[h][e], n + e);
-          best = k > best ? k : best;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
-          best = other > best ? other : best;
-        }
-        if (lane == 0 && best != 0) atomicMax(a.keys + m, best);
-      }
-      if (a.y == nullptr) continue;
-      if (quad) {
-        if (n >= a.N) continue;
-        if (a.res != nullptr) {
-          f[h][0] = round_bf16(f[h][0]) + __uint_as_float(res[h].x << 16);
-          f[h][1] = round_bf16(f[h][1]) + __uint_as_float(res[h].x & 0xffff0000u);
-          f[h][2] = round_bf16(f[h][2]) + __uint_as_float(res[h].y << 16);
-          f[h][3] = round_bf16(f[h][3]) + __uint_as_float(res[h].y & 0xffff0000u);
-        }
-        if (a.y_is_f32) {
-          *reinterpret_cast<float4*>(reinterpret_cast<float*>(a.y) + idx) = make_float4(f[h][0], f[h][1], f[h][2], f[h][3]);
-        } else {
-          const __nv_bfloat162 lo = __floats2bfloat162_rn(f[h][0], f[h][1]), hi = __floats2bfloat162_rn(f[h][2], f[h][3]);
-          *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.y) + idx) =
-              make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
-        }
-        continue;
-      }
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        if (n + e >= a.N) break;
-        float o = f[h][e];
-        if (a.res != nullptr) o = round_bf16(o) + __bfloat162float(a.res[idx + e]);
-        if (a.y_is_f32) reinterpret_cast<float*>(a.y)[idx + e] = o;
-        else reinterpret_cast<__nv_bfloat16*>(a.y)[idx + e] = __float2bfloat16_rn(o);
-      }
-    }
-  }
-}
-
-// SPLIT: k-ranges in a cluster (kWideStore only)
-template <bool SPLIT, int EPI>
+template <bool SPLIT, bool SWIGLU>
 __global__ void __launch_bounds__(kThreadsW, 1)
 tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const WideArgs a) {
-  constexpr bool SWIGLU = EPI == kWideSwiglu;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // the swizzle repeats every 1024 bytes
   const int b_half = a.brows / 2;                // rows of operand B of this CTA
@@ -291,8 +109,6 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   unsigned long long* s_best = reinterpret_cast<unsigned long long*>(acc_empty + 2);   // [4][256] arg-max keys of the row tile's rows, by quarter
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_best + 1024);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  int* s_out = reinterpret_cast<int*>(tmem_slot + 2);   // [2] of the share's first, second piece: warps whose sums are out;
-  volatile int* s_finish = s_out + 2;                   // [2] whether this CTA is its unit's last
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (warp: uniform)
   const int pair_x = (int)blockIdx.x & 1;
@@ -307,7 +123,6 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
 
   if (threadIdx.x == 0) {
     *abort_flag = 0;
-    s_out[0] = s_out[1] = s_finish[0] = s_finish[1] = 0;
     for (int s = 0; s < S; ++s) {
       mbar_init(w_full + s, 1);
       mbar_init(w_empty + s, 8);
@@ -337,9 +152,7 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   fence_after();
   const uint32_t tmem = *tmem_slot;
   const uint32_t tmem_a = tmem + (uint32_t)(a.accs * a.acc_cols);
-  // (A tcgen05 kernel behind this one waits for it while it holds tensor memory.  Behind the qkv projection it is the attention, which
-  // counts on everything in front of this kernel being complete: see below.)
-  if (EPI != kWideRope && threadIdx.x == 0) pdl_trigger();
+  if (threadIdx.x == 0) pdl_trigger();   // (a tcgen05 kernel behind this one waits for it while it holds tensor memory)
 
   if (warp == 0) {
     // ---- TMA producer ----
@@ -364,13 +177,10 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
 #pragma unroll
       for (int h = 0; h < 2; ++h) tma_load_2d_pair<false>(at + h * x_sub, &map_x, kb * 256 + h * 128, m0 + pair_x * b_half, bar, policy);
     };
-    WideWalk walk(a, first, kb0, kb1);
-    WidePiece p;
-    bool more = walk.next(a, step, p);
-    const int ahead = more ? min(S, p.k1 - p.k0) : 0;
+    const int ahead = first < a.units ? min(S, kb1 - kb0) : 0;
     if (a.early_weights) {   // the weights of the first stages do not depend on the kernel in front
       for (int i = 0; i < ahead; ++i) {
-        if (elect_one()) load_w(i, p.k0 + i, chan_of(p.u));
+        if (elect_one()) load_w(i, kb0 + i, chan_of(first));
         __syncwarp();
       }
     }
@@ -378,9 +188,9 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     int s = 0, issued = 0;
     uint32_t ph = 0;
     bool ok = true;
-    for (; more && ok; more = walk.next(a, step, p)) {
-      const int n0 = chan_of(p.u), m0 = row_of(p.u);
-      for (int kb = p.k0; kb < p.k1; ++kb) {
+    for (int u = first; u < a.units && ok; u += step) {
+      const int n0 = chan_of(u), m0 = row_of(u);
+      for (int kb = kb0; kb < kb1; ++kb) {
         const bool early = a.early_weights && issued < ahead;
         if (!early && !(ok = mbar_wait(w_empty + s, ph ^ 1u, abort_flag, a.error))) break;
         if (!early && elect_one()) load_w(s, kb, n0);
@@ -402,13 +212,11 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       int s = 0, buf = 0, piece = 0;
       uint32_t ph = 0, bph = 0, pph = 0;
       bool ok = true;
-      WideWalk walk(a, first, kb0, kb1);
-      WidePiece p;
-      while (ok && walk.next(a, step, p)) {
+      for (int u = first; u < a.units && ok; u += step) {
         if (!(ok = mbar_wait(acc_empty + buf, bph ^ 1u, abort_flag, a.error))) break;
         fence_after();
         const uint32_t d = tmem + (uint32_t)(buf * a.acc_cols);
-        for (int kb = p.k0; kb < p.k1 && ok; ++kb) {
+        for (int kb = kb0; kb < kb1 && ok; ++kb) {
           if (!(ok = mbar_wait(x_full + s, ph, abort_flag, a.error))) break;
           const uint64_t db = desc_sw128(smem + (size_t)s * stage_bytes + kWBytes);
 #pragma unroll
@@ -420,7 +228,7 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
               const uint32_t ta = tmem_a + (uint32_t)(piece * kPiece);
 #pragma unroll
               for (int j = 0; j < 4; ++j)   // 16 of K: 8 columns of A, 32 bytes along the rows of B
-                mma_f16_ts_pair(d, ta + (uint32_t)(8 * j), dbh + (uint64_t)(2 * j), id, (kb > p.k0 || h > 0 || j > 0) ? 1u : 0u);
+                mma_f16_ts_pair(d, ta + (uint32_t)(8 * j), dbh + (uint64_t)(2 * j), id, (kb > kb0 || h > 0 || j > 0) ? 1u : 0u);
               commit_pair(a_empty + piece, mask);
               if (h == 1) commit_pair(x_empty + s, mask);
             }
@@ -442,10 +250,8 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     uint32_t ph = 0, pph = 0;
     bool ok = true;
     int turn = g >> 1;   // 0: this stage is the group's
-    WideWalk walk(a, first, kb0, kb1);
-    WidePiece wp;
-    while (ok && walk.next(a, step, wp)) {
-      for (int kb = wp.k0; kb < wp.k1; ++kb, turn ^= 1) {
+    for (int u = first; u < a.units && ok; u += step) {
+      for (int kb = kb0; kb < kb1; ++kb, turn ^= 1) {
         if (turn != 0) {
           if (++s == S) { s = 0; ph ^= 1u; }
           continue;
@@ -479,14 +285,10 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     // ---- epilogue: a thread one channel, 16 rows at a time ----
     const int q = warp & 3, r = q * 32 + lane;
     pdl_wait();   // the residual comes from a kernel in front
-    if (EPI == kWideRope && threadIdx.x == 576) pdl_trigger();
     const bool one_row_tile = step % a.row_tiles == 0;
     int buf = 0;
     uint32_t bph = 0;
-    WideWalk walk(a, first, kb0, kb1);
-    WidePiece p;
-    while (walk.next(a, step, p)) {
-      const int u = p.u;
+    for (int u = first; u < a.units; u += step) {
       const int m0 = row_of(u), rows = min(a.rows, a.M - m0), n0 = chan_of(u), n = channel_of<SWIGLU>(n0, r, a.N);
       const int F = a.N / 2, unit = n0 / 2 + (r >> 5) * 16 + (r & 15);
       const bool live = SWIGLU ? unit < F : n < a.N;
@@ -494,18 +296,7 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       if (!__all_sync(0xffffffffu, mbar_wait(acc_full + buf, bph, abort_flag, a.error))) break;
       fence_after();
       const uint32_t t0 = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * a.acc_cols);
-      if (p.share >= 0) {   // the sums of a share: [row][channel], to be added by the last of its unit
-        float* to = part_slot(a, first, u, pair_x) + r;
-        for (int r0 = 0; r0 < rows; r0 += 16) {
-          uint32_t v[16];
-          tmem_ld16(t0 + (uint32_t)r0, v);
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (r0 + j < rows) to[(size_t)(r0 + j) * 128] = __uint_as_float(v[j]);
-        }
-        __threadfence();
-      }
-      for (int r0 = 0; EPI != kWideRope && p.share < 0 && r0 < rows; r0 += 16) {
+      for (int r0 = 0; r0 < rows; r0 += 16) {
         uint32_t v[16];
         tmem_ld16_async(t0 + (uint32_t)r0, v);
         const int count = rows - r0;
@@ -532,7 +323,7 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
           if (a.y != nullptr) store16(f, live, (size_t)(m0 + r0), n, a.N, count, a.y, a.y_is_f32 != 0, a.res != nullptr, res);
         }
       }
-      if (a.keys != nullptr && !one_row_tile && p.share < 0) {   // the next tile is of other rows: the warp hands on what it has
+      if (a.keys != nullptr && !one_row_tile) {   // the next tile is of other rows: the warp hands on what it has
         __syncwarp();
         for (int r0 = 0; r0 < rows; r0 += 16) {
           unsigned long long& k = s_best[q * 256 + r0 + lane % 16];
@@ -546,18 +337,8 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(cluster_map(smem_u32(acc_empty + buf), leader));
       if (++buf == a.accs) { buf = 0; bph ^= 1u; }
-      if (p.share >= 0 && lane == 0 && atomicAdd(s_out + p.share, 1) == 3) {   // the four warps' sums are out
-        __threadfence();
-        int p0, p1;
-        wide_sharers(a, u, p0, p1);
-        unsigned* count = a.arrived + 2 * (u - a.whole) + pair_x;
-        const bool last = p0 == p1 || (int)atomicAdd(count, 1u) == p1 - p0;
-        if (last && p0 != p1) *count = 0u;
-        __threadfence();
-        s_finish[p.share] = last ? 1 : 0;
-      }
     }
-    if (a.keys != nullptr && one_row_tile && first < a.whole) {
+    if (a.keys != nullptr && one_row_tile && first < a.units) {
       asm volatile("bar.sync 1, 128;\n" ::: "memory");   // (every epilogue warp comes here, one that has given up too)
       const int m0 = row_of(first);
       for (int t = (int)threadIdx.x - 576; t < min(a.rows, a.M - m0); t += 128) {
@@ -663,21 +444,10 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     cluster_arrive();   // nobody's shared memory goes away while another CTA may read it
     cluster_wait();
   }
-  if (!SPLIT && *abort_flag == 0 && (s_finish[0] | s_finish[1]) != 0) {
-    pdl_wait();   // (every thread: the residual comes from a kernel in front)
-    WideWalk walk(a, first, kb0, kb1);
-    WidePiece p;
-#pragma unroll 1
-    for (int i = 0; i < 2; ++i) {
-      if (!walk.next(a, step, p) || p.share != i) break;
-      if (s_finish[i] != 0) finish_shared<EPI>(a, p.u, pair_x, row_of(p.u), chan_of(p.u));
-    }
-  }
 }
 
 struct WidePlan {
   int row_tiles, rows, brows, nsplit, stages, accs, pieces, acc_cols, ctas, tiles;
-  int units, whole, sharers, longest;   // longest: stages that a sum runs over
   double cost;
 };
 
@@ -699,22 +469,16 @@ int max_pair_clusters(int s) {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, (const void*)tc_wide_kernel<true, kWideStore>, &cfg) != cudaSuccess) cudaGetLastError();
+    if (cudaOccupancyMaxActiveClusters(&n, (const void*)tc_wide_kernel<true, false>, &cfg) != cudaSuccess) cudaGetLastError();
     seen[s] = n < 1 ? 1 : n;
   }
   return seen[s];
 }
 
-constexpr int kPairs = 74;        // of SMs
-constexpr int kLeastShare = 3;    // stages
-
-// Row tiles, k-ranges and shares by an estimate of the time in us.  A stage (128 of K) takes its MMAs (7.0e6 multiply-adds per us on an
-// SM), or its way into the SM, or 0.41 us of the hand-overs from load to conversion to MMA.  Sharing (room: bytes there are for the parts)
-// costs its parts' way through L2 and a few round trips; it never makes the sums of a product longer, and with them less exact, than they
-// are without it.
-WidePlan plan_wide(int64_t M, int64_t N, int64_t K, int epi, bool keys, size_t room) {
-  WidePlan best = {}, shared = {};
-  const bool swiglu = epi == kWideSwiglu;
+// Row tiles and k-ranges by an estimate of the time in us.  A stage (128 of K) takes its MMAs (7.0e6 multiply-adds per us on an
+// SM), or its way into the SM, or 0.41 us of the hand-overs from load to conversion to MMA.
+WidePlan plan_wide(int64_t M, int64_t N, int64_t K, bool swiglu, bool keys) {
+  WidePlan best = {};
   const int kblocks = (int)((K + 127) / 128);
   const int tiles = (int)((N + 255) / 256);
   const int least = (int)((M + 255) / 256);
@@ -734,8 +498,6 @@ WidePlan plan_wide(int64_t M, int64_t N, int64_t K, int epi, bool keys, size_t r
     const double mma = p.brows * 128.0 * 128.0 / 7.0e6, intake = stage / 105e3;
     const double a = std::max(std::max(mma, intake), 0.41);
     const int units = tiles * t;
-    p.units = p.whole = units;
-    p.sharers = 0;
     for (int s = 1; s <= (swiglu ? 1 : 4) && s <= kblocks; ++s) {
       if (s == 1) {
         int n = 74;
@@ -746,23 +508,6 @@ WidePlan plan_wide(int64_t M, int64_t N, int64_t K, int epi, bool keys, size_t r
         const double drain = 0.006 * p.brows;   // of an accumulator
         p.cost = 4.0 + turns * (kblocks * a + (p.accs == 1 ? drain : 0.2)) + (p.accs == 2 ? drain : 0.0);
         p.ctas = 2 * n;
-        // the rest of the last turn shared
-        const int full = keys && kPairs / t > 0 ? kPairs / t * t : kPairs, rest = units % full;
-        const long long stages = (long long)rest * kblocks, fits = (long long)(room / ((size_t)p.rows * 1024)) - rest;
-        const int sharers = (int)std::min(std::min((long long)(units > full ? full : kPairs), std::max(stages / kLeastShare, 1LL)), fits);
-        if (rest > 0 && sharers >= rest && stages <= 0x7fffffffLL && (epi != kWideRope || units < full)) {
-          WidePlan q = p;
-          q.nsplit = 1;
-          q.whole = units - rest;
-          q.sharers = sharers;
-          q.ctas = 2 * (q.whole > 0 ? full : sharers);
-          const int per = (int)((stages + sharers - 1) / sharers);
-          q.longest = q.whole > 0 ? kblocks : per;
-          q.cost = 4.0 + (units / full + 1) * (p.accs == 1 ? drain : 0.2) + (p.accs == 2 ? drain : 0.0) + ((double)(units / full) * kblocks + per) * a +
-                   2.0 + 0.004 * p.brows * ((double)sharers / rest + 1.0);
-          q.cost = std::max(q.cost, (double)N * K / 6.3e6);
-          if (shared.sharers == 0 || q.cost < shared.cost * 0.99) shared = q;
-        }
       } else {
         const int fit = max_pair_clusters(s);
         const int waves = (units + fit - 1) / fit;
@@ -771,30 +516,26 @@ WidePlan plan_wide(int64_t M, int64_t N, int64_t K, int epi, bool keys, size_t r
       }
       p.cost = std::max(p.cost, (double)N * K / 6.3e6);
       p.nsplit = s;
-      p.longest = (kblocks + s - 1) / s;
       if (best.nsplit == 0 || p.cost < best.cost * 0.99) best = p;
     }
   }
-  if (shared.sharers > 0 && shared.longest <= best.longest && (epi == kWideRope || shared.cost < best.cost)) return shared;
   return best;
 }
 
-int launch_wide(int epi, const __nv_bfloat16* x, const int8_t* w, int64_t M, int64_t N, int64_t K, const WideScratch& scratch, WideArgs a, bool pdl,
-                cudaStream_t stream) {
+int launch_wide(const __nv_bfloat16* x, const int8_t* w, int64_t M, int64_t N, int64_t K, bool swiglu, WideArgs a, bool pdl, cudaStream_t stream) {
   static DeviceOnce once;
-  int rc = allow_shared_memory(once, kSmemW, true, {(const void*)tc_wide_kernel<true, kWideStore>, (const void*)tc_wide_kernel<false, kWideStore>,
-                                                    (const void*)tc_wide_kernel<false, kWideSwiglu>, (const void*)tc_wide_kernel<false, kWideRope>});
+  int rc = allow_shared_memory(once, kSmemW, true, {(const void*)tc_wide_kernel<false, false>, (const void*)tc_wide_kernel<true, false>,
+                                                    (const void*)tc_wide_kernel<false, true>});
   if (rc != QUASAR_OK) return rc;
-  const WidePlan p = plan_wide(M, N, K, epi, a.keys != nullptr, scratch.parts_bytes);
+  const WidePlan p = plan_wide(M, N, K, swiglu, a.keys != nullptr);
   CUtensorMap map_w, map_x;
-  rc = make_map_sw128(&map_w, w, (uint64_t)N, (uint64_t)K, epi == kWideSwiglu ? 16u : 128u);
+  rc = make_map_sw128(&map_w, w, (uint64_t)N, (uint64_t)K, swiglu ? 16u : 128u);
   if (rc != QUASAR_OK) return rc;
   rc = make_map_sw128(&map_x, x, (uint64_t)M, (uint64_t)K * 2, (uint32_t)(p.brows / 2));
   if (rc != QUASAR_OK) return rc;
   a.M = (int)M; a.N = (int)N; a.kblocks = (int)((K + 127) / 128);
   a.rows = p.rows; a.brows = p.brows; a.row_tiles = p.row_tiles; a.nsplit = p.nsplit; a.stages = p.stages;
-  a.accs = p.accs; a.pieces = p.pieces; a.acc_cols = p.acc_cols; a.units = p.units; a.whole = p.whole; a.sharers = p.sharers;
-  a.parts = scratch.parts; a.arrived = scratch.arrived;
+  a.accs = p.accs; a.pieces = p.pieces; a.acc_cols = p.acc_cols; a.units = p.tiles * p.row_tiles;
   a.early_weights = pdl ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)p.ctas, (unsigned)p.nsplit);
@@ -810,10 +551,9 @@ int launch_wide(int epi, const __nv_bfloat16* x, const int8_t* w, int64_t M, int
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 2u : 1u;
-  if (epi == kWideSwiglu) QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<false, kWideSwiglu>, map_w, map_x, a));
-  else if (epi == kWideRope) QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<false, kWideRope>, map_w, map_x, a));
-  else if (p.nsplit > 1) QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<true, kWideStore>, map_w, map_x, a));
-  else QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<false, kWideStore>, map_w, map_x, a));
+  if (swiglu) QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<false, true>, map_w, map_x, a));
+  else if (p.nsplit > 1) QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<true, false>, map_w, map_x, a));
+  else QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<false, false>, map_w, map_x, a));
   count_launch();
   return QUASAR_OK;
 }
@@ -830,29 +570,17 @@ int launch_wide(int epi, const __nv_bfloat16* x, const int8_t* w, int64_t M, int
 bool tc_wide_better(int64_t M, int64_t K) { return M > kDigitRows || K > 131071; }
 
 int launch_tc_wide(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t N, int64_t K, void* y, bool y_is_f32,
-                   const __nv_bfloat16* residual, unsigned long long* keys, const WideScratch& scratch, int32_t* error, bool pdl,
-                   cudaStream_t stream) {
+                   const __nv_bfloat16* residual, unsigned long long* keys, int32_t* error, bool pdl, cudaStream_t stream) {
   WideArgs a = {};
   a.dw = dw; a.y = y; a.res = residual; a.keys = keys; a.error = error; a.y_is_f32 = y_is_f32 ? 1 : 0;
-  return launch_wide(kWideStore, x, w, M, N, K, scratch, a, pdl, stream);
+  return launch_wide(x, w, M, N, K, false, a, pdl, stream);
 }
 
 int launch_tc_wide_swiglu(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t F, int64_t K, __nv_bfloat16* act,
-                          const WideScratch& scratch, int32_t* error, bool pdl, cudaStream_t stream) {
+                          int32_t* error, bool pdl, cudaStream_t stream) {
   WideArgs a = {};
   a.dw = dw; a.y = act; a.error = error;
-  return launch_wide(kWideSwiglu, x, w, M, 2 * F, K, scratch, a, pdl, stream);
-}
-
-bool tc_wide_rope_fits(int64_t M, int64_t N, int64_t K, const WideScratch& scratch) {
-  return plan_wide(M, N, K, kWideRope, false, scratch.parts_bytes).sharers > 0;
-}
-
-int launch_tc_wide_qkv_rope(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t K, const RopeArgs& rope,
-                            const WideScratch& scratch, int32_t* error, cudaStream_t stream) {
-  WideArgs a = {};
-  a.dw = dw; a.error = error; a.rope = rope;
-  return launch_wide(kWideRope, x, w, M, (int64_t)(rope.Hq + 2 * rope.Hkv) * rope.D, K, scratch, a, true, stream);
+  return launch_wide(x, w, M, 2 * F, K, true, a, pdl, stream);
 }
 
 }  // namespace quasar
