@@ -276,7 +276,7 @@ def test_w4_forms(m, n, k):
 def test_sequences_of_a_batch_attend_as_they_do_alone(batch, rows, prefixes):
     """Segments of one key tile and of several, whole on one thread block or shared, more sequences than a block keeps the places
     of: the first layer's attention, by the cache rows of the second and the logits, against each sequence in a batch of its own."""
-    shape, s_max = synth.SHAPES["tiny_qknorm"], 448
+    shape, s_max = synth.SHAPES["tiny_qknorm"], 960
     m = gpu_model(shape, seed=0, max_seq=s_max)
     kk, vv = synth.kv_prefix(shape, batch, s_max, seed=5, device="cuda")
     lens = torch.tensor([prefixes[0] + (prefixes[1] - prefixes[0]) * b // max(1, batch - 1) for b in range(batch)], dtype=torch.int32, device="cuda")
