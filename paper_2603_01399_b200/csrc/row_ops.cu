@@ -305,7 +305,6 @@ norm_kernel(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ g, int nve
   uint4 gain[V > 0 ? V : 1];
   load_gain<V>(gain, g, nvec);
   pdl_wait();
-  say_ahead(out.ahead);
   const int m = blockIdx.x;
   const uint4* row = reinterpret_cast<const uint4*>(x + (size_t)m * nvec * 8);
   norm_row<OP, V>([&](int i, float (&f)[8]) { unpack8(row[i], f); }, gain, g, nvec, eps, adders, m, out, s_buf);
@@ -350,7 +349,6 @@ operand_kernel(const __nv_bfloat16* x, const unsigned* row_max, int nvec, RowOpe
   float s[8];
   if (OP == kOperandCodes && i < nvec) load_smooth8(out.smooth, i, s);
   pdl_wait();
-  say_ahead(out.ahead);
   const uint32_t top = row_max[m];
   const float amax = __uint_as_float(top);
   float up = 1.f, scale = 1.f;
@@ -383,10 +381,7 @@ attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, Ro
   extern __shared__ __align__(16) unsigned char s_row[];   // this CTA's heads, bf16; then each warp's parts of a batch
   pdl_trigger();
   if (OP != kOperandBf16) tc::cluster_arrive();   // (every CTA of the cluster has started before one writes into another's memory)
-  if (!LIST) {
-    pdl_wait();
-    say_ahead(out.ahead);
-  }   // (the list's description is older than the kernel in front, see tc_attention_kernel)
+  if (!LIST) pdl_wait();   // (the list's description is older than the kernel in front, see tc_attention_kernel)
   const int rank = blockIdx.x % kMergeCtas, m = blockIdx.x / kMergeCtas, b = m / l.T_max, i = m % l.T_max;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
   const int Hq = l.Hkv * l.G, h0 = rank * Hq / kMergeCtas, h1 = (rank + 1) * Hq / kMergeCtas;
@@ -413,10 +408,7 @@ attention_merge_kernel(AttnList l, AttnParts parts, AttnChunks ch, int batch, Ro
     stride = ch.Rpad;
     row0 = i * l.G;
   }
-  if (LIST) {
-    pdl_wait();
-    say_ahead(out.ahead);
-  }
+  if (LIST) pdl_wait();
   float* s_o = reinterpret_cast<float*>(s_row + (size_t)((Hq + kMergeCtas - 1) / kMergeCtas) * D * 2) + (size_t)warp * batch * D;
   uint32_t top = 0;   // of the operand's values, head by head as they are made
   for (int hq = h0 + warp; hq < h1; hq += warps) {
@@ -636,7 +628,6 @@ embed_norm_kernel(BlockArgs a, int M, const __nv_bfloat16* __restrict__ embed, _
     __shared__ unsigned long long s_anc[kRowThreads / 32][QUASAR_MAX_BLOCK];
     const int warp = threadIdx.x >> 5;
     for (int k = threadIdx.x; k < a.n_clear; k += kRowThreads) a.clear[k] = 0u;
-    if (threadIdx.x == 0) *a.ahead_word = 0u;
     for (int b = warp; b < a.B; b += kRowThreads / 32) {
       prepare_sequence(a, b, s_parent[warp], s_anc[warp], s_depth[warp]);
       __syncwarp();

@@ -12,7 +12,7 @@ namespace quasar {
 // y may be nullptr and keys not: then only the rows' arg-max over the output channels is wanted.
 
 int launch_tc_linear_bf16(const __nv_bfloat16* x, const __nv_bfloat16* w, int64_t M, int64_t N, int64_t K, void* y, bool y_is_f32,
-                          const __nv_bfloat16* residual, unsigned long long* keys, int32_t* error, bool pdl, cudaStream_t stream, const Ahead& ahead = {});
+                          const __nv_bfloat16* residual, unsigned long long* keys, int32_t* error, bool pdl, cudaStream_t stream);
 
 // int8 weights, bf16 activations as digit rows: xd [kDigitPlanes M][K] int8 and row_scale [M], see write_digits8
 constexpr int kDigitPlanes = 4;
@@ -20,7 +20,7 @@ constexpr int kDigitRows = 256 / kDigitPlanes;   // rows of a block at most: ope
 int launch_digit_rows(const __nv_bfloat16* x, int64_t M, int64_t K, int8_t* xd, float* row_scale, cudaStream_t stream);
 int launch_tc_linear_digits(const int8_t* xd, const float* row_scale, const int8_t* w, const float* dw, int64_t M, int64_t N,
                             int64_t K, void* y, bool y_is_f32, const __nv_bfloat16* residual, unsigned long long* keys, int32_t* error, bool pdl,
-                            cudaStream_t stream, const Ahead& ahead = {});
+                            cudaStream_t stream);
 
 // the same on the bf16 rows themselves, in one launch, for blocks of up to 6 rows; *done false: not for this matrix, nothing launched
 int launch_tc_linear_direct(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t N, int64_t K, void* y, bool y_is_f32,
@@ -29,18 +29,18 @@ int launch_tc_linear_direct(const __nv_bfloat16* x, const int8_t* w, const float
 // int8 weights, int8 activations with their step sizes (Eq. 8, Eq. 10); acc_out: the raw sums, or nullptr
 int launch_tc_linear_w8a8(const int8_t* xq, const float* dx, const int8_t* w, const float* dw, int64_t M, int64_t N, int64_t K,
                           void* y, bool y_is_f32, const __nv_bfloat16* residual, int32_t* acc_out, unsigned long long* keys, int32_t* error, bool pdl,
-                          cudaStream_t stream, const Ahead& ahead = {});
+                          cudaStream_t stream);
 
 // Layers of the pass with the step that follows in their epilogue (form: OperandForm, which the operand is in; always
 // dependent launches), for blocks that tc_fusable accepts.
 // qkv projection: QK-norm, RoPE and KV append; writes q (into rope.qkv) and the cache rows.
 bool tc_fusable(int form, int64_t M);
 int launch_tc_qkv_rope(int form, const void* x, const float* dx, const void* w, const float* dw, int64_t M, int64_t K, const RopeArgs& rope,
-                       const Ahead& ahead, int32_t* error, cudaStream_t stream);
+                       int32_t* error, cudaStream_t stream);
 // gate+up projection: act = silu(gate) * up, [M][F] bf16; act_max [M] (zero before): bits of each row's largest magnitude,
 // times the smoothing factors of the down projection's input if there are any
 int launch_tc_gateup_swiglu(int form, const void* x, const float* dx, const void* w, const float* dw, int64_t M, int64_t F, int64_t K,
-                            __nv_bfloat16* act, unsigned* act_max, const float* smooth, const Ahead& ahead, int32_t* error, cudaStream_t stream);
+                            __nv_bfloat16* act, unsigned* act_max, const float* smooth, int32_t* error, cudaStream_t stream);
 
 #ifdef __CUDACC__
 // Order-preserving key of a value and its index: the larger key is the larger value and, among equals, the lower index.
