@@ -423,18 +423,11 @@ def quasar_kv_commit(model: Model, kv: KVCache, buf: VerifyBuffers, tree: bool =
                                   _ptr(buf.accept_path) if tree else None, buf.batch, buf.t_max, _stream()))
 
 
-def _row_ints(like: torch.Tensor, b: int, device) -> torch.Tensor:
-    """int32 [b] for a result.  (After a tensor of that kind: half the time of spelling out type and device.)"""
-    if like.dtype == torch.int32 and like.dim() == 1 and like.shape[0] == b and like.device == device and like.is_contiguous():
-        return torch.empty_like(like)
-    return torch.empty(b, dtype=torch.int32, device=device)
-
-
 def quasar_ngram_draft(history: torch.Tensor, hist_len: torch.Tensor, gamma: int, k_min: int, k_max: int):
     """history int32 [B][S], hist_len int32 [B] -> (draft int32 [B][gamma], draft_len int32 [B])."""
     b, s = history.shape
     draft = torch.empty(b, gamma, dtype=torch.int32, device=history.device)
-    dlen = _row_ints(hist_len, b, history.device)
+    dlen = torch.empty(b, dtype=torch.int32, device=history.device)
     _check(lib().quasar_ngram_draft(_ptr(history), _ptr(hist_len), b, s, gamma, k_min, k_max, _ptr(draft), _ptr(dlen), _stream()))
     return draft, dlen
 
@@ -444,8 +437,8 @@ def quasar_accept_stochastic(logits: torch.Tensor, tokens: torch.Tensor, block_l
     """logits fp32 [B][T][V]; tokens int32 [B][T]; block_len int32 [B]; q_probs fp32 [B][T][V] or None;
     r_accept fp32 [B][T]; r_sample fp32 [B].  Returns (accept_len, next_token), int32 [B]."""
     b, t, v = logits.shape
-    accept_len = _row_ints(block_len, b, logits.device)
-    nxt = _row_ints(block_len, b, logits.device)
+    accept_len = torch.empty(b, dtype=torch.int32, device=logits.device)
+    nxt = torch.empty(b, dtype=torch.int32, device=logits.device)
     ws = torch.empty(_bytes("quasar_accept_stochastic_workspace_bytes", b, t), dtype=torch.uint8, device=logits.device)
     _check(lib().quasar_accept_stochastic(_ptr(logits), _ptr(tokens), _ptr(block_len), _ptr(q_probs), b, t, v, temperature,
                                           _ptr(r_accept), _ptr(r_sample), _ptr(accept_len), _ptr(nxt), _ptr(ws), ws.numel(),
