@@ -27,6 +27,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "rope.cuh"
 #include "tc_common.cuh"
 #include "tc_linear.cuh"
 #include "tc_wide.cuh"
@@ -56,7 +57,14 @@ struct WideArgs {
   int acc_cols;                // columns from one accumulator to the next
   int units;
   int y_is_f32, early_weights;
+  RopeArgs rope;               // kWideRope
 };
+
+// What is done with a unit's finished sums: stored; multiplied as gate and up units; or made q, k and v (QK-norm, RoPE, cache
+// append: only behind ranges, whose exchange leaves whole rows of a head to a warp; a kernel and a pass over q, k and v less.  A pass
+// of 8 x 9 rows through the 8B shape 4104 -> 3953 us, of a 17-node tree x 4 through the 14B shape 5523 -> 5364; 8 x 64 rows 9681 -> 9638,
+// within the noise.  Tiles in turn keep the separate kernel: their epilogue has a channel a lane)
+enum WideEpilogue { kWideStore = 0, kWideSwiglu = 1, kWideRope = 2 };
 
 // four int8 -> four bf16, exactly: 0x43bb is 128 + bb for the low seven bits, and the sign bit asks for 256 instead of 128 to go
 __device__ __forceinline__ void bf16x4(uint32_t w, uint32_t& lo, uint32_t& hi) {
@@ -89,9 +97,10 @@ __device__ __forceinline__ int channel_of(int n0, int r, int N) {
   return (r & 16) ? N / 2 + u : u;
 }
 
-template <bool SPLIT, bool SWIGLU>
+template <bool SPLIT, int EPI>
 __global__ void __launch_bounds__(kThreadsW, 1)
 tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const WideArgs a) {
+  constexpr bool SWIGLU = EPI == kWideSwiglu;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // the swizzle repeats every 1024 bytes
   const int b_half = a.brows / 2;                // rows of operand B of this CTA
@@ -152,7 +161,9 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   fence_after();
   const uint32_t tmem = *tmem_slot;
   const uint32_t tmem_a = tmem + (uint32_t)(a.accs * a.acc_cols);
-  if (threadIdx.x == 0) pdl_trigger();   // (a tcgen05 kernel behind this one waits for it while it holds tensor memory)
+  // (A tcgen05 kernel behind this one waits for it while it holds tensor memory.  Behind the qkv projection it is the attention, which
+  // counts on everything in front of THIS kernel being complete: see below.)
+  if (EPI != kWideRope && threadIdx.x == 0) pdl_trigger();
 
   if (warp == 0) {
     // ---- TMA producer ----
@@ -349,6 +360,10 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       }
     }
   }
+  if (EPI == kWideRope && warp == 18) {
+    pdl_wait();
+    if (lane == 0) pdl_trigger();
+  }
   if (SPLIT && warp >= 2) {
     // ---- this range's sums to shared memory, [row][channel] (the ring is idle then: every load has landed and every MMA read it) ----
     const int q = warp & 3, r = q * 32 + lane;
@@ -383,6 +398,8 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
 #pragma unroll
       for (int e = 0; e < 4; ++e) dw[e] = n + e < a.N ? __ldg(a.dw + n + e) : 1.f;
       for (int m = split * per + warp; m < r_end; m += kThreadsW / 32) {
+        RopeRow rope;
+        if constexpr (EPI == kWideRope) rope_row_load(rope, a.rope, m0 + m, chan_of(first));
         uint4 p[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k)
@@ -394,6 +411,13 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
           const uint32_t v[4] = {p[k].x, p[k].y, p[k].z, p[k].w};
 #pragma unroll
           for (int e = 0; e < 4; ++e) f[e] = k == 0 ? __uint_as_float(v[e]) : f[e] + __uint_as_float(v[e]);
+        }
+        if constexpr (EPI == kWideRope) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) f[e] = round_bf16(f[e] * dw[e]);
+          if (a.rope.D == 128) rope_row_store<128>(a.rope, f, m0 + m, chan_of(first), rope);
+          else rope_row_store<64>(a.rope, f, m0 + m, chan_of(first), rope);
+          continue;
         }
         unsigned long long best = 0;
         const size_t idx = (size_t)(m0 + m) * a.N + n;
@@ -451,7 +475,14 @@ struct WidePlan {
   double cost;
 };
 
-// Clusters of s pairs that the device holds at once (they lie within a group of SMs, so long ones leave SMs unused).
+int allow_wide() {
+  static DeviceOnce once;
+  return allow_shared_memory(once, kSmemW, true, {(const void*)tc_wide_kernel<false, kWideStore>, (const void*)tc_wide_kernel<true, kWideStore>,
+                                                  (const void*)tc_wide_kernel<false, kWideSwiglu>, (const void*)tc_wide_kernel<true, kWideRope>});
+}
+
+// Clusters of s pairs that the device holds at once (they lie within a group of SMs, so long ones leave SMs unused).  The kernels'
+// shared memory is allowed first, whoever asks: without it the answer is none, and it is kept.
 int max_pair_clusters(int s) {
   static std::mutex mu;
   static int seen[5] = {};
@@ -469,7 +500,8 @@ int max_pair_clusters(int s) {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, (const void*)tc_wide_kernel<true, false>, &cfg) != cudaSuccess) cudaGetLastError();
+    if (allow_wide() != QUASAR_OK || cudaOccupancyMaxActiveClusters(&n, (const void*)tc_wide_kernel<true, kWideStore>, &cfg) != cudaSuccess)
+      cudaGetLastError();
     seen[s] = n < 1 ? 1 : n;
   }
   return seen[s];
@@ -522,10 +554,9 @@ WidePlan plan_wide(int64_t M, int64_t N, int64_t K, bool swiglu, bool keys) {
   return best;
 }
 
-int launch_wide(const __nv_bfloat16* x, const int8_t* w, int64_t M, int64_t N, int64_t K, bool swiglu, WideArgs a, bool pdl, cudaStream_t stream) {
-  static DeviceOnce once;
-  int rc = allow_shared_memory(once, kSmemW, true, {(const void*)tc_wide_kernel<false, false>, (const void*)tc_wide_kernel<true, false>,
-                                                    (const void*)tc_wide_kernel<false, true>});
+int launch_wide(int epi, const __nv_bfloat16* x, const int8_t* w, int64_t M, int64_t N, int64_t K, WideArgs a, bool pdl, cudaStream_t stream) {
+  const bool swiglu = epi == kWideSwiglu;
+  int rc = allow_wide();
   if (rc != QUASAR_OK) return rc;
   const WidePlan p = plan_wide(M, N, K, swiglu, a.keys != nullptr);
   CUtensorMap map_w, map_x;
@@ -551,9 +582,10 @@ int launch_wide(const __nv_bfloat16* x, const int8_t* w, int64_t M, int64_t N, i
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 2u : 1u;
-  if (swiglu) QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<false, true>, map_w, map_x, a));
-  else if (p.nsplit > 1) QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<true, false>, map_w, map_x, a));
-  else QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<false, false>, map_w, map_x, a));
+  if (swiglu) QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<false, kWideSwiglu>, map_w, map_x, a));
+  else if (epi == kWideRope) QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<true, kWideRope>, map_w, map_x, a));
+  else if (p.nsplit > 1) QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<true, kWideStore>, map_w, map_x, a));
+  else QUASAR_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tc_wide_kernel<false, kWideStore>, map_w, map_x, a));
   count_launch();
   return QUASAR_OK;
 }
@@ -573,14 +605,23 @@ int launch_tc_wide(const __nv_bfloat16* x, const int8_t* w, const float* dw, int
                    const __nv_bfloat16* residual, unsigned long long* keys, int32_t* error, bool pdl, cudaStream_t stream) {
   WideArgs a = {};
   a.dw = dw; a.y = y; a.res = residual; a.keys = keys; a.error = error; a.y_is_f32 = y_is_f32 ? 1 : 0;
-  return launch_wide(x, w, M, N, K, false, a, pdl, stream);
+  return launch_wide(kWideStore, x, w, M, N, K, a, pdl, stream);
 }
 
 int launch_tc_wide_swiglu(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t F, int64_t K, __nv_bfloat16* act,
                           int32_t* error, bool pdl, cudaStream_t stream) {
   WideArgs a = {};
   a.dw = dw; a.y = act; a.error = error;
-  return launch_wide(x, w, M, 2 * F, K, true, a, pdl, stream);
+  return launch_wide(kWideSwiglu, x, w, M, 2 * F, K, a, pdl, stream);
+}
+
+bool tc_wide_rope_fits(int64_t M, int64_t N, int64_t K) { return plan_wide(M, N, K, false, false).nsplit > 1; }
+
+int launch_tc_wide_qkv_rope(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t K, const RopeArgs& rope, int32_t* error,
+                            cudaStream_t stream) {
+  WideArgs a = {};
+  a.dw = dw; a.error = error; a.rope = rope;
+  return launch_wide(kWideRope, x, w, M, (int64_t)(rope.Hq + 2 * rope.Hkv) * rope.D, K, a, true, stream);
 }
 
 }  // namespace quasar

@@ -2,6 +2,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "rope.cuh"
 
 namespace quasar {
 
@@ -14,5 +15,10 @@ int launch_tc_wide(const __nv_bfloat16* x, const int8_t* w, const float* dw, int
 // gate+up projection: act = silu(gate) * up, [M][F] bf16
 int launch_tc_wide_swiglu(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t F, int64_t K, __nv_bfloat16* act,
                           int32_t* error, bool pdl, cudaStream_t stream);
+// qkv projection with QK-norm, RoPE and KV append (a dependent launch), where tc_wide_rope_fits says that the layer runs as k-ranges;
+// writes q (into rope.qkv) and the cache rows
+bool tc_wide_rope_fits(int64_t M, int64_t N, int64_t K);
+int launch_tc_wide_qkv_rope(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t K, const RopeArgs& rope, int32_t* error,
+                            cudaStream_t stream);
 
 }  // namespace quasar
