@@ -235,9 +235,9 @@ def test_a_workspace_that_holds_some_of_the_rows(room):
     assert bool((ws[65536 + room:] == 7).all())
 
 
-# rows: one, two blocks of 16, the most that two accumulators hold; channels: the narrowest tiles of the form, and a last one that is cut
+# rows: one, some, the most of the form and one more; channels: the narrowest tiles of the form, and a last one that is cut
 @pytest.mark.parametrize("ffn", [9536, 12288])
-@pytest.mark.parametrize("batch,rows", [(1, 1), (1, 6), (2, 16), (3, 11), (2, 64)])
+@pytest.mark.parametrize("batch,rows", [(1, 1), (1, 6), (2, 4), (3, 3)])
 def test_gateup_on_bf16_weights_in_one_wave_of_wide_tiles(batch, rows, ffn):
     """Two gate+up tiles on one thread block (SwiGLU in the epilogue) against the plain layer and SwiGLU behind it, which a trace
     asks for: the same sums in another order, so the logits agree as the forms of a layer do."""
