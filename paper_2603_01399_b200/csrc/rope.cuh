@@ -83,13 +83,13 @@ __device__ __forceinline__ void rope_row_load(RopeRow& p, const RopeArgs& r, int
   }
 }
 
-// The row, four channels a lane, f as the linear layer's bf16 output: q and k heads normalised, rotated and put in their places,
-// v heads copied.
+// The row (of `width` channels in all), four channels a lane, f as the linear layer's bf16 output: q and k heads normalised, rotated
+// and put in their places, v heads copied.
 template <int D>
-__device__ __forceinline__ void rope_row_store(const RopeArgs& r, const float (&f)[4], int m, int n0, const RopeRow& p) {
+__device__ __forceinline__ void rope_row_store(const RopeArgs& r, const float (&f)[4], int m, int n0, int width, const RopeRow& p) {
   const int lane = threadIdx.x & 31;
   if (p.slot < 0) return;
-  const int b = m / r.T_max, width = (r.Hq + 2 * r.Hkv) * r.D;
+  const int b = m / r.T_max;
 #pragma unroll
   for (int h = 0; h < 128 / D; ++h) {
     const int head = n0 / D + h;

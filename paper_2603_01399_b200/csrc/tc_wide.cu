@@ -415,8 +415,8 @@ tc_wide_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         if constexpr (EPI == kWideRope) {
 #pragma unroll
           for (int e = 0; e < 4; ++e) f[e] = round_bf16(f[e] * dw[e]);
-          if (a.rope.D == 128) rope_row_store<128>(a.rope, f, m0 + m, chan_of(first), rope);
-          else rope_row_store<64>(a.rope, f, m0 + m, chan_of(first), rope);
+          if (a.rope.D == 128) rope_row_store<128>(a.rope, f, m0 + m, chan_of(first), a.N, rope);
+          else rope_row_store<64>(a.rope, f, m0 + m, chan_of(first), a.N, rope);
           continue;
         }
         unsigned long long best = 0;
