@@ -63,7 +63,8 @@ struct WideArgs {
 // What is done with a unit's finished sums: stored; multiplied as gate and up units; or made q, k and v (QK-norm, RoPE, cache
 // append: only behind ranges, whose exchange leaves whole rows of a head to a warp; a kernel and a pass over q, k and v less.  A pass
 // of 8 x 9 rows through the 8B shape 4104 -> 3953 us, of a 17-node tree x 4 through the 14B shape 5523 -> 5364; 8 x 64 rows 9681 -> 9638,
-// within the noise.  Tiles in turn keep the separate kernel: their epilogue has a channel a lane)
+// within the noise.  Tiles without ranges keep the separate kernel: eight rows a warp, one after the other, cost more than it does, 8 x 64
+// rows 9592 -> 9765)
 enum WideEpilogue { kWideStore = 0, kWideSwiglu = 1, kWideRope = 2 };
 
 // four int8 -> four bf16, exactly: 0x43bb is 128 + bb for the low seven bits, and the sign bit asks for 256 instead of 128 to go
