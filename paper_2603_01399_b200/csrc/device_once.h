@@ -1,4 +1,4 @@
-// What has to be done once on every device of a process (host code, no CUDA headers).
+// What has to be done once, or asked once, on every device of a process (host code, no CUDA headers).
 #pragma once
 
 #include <stdint.h>
@@ -22,6 +22,27 @@ class DeviceOnce {
 
  private:
   std::atomic<uint64_t> done_{0};
+};
+
+// Whole numbers that depend on nothing but the device: N questions.
+template <int N>
+class DeviceAnswers {
+ public:
+  // ask() returns a positive number, which is kept for `device`, or 0 where it could not be had: then the next call asks again.
+  template <typename F>
+  int get(int device, int question, F&& ask) {
+    const bool kept = device >= 0 && device < 64 && question >= 0 && question < N;
+    if (kept) {
+      const int n = seen_[device][question].load(std::memory_order_relaxed);
+      if (n > 0) return n;
+    }
+    const int n = ask();
+    if (kept && n > 0) seen_[device][question].store(n, std::memory_order_relaxed);
+    return n;
+  }
+
+ private:
+  std::atomic<int> seen_[64][N] = {};
 };
 
 }  // namespace quasar

@@ -14,7 +14,6 @@
 // accumulation per group, folded into the running sum with the group's step size.  The ranges of a channel block form a
 // cluster and add their sums through distributed shared memory in the order of the ranges.
 #include <algorithm>
-#include <mutex>
 
 #include "common.cuh"
 #include "quant.cuh"
@@ -238,29 +237,11 @@ __global__ void __launch_bounds__(kW4Threads) w4_gemm_kernel(W4Args a) {
 }
 
 // Clusters of s CTAs with this much shared memory that the device holds at once (they lie within a group of SMs, so long ones
-// leave SMs unused).
+// leave SMs unused); 1 for a call where that cannot be found out.
 template <int NT>
-int w4_clusters(int s, int chunk, size_t smem) {
-  static std::mutex mu;
-  static int seen[9][64] = {};
-  std::lock_guard<std::mutex> lock(mu);
-  int& n = seen[s][chunk];
-  if (n == 0) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(1, (unsigned)s);
-    cfg.blockDim = dim3(kW4Threads);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = 1;
-    attr.val.clusterDim.y = (unsigned)s;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, w4_gemm_kernel<NT>, &cfg) != cudaSuccess) cudaGetLastError();
-    if (n < 1) n = 1;
-  }
-  return n;
+int w4_clusters(int device, int s, int chunk, size_t smem) {
+  static DeviceAnswers<9 * 64> kept;
+  return std::max(1, clusters_at_once(kept, device, s * 64 + chunk, (const void*)w4_gemm_kernel<NT>, kW4Threads, smem, 1, (unsigned)s));
 }
 
 template <int NT>
@@ -268,6 +249,7 @@ int launch_w4_nt(W4Args a, cudaStream_t stream) {
   static DeviceOnce once;
   const int rc = allow_shared_memory(once, 100 * 1024, false, {(const void*)w4_gemm_kernel<NT>});
   if (rc != QUASAR_OK) return rc;
+  const int device = current_device();
   const int nblocks = (a.N + kW4BlockN - 1) / kW4BlockN, ngroups = a.K / kGroup;
   // Ranges: a launch takes the waves of clusters that the device holds at once - where they do not all fit, half a one more, as
   // CTAs follow one another - times the groups of a range and what a range costs besides, about three groups.  No range shorter
@@ -283,7 +265,7 @@ int launch_w4_nt(W4Args a, cudaStream_t stream) {
     if (chunk > kW4Ahead) chunk = chunk / kW4Ahead * kW4Ahead;
     chunk = std::min(chunk, per);
     const size_t need = std::max((size_t)chunk * kGroupBytes, (size_t)NT * 8 * kW4BlockN * 4);
-    const double waves = (double)nblocks / w4_clusters<NT>(s, chunk, need);
+    const double waves = (double)nblocks / w4_clusters<NT>(device, s, chunk, need);
     const double cost = (waves > 1 ? waves + 0.5 : 1.0) * (per + 3);
     if (a.nsplit == 0 || cost < best) {
       best = cost;

@@ -25,7 +25,6 @@
 #include <math.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "rope.cuh"
 #include "tc_common.cuh"
@@ -483,35 +482,18 @@ int allow_wide() {
 }
 
 // Clusters of s pairs that the device holds at once (they lie within a group of SMs, so long ones leave SMs unused).  The kernels'
-// shared memory is allowed first, whoever asks: without it the answer is none, and it is kept.
-int max_pair_clusters(int s) {
-  static std::mutex mu;
-  static int seen[5] = {};
-  std::lock_guard<std::mutex> lock(mu);
-  if (seen[s] == 0) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2, (unsigned)s);
-    cfg.blockDim = dim3(kThreadsW);
-    cfg.dynamicSmemBytes = kSmemW;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = 2;
-    attr.val.clusterDim.y = (unsigned)s;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (allow_wide() != QUASAR_OK || cudaOccupancyMaxActiveClusters(&n, (const void*)tc_wide_kernel<true, kWideStore>, &cfg) != cudaSuccess)
-      cudaGetLastError();
-    seen[s] = n < 1 ? 1 : n;
-  }
-  return seen[s];
+// shared memory has to be allowed first.  Where the question fails this plan goes by one, and the next one asks again.
+int max_pair_clusters(int device, int s) {
+  static DeviceAnswers<5> kept;
+  return std::max(1, clusters_at_once(kept, device, s, (const void*)tc_wide_kernel<true, kWideStore>, kThreadsW, kSmemW, 2, (unsigned)s));
 }
 
 // Row tiles and k-ranges by an estimate of the time in us.  A stage (128 of K) takes its MMAs (7.0e6 multiply-adds per us on an
 // SM), or its way into the SM, or 0.41 us of the hand-overs from load to conversion to MMA.
 WidePlan plan_wide(int64_t M, int64_t N, int64_t K, bool swiglu, bool keys) {
   WidePlan best = {};
+  const int device = current_device();
+  const bool allowed = allow_wide() == QUASAR_OK;
   const int kblocks = (int)((K + 127) / 128);
   const int tiles = (int)((N + 255) / 256);
   const int least = (int)((M + 255) / 256);
@@ -542,7 +524,7 @@ WidePlan plan_wide(int64_t M, int64_t N, int64_t K, bool swiglu, bool keys) {
         p.cost = 4.0 + turns * (kblocks * a + (p.accs == 1 ? drain : 0.2)) + (p.accs == 2 ? drain : 0.0);
         p.ctas = 2 * n;
       } else {
-        const int fit = max_pair_clusters(s);
+        const int fit = allowed ? max_pair_clusters(device, s) : 1;
         const int waves = (units + fit - 1) / fit;
         p.cost = waves * (6.0 + (kblocks + s - 1) / s * a + 0.012 * p.brows) + 0.3 * s;
         p.ctas = 2 * units;

@@ -30,6 +30,44 @@ def test_work_runs_once_on_each_device_and_again_after_a_failure(tmp_path):
     assert subprocess.check_output([str(exe)], text=True) == "5 2"
 
 
+ANSWERS = r'''
+#include <stdio.h>
+#include "device_once.h"
+int main() {
+  static quasar::DeviceAnswers<5> kept;
+  int asked = 0, next = 0;
+  auto ask = [&] { ++asked; return next; };
+  if (kept.get(0, 2, ask) != 0 || asked != 1) return 1;                       // could not be had: not kept
+  next = 33;
+  if (kept.get(0, 2, ask) != 33 || kept.get(0, 2, ask) != 33 || asked != 2) return 2;
+  next = 15;
+  if (kept.get(0, 4, ask) != 15 || kept.get(0, 2, ask) != 33 || asked != 3) return 3;      // another question
+  if (kept.get(1, 2, ask) != 15 || kept.get(0, 2, ask) != 33 || kept.get(1, 2, ask) != 15 || asked != 4) return 4;   // another device
+  if (kept.get(63, 0, ask) != 15 || kept.get(63, 0, ask) != 15 || asked != 5) return 5;
+  if (kept.get(64, 0, ask) != 15 || kept.get(64, 0, ask) != 15 || kept.get(-1, 0, ask) != 15 || asked != 8) return 6;   // beyond what is kept: each time
+  printf("ok");
+  return 0;
+}
+'''
+
+
+def test_answers_are_kept_for_their_device_and_only_when_there_is_one(tmp_path):
+    src, exe = tmp_path / "answers.cpp", tmp_path / "answers"
+    src.write_text(ANSWERS)
+    subprocess.check_call(["g++", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)])
+    assert subprocess.check_output([str(exe)], text=True) == "ok"
+
+
+def test_what_a_device_holds_at_once_is_asked_in_one_place():
+    """clusters_at_once, which keeps answers only: a function of its own beside it once kept a failed question for the process."""
+    found = []
+    for name in sorted(os.listdir(CSRC)):
+        if name.endswith((".cu", ".cuh", ".h")):
+            text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+            found += [name] * text.count("cudaOccupancyMaxActiveClusters")
+    assert found == ["common.cuh"]
+
+
 def test_no_kernel_sets_its_attributes_any_other_way():
     found = []
     for name in sorted(os.listdir(CSRC)):
