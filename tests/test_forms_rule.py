@@ -1,0 +1,58 @@
+"""Which form the gate+up projection on bf16 weights takes (host code, no GPU needed): one wave of wide tiles only where that was
+measured to be the quicker one."""
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2603_01399_b200", "csrc")
+
+PROGRAM = r'''
+#include <stdio.h>
+#include "tc_dual.h"
+int main() {
+  long long m, n, k;
+  while (scanf("%lld %lld %lld", &m, &n, &k) == 3) printf("%d\n", quasar::dual_channels(m, n, k));
+  return 0;
+}
+'''
+
+
+@pytest.fixture(scope="module")
+def channels(tmp_path_factory):
+    where = tmp_path_factory.mktemp("rule")
+    src, exe = where / "rule.cpp", where / "rule"
+    src.write_text(PROGRAM)
+    subprocess.check_call(["g++", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)])
+
+    def ask(cases):
+        text = "".join("%d %d %d\n" % c for c in cases)
+        return [int(x) for x in subprocess.run([str(exe)], input=text, text=True, check=True, capture_output=True).stdout.split()]
+
+    return ask
+
+
+def test_wide_tiles_where_they_won(channels):
+    cases = [(m, 24576, 4096) for m in (1, 2, 4, 6, 8)] + [(8, 19072, 4096), (8, 28672, 4096), (3, 22016, 3584), (1, 24576, 5120)]
+    cases += [(m, n, k) for m in (1, 8) for n, k in ((19072, 4096), (22016, 3600), (30784, 4096))]     # as the GPU test runs them
+    assert channels(cases) == [176] * 5 + [144, 208, 160, 176] + [144, 160, 208] * 2
+
+
+def test_tiles_of_128_where_wide_ones_lost(channels):
+    """34,816 x 5120 (the 14B shape): 117 us a layer and 0.3 to 1.7 more in tiles of 240."""
+    cases = [(m, 34816, 5120) for m in (1, 2, 4, 6, 8)]
+    cases += [(m, n, k) for m in (1, 8) for n in (34816, 37888) for k in (3584, 4096)]              # 240 and 256 channels
+    cases += [(6, 24576, 5120), (8, 24576, 4608), (3, 24576, 5120), (1, 24576, 8192)]               # long contractions
+    cases += [(1, 19072, 2048), (4, 37888, 2048), (1, 24576, 512), (8, 19456, 2560)]                # short ones
+    cases += [(9, 24576, 4096), (64, 24576, 4096), (1, 18944, 4096), (1, 1376, 256), (0, 24576, 4096)]   # rows; tiles of 128 do
+    assert channels(cases) == [0] * len(cases)
+
+
+def test_the_tiles_of_one_wave(channels):
+    """Multiples of 16 that cover all channels with at most 148 tiles, and what a ring and two accumulators have room for."""
+    cases = [(1, 2 * f, 4096) for f in range(9000, 20000, 16)]
+    for (_, n, _), c in zip(cases, channels(cases)):
+        if c:
+            assert c % 16 == 0 and 128 < c <= 208 and 148 * c >= n and 148 * (c - 16) < n
+        else:
+            assert n <= 148 * 128 or n > 148 * 208
