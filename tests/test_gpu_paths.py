@@ -265,36 +265,49 @@ def test_gateup_on_bf16_weights_in_one_wave_of_wide_tiles(batch, rows, hidden, f
     assert bool(((fused - plain).abs() <= 2.0 ** -6 * plain.pow(2).mean(dim=-1, keepdim=True).sqrt() + 1e-2 * plain.abs()).all())
 
 
-# rows: the fewest of the wide form, two row tiles with blocks that end early; heads: whole tiles of 256 channels, and a last one cut
+# rows: the fewest of the wide form, one row tile with several rows a warp, two row tiles, blocks that end early; heads: whole tiles
+# of 256 channels, and a last one cut
 @pytest.mark.parametrize("heads,kv_heads,dim,norm", [(8, 2, 128, True), (6, 2, 64, False)])
-@pytest.mark.parametrize("batch,rows", [(5, 13), (2, 40), (5, 60)])
-def test_wide_qkv_rows_finish_as_those_of_the_layer_and_the_kernel_behind_it(batch, rows, heads, kv_heads, dim, norm):
-    """QK-norm, RoPE and cache append where the sums of the k-ranges join, against the two kernels that a trace asks for: the cache
-    rows of the first layer are the same bits, and no other rows of the cache are written."""
+@pytest.mark.parametrize("batch,rows,tree", [(5, 13, False), (2, 40, False), (5, 60, False), (4, 17, True), (8, 24, False)])
+def test_wide_qkv_rows_finish_as_those_of_the_layer_and_the_kernel_behind_it(batch, rows, tree, heads, kv_heads, dim, norm):
+    """QK-norm, RoPE and cache append where the sums of the k-ranges join, against the two kernels that a trace asks for: the same
+    bits.  The FFNs give zeros, so what stands between one layer's q, k and v and the next one's are the same kernels on both sides:
+    a q head in the wrong place or with the wrong gain shows in the second layer's cache rows and in the logits.  No other rows of
+    the cache are written."""
     shape, s_max = synth.ModelShape("wide_qkv", 2, 2048, heads, kv_heads, dim, 512, 512, norm), 128
     m = gpu_model(shape, seed=0, int8=True, max_seq=s_max, gen_device="cuda")
+    for layer in range(2):
+        m.tensors[f"l{layer}.gateup_delta"].zero_()
     kk, vv = synth.kv_prefix(shape, batch, s_max, seed=3, device="cuda")
     tokens = synth.uniform_tokens((batch, rows), shape.vocab, 5).to(torch.int32)
     lens = torch.tensor([rows - b % 3 for b in range(batch)], dtype=torch.int32)
+    g = torch.Generator().manual_seed(rows)
+    parents = torch.tensor([[-1] + [int(torch.randint(0, i, (1,), generator=g)) for i in range(1, rows)] for _ in range(batch)], dtype=torch.int32)
 
     def run(traced):
         seq = torch.arange(30, 30 + batch, dtype=torch.int32, device="cuda")
         kv = binding.KVCache(shape, batch, s_max, k=kk.clone(), v=vv.clone(), seq_len=seq)
-        buf = binding.VerifyBuffers(m, batch, rows)
+        buf = binding.VerifyBuffers(m, batch, rows, tree=tree)
         buf.tokens.copy_(tokens)
         buf.block_len.copy_(lens)
+        if tree:
+            buf.parents.copy_(parents)
         if traced:
             m.set_trace(torch.empty(m.trace_bytes(batch, rows), dtype=torch.uint8, device="cuda"))
+        before = binding.kernel_launches()
         binding.quasar_verify(m, kv, buf)
+        launches = binding.kernel_launches() - before
         torch.cuda.synchronize()
         m.set_trace(None)
         assert int(buf.status[0]) == 0
-        return kv
+        return kv, buf.logits, launches
 
-    kv, kv_t = run(False), run(True)
-    assert torch.equal(kv.k[0], kv_t.k[0]) and torch.equal(kv.v[0], kv_t.v[0])
+    (kv, logits, launches), (kv_t, logits_t, launches_t) = run(False), run(True)
+    assert launches_t - launches == 2 * 2     # a layer's RoPE kernel and its SwiGLU kernel: both forms ran
+    assert torch.equal(kv.k, kv_t.k) and torch.equal(kv.v, kv_t.v)
     rows_written = torch.zeros(batch, s_max, dtype=torch.bool)
     for b in range(batch):
         rows_written[b, 30 + b:30 + b + int(lens[b])] = True
+        assert torch.equal(logits[b, :int(lens[b])], logits_t[b, :int(lens[b])])
     for new, old in ((kv.k, kk), (kv.v, vv)):   # [layer][sequence][head][position][channel]
         assert torch.equal((new != old).any(dim=-1).any(dim=2).any(dim=0).cpu(), rows_written)
