@@ -311,3 +311,69 @@ def test_wide_qkv_rows_finish_as_those_of_the_layer_and_the_kernel_behind_it(bat
         assert torch.equal(logits[b, :int(lens[b])], logits_t[b, :int(lens[b])])
     for new, old in ((kv.k, kk), (kv.v, vv)):   # [layer][sequence][head][position][channel]
         assert torch.equal((new != old).any(dim=-1).any(dim=2).any(dim=0).cpu(), rows_written)
+
+
+@pytest.mark.parametrize("top", [254.0, 255.0, 128.0, 129.0])
+@pytest.mark.parametrize("k", [256, 4096, 12288])
+def test_quantiser_at_the_middles_between_codes(top, k):
+    """A row whose maximum is 254 / 256 of a power of two has step sizes that put bf16 values on exact middles all along, other
+    maxima near them now and then: the codes are those of the rounded quotient everywhere, of the 4-bit groups too."""
+    n = 37
+    g = torch.Generator().manual_seed(int(top) + k)
+    w = (torch.randint(-int(top), int(top) + 1, (n, k), generator=g).float() * 2.0 ** torch.randint(-9, 1, (n, k), generator=g)).to(torch.bfloat16)
+    w[:, ::128] = top
+    w = w * 2.0 ** -12
+    q, d = binding.quasar_quantize(w.cuda())
+    delta = w.float().abs().amax(1) / 127.0
+    assert torch.equal(d.cpu(), delta)
+    assert torch.equal(q.cpu(), torch.round(w.float() / delta[:, None]).to(torch.int8))
+    packed, d4 = binding.quasar_quantize_int4(w.cuda())
+    groups = w.float().view(n, k // 128, 128)
+    delta4 = groups.abs().amax(2) / 7.0
+    codes = torch.round(groups / delta4[..., None]).to(torch.int32).view(n, k)
+    assert torch.equal(d4.cpu(), delta4)
+    assert torch.equal(packed.cpu().to(torch.int32), (codes[:, ::2] & 15) | ((codes[:, 1::2] & 15) << 4))
+
+
+# rows: one block of 16 and its edges, two launches; channels: part of a tile, an odd count, more tiles than SMs; groups: one, odd, ranges
+@pytest.mark.parametrize("m,n,k", [(1, 129, 128), (15, 1001, 384), (16, 4096, 1152), (17, 130, 640), (33, 19077, 256), (48, 515, 2048),
+                                   (64, 20480, 384), (65, 300, 896), (5, 1376, 12288)])
+def test_w4_forms(m, n, k):
+    x = synth.normal_bf16((m, k), 1.0, seed=m + n, device="cuda")
+    packed, d = binding.quasar_quantize_int4(synth.normal_bf16((n, k), 0.02, seed=n + k, device="cuda"))
+    p = packed.to(torch.int32)
+    codes = torch.stack([p & 15, p >> 4], dim=2).view(n, k)
+    w = (codes - 16 * (codes > 7)).double() * d.double().repeat_interleave(128, dim=1)
+    res = synth.normal_bf16((m, n), 1.0, seed=7, device="cuda")
+    one = torch.ones(n, dtype=torch.float64, device="cuda")
+    _within(binding.quasar_linear_w4(x, packed, d, out_f32=True), x, w, one)
+    _within(binding.quasar_linear_w4(x, packed, d, residual=res), x, w, one, res)
+
+
+@pytest.mark.parametrize("batch,rows,prefixes", [(50, 1, (0, 40)), (3, 2, (120, 300)), (1, 6, (900, 900)), (60, 3, (0, 260)), (5, 33, (100, 390))])
+def test_sequences_of_a_batch_attend_as_they_do_alone(batch, rows, prefixes):
+    """Segments of one key tile and of several, whole on one thread block or shared, more sequences than a block keeps the places
+    of: the first layer's attention, by the cache rows of the second and the logits, against each sequence in a batch of its own."""
+    shape, s_max = synth.SHAPES["tiny_qknorm"], 960
+    m = gpu_model(shape, seed=0, max_seq=s_max)
+    kk, vv = synth.kv_prefix(shape, batch, s_max, seed=5, device="cuda")
+    lens = torch.tensor([prefixes[0] + (prefixes[1] - prefixes[0]) * b // max(1, batch - 1) for b in range(batch)], dtype=torch.int32, device="cuda")
+    tokens = synth.uniform_tokens((batch, rows), shape.vocab, 5).to(torch.int32)
+
+    def run(which):
+        kv = binding.KVCache(shape, len(which), s_max, k=kk[:, which].contiguous().clone(), v=vv[:, which].contiguous().clone(), seq_len=lens[which].clone())
+        buf = binding.VerifyBuffers(m, len(which), rows)
+        buf.tokens.copy_(tokens[which])
+        binding.quasar_verify(m, kv, buf)
+        torch.cuda.synchronize()
+        assert int(buf.status[0]) == 0
+        return buf.logits, kv.k, kv.v
+
+    logits, kc, vc = run(list(range(batch)))
+    for b in list(range(0, batch, 7)) + [batch - 1]:
+        one, k1, v1 = run([b])
+        assert bool(((logits[b] - one[0]).abs() <= torch.clamp(1e-2 * one[0].abs(), min=2e-2)).all())
+        at = slice(int(lens[b]), int(lens[b]) + rows)
+        for got, want in ((kc[1, b, :, at], k1[1, 0, :, at]), (vc[1, b, :, at], v1[1, 0, :, at])):   # two roundings of bf16 apart at most, of the rms where small
+            floor = want.float().pow(2).mean().sqrt()
+            assert bool(((got.float() - want.float()).abs() <= 2.0 ** -6 * torch.maximum(want.float().abs(), floor)).all())
