@@ -22,7 +22,8 @@ __global__ void rope_table_kernel(float2* table, int max_pos, int D, double thet
   table[idx] = make_float2((float)c, (float)s);
 }
 
-// ---- QK-RMSNorm + RoPE + KV append (blocks too wide for the fused epilogue, traces): a warp per row and six neighbouring heads,
+// ---- QK-RMSNorm + RoPE + KV append (where the qkv projection does not finish its rows itself: traces, wide int8 blocks that run
+//      as one range, W8A8 and bf16 blocks of more than 128 rows): a warp per row and six neighbouring heads,
 //      whose vectors are asked for at once, beside what says where the row goes.  One head a warp was a chain of round trips for
 //      a kilobyte: 9.1 us at 512 rows of 48 heads. ----
 constexpr int kRopeHeads = 6;

@@ -60,10 +60,15 @@ struct WideArgs {
 };
 
 // What is done with a unit's finished sums: stored; multiplied as gate and up units; or made q, k and v (QK-norm, RoPE, cache
-// append: only behind ranges, whose exchange leaves whole rows of a head to a warp; a kernel and a pass over q, k and v less.  A pass
-// of 8 x 9 rows through the 8B shape 4104 -> 3953 us, of a 17-node tree x 4 through the 14B shape 5523 -> 5364; 8 x 64 rows 9681 -> 9638,
-// within the noise.  Tiles without ranges keep the separate kernel: eight rows a warp, one after the other, cost more than it does, 8 x 64
-// rows 9592 -> 9765)
+// append: only behind ranges, whose exchange leaves whole rows of a head to a warp; a kernel and a pass over q, k and v less).
+// A warp finishes its rows one after the other, so the gain shrinks with the rows, but the plan goes over to one range before it is
+// gone.  us a layer against the separate kernel (passes of 4 layers on 256 positions; rows a warp in brackets):
+//   rows                  65-72        96          128         176         208         224         240
+//   6144 x 4096           -2.7 (1.6)   -2.4 (2.2)  -3.0 (2.9)  -2.0 (4.0)  -1.4 (4.7)  -1.0 (5.1)  one range
+//   7168 x 5120           -3.1 (1.6)   -3.9 (2.2)  -2.7 (2.9)  -2.2 (4.0)  -1.2 (4.7)  -0.8 (5.1)  -0.8 (5.5)
+//   3072 x 2048, heads of 64: -0.6 at 72 rows, -1.7 at 128, -2.3 at 176 in four ranges; -1.1 at 192 to 224 in two row tiles of two
+// A pass of 8 x 9 rows through the 8B shape 4104 -> 3953 us, of a 17-node tree x 4 through the 14B shape 5523 -> 5364.  Tiles without
+// ranges keep the separate kernel: eight rows a warp cost more than it does (8 x 64 rows 9592 -> 9765).
 enum WideEpilogue { kWideStore = 0, kWideSwiglu = 1, kWideRope = 2 };
 
 // four int8 -> four bf16, exactly: 0x43bb is 128 + bb for the low seven bits, and the sign bit asks for 256 instead of 128 to go
