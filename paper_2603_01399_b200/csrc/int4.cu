@@ -247,9 +247,9 @@ int w4_clusters(int device, int s, int chunk, size_t smem) {
 template <int NT>
 int launch_w4_nt(W4Args a, cudaStream_t stream) {
   static DeviceOnce once;
-  const int rc = allow_shared_memory(once, 100 * 1024, false, {(const void*)w4_gemm_kernel<NT>});
+  int device = 0;
+  const int rc = allow_shared_memory(once, 100 * 1024, false, {(const void*)w4_gemm_kernel<NT>}, &device);
   if (rc != QUASAR_OK) return rc;
-  const int device = current_device();
   const int nblocks = (a.N + kW4BlockN - 1) / kW4BlockN, ngroups = a.K / kGroup;
   // Ranges: a launch takes the waves of clusters that the device holds at once - where they do not all fit, half a one more, as
   // CTAs follow one another - times the groups of a range and what a range costs besides, about three groups.  No range shorter

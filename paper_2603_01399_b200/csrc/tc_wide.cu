@@ -480,14 +480,14 @@ struct WidePlan {
   double cost;
 };
 
-int allow_wide() {
+int allow_wide(int* device) {
   static DeviceOnce once;
   return allow_shared_memory(once, kSmemW, true, {(const void*)tc_wide_kernel<false, kWideStore>, (const void*)tc_wide_kernel<true, kWideStore>,
-                                                  (const void*)tc_wide_kernel<false, kWideSwiglu>, (const void*)tc_wide_kernel<true, kWideRope>});
+                                                  (const void*)tc_wide_kernel<false, kWideSwiglu>, (const void*)tc_wide_kernel<true, kWideRope>}, device);
 }
 
-// Clusters of s pairs that the device holds at once (they lie within a group of SMs, so long ones leave SMs unused).  The kernels'
-// shared memory has to be allowed first.  Where the question fails this plan goes by one, and the next one asks again.
+// Clusters of s pairs that the device holds at once (they lie within a group of SMs, so long ones leave SMs unused).  Behind
+// allow_wide, without which it holds none.  Where the question fails this plan goes by one, and the next one asks again.
 int max_pair_clusters(int device, int s) {
   static DeviceAnswers<5> kept;
   return std::max(1, clusters_at_once(kept, device, s, (const void*)tc_wide_kernel<true, kWideStore>, kThreadsW, kSmemW, 2, (unsigned)s));
@@ -495,10 +495,8 @@ int max_pair_clusters(int device, int s) {
 
 // Row tiles and k-ranges by an estimate of the time in us.  A stage (128 of K) takes its MMAs (7.0e6 multiply-adds per us on an
 // SM), or its way into the SM, or 0.41 us of the hand-overs from load to conversion to MMA.
-WidePlan plan_wide(int64_t M, int64_t N, int64_t K, bool swiglu, bool keys) {
+WidePlan plan_wide(int device, int64_t M, int64_t N, int64_t K, bool swiglu, bool keys) {
   WidePlan best = {};
-  const int device = current_device();
-  const bool allowed = allow_wide() == QUASAR_OK;
   const int kblocks = (int)((K + 127) / 128);
   const int tiles = (int)((N + 255) / 256);
   const int least = (int)((M + 255) / 256);
@@ -529,7 +527,7 @@ WidePlan plan_wide(int64_t M, int64_t N, int64_t K, bool swiglu, bool keys) {
         p.cost = 4.0 + turns * (kblocks * a + (p.accs == 1 ? drain : 0.2)) + (p.accs == 2 ? drain : 0.0);
         p.ctas = 2 * n;
       } else {
-        const int fit = allowed ? max_pair_clusters(device, s) : 1;
+        const int fit = max_pair_clusters(device, s);
         const int waves = (units + fit - 1) / fit;
         p.cost = waves * (6.0 + (kblocks + s - 1) / s * a + 0.012 * p.brows) + 0.3 * s;
         p.ctas = 2 * units;
@@ -544,9 +542,9 @@ WidePlan plan_wide(int64_t M, int64_t N, int64_t K, bool swiglu, bool keys) {
 
 int launch_wide(int epi, const __nv_bfloat16* x, const int8_t* w, int64_t M, int64_t N, int64_t K, WideArgs a, bool pdl, cudaStream_t stream) {
   const bool swiglu = epi == kWideSwiglu;
-  int rc = allow_wide();
+  int device = 0, rc = allow_wide(&device);
   if (rc != QUASAR_OK) return rc;
-  const WidePlan p = plan_wide(M, N, K, swiglu, a.keys != nullptr);
+  const WidePlan p = plan_wide(device, M, N, K, swiglu, a.keys != nullptr);
   CUtensorMap map_w, map_x;
   rc = make_map_sw128(&map_w, w, (uint64_t)N, (uint64_t)K, swiglu ? 16u : 128u);
   if (rc != QUASAR_OK) return rc;
@@ -603,7 +601,10 @@ int launch_tc_wide_swiglu(const __nv_bfloat16* x, const int8_t* w, const float* 
   return launch_wide(kWideSwiglu, x, w, M, 2 * F, K, a, pdl, stream);
 }
 
-bool tc_wide_rope_fits(int64_t M, int64_t N, int64_t K) { return plan_wide(M, N, K, false, false).nsplit > 1; }
+bool tc_wide_rope_fits(int64_t M, int64_t N, int64_t K) {
+  int device = 0;
+  return allow_wide(&device) == QUASAR_OK && plan_wide(device, M, N, K, false, false).nsplit > 1;   // (a failure is the launch's to report)
+}
 
 int launch_tc_wide_qkv_rope(const __nv_bfloat16* x, const int8_t* w, const float* dw, int64_t M, int64_t K, const RopeArgs& rope, int32_t* error,
                             cudaStream_t stream) {
