@@ -12,7 +12,9 @@
 // i + 4, so the activations are staged in that order (0,4,1,5,2,6,3,7 within eight) and the operands of mma.m16n8k16 line
 // up without further moves; the contraction index may be permuted freely as long as both operands agree.  fp32
 // accumulation per group, folded into the running sum with the group's step size.  The ranges of a channel block form a
-// cluster and add their sums through distributed shared memory in the order of the ranges.
+// cluster and add their sums through distributed shared memory in the order of the ranges.  What bounds it (16 x 4096 x 12288,
+// 17.9 us): waiting for weights - a range of twelve groups asks for four at a time, one after the other; a scheduler has 3.5
+// warps and issues in 36 % of its cycles, the integer pipes are 29 % busy, the tensor pipe 14 %, the memory 17 %.
 #include <algorithm>
 
 #include "common.cuh"

@@ -1,10 +1,11 @@
 // Symmetric uniform quantisation of rows, one step size per row (Section 3.2 Eq. 6): offline weight preparation (Section
 // 3.3; plain, or of W / s for the W8A8 form, Eq. 4) and the online quantisation of activations X * s (Eq. 9).
 //
-// 2 B read + 1 B written per element and nothing else to pay for: every row stays in registers between its maximum and its
-// codes, 1 to 8 warps a row so that a lane holds up to 4 (12 on the longest rows) 16-byte pieces, all of them in flight at
-// once, and the quotients are rounded without a division (quant.cuh).  A CTA per row that read it twice and divided took
-// 88 us for 24,576 x 4096; the memory needs 47.
+// 2 B read + 1 B written per element: every row stays in registers between its maximum and its codes, 1 to 8 warps a row so
+// that a lane holds up to 4 (12 on the longest rows) 16-byte pieces, all of them in flight at once, and the quotients are
+// rounded without a division (quant.cuh).  What bounds it: issuing some 17 instructions an element, 71 % of the slots of the
+// whole launch, at half the warps an SM could hold (56 registers); the memory is half busy.  24,576 x 4096 takes 68 us, of which the
+// memory needs 47; a CTA per row that read it twice and divided took 88.
 #include "common.cuh"
 #include "quant.cuh"
 #include "tc_common.cuh"
