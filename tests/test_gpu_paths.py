@@ -236,8 +236,8 @@ def test_a_workspace_that_holds_some_of_the_rows(room):
 
 
 # rows: one, some, the most of the form and one more; channels: the narrowest tiles of the form (144), last ones that are cut (160,
-# 176), the widest (208); contraction: many turns of the ring, with a remainder; the last two sizes run in tiles of 128
-@pytest.mark.parametrize("hidden,ffn", [(4096, 9536), (3600, 11008), (4096, 12288), (4096, 15392), (256, 9536), (256, 12288)])
+# 176), wide ones (208, 256); contraction: many turns of the ring, with a remainder; the last two sizes run in tiles of 128
+@pytest.mark.parametrize("hidden,ffn", [(4096, 9536), (3600, 11008), (4096, 12288), (4096, 15392), (1024, 18944), (256, 9536), (256, 12288)])
 @pytest.mark.parametrize("batch,rows", [(1, 1), (1, 6), (2, 4), (3, 3)])
 def test_gateup_on_bf16_weights_in_one_wave_of_wide_tiles(batch, rows, hidden, ffn):
     """Two gate+up tiles on one thread block (SwiGLU in the epilogue; tests/test_forms_rule.py says which sizes run so) against the
